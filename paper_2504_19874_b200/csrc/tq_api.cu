@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "tq_attend_simt.cuh"
+#include "tq_dequant_tc.h"
 #include "tq_gemm_simt.cuh"
 #include "tq_internal.h"
 #include "tq_quantize_tc.h"
@@ -586,6 +587,7 @@ extern "C" int tq_plan_create(int d, int bits, int mode, const float* Pi, const 
       PLAN_CUDA(tc::build_matrix_limbs(p->dSp, d, d, p->dpad, p->tc_bn, &p->sp_limbs), "bf16 limbs of S'");
     p->tc_ok = 1;
   }
+  PLAN_CUDA(dq::plan_init(p, Pi, mode == TQ_PROD ? S : nullptr), "fp16 limbs of Pi^T and S^T");
   mscan::plan_init(p);
   nscan::plan_init(p);
   PLAN_CUDA(cudaDeviceSynchronize(), "synchronize");
@@ -603,6 +605,7 @@ extern "C" int tq_plan_destroy(tq_plan* plan) {
   cudaFree(plan->d_status);
   tc::free_matrix_limbs(&plan->pi_limbs);
   tc::free_matrix_limbs(&plan->sp_limbs);
+  dq::plan_free(plan);
   delete plan;
   return TQ_OK;
 }
@@ -830,6 +833,7 @@ extern "C" int tq_dequantize(const tq_plan* plan, int64_t n, const uint8_t* idx,
   TQ_REQUIRE(ldxh >= plan->d, TQ_ERR_INVALID_ARG, "%s: ldxh < d", who);
   TQ_REQUIRE(aligned(Xhat, 16), TQ_ERR_ALIGNMENT, "%s: Xhat is not 16-byte aligned", who);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (plan->dq.ok) return dq::dequantize(plan, n, idx, qjl, gamma, norms, Xhat, ldxh, st, who);
   const int ncols = plan->ncat * plan->dpad;
   simt::Codes A = make_codes(plan, n, idx, qjl, gamma);
   simt::RowsF32 B{plan->dBackT, ncols, plan->d, ncols};

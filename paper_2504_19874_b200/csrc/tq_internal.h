@@ -4,6 +4,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <nvtx3/nvToolsExt.h>
 
 #include <cstdarg>
@@ -108,6 +109,15 @@ struct tq_plan {
     uint32_t hi_a, hi_b, lo_a, lo_b;   // 16-bit centroid table t_i = 256 h_i + l_i as bytes: h of entries 0..3, 4..7, l alike
     double delta;                      // c_i ~ delta * t_i
   } nb;
+  // tensor-core reconstruction (d >= 128)
+  struct {
+    int ok;
+    int pitch;                         // row pitch of the limb matrices, elements
+    __half *p_hi, *p_lo, *s_hi, *s_lo; // fp16 limbs of Pi^T and S^T, scaled by powers of two
+    alignas(64) CUtensorMap map_p_hi, map_p_lo, map_s_hi, map_s_lo;
+    uint32_t tab[4][4];                // bytes of the codebook's limbs: hi low / high byte, lo low / high byte, 16 entries each
+    float gscale, oscale;              // weight of the sign term per unit of gamma; scale of the result
+  } dq;
   int* d_status;   // device word: set to TQ_ERR_TIMEOUT by a kernel whose bounded wait ran out
 };
 
