@@ -1,4 +1,5 @@
-"""ctypes binding of include/tq.h.  Argument marshalling only."""
+"""Python binding of include/tq.h.  Argument marshalling only: the calls a program makes again and again go through the
+extension module _tqbind (csrc/tq_bind.cpp), set-up and size queries through ctypes."""
 from __future__ import annotations
 
 import ctypes
@@ -18,6 +19,7 @@ TQ_STATIC_SCRATCH_BYTES = 1 << 20
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)),
                          "libtq_debug.so" if os.environ.get("TQ_LIB_VARIANT") == "debug" else "libtq.so")
 _lib = None
+_n = None        # the _tqbind module, bound to the loaded library
 
 c_void_p, c_int, c_int64, c_size_t, c_u64 = ctypes.c_void_p, ctypes.c_int, ctypes.c_int64, ctypes.c_size_t, ctypes.c_uint64
 _F = ctypes.POINTER(ctypes.c_float)
@@ -95,6 +97,21 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def _native():
+    """The marshalling module, bound to the library that lib() loads."""
+    global _n
+    if _n is None:
+        lib()
+        try:
+            from . import _tqbind
+        except ImportError as e:
+            raise RuntimeError("_tqbind.so is missing or does not load: run `python -m paper_2504_19874_b200.build` first "
+                               f"(there is no fallback path): {e}") from e
+        _tqbind.bind(_LIB_PATH)
+        _n = _tqbind
+    return _n
+
+
 def _check(code: int):
     if code != 0:
         raise TqError(code, lib().tq_last_error().decode())
@@ -111,20 +128,6 @@ def _dev(t):
     if not t.is_cuda:
         raise ValueError("expected a CUDA tensor (this library has no CPU path)")
     return t.data_ptr()
-
-
-def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return TQ_F32
-    if t.dtype == torch.bfloat16:
-        return TQ_BF16
-    raise ValueError(f"unsupported dtype {t.dtype}")
-
-
-def _rows(t: torch.Tensor):
-    if t.dim() != 2 or t.stride(1) != 1:
-        raise ValueError("expected a 2-D tensor with unit inner stride")
-    return t.shape[0], t.stride(0) if t.shape[0] > 1 else max(t.stride(0), t.shape[1])
 
 
 def _stream():
@@ -176,7 +179,7 @@ class Plan:
         h = c_void_p()
         _check(lib().tq_plan_create(d, bits, mode, _fptr(Pi), None if Sp is None else _fptr(Sp), _fptr(cent),
                                     ctypes.byref(h)))
-        self.handle = h
+        self.handle = h.value
 
     def set_layout(self, layout: int) -> None:
         """TQ_LAYOUT_CANONICAL or TQ_LAYOUT_NIBBLE (TQ_PROD with b = 4 only): arrangement of the code rows."""
@@ -212,41 +215,26 @@ def tq_workspace_bytes(plan: Plan, op: int, n: int, nq: int = 0, k: int = 0) -> 
     return lib().tq_workspace_bytes(plan.handle, op, n, nq, k)
 
 
-def _scratch_args(t):
-    return (_dev(t), 0 if t is None else t.numel() * t.element_size())
-
-
 def tq_quantize_mse(plan: Plan, X, idx, norms=None, scratch=None):
-    n, ldx = _rows(X)
-    _check(lib().tq_quantize_mse(plan.handle, _dev(X), _dtype_code(X), n, ldx, _dev(idx), _dev(norms),
-                                 *_scratch_args(scratch), _stream()))
+    _check((_n or _native()).quantize_mse(plan.handle, X, idx, norms, scratch))
 
 
 def tq_quantize_prod(plan: Plan, X, idx, qjl, gamma, norms=None, scratch=None):
-    n, ldx = _rows(X)
-    _check(lib().tq_quantize_prod(plan.handle, _dev(X), _dtype_code(X), n, ldx, _dev(idx), _dev(qjl), _dev(gamma),
-                                  _dev(norms), *_scratch_args(scratch), _stream()))
+    _check((_n or _native()).quantize_prod(plan.handle, X, idx, qjl, gamma, norms, scratch))
 
 
 def tq_dequantize(plan: Plan, n: int, idx, qjl, gamma, norms, Xhat):
-    _, ld = _rows(Xhat)
-    _check(lib().tq_dequantize(plan.handle, n, _dev(idx), _dev(qjl), _dev(gamma), _dev(norms), _dev(Xhat), ld, _stream()))
+    _check((_n or _native()).dequantize(plan.handle, n, idx, qjl, gamma, norms, Xhat))
 
 
 def tq_score(plan: Plan, Q, n: int, idx, qjl, gamma, norms, scores, workspace):
-    nq, ldq = _rows(Q)
-    _, lds = _rows(scores)
-    _check(lib().tq_score(plan.handle, _dev(Q), _dtype_code(Q), nq, ldq, n, _dev(idx), _dev(qjl), _dev(gamma),
-                          _dev(norms), _dev(scores), lds, *_scratch_args(workspace), _stream()))
+    _check((_n or _native()).score(plan.handle, Q, n, idx, qjl, gamma, norms, scores, workspace))
 
 
 def tq_score_static(plan: Plan, Q, n: int, idx, qjl, gamma, norms, scores):
     """tq_score for callers that cannot allocate device memory: the rotated-query workspace is an
     array built into the library (TQ_STATIC_SCRATCH_BYTES), shared by every call on the device."""
-    nq, ldq = _rows(Q)
-    _, lds = _rows(scores)
-    _check(lib().tq_score_static(plan.handle, _dev(Q), _dtype_code(Q), nq, ldq, n, _dev(idx), _dev(qjl), _dev(gamma),
-                                 _dev(norms), _dev(scores), lds, _stream()))
+    _check((_n or _native()).score_static(plan.handle, Q, n, idx, qjl, gamma, norms, scores))
 
 
 def tq_score_static_max_queries(plan: Plan) -> int:
@@ -259,14 +247,11 @@ def tq_query_bytes(plan: Plan, nq: int) -> int:
 
 def tq_query_prepare(plan: Plan, Q, prepared):
     """Query-side work of tq_score (rotations, scan operand) into `prepared` (>= tq_query_bytes(plan, nq) bytes)."""
-    nq, ldq = _rows(Q)
-    _check(lib().tq_query_prepare(plan.handle, _dev(Q), _dtype_code(Q), nq, ldq, *_scratch_args(prepared), _stream()))
+    _check((_n or _native()).query_prepare(plan.handle, Q, prepared))
 
 
 def tq_score_prepared(plan: Plan, prepared, nq: int, n: int, idx, qjl, gamma, norms, scores):
-    _, lds = _rows(scores)
-    _check(lib().tq_score_prepared(plan.handle, _dev(prepared), nq, n, _dev(idx), _dev(qjl), _dev(gamma), _dev(norms),
-                                   _dev(scores), lds, _stream()))
+    _check((_n or _native()).score_prepared(plan.handle, prepared, nq, n, idx, qjl, gamma, norms, scores))
 
 
 def tq_selftest_wait_timeout(plan: Plan, limit_cycles: int = 20000) -> None:
@@ -275,64 +260,32 @@ def tq_selftest_wait_timeout(plan: Plan, limit_cycles: int = 20000) -> None:
 
 
 def tq_topk(plan: Plan, Q, n: int, idx, qjl, gamma, norms, k: int, top_scores, top_ids, workspace):
-    nq, ldq = _rows(Q)
-    _check(lib().tq_topk(plan.handle, _dev(Q), _dtype_code(Q), nq, ldq, n, _dev(idx), _dev(qjl), _dev(gamma),
-                         _dev(norms), k, _dev(top_scores), _dev(top_ids), *_scratch_args(workspace), _stream()))
+    _check((_n or _native()).topk(plan.handle, Q, n, idx, qjl, gamma, norms, k, top_scores, top_ids, workspace))
 
 
 def tq_wsum(plan: Plan, W, n: int, idx, qjl, gamma, norms, out, workspace):
-    nw, ldo = _rows(out)
-    ldw = _rows(W)[1] if W is not None else n
-    _check(lib().tq_wsum(plan.handle, _dev(W), nw, ldw, n, _dev(idx), _dev(qjl), _dev(gamma), _dev(norms),
-                         _dev(out), ldo, *_scratch_args(workspace), _stream()))
+    _check((_n or _native()).wsum(plan.handle, W, n, idx, qjl, gamma, norms, out, workspace))
 
 
 def tq_softmax(s1, s2, scale: float, W):
-    nw, lds = _rows(s1)
-    _, ldw = _rows(W)
-    n = s1.shape[1]
-    if s2 is not None and (_rows(s2)[1] != lds or s2.shape != s1.shape):
-        raise ValueError("s2 must have the shape and row stride of s1")
-    _check(lib().tq_softmax(_dev(s1), _dev(s2), nw, n, lds, scale, _dev(W), ldw, _stream()))
+    _check((_n or _native()).softmax(s1, s2, scale, W))
 
 
 def tq_attend_decode_workspace_bytes(ngroups: int, heads: int, tokens: int, d: int) -> int:
     return lib().tq_attend_decode_workspace_bytes(ngroups, heads, tokens, d)
 
 
-def _kv_groups(groups):
-    arr = (KvGroup * len(groups))()
-    for dst, g in zip(arr, groups):
-        dst.plan_k, dst.plan_v = g["plan_k"].handle, g["plan_v"].handle
-        for name in ("k_idx", "k_qjl", "k_gamma", "k_norms", "v_idx", "v_norms", "k_channels", "v_channels"):
-            setattr(dst, name, _dev(g.get(name)))
-        for name in ("k_channels", "v_channels"):
-            if g[name].dtype != torch.int32 or not g[name].is_contiguous():
-                raise ValueError(f"{name} must be a contiguous int32 tensor")
-    return arr
-
-
 def tq_attend_decode(groups, heads: int, tokens: int, q_per_kv: int, Q, scale: float, out, workspace, head_stride=None):
     """groups: sequence of dicts with keys plan_k, plan_v (Plan) and k_idx, k_qjl, k_gamma, k_norms, v_idx,
     v_norms, k_channels, v_channels (CUDA tensors or None); rows of all heads head-major, head_stride rows
     per head (default: tokens)."""
-    arr = _kv_groups(groups)
-    _, ldq = _rows(Q)
-    _, ldo = _rows(out)
-    _check(lib().tq_attend_decode(ctypes.cast(arr, c_void_p), len(groups), heads, tokens,
-                                  tokens if head_stride is None else head_stride, q_per_kv, _dev(Q), _dtype_code(Q),
-                                  ldq, scale, _dev(out), ldo, *_scratch_args(workspace), _stream()))
+    _check((_n or _native()).attend_decode(groups, heads, tokens, tokens if head_stride is None else head_stride, q_per_kv, Q, scale,
+                                           out, workspace))
 
 
 def tq_kv_append(groups, heads: int, head_stride: int, position: int, K, V):
     """Quantises one new token per KV head (K, V: [heads, head_dim]) into row `position` of every head."""
-    arr = _kv_groups(groups)
-    _, ldk = _rows(K)
-    _, ldv = _rows(V)
-    if K.dtype != V.dtype:
-        raise ValueError("K and V must have one dtype")
-    _check(lib().tq_kv_append(ctypes.cast(arr, c_void_p), len(groups), heads, head_stride, position, _dev(K), _dev(V),
-                              _dtype_code(K), ldk, ldv, _stream()))
+    _check((_n or _native()).kv_append(groups, heads, head_stride, position, K, V))
 
 
 def tq_entropy_lengths(d: int, bits: int, centroids) -> np.ndarray:
@@ -346,26 +299,16 @@ def tq_entropy_lengths(d: int, bits: int, centroids) -> np.ndarray:
 def tq_entropy_pack(plan: Plan, lengths, n: int, idx):
     """(packed uint8 tensor, row_offsets int64 tensor of n + 1 byte offsets): the entropy-coded index rows."""
     ln = np.ascontiguousarray(lengths, dtype=np.uint8)
-    lp = ln.ctypes.data_as(c_void_p)
-    dev = idx.device
-    offsets = torch.empty(n + 1, dtype=torch.int64, device=dev)
-    ws = torch.empty(max(lib().tq_entropy_workspace_bytes(n), 256), dtype=torch.uint8, device=dev)
-    _check(lib().tq_entropy_measure(plan.handle, lp, n, _dev(idx), _dev(offsets), *_scratch_args(ws), _stream()))
-    total = int(offsets[n].item())
-    out = torch.empty(max(total, 4), dtype=torch.uint8, device=dev)
-    _check(lib().tq_entropy_pack(plan.handle, lp, n, _dev(idx), _dev(offsets), _dev(out), total, _stream()))
-    return out[:total], offsets
+    got = (_n or _native()).entropy_pack(plan.handle, ln.ctypes.data, n, idx)
+    if not isinstance(got, tuple):
+        _check(got)
+    return got
 
 
 def tq_entropy_unpack(plan: Plan, lengths, n: int, packed, offsets, idx_out):
     ln = np.ascontiguousarray(lengths, dtype=np.uint8)
-    _check(lib().tq_entropy_unpack(plan.handle, ln.ctypes.data_as(c_void_p), n, _dev(packed), _dev(offsets), _dev(idx_out),
-                                   _stream()))
+    _check((_n or _native()).entropy_unpack(plan.handle, ln.ctypes.data, n, packed, offsets, idx_out))
 
 
 def tq_select_topk(cand_scores, cand_ids, k: int, top_scores, top_ids):
-    nq, ld = _rows(cand_scores)
-    if _rows(cand_ids)[1] != ld or cand_ids.shape != cand_scores.shape:
-        raise ValueError("cand_ids must have the shape and row stride of cand_scores")
-    _check(lib().tq_select_topk(_dev(cand_scores), _dev(cand_ids), nq, cand_scores.shape[1], ld, k, _dev(top_scores),
-                                _dev(top_ids), _stream()))
+    _check((_n or _native()).select_topk(cand_scores, cand_ids, k, top_scores, top_ids))

@@ -1,15 +1,21 @@
-"""Builds libtq.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libtq.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _tqbind.so (the marshalling half of the
+Python binding) with the host compiler."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 LIB = os.path.join(PKG, "libtq.so")
 LIB_DEBUG = os.path.join(PKG, "libtq_debug.so")   # the same sources with -DTQ_DEBUG (device-side index checks)
+
+
+BIND = os.path.join(PKG, "_tqbind.so")
+BIND_SRC = os.path.join(PKG, "csrc", "tq_bind.cpp")
 
 
 def sources():
@@ -25,8 +31,25 @@ def _stale(lib: str = LIB) -> bool:
     return any(os.path.getmtime(p) > t for p in deps)
 
 
+def build_binding(force: bool = False) -> str:
+    header = os.path.join(ROOT, "include", "tq.h")
+    if not force and os.path.exists(BIND) and all(os.path.getmtime(p) <= os.path.getmtime(BIND) for p in (BIND_SRC, header)):
+        return BIND
+    import torch
+    torch_dir = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(ROOT, "include"), "-isystem", os.path.join(torch_dir, "include"),
+           "-isystem", os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"), "-isystem", os.path.join(cuda, "include"),
+           "-I", sysconfig.get_paths()["include"], BIND_SRC, "-o", BIND, "-L", os.path.join(torch_dir, "lib"),
+           "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-L", os.path.join(cuda, "lib64"), "-lcudart", "-ldl"]
+    subprocess.run(cmd, check=True)
+    return BIND
+
+
 def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
     lib = LIB_DEBUG if debug else LIB
+    build_binding(force)
     if not force and not _stale(lib):
         return lib
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
