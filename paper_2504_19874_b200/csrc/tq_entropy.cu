@@ -8,18 +8,21 @@
 // parallel.  Row stream: bit p is bit (p & 7) of byte (p >> 3); code words follow one another without gaps,
 // each written from its most significant bit; a row occupies a whole number of 32-bit words.
 //
-//   measure   one warp per row: lane l sums the code lengths of its chunk of coordinates; row bytes -> sizes
-//   offsets   exclusive prefix sum of the row sizes (one CTA walks the rows in pieces of 1024 with a carry)
-//   pack      one warp per row: warp scan of the lanes' bit counts gives every lane its bit offset; a lane
-//             shifts its code words into a 64-bit buffer and flushes whole words (the first and last word of
-//             a lane's chunk, shared with its neighbours, by atomic OR into the zeroed output)
-//   unpack    one thread per row: table look-up on the next maxlen bits gives (symbol, length)
+//   measure   one warp per row: eight coordinates become a word of nibbles, byte permutes look up four code lengths at a time
+//             and dp4a adds them; a CTA also leaves the total of its rows
+//   offsets   exclusive prefix sum of the row sizes: a CTA of 1024 rows adds up the CTA totals before it, then scans its own
+//   pack      one warp per row: code words are looked up two at a time, a lane joins the eight of its group, a warp scan of the
+//             lengths places them in a shared-memory image of the row (atomic OR), which leaves in one coalesced sweep
+//   unpack    one thread per row: a look-up on the next 10 (12) stream bits gives as many whole symbols as they hold
+// Bound by instruction issue, not by memory.  Measured at n = 100,000, d = 1536, b = 4 (76.8 MB of indices), before -> now:
+// measure 121 -> 33 us, offsets 83 (one CTA) -> 3, clearing the output 13 -> 0, pack 396 -> 112, unpack 471 -> 150.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
 
 #include "tq_internal.h"
+#include "tq_quantize_tc.h"
 
 namespace tq {
 namespace entropy {
@@ -33,6 +36,7 @@ struct Code {
   uint16_t word[16];   // canonical code word, most significant bit first
   int bits;            // b_m
   int maxlen;
+  uint32_t len4[4];    // the lengths again, four to a word
 };
 
 struct Args {
@@ -43,157 +47,336 @@ struct Args {
   Code code;
 };
 
-__device__ __forceinline__ int symbol_at(const uint8_t* row, int j, int bits) {
-  const int bp = j * bits, b0 = bp >> 3, sh = bp & 7;
-  unsigned v = row[b0];
-  if (sh + bits > 8) v |= (unsigned)row[b0 + 1] << 8;
-  return (v >> sh) & ((1u << bits) - 1u);
+__device__ __forceinline__ uint32_t spread3(uint32_t x) {   // eight 3-bit codes (low 24 bits) as nibbles
+  x = (x & 0x00000fffu) | ((x & 0x00fff000u) << 4);
+  x = (x & 0x003f003fu) | ((x & 0x0fc00fc0u) << 2);
+  return (x & 0x07070707u) | ((x & 0x38383838u) << 1);
+}
+__device__ __forceinline__ uint32_t spread2(uint32_t x) {
+  x = (x & 0x000000ffu) | ((x & 0x0000ff00u) << 8);
+  x = (x & 0x000f000fu) | ((x & 0x00f000f0u) << 4);
+  return (x & 0x03030303u) | ((x & 0x0c0c0c0cu) << 2);
+}
+__device__ __forceinline__ uint32_t spread1(uint32_t x) {
+  x = (x & 0x0fu) | ((x & 0xf0u) << 12);
+  x = (x & 0x00030003u) | ((x & 0x000c000cu) << 6);
+  return (x & 0x01010101u) | ((x & 0x02020202u) << 3);
 }
 
-// Row sizes in bytes (multiple of 4).
-__global__ void __launch_bounds__(256) measure_kernel(Args a, uint32_t* __restrict__ sizes) {
-  const int lane = threadIdx.x & 31;
-  const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (row >= a.n) return;
-  const uint8_t* r = a.idx + (size_t)row * a.idx_rb;
-  const int chunk = (a.d + 31) / 32;
-  int bits = 0;
-  for (int j = lane * chunk; j < min(a.d, (lane + 1) * chunk); ++j) bits += a.code.len[symbol_at(r, j, a.code.bits)];
+// Coordinates 8 g .. 8 g + 7 of a packed row as eight nibbles (row: 4-byte aligned, row_words words; whole groups of the row
+// lie inside it because its stride covers ceil(d BITS / 8) bytes rounded up to words).
+template <int BITS>
+__device__ __forceinline__ uint32_t nibbles(const uint32_t* __restrict__ row, int row_words, int g) {
+  if (BITS == 4) return __ldg(row + g);
+  const int bit = 8 * BITS * g, w = bit >> 5, sh = bit & 31;
+  const uint32_t x = __ldg(row + w);
+  if (BITS == 3) return spread3(__funnelshift_r(x, sh > 8 && w + 1 < row_words ? __ldg(row + w + 1) : 0u, sh) & 0x00ffffffu);
+  return BITS == 2 ? spread2((x >> sh) & 0xffffu) : spread1((x >> sh) & 0xffu);
+}
+
+// acc + the code lengths of the eight nibbles of x.
+template <int BITS>
+__device__ __forceinline__ uint32_t code_bits(const Code& c, uint32_t x, uint32_t acc) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) bits += __shfl_xor_sync(0xffffffffu, bits, o);
-  if (lane == 0) sizes[row] = (uint32_t)((bits + 31) / 32 * 4);
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t four = h ? x >> 16 : x;
+    uint32_t v = __byte_perm(c.len4[0], c.len4[1], BITS == 4 ? four & 0x7777u : four);
+    if (BITS == 4) {
+      const uint32_t up = __byte_perm(0x0000ff00u, 0u, (four >> 3) & 0x1111u);
+      v = (v & ~up) | (__byte_perm(c.len4[2], c.len4[3], four & 0x7777u) & up);
+    }
+    acc = __dp4a(v, 0x01010101u, acc);
+  }
+  return acc;
 }
 
-// offsets[i] = sum of sizes[0 .. i-1], offsets[n] = total.  One CTA of 1024 threads.
-__global__ void __launch_bounds__(1024) offsets_kernel(const uint32_t* __restrict__ sizes, int64_t n, uint64_t* __restrict__ offsets) {
-  __shared__ unsigned long long warp_tot[32];
-  __shared__ unsigned long long carry;
+// Row sizes in bytes (multiples of 4) and the total of each CTA's 8 R rows.
+template <int BITS>
+__global__ void __launch_bounds__(256) measure_kernel(Args a, int R, uint32_t* __restrict__ sizes, uint64_t* __restrict__ totals) {
+  __shared__ uint32_t warp_tot[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int groups = (a.d + 7) / 8, row_words = (int)(a.idx_rb / 4);
+  const int absent = 8 * groups - a.d;   // coordinates of the last group past the row's end: index 0 (pad bits are 0)
+  uint32_t tot = 0;
+  for (int r = 0; r < R; ++r) {
+    const int64_t row = ((int64_t)blockIdx.x * R + r) * 8 + warp;
+    if (row >= a.n) break;
+    const uint32_t* p = reinterpret_cast<const uint32_t*>(a.idx + (size_t)row * a.idx_rb);
+    uint32_t bits = 0;
+    for (int g0 = 0; g0 < groups; g0 += 256) {   // eight loads per lane in flight
+      uint32_t x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int g = g0 + 32 * i + lane;
+        x[i] = g < groups ? nibbles<BITS>(p, row_words, g) : 0u;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (g0 + 32 * i + lane < groups) bits = code_bits<BITS>(a.code, x[i], bits);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) bits += __shfl_xor_sync(0xffffffffu, bits, o);
+    bits -= (uint32_t)absent * a.code.len[0];
+    const uint32_t bytes = (bits + 31) / 32 * 4;
+    if (lane == 0) sizes[row] = bytes;
+    tot += bytes;
+  }
+  if (lane == 0) warp_tot[warp] = tot;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint64_t t = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += warp_tot[w];
+    totals[blockIdx.x] = t;
+  }
+}
+
+__device__ __forceinline__ unsigned long long warp_inclusive(unsigned long long v, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
+  }
+  return v;
+}
+
+// Exclusive prefix sums of `count` totals in place, by one CTA that walks them in pieces of 1024 with a carry: only for so
+// many rows that every CTA of offsets_kernel adding up its predecessors' totals would cost more (see tq_entropy_measure).
+__global__ void __launch_bounds__(1024) prefix_totals_kernel(uint64_t* __restrict__ totals, int64_t count) {
+  __shared__ unsigned long long warp_tot[32], carry;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) carry = 0ull;
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int64_t base = 0; base < n; base += 1024) {
+  for (int64_t base = 0; base < count; base += 1024) {
     const int64_t i = base + threadIdx.x;
-    const unsigned long long v = i < n ? sizes[i] : 0ull;
-    unsigned long long incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
+    const unsigned long long v = i < count ? totals[i] : 0ull, incl = warp_inclusive(v, lane);
     if (lane == 31) warp_tot[warp] = incl;
     __syncthreads();
     if (warp == 0) {
-      unsigned long long w = warp_tot[lane], wi = w;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long t = __shfl_up_sync(0xffffffffu, wi, o);
-        if (lane >= o) wi += t;
-      }
-      warp_tot[lane] = wi - w;   // exclusive
+      const unsigned long long w = warp_tot[lane];
+      warp_tot[lane] = warp_inclusive(w, lane) - w;
     }
     __syncthreads();
     const unsigned long long excl = carry + warp_tot[warp] + incl - v;
-    if (i < n) offsets[i] = excl;
+    if (i < count) totals[i] = excl;
     __syncthreads();
     if (threadIdx.x == 1023) carry = excl + v;
     __syncthreads();
   }
-  if (threadIdx.x == 0) offsets[n] = carry;
 }
 
-__global__ void __launch_bounds__(256) pack_kernel(Args a, const uint64_t* __restrict__ offsets, uint8_t* __restrict__ out,
-                                                   size_t out_bytes, int* status) {
-  const int lane = threadIdx.x & 31;
-  const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (row >= a.n) return;
-  if (offsets[row + 1] > out_bytes) {   // the caller's buffer is smaller than the measured total
-    if (lane == 0) atomicExch(status, TQ_ERR_WORKSPACE);
-    return;
-  }
-  const uint8_t* r = a.idx + (size_t)row * a.idx_rb;
-  uint32_t* dst = reinterpret_cast<uint32_t*>(out + offsets[row]);
-  const int chunk = (a.d + 31) / 32;
-  const int j0 = lane * chunk, j1 = min(a.d, (lane + 1) * chunk);
-  int bits = 0;
-  for (int j = j0; j < j1; ++j) bits += a.code.len[symbol_at(r, j, a.code.bits)];
-  int incl = bits;
+// offsets[i] = sum of sizes[0 .. i-1], offsets[n] = total; a CTA of 1024 threads takes 1024 rows.  totals[g]: bytes of rows
+// [g rows_per_total, (g + 1) rows_per_total), or with `prefixed` the bytes before that group.
+__global__ void __launch_bounds__(1024) offsets_kernel(const uint32_t* __restrict__ sizes, const uint64_t* __restrict__ totals,
+                                                       int rows_per_total, int prefixed, int64_t n, uint64_t* __restrict__ offsets) {
+  __shared__ unsigned long long warp_tot[32], before[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t base = (int64_t)blockIdx.x * 1024, first = base / rows_per_total;   // rows_per_total divides 1024
+  unsigned long long b = 0ull;
+  if (!prefixed)
+    for (int64_t g = threadIdx.x; g < first; g += 1024) b += totals[g];
+  else if (threadIdx.x == 0 && base < n) b = totals[first];
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
+  for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+  const int64_t i = base + threadIdx.x;
+  const unsigned long long v = i < n ? sizes[i] : 0ull, incl = warp_inclusive(v, lane);
+  if (lane == 0) before[warp] = b;
+  if (lane == 31) warp_tot[warp] = incl;
+  __syncthreads();
+  if (warp == 0) {
+    const unsigned long long w = warp_tot[lane];
+    unsigned long long s = before[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    warp_tot[lane] = s + warp_inclusive(w, lane) - w;
   }
-  const int start = incl - bits, end = incl;   // this lane's bits occupy [start, end) of the row stream
-  if (bits == 0) return;
-  int word = start >> 5, fill = start & 31;    // current output word and the bits of it already in `buf`
-  unsigned long long buf = 0ull;
-  const int first_word = word, last_word = (end - 1) >> 5;
-  auto flush = [&](uint32_t v) {
-    // words shared with a neighbouring lane: the first of the chunk (unless it starts on a word boundary) and the last
-    // (unless it ends on one); the output was zeroed, so OR composes them
-    if ((word == first_word && (start & 31)) || (word == last_word && (end & 31))) atomicOr(dst + word, v);
-    else dst[word] = v;
-    ++word;
-  };
-  for (int j = j0; j < j1; ++j) {
-    const int s = symbol_at(r, j, a.code.bits);
-    const int l = a.code.len[s];
-    // the code word from its most significant bit = stream order: reverse its l bits into LSB-first order
-    const unsigned rev = __brev((unsigned)a.code.word[s]) >> (32 - l);
-    buf |= (unsigned long long)rev << fill;
-    fill += l;
-    if (fill >= 32) {
-      flush((uint32_t)buf);
-      buf >>= 32;
-      fill -= 32;
-    }
+  __syncthreads();
+  if (i < n) {
+    const unsigned long long excl = warp_tot[warp] + incl - v;
+    offsets[i] = excl;
+    if (i == n - 1) offsets[n] = excl + v;
   }
-  if (fill > 0) flush((uint32_t)buf);
+  if (n == 0 && i == 0) offsets[0] = 0ull;
 }
 
-__global__ void __launch_bounds__(128) unpack_kernel(Args a, const uint64_t* __restrict__ offsets, const uint8_t* __restrict__ packed,
-                                                     uint8_t* __restrict__ idx_out) {
-  __shared__ uint16_t lut[1 << kMaxLen];   // next maxlen stream bits (LSB first) -> symbol | length << 8
-  const int L = a.code.maxlen;
-  for (int u = threadIdx.x; u < (1 << L); u += blockDim.x) {
-    uint16_t e = 0;
-    for (int s = 0; s < (1 << a.code.bits); ++s) {
-      const int l = a.code.len[s];
-      if (l == 0) continue;
-      const unsigned rev = __brev((unsigned)a.code.word[s]) >> (32 - l);
-      if ((u & ((1u << l) - 1u)) == rev) e = (uint16_t)(s | (l << 8));
+// Persistent over rows.  Shared memory: 256 pairs of code words x 32 copies (no two lanes meet in a bank), then one row image
+// per warp.  A pair entry holds the two code words in stream order (up to 24 bits) and their length above.  A lane takes every
+// 32nd group of eight coordinates; a warp scan of the groups' lengths places them.  Everything is straight-line code: a version
+// that appended to a 64-bit buffer and flushed it word by word took 1,560 instructions per row of 1536 coordinates, because
+// some lane flushed at every step.
+constexpr int kPackWarps = 8;
+template <int BITS, bool LONG>   // LONG: eight code words may take more than 64 bits (a code word of more than 8)
+__global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(Args a, const uint64_t* __restrict__ offsets, uint8_t* __restrict__ out,
+                                                               size_t out_bytes, int image_words, int* status) {
+  extern __shared__ uint32_t pack_smem[];
+  uint32_t* pairs = pack_smem;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t* image = pack_smem + 256 * 32 + warp * (image_words + 4);
+  for (int e = warp; e < 256; e += kPackWarps) {
+    const int s0 = e & 15, s1 = e >> 4;
+    const int l0 = a.code.len[s0], l1 = a.code.len[s1];
+    // a code word from its most significant bit = stream order: its bits reversed into LSB-first order
+    const uint32_t r0 = l0 ? __brev((uint32_t)a.code.word[s0]) >> (32 - l0) : 0u, r1 = l1 ? __brev((uint32_t)a.code.word[s1]) >> (32 - l1) : 0u;
+    pairs[e * 32 + lane] = r0 | (r1 << l0) | ((uint32_t)(l0 + l1) << 24);
+  }
+  __syncthreads();
+  const uint32_t* mine = pairs + lane;
+  const int groups = (a.d + 7) / 8, row_words = (int)(a.idx_rb / 4);
+  for (int64_t row = (int64_t)blockIdx.x * kPackWarps + warp; row < a.n; row += (int64_t)gridDim.x * kPackWarps) {
+    const uint64_t off = offsets[row], off_end = offsets[row + 1];
+    if (off_end > out_bytes) {   // the caller's buffer is smaller than the measured total
+      if (lane == 0) atomicExch(status, TQ_ERR_WORKSPACE);
+      continue;
     }
-    lut[u] = e;
+    const int words = min((int)((off_end - off) / 4), image_words);
+    const uint32_t* p = reinterpret_cast<const uint32_t*>(a.idx + (size_t)row * a.idx_rb);
+    for (int w = lane; w < words; w += 32) image[w] = 0u;
+    __syncwarp();
+    int base = 0;   // stream bits before this sweep's groups
+    uint32_t next = lane < groups ? nibbles<BITS>(p, row_words, lane) : 0u;
+    for (int g0 = 0; g0 < groups; g0 += 32) {
+      const int g = g0 + lane;
+      const uint32_t x = next;
+      if (g + 32 < groups) next = nibbles<BITS>(p, row_words, g + 32);   // requested one sweep ahead
+      unsigned long long half[2];   // four code words each, at most 48 bits
+      int len[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t e0 = mine[((x >> (16 * h)) & 255u) * 32], e1 = mine[((x >> (16 * h + 8)) & 255u) * 32];
+        if (8 * (g0 + 32) > a.d) {   // the last sweep: coordinates past the row's end have no code word
+          const int left = a.d - 8 * g - 4 * h;
+          const uint32_t four = x >> (16 * h);
+          if (left < 4) {
+            if (left <= 0) e0 = 0u;
+            else if (left == 1) { const uint32_t l = a.code.len[four & 15u]; e0 = (e0 & ((1u << l) - 1u)) | (l << 24); }
+            if (left <= 2) e1 = 0u;
+            else { const uint32_t l = a.code.len[(four >> 8) & 15u]; e1 = (e1 & ((1u << l) - 1u)) | (l << 24); }
+          }
+        }
+        const int l0 = (int)(e0 >> 24);
+        half[h] = (unsigned long long)(e0 & 0x00ffffffu) | ((unsigned long long)(e1 & 0x00ffffffu) << l0);
+        len[h] = l0 + (int)(e1 >> 24);
+      }
+      const int mine_bits = len[0] + len[1];
+      int incl = mine_bits;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      int pos = base + incl - mine_bits;
+      base += __shfl_sync(0xffffffffu, incl, 31);
+      // up to 64 bits shifted by up to 31: two words, rarely a third (the image has room for zero parts past its end)
+      auto place = [&](unsigned long long v) {
+        const int w = pos >> 5, sh = pos & 31;
+        const unsigned long long lo = v << sh;
+        atomicOr(image + w, (uint32_t)lo);
+        atomicOr(image + w + 1, (uint32_t)(lo >> 32));
+        const uint32_t v2 = __funnelshift_l((uint32_t)(v >> 32), 0u, sh);
+        if (v2) atomicOr(image + w + 2, v2);
+      };
+      if (LONG) {
+        place(half[0]);
+        pos += len[0];
+        place(half[1]);
+      } else {
+        place(half[0] | (half[1] << len[0]));
+      }
+    }
+    __syncwarp();
+    uint32_t* dst = reinterpret_cast<uint32_t*>(out + off);
+    for (int w = lane; w < words; w += 32) dst[w] = image[w];
+    __syncwarp();
+  }
+}
+
+// One thread per row.  Look-up on the next K = 10 bits (12 where a code word is longer than 10; always 12 measured 322 us: the
+// larger table takes L1 away from the rows' lines): up to 16 bits of whole
+// symbols, their number of output bits and the stream bits they take.  The lanes of a warp run in step by output word, so that
+// filling and emitting words is the same instruction for all of them; only the number of look-ups per word differs.
+constexpr int kUnpackThreads = 128;
+__global__ void __launch_bounds__(kUnpackThreads) unpack_kernel(Args a, int K, const uint64_t* __restrict__ offsets,
+                                                                const uint8_t* __restrict__ packed, uint8_t* __restrict__ idx_out) {
+  extern __shared__ uint32_t unpack_smem[];
+  uint32_t* lut = unpack_smem;                                            // [2^K]: symbols | output bits << 16 | stream bits << 24
+  uint16_t* single = reinterpret_cast<uint16_t*>(unpack_smem + (1 << K)); // [2^maxlen]: symbol | length << 8
+  const int L = a.code.maxlen, bits = a.code.bits;
+  for (int u = threadIdx.x; u < (1 << L); u += blockDim.x) {
+    uint16_t e = 1 << 8;   // no code word (an incomplete code): one bit, symbol 0
+    for (int s = 0; s < (1 << bits); ++s) {
+      const int l = a.code.len[s];
+      if ((u & ((1u << l) - 1u)) == __brev((unsigned)a.code.word[s]) >> (32 - l)) e = (uint16_t)(s | (l << 8));
+    }
+    single[u] = e;
+  }
+  __syncthreads();
+  for (int u = threadIdx.x; u < (1 << K); u += blockDim.x) {
+    uint32_t sym = 0u;
+    int used = 0, produced = 0;
+    while (produced + bits <= 16) {
+      const uint16_t e = single[(u >> used) & ((1u << L) - 1u)];
+      const int l = e >> 8;
+      if (used + l > K) break;   // the word may go on past the look-up window
+      sym |= (uint32_t)(e & 255u) << produced;
+      used += l;
+      produced += bits;
+    }
+    lut[u] = sym | ((uint32_t)produced << 16) | ((uint32_t)used << 24);
   }
   __syncthreads();
   const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= a.n) return;
-  const uint32_t* src = reinterpret_cast<const uint32_t*>(packed + offsets[row]);
-  const int nwords = (int)((offsets[row + 1] - offsets[row]) / 4);
+  const uint64_t off = offsets[row];
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(packed + off);
+  const int nwords = (int)((offsets[row + 1] - off) / 4);
   uint32_t* dst = reinterpret_cast<uint32_t*>(idx_out + (size_t)row * a.idx_rb);
-  const int row_words = (int)(a.idx_rb / 4);
+  const int row_words = (int)(a.idx_rb / 4), total_bits = a.d * bits, out_words = (total_bits + 31) / 32;
+  const uint32_t last_mask = (total_bits & 31) ? (1u << (total_bits & 31)) - 1u : 0xffffffffu;
+  // The stream window is filled at the start of every output word by all lanes together, and only rarely inside a word: a
+  // load that some lane issues at every look-up makes the other lanes of the warp wait for it (267 against 150 us).
   unsigned long long in = 0ull, outbuf = 0ull;
-  int have = 0, rd = 0, ofill = 0, ow = 0;
-  const unsigned mask = (1u << L) - 1u;
-  for (int j = 0; j < a.d; ++j) {
-    if (have < L) {   // a zero word past the end of the row stream only pads the look-up of the last code words
-      in |= (unsigned long long)(rd < nwords ? src[rd] : 0u) << have;
-      ++rd;
-      have += 32;
-    }
-    const uint16_t e = lut[(unsigned)in & mask];
-    const int l = e >> 8;
-    in >>= l;
-    have -= l;
-    outbuf |= (unsigned long long)(e & 255u) << ofill;
-    ofill += a.code.bits;
-    if (ofill >= 32) {
-      dst[ow++] = (uint32_t)outbuf;
-      outbuf >>= 32;
-      ofill -= 32;
+  int have = 0, rd = 0, ofill = 0;
+  const unsigned mask = (1u << K) - 1u;
+  uint32_t ahead = nwords > 0 ? __ldg(src) : 0u;   // the next word, requested one word early
+  auto refill = [&]() {   // zero words past the end of the row stream only pad the look-up of its last code words
+    in |= (unsigned long long)ahead << have;
+    have += 32;
+    ++rd;
+    ahead = rd < nwords ? __ldg(src + rd) : 0u;
+  };
+  auto next_word = [&]() -> uint32_t {
+    if (have < 32) refill();
+    do {
+      if (have < K) refill();
+      const uint32_t e = lut[(unsigned)in & mask];
+      const int used = e >> 24;
+      in >>= used;
+      have -= used;
+      outbuf |= (unsigned long long)(e & 0xffffu) << ofill;
+      ofill += (e >> 16) & 255u;
+    } while (ofill < 32);
+    const uint32_t v = (uint32_t)outbuf;
+    outbuf >>= 32;
+    ofill -= 32;
+    return v;
+  };
+  auto checked_word = [&](int ow) -> uint32_t {
+    if (ow >= out_words) return 0u;   // pad words of the row
+    const uint32_t v = next_word();
+    return ow == out_words - 1 ? v & last_mask : v;   // what follows the last coordinate is not a symbol
+  };
+  int ow = 0;
+  if (row_words % 4 == 0) {
+    for (; ow + 4 <= total_bits / 32; ow += 4) {
+      uint4 v;
+      v.x = next_word();
+      v.y = next_word();
+      v.z = next_word();
+      v.w = next_word();
+      *reinterpret_cast<uint4*>(dst + ow) = v;
     }
   }
-  if (ofill > 0) dst[ow++] = (uint32_t)outbuf;
-  for (; ow < row_words; ++ow) dst[ow] = 0u;   // pad words of the row
+  for (; ow < row_words; ++ow) dst[ow] = checked_word(ow);
 }
 
 int make_code(const tq_plan* plan, const uint8_t* lengths, Code* c, const char* who) {
@@ -206,6 +389,7 @@ int make_code(const tq_plan* plan, const uint8_t* lengths, Code* c, const char* 
     TQ_REQUIRE(lengths[s] >= 1 && lengths[s] <= kMaxLen, TQ_ERR_UNSUPPORTED, "%s: code length %d of symbol %d outside 1..%d", who,
                (int)lengths[s], s, kMaxLen);
     c->len[s] = lengths[s];
+    c->len4[s >> 2] |= (uint32_t)lengths[s] << (8 * (s & 3));
     c->maxlen = std::max(c->maxlen, (int)lengths[s]);
     kraft += std::ldexp(1.0, -(int)lengths[s]);
     order.push_back({(int)lengths[s], s});
@@ -270,7 +454,11 @@ extern "C" int tq_entropy_lengths(int d, int bits, const float* centroids, uint8
   return TQ_OK;
 }
 
-extern "C" size_t tq_entropy_workspace_bytes(int64_t n) { return n > 0 ? (size_t)((n * 4 + 255) / 256 * 256) : 0; }
+// Row sizes (4 bytes each), then the totals of groups of at least eight rows (8 bytes each).
+static size_t sizes_bytes(int64_t n) { return (size_t)((n * 4 + 255) / 256 * 256); }
+extern "C" size_t tq_entropy_workspace_bytes(int64_t n) {
+  return n > 0 ? sizes_bytes(n) + (size_t)(((n + 7) / 8 * 8 + 255) / 256 * 256) : 0;
+}
 
 extern "C" int tq_entropy_measure(const tq_plan* plan, const uint8_t* lengths, int64_t n, const uint8_t* idx, uint64_t* row_offsets,
                                   void* workspace, size_t workspace_bytes, void* stream) {
@@ -286,12 +474,28 @@ extern "C" int tq_entropy_measure(const tq_plan* plan, const uint8_t* lengths, i
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   a.n = n; a.d = plan->d; a.idx = idx; a.idx_rb = plan->idx_row_bytes;
   uint32_t* sizes = static_cast<uint32_t*>(workspace);
+  uint64_t* totals = reinterpret_cast<uint64_t*>(static_cast<char*>(workspace) + sizes_bytes(n));
+  // eight rows per warp once that still fills the chip four times over
+  const int R = n >= 8 * 8 * 4 * 148 ? 8 : 1;
+  const int64_t groups = (n + 8 * R - 1) / (8 * R);
+  // CTA j of offsets_kernel adds up the j 1024 / (8 R) totals before it: 2^21 rows make 2,048 CTAs read 16,384 totals on
+  // average (0.27 GB from L2); from there on one launch turns the totals into prefix sums first
+  const int prefixed = n > ((int64_t)1 << 21) ? 1 : 0;
   if (n > 0) {
-    entropy::measure_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(a, sizes);
+    switch (a.code.bits) {
+      case 1: entropy::measure_kernel<1><<<(unsigned)groups, 256, 0, st>>>(a, R, sizes, totals); break;
+      case 2: entropy::measure_kernel<2><<<(unsigned)groups, 256, 0, st>>>(a, R, sizes, totals); break;
+      case 3: entropy::measure_kernel<3><<<(unsigned)groups, 256, 0, st>>>(a, R, sizes, totals); break;
+      default: entropy::measure_kernel<4><<<(unsigned)groups, 256, 0, st>>>(a, R, sizes, totals); break;
+    }
     TQ_CHECK_CUDA(cudaGetLastError(), who);
+    if (prefixed) {
+      entropy::prefix_totals_kernel<<<1, 1024, 0, st>>>(totals, groups);
+      TQ_CHECK_CUDA(cudaGetLastError(), who);
+    }
   }
-  entropy::offsets_kernel<<<1, 1024, 0, st>>>(sizes, n, row_offsets);
-  count_launches(n > 0 ? 2 : 1);
+  entropy::offsets_kernel<<<(unsigned)std::max<int64_t>(1, (n + 1023) / 1024), 1024, 0, st>>>(sizes, totals, 8 * R, prefixed, n, row_offsets);
+  count_launches(n > 0 ? 2 + prefixed : 1);
   TQ_CHECK_CUDA(cudaGetLastError(), who);
   return TQ_OK;
 }
@@ -309,8 +513,17 @@ extern "C" int tq_entropy_pack(const tq_plan* plan, const uint8_t* lengths, int6
   if ((rc = entropy::make_code(plan, lengths, &a.code, who))) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   a.n = n; a.d = plan->d; a.idx = idx; a.idx_rb = plan->idx_row_bytes;
-  TQ_CHECK_CUDA(cudaMemsetAsync(out, 0, out_bytes, st), who);
-  entropy::pack_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(a, row_offsets, out, out_bytes, plan->d_status);
+  const int image_words = (int)(((int64_t)a.d * a.code.maxlen + 31) / 32);   // the longest row stream
+  const size_t smem = (256 * 32 + (size_t)entropy::kPackWarps * (image_words + 4)) * sizeof(uint32_t);
+  const int per_sm = std::max(1, std::min(8, (int)(228 * 1024 / (smem + 1024))));
+  const int64_t ctas = std::min<int64_t>((n + entropy::kPackWarps - 1) / entropy::kPackWarps, (int64_t)tc::sm_count() * per_sm);
+  const bool wide = a.code.maxlen > 8;
+  const auto kernel = a.code.bits == 1   ? (wide ? entropy::pack_kernel<1, true> : entropy::pack_kernel<1, false>)
+                      : a.code.bits == 2 ? (wide ? entropy::pack_kernel<2, true> : entropy::pack_kernel<2, false>)
+                      : a.code.bits == 3 ? (wide ? entropy::pack_kernel<3, true> : entropy::pack_kernel<3, false>)
+                                         : (wide ? entropy::pack_kernel<4, true> : entropy::pack_kernel<4, false>);
+  if (smem > 48 * 1024) TQ_CHECK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), who);
+  kernel<<<(unsigned)ctas, 32 * entropy::kPackWarps, smem, st>>>(a, row_offsets, out, out_bytes, image_words, plan->d_status);
   count_launches(1);
   TQ_CHECK_CUDA(cudaGetLastError(), who);
   return TQ_OK;
@@ -329,7 +542,10 @@ extern "C" int tq_entropy_unpack(const tq_plan* plan, const uint8_t* lengths, in
   entropy::Args a;
   if ((rc = entropy::make_code(plan, lengths, &a.code, who))) return rc;
   a.n = n; a.d = plan->d; a.idx = nullptr; a.idx_rb = plan->idx_row_bytes;
-  entropy::unpack_kernel<<<(unsigned)((n + 127) / 128), 128, 0, static_cast<cudaStream_t>(stream)>>>(a, row_offsets, packed, idx);
+  const int K = a.code.maxlen <= 10 ? 10 : 12;
+  const size_t smem = sizeof(uint32_t) * ((size_t)1 << K) + sizeof(uint16_t) * ((size_t)1 << a.code.maxlen);   // at most 24 KB
+  const int64_t ctas = (n + entropy::kUnpackThreads - 1) / entropy::kUnpackThreads;
+  entropy::unpack_kernel<<<(unsigned)ctas, entropy::kUnpackThreads, smem, static_cast<cudaStream_t>(stream)>>>(a, K, row_offsets, packed, idx);
   count_launches(1);
   TQ_CHECK_CUDA(cudaGetLastError(), who);
   return TQ_OK;
