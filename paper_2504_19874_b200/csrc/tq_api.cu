@@ -10,6 +10,7 @@
 #include "tq_dequant_tc.h"
 #include "tq_gemm_simt.cuh"
 #include "tq_internal.h"
+#include "tq_quantize_small.h"
 #include "tq_quantize_tc.h"
 #include "tq_scan_mma.h"
 #include "tq_scan_nib.h"
@@ -587,6 +588,7 @@ extern "C" int tq_plan_create(int d, int bits, int mode, const float* Pi, const 
       PLAN_CUDA(tc::build_matrix_limbs(p->dSp, d, d, p->dpad, p->tc_bn, &p->sp_limbs), "bf16 limbs of S'");
     p->tc_ok = 1;
   }
+  PLAN_CUDA(sq::plan_init(p), "fp16 limb images of Pi and S'");
   PLAN_CUDA(dq::plan_init(p, Pi, mode == TQ_PROD ? S : nullptr), "fp16 limbs of Pi^T and S^T");
   mscan::plan_init(p);
   nscan::plan_init(p);
@@ -606,6 +608,7 @@ extern "C" int tq_plan_destroy(tq_plan* plan) {
   tc::free_matrix_limbs(&plan->pi_limbs);
   tc::free_matrix_limbs(&plan->sp_limbs);
   dq::plan_free(plan);
+  sq::plan_free(plan);
   delete plan;
   return TQ_OK;
 }
@@ -747,8 +750,10 @@ extern "C" int tq_quantize_mse(const tq_plan* plan, const void* X, int x_dtype, 
     TQ_REQUIRE(scratch != nullptr && scratch_bytes >= need, TQ_ERR_WORKSPACE, "%s: scratch of %zu bytes, at least %zu needed",
                who, scratch_bytes, need);
     TQ_REQUIRE(aligned(scratch, 256), TQ_ERR_ALIGNMENT, "%s: scratch is not 256-byte aligned", who);
+    if (sq::preferred(plan, x_dtype, n)) return sq::quantize(plan, X, x_dtype, n, ldx, idx, nullptr, nullptr, norms, st, who);
     return tc::quantize(plan, X, x_dtype, n, ldx, idx, nullptr, nullptr, norms, scratch, scratch_bytes, st, who);
   }
+  if (plan->sq.ok) return sq::quantize(plan, X, x_dtype, n, ldx, idx, nullptr, nullptr, norms, st, who);
   if (norms) TQ_CHECK_CUDA(compute_norms(X, x_dtype, n, ldx, plan->d, norms, st), who);
   if (has_pad_words(plan->d, plan->mse_bits, plan->idx_row_bytes))
     TQ_CHECK_CUDA(cudaMemsetAsync(idx, 0, (size_t)n * plan->idx_row_bytes, st), who);
@@ -775,6 +780,8 @@ extern "C" int tq_quantize_prod(const tq_plan* plan, const void* X, int x_dtype,
     TQ_REQUIRE(scratch != nullptr && scratch_bytes >= least, TQ_ERR_WORKSPACE,
                "%s: scratch of %zu bytes, at least %zu needed", who, scratch_bytes, least);
     TQ_REQUIRE(aligned(scratch, 256), TQ_ERR_ALIGNMENT, "%s: scratch is not 256-byte aligned", who);
+    if (sq::preferred(plan, x_dtype, n))
+      return sq::quantize(plan, X, x_dtype, n, ldx, idx, qjl, gamma, norms, st, who);
     // (the GEMM epilogues write whichever layout the plan has)
     return tc::quantize(plan, X, x_dtype, n, ldx, idx, qjl, gamma, norms, scratch, scratch_bytes, st, who);
   }
@@ -782,6 +789,7 @@ extern "C" int tq_quantize_prod(const tq_plan* plan, const void* X, int x_dtype,
   TQ_REQUIRE(scratch != nullptr && scratch_bytes >= need, TQ_ERR_WORKSPACE, "%s: scratch of %zu bytes, %zu needed", who,
              scratch_bytes, need);
   TQ_REQUIRE(aligned(scratch, 16), TQ_ERR_ALIGNMENT, "%s: scratch is not 16-byte aligned", who);
+  if (plan->sq.ok) return sq::quantize(plan, X, x_dtype, n, ldx, idx, qjl, gamma, norms, st, who);
   const int d = plan->d;
   const int64_t ldE = plan->dpad;
   float* E = static_cast<float*>(scratch);
