@@ -588,7 +588,7 @@ extern "C" int tq_plan_create(int d, int bits, int mode, const float* Pi, const 
       PLAN_CUDA(tc::build_matrix_limbs(p->dSp, d, d, p->dpad, p->tc_bn, &p->sp_limbs), "bf16 limbs of S'");
     p->tc_ok = 1;
   }
-  PLAN_CUDA(sq::plan_init(p), "fp16 limb images of Pi and S'");
+  PLAN_CUDA(sq::plan_init(p), "transpose of S'");
   PLAN_CUDA(dq::plan_init(p, Pi, mode == TQ_PROD ? S : nullptr), "fp16 limbs of Pi^T and S^T");
   mscan::plan_init(p);
   nscan::plan_init(p);
@@ -750,7 +750,6 @@ extern "C" int tq_quantize_mse(const tq_plan* plan, const void* X, int x_dtype, 
     TQ_REQUIRE(scratch != nullptr && scratch_bytes >= need, TQ_ERR_WORKSPACE, "%s: scratch of %zu bytes, at least %zu needed",
                who, scratch_bytes, need);
     TQ_REQUIRE(aligned(scratch, 256), TQ_ERR_ALIGNMENT, "%s: scratch is not 256-byte aligned", who);
-    if (sq::preferred(plan, x_dtype, n)) return sq::quantize(plan, X, x_dtype, n, ldx, idx, nullptr, nullptr, norms, st, who);
     return tc::quantize(plan, X, x_dtype, n, ldx, idx, nullptr, nullptr, norms, scratch, scratch_bytes, st, who);
   }
   if (plan->sq.ok) return sq::quantize(plan, X, x_dtype, n, ldx, idx, nullptr, nullptr, norms, st, who);
@@ -780,8 +779,6 @@ extern "C" int tq_quantize_prod(const tq_plan* plan, const void* X, int x_dtype,
     TQ_REQUIRE(scratch != nullptr && scratch_bytes >= least, TQ_ERR_WORKSPACE,
                "%s: scratch of %zu bytes, at least %zu needed", who, scratch_bytes, least);
     TQ_REQUIRE(aligned(scratch, 256), TQ_ERR_ALIGNMENT, "%s: scratch is not 256-byte aligned", who);
-    if (sq::preferred(plan, x_dtype, n))
-      return sq::quantize(plan, X, x_dtype, n, ldx, idx, qjl, gamma, norms, st, who);
     // (the GEMM epilogues write whichever layout the plan has)
     return tc::quantize(plan, X, x_dtype, n, ldx, idx, qjl, gamma, norms, scratch, scratch_bytes, st, who);
   }

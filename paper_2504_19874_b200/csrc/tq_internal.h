@@ -118,11 +118,10 @@ struct tq_plan {
     uint32_t tab[4][4];                // bytes of the codebook's limbs: hi low / high byte, lo low / high byte, 16 entries each
     float gscale, oscale;              // weight of the sign term per unit of gamma; scale of the result
   } dq;
-  // one-launch quantiser for short vectors (d = 32, 64, 96, 128)
+  // one-launch quantiser for short vectors (d = 32, 64, 96)
   struct {
     int ok;
-    void *pi_img, *sp_img;             // fp16 limb images of Pi and S' as the kernel stages them
-    float pi_unscale;                  // inverse of Pi's power-of-two scale
+    float* spt;                        // [d, d] transpose of S' (TQ_PROD)
   } sq;
   int* d_status;   // device word: set to TQ_ERR_TIMEOUT by a kernel whose bounded wait ran out
 };

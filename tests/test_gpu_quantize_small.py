@@ -1,4 +1,4 @@
-"""The one-launch quantiser (d = 32, 64, 96, 128) at the edges of its 16-row tiles and over its bit widths, types and strides,
+"""The one-launch quantiser (d = 32, 64, 96) at the edges of its 64-row tiles and over its bit widths, types and strides,
 against the oracle by the criteria of the other quantiser tests."""
 import pytest
 import torch
@@ -10,12 +10,12 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-@pytest.mark.parametrize("d", [32, 64, 96, 128])
+@pytest.mark.parametrize("d", [32, 64, 96])
 @pytest.mark.parametrize("bits,mode", [(1, tq.TQ_MSE), (2, tq.TQ_MSE), (3, tq.TQ_MSE), (4, tq.TQ_MSE),
                                        (1, tq.TQ_PROD), (2, tq.TQ_PROD), (3, tq.TQ_PROD), (4, tq.TQ_PROD), (5, tq.TQ_PROD)])
 def test_codes_norms_and_residuals(d, bits, mode):
     su = P.Setup(d, bits, mode)
-    for n, dtype, pad in ((1, torch.float32, 0), (17, torch.bfloat16, 0), (127, torch.float32, 1), (130, torch.bfloat16, 3)):
+    for n, dtype, pad in ((1, torch.float32, 0), (63, torch.bfloat16, 0), (127, torch.float32, 1), (130, torch.bfloat16, 3)):
         g = torch.Generator(device="cpu").manual_seed(100 * d + 10 * bits + n)
         X = torch.randn((n, d + pad), generator=g)
         X[:, :4] *= 10.0                                        # outlier channels
