@@ -31,6 +31,7 @@ struct Cfg {
 struct Args {
   const void* X;
   int64_t n, ldx;
+  int vec;                          // rows are 16-byte aligned
   const float* backt;               // [D, ncols]: row k holds Pi[:, k]
   int ncols;
   const float* spt;                 // [D, D]: row k holds S'[:, k]
@@ -47,38 +48,57 @@ __device__ __forceinline__ float element(const void* X, int64_t at) {
   if (BF16) return __bfloat162float(static_cast<const __nv_bfloat16*>(X)[at]);
   return __ldg(static_cast<const float*>(X) + at);
 }
-__device__ __forceinline__ float warp_sum(float v) {
+// Sum of squares of one row of xs by four threads (j = 0..3 of a lane quad), added as a warp with element 32 w + l in lane l
+// would: per lane in ascending order, then the xor butterfly over lane distances 16, 8, 4, 2, 1.  Whole quads call it.
+template <int D>
+__device__ __forceinline__ float row_squares(const float* row, int j) {
+  float s[8];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-// Four BITS-bit codes of coordinates 4 t .. 4 t + 3 (t = lane & 7) of a group of 32: the BITS words of the group, combined over
-// the eight lanes; lane t < BITS returns word t.
-template <int BITS>
-__device__ __forceinline__ uint32_t group_words(uint32_t four, int t) {
-  uint32_t mine = 0u;
-  const int at = 4 * BITS * t;
+  for (int m = 0; m < 8; ++m) {
+    s[m] = 0.f;
 #pragma unroll
-  for (int m = 0; m < BITS; ++m) {
-    const int sh = at - 32 * m;
-    uint32_t v = sh >= 32 || sh <= -4 * BITS ? 0u : sh >= 0 ? four << sh : four >> -sh;
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) v |= __shfl_xor_sync(0xffffffffu, v, o);
-    if (t == m) mine = v;
+    for (int w = 0; w < D / 32; ++w) {
+      const float x = row[32 * w + 4 * m + j];
+      s[m] = fmaf(x, x, s[m]);
+    }
   }
-  return mine;
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int m = 0; m < o; ++m) s[m] += s[m + o];
+  s[0] += __shfl_xor_sync(0xffffffffu, s[0], 2);
+  return s[0] + __shfl_xor_sync(0xffffffffu, s[0], 1);
+}
+// Four BITS-bit codes of coordinates 4 t .. 4 t + 3 (t = lane & 7) of a group of 32 -> the group's BITS words.  Returns one word
+// and its number in `which` (-1: this lane has none).
+template <int BITS>
+__device__ __forceinline__ uint32_t group_words(uint32_t four, int t, int& which) {
+  if (BITS == 3) {   // pairs of lanes hold 24 bits; word k = bits of pairs k and k + 1
+    const uint32_t other = __shfl_xor_sync(0xffffffffu, four, 1);
+    const uint32_t pair = (t & 1) ? other | (four << 12) : four | (other << 12);
+    const uint32_t next = __shfl_down_sync(0xffffffffu, pair, 2);
+    const int k = t >> 1;
+    which = (t & 1) == 0 && k < 3 ? k : -1;
+    return (pair >> (8 * k)) | (next << ((24 - 8 * k) & 31));
+  }
+  constexpr int LANES = 8 / BITS;   // lanes of one word
+  uint32_t v = four << (4 * BITS * (t & (LANES - 1)));
+#pragma unroll
+  for (int o = 1; o < LANES; o <<= 1) v |= __shfl_xor_sync(0xffffffffu, v, o);
+  which = (t & (LANES - 1)) == 0 ? t / LANES : -1;
+  return v;
 }
 
 template <int D, int BITS, bool PROD, bool BF16>
 __global__ void __launch_bounds__(Cfg<D>::kThreads) small_quantize_kernel(Args a) {
-  constexpr int T = Cfg<D>::kThreads, TX = D / 4, S = Cfg<D>::kStride, NWARP = T / 32;
+  constexpr int T = Cfg<D>::kThreads, TX = D / 4, S = Cfg<D>::kStride;
   extern __shared__ __align__(16) float smem[];
   float* xs = smem;                        // [RT][S]  rows, later the residuals
   float* bs = xs + RT * S;                 // [D][D]   Pi^T
   float* ss = bs + D * D;                  // [D][D]   S'^T (PROD)
   float* vs = bs + (PROD ? 2 : 1) * D * D; // [RT]     nu as the comparisons take it (1 for a zero row)
   float* is = vs + RT;                     // [RT]     1 / nu (0 for a zero row)
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   const int tx = tid % TX, ty = tid / TX, t8 = lane & 7;
   const int64_t row0 = (int64_t)blockIdx.x * RT;
   {
@@ -92,21 +112,38 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads) small_quantize_kernel(Args a
       asm volatile("cp.async.commit_group;" ::: "memory");
     }
   }
-  // ---- rows to shared memory, their norms (lane l: elements l, l + 32, ..)
-#pragma unroll 4
-  for (int r = warp; r < RT; r += NWARP) {
-    const int64_t row = min(row0 + r, a.n - 1);   // rows past the end repeat the last one
-    float x[D / 32], s = 0.f;
+  // ---- rows to shared memory, then their norms
+  constexpr int PE = BF16 ? 8 : 4;   // elements of a 16-byte piece
 #pragma unroll
-    for (int w = 0; w < D / 32; ++w) x[w] = element<BF16>(a.X, row * a.ldx + 32 * w + lane);
+  for (int p = tid; p < RT * D / PE; p += T) {
+    const int r = p / (D / PE), c = PE * (p % (D / PE));
+    const int64_t at = min(row0 + r, a.n - 1) * a.ldx + c;   // rows past the end repeat the last one
+    float x[PE];
+    if (a.vec) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(static_cast<const unsigned char*>(a.X) + at * (16 / PE)));
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int w = 0; w < D / 32; ++w) {
-      s = fmaf(x[w], x[w], s);
-      xs[r * S + 32 * w + lane] = x[w];
+      for (int i = 0; i < 4; ++i) {
+        if (BF16) {
+          x[2 * i] = __uint_as_float(w[i] << 16);
+          x[(2 * i + 1) % PE] = __uint_as_float(w[i] & 0xffff0000u);
+        } else {
+          x[i] = __uint_as_float(w[i]);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < PE; ++i) x[i] = element<BF16>(a.X, at + i);
     }
+#pragma unroll
+    for (int i = 0; i < PE; i += 4) *reinterpret_cast<float4*>(xs + r * S + c + i) = make_float4(x[i], x[i + 1], x[i + 2], x[i + 3]);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = tid >> 2; r < RT; r += T / 4) {   // whole warps
     float nu = 1.f;
-    if (a.norms != nullptr) nu = sqrtf(warp_sum(s));
-    if (lane == 0) {
+    if (a.norms != nullptr) nu = sqrtf(row_squares<D>(xs + r * S, tid & 3));
+    if ((tid & 3) == 0) {
       if (a.norms != nullptr && row0 + r < a.n) a.norms[row0 + r] = nu;
       vs[r] = nu > 0.f ? nu : 1.f;
       is[r] = nu > 0.f ? 1.f / nu : 0.f;
@@ -168,11 +205,13 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads) small_quantize_kernel(Args a
       if (PROD) e[c] = inv > 0.f ? fmaf(y, inv, -cent) : 0.f;
     }
     if (BITS > 0) {
-      const uint32_t word = group_words<BITS>(four, t8);
+      int which;
+      const uint32_t word = group_words<BITS == 0 ? 1 : BITS>(four, t8, which);
       uint32_t* dst = reinterpret_cast<uint32_t*>(a.idx + (size_t)row * a.idx_rb);
-      if (row < a.n && t8 < BITS) dst[(tx >> 3) * BITS + t8] = word;
-      if (row < a.n)
-        for (int w = D * BITS / 32 + tx; w < a.idx_rb / 4; w += TX) dst[w] = 0u;   // pad words
+      if (row < a.n) {
+        if (which >= 0) dst[(tx >> 3) * BITS + which] = word;
+        if (D * BITS / 32 + tx < a.idx_rb / 4) dst[D * BITS / 32 + tx] = 0u;   // pad words (fewer than four)
+      }
     }
     if (PROD) *reinterpret_cast<float4*>(xs + r * S + 4 * tx) = make_float4(e[0], e[1], e[2], e[3]);
   }
@@ -180,16 +219,10 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads) small_quantize_kernel(Args a
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     // ---- gamma = |r|, then z = sign(S' r)
-#pragma unroll 4
-    for (int r = warp; r < RT; r += NWARP) {
-      float s = 0.f;
 #pragma unroll
-      for (int w = 0; w < D / 32; ++w) {
-        const float e = xs[r * S + 32 * w + lane];
-        s = fmaf(e, e, s);
-      }
-      s = warp_sum(s);
-      if (lane == 0 && row0 + r < a.n) a.gamma[row0 + r] = sqrtf(s);
+    for (int r = tid >> 2; r < RT; r += T / 4) {
+      const float s = row_squares<D>(xs + r * S, tid & 3);
+      if ((tid & 3) == 0 && row0 + r < a.n) a.gamma[row0 + r] = sqrtf(s);
     }
     product(ss);
 #pragma unroll
@@ -198,11 +231,13 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads) small_quantize_kernel(Args a
       uint32_t four = 0u;
 #pragma unroll
       for (int c = 0; c < 4; ++c) four |= acc[i][c] >= 0.f ? 1u << c : 0u;
-      const uint32_t word = group_words<1>(four, t8);
+      int which;
+      const uint32_t word = group_words<1>(four, t8, which);
       uint32_t* dst = reinterpret_cast<uint32_t*>(a.qjl + (size_t)row * a.qjl_rb);
-      if (row < a.n && t8 == 0) dst[tx >> 3] = word;
-      if (row < a.n)
-        for (int w = D / 32 + tx; w < a.qjl_rb / 4; w += TX) dst[w] = 0u;
+      if (row < a.n) {
+        if (which == 0) dst[tx >> 3] = word;
+        if (D / 32 + tx < a.qjl_rb / 4) dst[D / 32 + tx] = 0u;
+      }
     }
   }
 }
@@ -273,6 +308,7 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
   a.X = X;
   a.n = n;
   a.ldx = ldx;
+  a.vec = (ldx * (x_dtype == TQ_F32 ? 4 : 2)) % 16 == 0;
   a.backt = plan->dBackT;
   a.ncols = plan->ncat * plan->dpad;
   a.spt = plan->sq.spt;
