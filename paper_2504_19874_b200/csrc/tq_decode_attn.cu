@@ -619,23 +619,6 @@ size_t workspace_bytes(int ngroups, int heads, int64_t tokens, int d) {
 }
 
 
-// Launch with the programmatic-stream-serialisation attribute.
-template <typename... KArgs, typename... LArgs>
-cudaError_t launch_after(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, LArgs... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
-  return e != cudaSuccess ? e : cudaGetLastError();
-}
-
 // Walsh coefficients of an antisymmetric codebook of 2^bits entries (see tq_decode_mma.cuh); false if it is not one.
 bool walsh_coefficients(const float* c, int bits, float* alpha) {
   for (int i = 0; i < 8; ++i) alpha[i] = 0.f;
@@ -866,10 +849,10 @@ extern "C" int tq_attend_decode(const tq_kv_group* groups, int ngroups, int head
     // all three launches may be scheduled while their predecessor in the stream drains; each orders itself with
     // griddepcontrol.wait before it reads or writes global memory that another kernel touches
     if (q_dtype == TQ_F32)
-      TQ_CHECK_CUDA(launch_after(prepare_mma_kernel<float>, dim3((unsigned)(heads * ngroups)), dim3(256), 0, st, a, ma,
+      TQ_CHECK_CUDA(launch_dependent(prepare_mma_kernel<float>, dim3((unsigned)(heads * ngroups)), dim3(256), 0, st, a, ma,
                                  static_cast<const float*>(Q), ldq), who);
     else
-      TQ_CHECK_CUDA(launch_after(prepare_mma_kernel<__nv_bfloat16>, dim3((unsigned)(heads * ngroups)), dim3(256), 0, st, a, ma,
+      TQ_CHECK_CUDA(launch_dependent(prepare_mma_kernel<__nv_bfloat16>, dim3((unsigned)(heads * ngroups)), dim3(256), 0, st, a, ma,
                                  static_cast<const __nv_bfloat16*>(Q), ldq), who);
     static std::atomic<size_t> mma_smem_set[16];
     if (dev >= 16 || mma_smem > mma_smem_set[dev].load(std::memory_order_relaxed)) {
@@ -878,8 +861,8 @@ extern "C" int tq_attend_decode(const tq_kv_group* groups, int ngroups, int head
       TQ_CHECK_CUDA(cudaFuncSetAttribute(partial_mma_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared), who);
       if (dev < 16) mma_smem_set[dev].store(mma_smem, std::memory_order_relaxed);
     }
-    TQ_CHECK_CUDA(launch_after(partial_mma_kernel, dim3((unsigned)(heads * nslices)), dim3(NT), mma_smem, st, a, ma), who);
-    TQ_CHECK_CUDA(launch_after(merge_kernel, dim3((unsigned)(heads * ngroups)), dim3(MERGE_NT), merge_smem, st, a, out, ldo), who);
+    TQ_CHECK_CUDA(launch_dependent(partial_mma_kernel, dim3((unsigned)(heads * nslices)), dim3(NT), mma_smem, st, a, ma), who);
+    TQ_CHECK_CUDA(launch_dependent(merge_kernel, dim3((unsigned)(heads * ngroups)), dim3(MERGE_NT), merge_smem, st, a, out, ldo), who);
     count_launches(3);
     return TQ_OK;
   }

@@ -61,6 +61,30 @@ __device__ __forceinline__ bool device_check_failed(int* status) {
 #endif
 #endif
 
+#ifdef __CUDACC__
+// Programmatic dependent launch: the grid may be scheduled while the kernel ahead of it in the stream drains.  Such a kernel
+// calls wait_for_predecessor() in every thread before it touches global memory that another kernel writes or reads (constants
+// of a plan may be read before); the call returns once the kernel ahead -- and with it, by the same rule, everything before --
+// has completed.  allow_successor() lets the next such kernel be scheduled.
+__device__ __forceinline__ void allow_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... KArgs, typename... LArgs>
+cudaError_t launch_dependent(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, LArgs... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+#endif
+
 struct MatrixLimbs {
   __nv_bfloat16* hi;
   __nv_bfloat16* lo;
