@@ -215,22 +215,26 @@ bool has_pad_words(int d, int bits, size_t row_bytes) {
 // of the queries in shared memory; each lane sums its products in fp32, the 32 partial sums are
 // added in fp64.  The matrix is read once per 8 queries.
 constexpr int kRotQ = 8, kRotChunk = 2048;   // 64 KB of queries per chunk (dynamic shared memory)
-constexpr int kRotQPerBlock = 64;            // queries per CTA (grid.y covers the rest)
+constexpr int kRotQPerBlock = 64;            // most queries per CTA (grid.y covers the rest)
+// Queries per CTA: 64 (eight rounds, the matrix is read once for all of them) where that still gives every SM two CTAs, else
+// fewer rounds in more CTAs: 64 queries of d = 128 took four CTAs 33 us for eight rounds each, 32 CTAs take 3.4 us.
+inline int rotate_queries_per_cta(int64_t column_ctas, int nq) {
+  int per = kRotQPerBlock;
+  while (per > kRotQ && column_ctas * ((nq + per - 1) / per) < 2 * 148) per /= 2;
+  return per;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(256) rotate_queries_kernel(const float* __restrict__ Rot, int nrows, int d,
                                                              const T* __restrict__ Q, int64_t ldq, int nq,
-                                                             float* __restrict__ Qcat, int64_t ldo) {
-  extern __shared__ __align__(16) float qs_raw[];
-  float (*qs)[kRotChunk] = reinterpret_cast<float (*)[kRotChunk]>(qs_raw);
-  // a successor launched as a programmatic dependent may be scheduled while this grid drains (it waits for
-  // this grid's completion before it reads Qcat)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+                                                             float* __restrict__ Qcat, int64_t ldo, int per_cta, int stride) {
+  extern __shared__ __align__(16) float qs_raw[];   // [queries of a round][stride]
+  auto qs = [&](int qq, int c) -> float* { return qs_raw + qq * stride + c; };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int j = blockIdx.x * 8 + warp;
   const float* row = Rot + (size_t)min(j, nrows - 1) * d;
   const bool vec = (d & 3) == 0;   // rows are 16-byte aligned
-  const int q_begin = blockIdx.y * kRotQPerBlock, q_end = min(nq, q_begin + kRotQPerBlock);
+  const int q_begin = blockIdx.y * per_cta, q_end = min(nq, q_begin + per_cta);
   for (int q0 = q_begin; q0 < q_end; q0 += kRotQ) {
     float acc[kRotQ];
 #pragma unroll
@@ -247,9 +251,13 @@ __global__ void __launch_bounds__(256) rotate_queries_kernel(const float* __rest
           r[i] = (4 * c4 < len) ? __ldg(row4 + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
       }
+      if (q0 == q_begin && c0 == 0) {   // the first piece of the matrix (the plan's) is on its way
+        wait_for_predecessor();         // it may write the queries
+        allow_successor();              // (only now: a successor may start reading the codes, see nscan::run)
+      }
       __syncthreads();
-      for (int e = threadIdx.x; e < nact * (kRotChunk / 4); e += blockDim.x) {
-        const int qq = e / (kRotChunk / 4), c = 4 * (e % (kRotChunk / 4));
+      for (int e = threadIdx.x; e < nact * (stride / 4); e += blockDim.x) {
+        const int qq = e / (stride / 4), c = 4 * (e % (stride / 4));
         float v[4] = {0.f, 0.f, 0.f, 0.f};
         if (q0 + qq < q_end && c < len) {
           const T* src = Q + (int64_t)(q0 + qq) * ldq + c0 + c;
@@ -257,7 +265,7 @@ __global__ void __launch_bounds__(256) rotate_queries_kernel(const float* __rest
           for (int t = 0; t < 4; ++t)
             if (c + t < len) v[t] = scan::to_f32<T>(src[t]);
         }
-        *reinterpret_cast<float4*>(&qs[qq][c]) = make_float4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<float4*>(qs(qq, c)) = make_float4(v[0], v[1], v[2], v[3]);
       }
       __syncthreads();
       if (vec) {
@@ -268,7 +276,7 @@ __global__ void __launch_bounds__(256) rotate_queries_kernel(const float* __rest
 #pragma unroll
             for (int qq = 0; qq < kRotQ; ++qq) {
               if (qq < nact) {
-                const float4 v = *reinterpret_cast<const float4*>(&qs[qq][4 * c4]);
+                const float4 v = *reinterpret_cast<const float4*>(qs(qq, 4 * c4));
                 acc[qq] = fmaf(r[i].x, v.x, fmaf(r[i].y, v.y, fmaf(r[i].z, v.z, fmaf(r[i].w, v.w, acc[qq]))));
               }
             }
@@ -279,7 +287,7 @@ __global__ void __launch_bounds__(256) rotate_queries_kernel(const float* __rest
           const float rv = __ldg(row + c0 + c);
 #pragma unroll
           for (int qq = 0; qq < kRotQ; ++qq)
-            if (qq < nact) acc[qq] = fmaf(rv, qs[qq][c], acc[qq]);
+            if (qq < nact) acc[qq] = fmaf(rv, *qs(qq, c), acc[qq]);
         }
       }
     }
@@ -305,13 +313,14 @@ constexpr int kRotManyFrom = 64;   // queries from which the blocked kernel is u
 template <typename T>
 __global__ void __launch_bounds__(32 * kRmWarps) rotate_many_kernel(const float* __restrict__ Rot, int nrows, int d,
                                                                     const T* __restrict__ Q, int64_t ldq, int nq,
-                                                                    float* __restrict__ Qcat, int64_t ldo) {
-  extern __shared__ __align__(16) float qs_raw[];
-  float (*qs)[kRotChunk] = reinterpret_cast<float (*)[kRotChunk]>(qs_raw);
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+                                                                    float* __restrict__ Qcat, int64_t ldo, int per_cta, int stride) {
+  extern __shared__ __align__(16) float qs_raw[];   // [queries of a round][stride]
+  auto qs = [&](int qq, int c) -> float* { return qs_raw + qq * stride + c; };
+  wait_for_predecessor();   // it may write the queries
+  allow_successor();        // (only now: a successor may start reading the codes, see nscan::run)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int j0 = blockIdx.x * kRmRowsPerBlock + warp * kRmRows;
-  const int q_begin = blockIdx.y * kRotQPerBlock, q_end = min(nq, q_begin + kRotQPerBlock);
+  const int q_begin = blockIdx.y * per_cta, q_end = min(nq, q_begin + per_cta);
   for (int q0 = q_begin; q0 < q_end; q0 += kRotQ) {
     float acc[kRmRows][kRotQ];
 #pragma unroll
@@ -322,14 +331,14 @@ __global__ void __launch_bounds__(32 * kRmWarps) rotate_many_kernel(const float*
     for (int c0 = 0; c0 < d; c0 += kRotChunk) {
       const int len = min(kRotChunk, d - c0);
       __syncthreads();
-      for (int e = threadIdx.x; e < nact * (kRotChunk / 4); e += blockDim.x) {
-        const int qq = e / (kRotChunk / 4), c = 4 * (e % (kRotChunk / 4));
+      for (int e = threadIdx.x; e < nact * (stride / 4); e += blockDim.x) {
+        const int qq = e / (stride / 4), c = 4 * (e % (stride / 4));
         if (c >= len) continue;   // columns past the chunk's end are not read below
         const T* src = Q + (int64_t)(q0 + qq) * ldq + c0 + c;
         float v[4];
 #pragma unroll
         for (int t = 0; t < 4; ++t) v[t] = scan::to_f32<T>(src[t]);   // d is a multiple of 4: whole groups of four
-        *reinterpret_cast<float4*>(&qs[qq][c]) = make_float4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<float4*>(qs(qq, c)) = make_float4(v[0], v[1], v[2], v[3]);
       }
       __syncthreads();
 #pragma unroll 2
@@ -343,7 +352,7 @@ __global__ void __launch_bounds__(32 * kRmWarps) rotate_many_kernel(const float*
 #pragma unroll
         for (int qq = 0; qq < kRotQ; ++qq) {
           if (qq < nact) {
-            const float4 v = *reinterpret_cast<const float4*>(&qs[qq][4 * c4]);
+            const float4 v = *reinterpret_cast<const float4*>(qs(qq, 4 * c4));
 #pragma unroll
             for (int rr = 0; rr < kRmRows; ++rr)
               acc[rr][qq] = fmaf(r[rr].x, v.x, fmaf(r[rr].y, v.y, fmaf(r[rr].z, v.z, fmaf(r[rr].w, v.w, acc[rr][qq]))));
@@ -383,32 +392,35 @@ __global__ void __launch_bounds__(32 * kRmWarps) rotate_many_kernel(const float*
 template <typename T>
 cudaError_t launch_rotate_queries(const tq_plan* plan, const T* Q, int64_t ldq, int nq, float* Qcat, cudaStream_t st) {
   const int ncols = plan->ncat * plan->dpad;
-  constexpr int smem = kRotQ * kRotChunk * (int)sizeof(float);
+  constexpr int smem_max = kRotQ * kRotChunk * (int)sizeof(float);
+  const int stride = std::min(round_up(plan->d, 4), kRotChunk), smem = std::min(nq, kRotQ) * stride * (int)sizeof(float);
   // function attributes are per device: remember the devices this launcher has prepared
   static std::atomic<unsigned long long> attr_devices{0};   // written by any thread that launches
   int attr_dev = 0;
   if (cudaGetDevice(&attr_dev) != cudaSuccess) return cudaErrorInvalidDevice;
   if (attr_dev >= 64 || !((attr_devices.load(std::memory_order_relaxed) >> attr_dev) & 1ull)) {
-    cudaError_t e = cudaFuncSetAttribute(rotate_queries_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(rotate_queries_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
     if (e != cudaSuccess) return e;
     if (attr_dev < 64) attr_devices.fetch_or(1ull << attr_dev, std::memory_order_relaxed);
   }
   if (nq >= kRotManyFrom && (plan->d & 3) == 0) {
     static std::atomic<unsigned long long> many_devices{0};
     if (attr_dev >= 64 || !((many_devices.load(std::memory_order_relaxed) >> attr_dev) & 1ull)) {
-      cudaError_t e = cudaFuncSetAttribute(rotate_many_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      cudaError_t e = cudaFuncSetAttribute(rotate_many_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
       if (e != cudaSuccess) return e;
       if (attr_dev < 64) many_devices.fetch_or(1ull << attr_dev, std::memory_order_relaxed);
     }
-    const dim3 grid((unsigned)((ncols + kRmRowsPerBlock - 1) / kRmRowsPerBlock), (unsigned)((nq + kRotQPerBlock - 1) / kRotQPerBlock));
-    rotate_many_kernel<T><<<grid, 32 * kRmWarps, smem, st>>>(plan->dRotCat, ncols, plan->d, Q, ldq, nq, Qcat, ncols);
+    const int cols = (ncols + kRmRowsPerBlock - 1) / kRmRowsPerBlock, per = rotate_queries_per_cta(cols, nq);
+    const dim3 grid((unsigned)cols, (unsigned)((nq + per - 1) / per));
     count_launches(1);
-    return cudaGetLastError();
+    return launch_dependent(rotate_many_kernel<T>, grid, dim3(32 * kRmWarps), smem, st, plan->dRotCat, ncols, plan->d, Q, ldq, nq, Qcat,
+                            (int64_t)ncols, per, stride);
   }
-  const dim3 grid((unsigned)((ncols + 7) / 8), (unsigned)((nq + kRotQPerBlock - 1) / kRotQPerBlock));
-  rotate_queries_kernel<T><<<grid, 256, smem, st>>>(plan->dRotCat, ncols, plan->d, Q, ldq, nq, Qcat, ncols);
+  const int cols = (ncols + 7) / 8, per = rotate_queries_per_cta(cols, nq);
+  const dim3 grid((unsigned)cols, (unsigned)((nq + per - 1) / per));
   count_launches(1);
-  return cudaGetLastError();
+  return launch_dependent(rotate_queries_kernel<T>, grid, dim3(256), smem, st, plan->dRotCat, ncols, plan->d, Q, ldq, nq, Qcat, (int64_t)ncols,
+                          per, stride);
 }
 
 // Q' = Q Pi^T and Q'' = Q S^T side by side: Qcat[nq, ncat*dpad].
@@ -1017,14 +1029,16 @@ static int topk_ms(const tq_plan* plan, const float* Qcat, int nq, int64_t n, co
     const bool use_filter = n >= kFilterMinN && dense_rows >= std::min<int64_t>(n, eng.dense_rows_pref);
     const int* guard = nullptr;
     if (use_filter) {
-      int64_t m = std::max<int64_t>(round_up64(n / 64, 256), round_up64(std::max(k, 4096), 256));
+      // pilot rows: about 8192 candidates are then expected from the full pass (n k / m), well inside the lists' 32,768 (the
+      // k-th best of the pilot varies by 1 / sqrt(k)) and what the final selection keeps in registers; a larger pilot costs a
+      // longer pilot scan and selection
+      int64_t m = std::max<int64_t>(round_up64((int64_t)((double)n * k / 8192.0), 256), 4096);
       m = std::min<int64_t>(m, std::min<int64_t>(dense_rows / 256 * 256, n));
       if ((rc = engine_run(eng, q0, nqp, m, idx, qjl, gamma, norms, dense, m, nullptr, nullptr, msw, st, who))) return rc;
-      TQ_CHECK_CUDA(mscan::select_topk(dense, nullptr, nullptr, (int)m, (int)m, 0, nqp, k, 0, ts, ti, tau, nullptr, nullptr, st), who);
-      TQ_CHECK_CUDA(cudaMemsetAsync(count, 0, (size_t)(qpp + 1) * sizeof(int), st), who);   // counters and the overflow flag
+      TQ_CHECK_CUDA(mscan::select_topk(dense, nullptr, nullptr, (int)m, (int)m, 0, nqp, k, 0, nullptr, nullptr, tau, nullptr, nullptr, count, overflow, st), who);
       mscan::Filter f{tau, count, cand_s, cand_i, kCandCap};
       if ((rc = engine_run(eng, q0, nqp, n, idx, qjl, gamma, norms, nullptr, 0, &f, nullptr, msw, st, who))) return rc;
-      TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count, kCandCap, 0, 0, nqp, k, 0, ts, ti, nullptr, overflow, nullptr, st), who);
+      TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count, kCandCap, 0, 0, nqp, k, 0, ts, ti, nullptr, overflow, nullptr, nullptr, nullptr, st), who);
       guard = overflow;
     }
     // dense block flow: the whole job for small n, the guarded rescue otherwise
@@ -1036,7 +1050,7 @@ static int topk_ms(const tq_plan* plan, const float* Qcat, int nq, int64_t n, co
                            gamma ? gamma + v0 : nullptr, norms ? norms + v0 : nullptr, dense, block, nullptr, guard, msw, st, who)))
         return rc;
       TQ_CHECK_CUDA(mscan::select_topk(dense, nullptr, nullptr, (int)block, (int)cn, (int)v0, nqp, k, v0 > 0 ? 1 : 0, ts, ti,
-                                       nullptr, nullptr, guard, st), who);
+                                       nullptr, nullptr, guard, nullptr, nullptr, st), who);
     }
   }
   return TQ_OK;

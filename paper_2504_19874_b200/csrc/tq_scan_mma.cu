@@ -29,6 +29,7 @@
 // per-query threshold to a candidate list (top-k).
 #include <atomic>
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 
 #include "tq_quantize_tc.h"
@@ -184,6 +185,8 @@ __device__ __forceinline__ int digit_of(long long J, int limb) {
 // long, and this kernel sits in front of every scan call; the 8 bytes meet by a shuffle-OR.
 __global__ void __launch_bounds__(256) bprep_kernel(BPrepArgs a) {
   __shared__ QConst sc[kMaxPassQueries];
+  allow_successor();
+  wait_for_predecessor();   // the rotated queries are its output; the operand may still be read by it
   query_constants(a, sc);
   const int ksa = ks_a(a.bm), kss = ks_s(a.prod != 0), KS = ksa + kss;
   const int64_t total = (int64_t)a.NT * a.R * KS * 32;
@@ -288,7 +291,11 @@ scan_mma_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
   constexpr int KSA = ks_a(BM), KSS = ks_s(PROD), KS = KSA + KSS;
   constexpr int NQP = NT * 8 / LIMBS;              // queries per pass
 
-  if (a.run_if != nullptr && *a.run_if == 0) return;
+  allow_successor();
+  if (a.run_if != nullptr) {
+    wait_for_predecessor();   // it may write the switch
+    if (*a.run_if == 0) return;
+  }
 
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -311,6 +318,7 @@ scan_mma_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
     if (BM > 0) tc::tma_prefetch_desc(&tmIdx);
     if (PROD) tc::tma_prefetch_desc(&tmQjl);
   }
+  wait_for_predecessor();   // every input may be its output
   {
     const uint4* src = reinterpret_cast<const uint4*>(a.Bfrag);
     uint4* dst = reinterpret_cast<uint4*>(Bs);
@@ -572,11 +580,13 @@ struct SelArgs {
   const int* cand_i;      // nullptr: dense row, id = id0 + position
   const int* count;       // nullptr: m elements
   int cap, m, id0, k, merge;
-  float* top_s;
+  float* top_s;           // nullable (with top_i, merge = 0): only kth is wanted, and any lower bound reached by k entries will do
   int* top_i;
   float* kth;             // nullable
   int* overflow;          // nullable: set to 1 when count > cap for this query
   const int* run_if;      // nullable
+  int* clear_count;       // nullable: [nq] counters to zero, and with them the flag
+  int* clear_flag;
 };
 
 __device__ __forceinline__ unsigned long long make_key(float s, int id) {
@@ -586,13 +596,35 @@ __device__ __forceinline__ unsigned long long make_key(float s, int id) {
   return ((unsigned long long)u << 32) | (uint32_t)(~(uint32_t)id);
 }
 
+__device__ __forceinline__ float key_score(unsigned long long key) {
+  uint32_t u = (uint32_t)(key >> 32);
+  u = (u & 0x80000000u) ? (u & 0x7fffffffu) : ~u;
+  return __uint_as_float(u);
+}
+
+// One CTA per query: the k largest keys, sorted.
+// Usual case: the scores are counted in kSelBins equal steps between their minimum and maximum; the bin that holds the k-th
+// largest is found by a suffix sum, and everything in it and above is sorted (scores of a search thin out towards the top, so
+// that is hardly more than k).  Three sweeps over the list; lists of up to 16,384 entries stay in registers.  If more than
+// 1024 entries would have to be sorted (ties, a few far outliers) or a score is not finite, a radix select over the key's
+// bytes does the job (up to eight sweeps, each with lane-matching and a histogram of its own: 20 us for 15,616 scores
+// against 15).
+constexpr int kSelBins = 2048;
 __global__ void __launch_bounds__(1024) select_kernel(SelArgs a) {
-  __shared__ int hist[256];
+  __shared__ int hist[kSelBins];
   __shared__ unsigned long long s_prefix;
   __shared__ int s_kk, s_done, s_cnt;
   __shared__ unsigned long long skey[1024];
+  __shared__ float wmin[32], wmax[32];
+  __shared__ int wsum[32];
+  allow_successor();
+  wait_for_predecessor();   // all inputs are outputs of kernels ahead in the stream
   if (a.run_if != nullptr && *a.run_if == 0) return;
-  const int q = blockIdx.x, tid = threadIdx.x;
+  const int q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (a.clear_count != nullptr && tid == 0) {   // the candidate counters of the pass that follows
+    a.clear_count[q] = 0;
+    if (q == 0) *a.clear_flag = 0;
+  }
   int m_new = a.m;
   if (a.count != nullptr) {
     const int c = a.count[q];
@@ -622,38 +654,135 @@ __global__ void __launch_bounds__(1024) select_kernel(SelArgs a) {
       kc[u] = (i < total) ? key_at(i) : 0ull;
     }
   }
-  int kk = min(a.k, total);
-  const int k_target = kk;
-  unsigned long long prefix = 0ull;
-  int shift = 56;
-  if (kk > 0) {
+  // f(key) for every entry of the list (0 where there is none), all threads of a warp together
+  auto sweep = [&](auto&& f) {
+    if (cached) {
+#pragma unroll
+      for (int u = 0; u < 16; ++u)
+        if (u * 1024 < total) f(kc[u]);
+    } else {
+      // batches of 8 independent loads per thread, then the (convergent) uses
+      for (int base = 0; base < total; base += 8 * 1024) {
+        unsigned long long keys[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int i = base + u * 1024 + tid;
+          keys[u] = (i < total) ? key_at(i) : 0ull;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) f(keys[u]);
+      }
+    }
+  };
+  const int k_target = min(a.k, total);
+  bool sorted_set = false;   // skey holds the survivors
+  if (tid == 0) s_cnt = 0;
+  skey[tid] = 0ull;
+  if (k_target > 0) {
+    // ---- range of the scores
+    float mn = INFINITY, mx = -INFINITY;
+    int odd = 0;
+    sweep([&](unsigned long long key) {
+      if (key != 0ull) {
+        const float v = key_score(key);
+        odd |= !(fabsf(v) <= FLT_MAX);
+        mn = fminf(mn, v);
+        mx = fmaxf(mx, v);
+      }
+    });
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    if (lane == 0) { wmin[warp] = mn; wmax[warp] = mx; }
+    for (int b = tid; b < kSelBins; b += 1024) hist[b] = 0;
+    odd = __syncthreads_or(odd);
+    mn = wmin[lane];
+    mx = wmax[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    const float scale = (float)kSelBins / (mx - mn);
+    if (!odd && mx > mn && scale <= FLT_MAX) {
+      // the bin of a score never decreases with the score: subtraction, product and truncation round monotonically
+      auto bin_of = [&](unsigned long long key) { return min(kSelBins - 1, (int)((key_score(key) - mn) * scale)); };
+      sweep([&](unsigned long long key) {
+        if (key != 0ull) atomicAdd(&hist[bin_of(key)], 1);
+      });
+      __syncthreads();
+      // thread t owns bins B - 1 - 2 t and B - 2 - 2 t: counts from the top by a block-wide prefix sum
+      const int hi = hist[kSelBins - 1 - 2 * tid], lo = hist[kSelBins - 2 - 2 * tid];
+      int incl = hi + lo;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      if (lane == 31) wsum[warp] = incl;
+      __syncthreads();
+      int before = lane < warp ? wsum[lane] : 0, all = wsum[lane];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        before += __shfl_xor_sync(0xffffffffu, before, o);
+        all += __shfl_xor_sync(0xffffffffu, all, o);
+      }
+      const int above = before + incl - hi - lo;   // entries in higher bins than this thread's
+      if (above < k_target && above + hi + lo >= k_target) {   // the k-th largest is in one of this thread's bins
+        const bool first = above + hi >= k_target;
+        s_kk = kSelBins - (first ? 1 : 2) - 2 * tid;
+        s_done = above + hi + (first ? 0 : lo);                // entries to sort
+      }
+      __syncthreads();
+      if (a.top_s == nullptr && all >= k_target) {
+        // only a lower bound of the k-th score is wanted: the smallest score in the bins from that of the k-th on
+        const int cut = s_kk;
+        float low = INFINITY;
+        sweep([&](unsigned long long key) {
+          if (key != 0ull && bin_of(key) >= cut) low = fminf(low, key_score(key));
+        });
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) low = fminf(low, __shfl_xor_sync(0xffffffffu, low, o));
+        if (lane == 0) wmin[warp] = low;
+        __syncthreads();
+        if (warp == 0) {
+          low = wmin[lane];
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) low = fminf(low, __shfl_xor_sync(0xffffffffu, low, o));
+          if (lane == 0) a.kth[q] = low;
+        }
+        return;
+      }
+      const bool few = all < k_target;   // fewer entries than k (empty slots in the list): all of them
+      const int cut = few ? 0 : s_kk;
+      if ((few ? all : s_done) <= 1024) {
+        sweep([&](unsigned long long key) {
+          if (key != 0ull && bin_of(key) >= cut) skey[atomicAdd(&s_cnt, 1)] = key;
+        });
+        sorted_set = true;
+      }
+    }
+  }
+  if (!sorted_set && k_target > 0) {
+    // ---- radix select over the key's bytes, from the top
+    int kk = k_target;
+    unsigned long long prefix = 0ull;
+    int shift = 56;
     for (int round = 0; round < 8; ++round) {
       shift = 56 - 8 * round;
+      __syncthreads();
       if (tid < 256) hist[tid] = 0;
       __syncthreads();
-      auto tally = [&](unsigned long long key, bool valid) {
-        const bool in = valid && (round == 0 || (key >> (shift + 8)) == prefix);
+      sweep([&](unsigned long long key) {
+        const bool in = key != 0ull && (round == 0 || (key >> (shift + 8)) == prefix);
         // lanes with the same digit add once (scores of one query crowd into a few bins)
         const int dg = in ? (int)((key >> shift) & 255ull) : -1;
         const unsigned peers = __match_any_sync(0xffffffffu, dg);
-        if (in && (int)(__ffs(peers) - 1) == (tid & 31)) atomicAdd(&hist[dg], __popc(peers));
-      };
-      if (cached) {
-#pragma unroll
-        for (int u = 0; u < 16; ++u) tally(kc[u], u * 1024 + tid < total);
-      } else {
-        // batches of 8 independent loads per thread, then the (convergent) histogram updates
-        for (int base = 0; base < total; base += 8 * blockDim.x) {
-          unsigned long long keys[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int i = base + u * blockDim.x + tid;
-            keys[u] = (i < total) ? key_at(i) : 0ull;
-          }
-#pragma unroll
-          for (int u = 0; u < 8; ++u) tally(keys[u], base + u * (int)blockDim.x + tid < total);
-        }
-      }
+        if (in && (int)(__ffs(peers) - 1) == lane) atomicAdd(&hist[dg], __popc(peers));
+      });
+      if (tid == 0) s_done = -1;
       __syncthreads();
       if (tid < 32) {
         // lane l owns bins 255 - 8l ... 248 - 8l (descending); exclusive prefix of the lane totals by shuffles
@@ -685,39 +814,23 @@ __global__ void __launch_bounds__(1024) select_kernel(SelArgs a) {
         }
       }
       __syncthreads();
+      if (s_done < 0) {   // fewer entries than k in the list: all of them
+        prefix = 0ull;
+        shift = 63;
+        break;
+      }
       prefix = s_prefix;
       kk = s_kk;
-      const int done = s_done;
-      __syncthreads();
-      if (done) break;
+      if (s_done) break;
     }
-  }
-  // survivors: (key >> shift) >= prefix
-  if (tid == 0) s_cnt = 0;
-  skey[tid] = 0ull;
-  __syncthreads();
-  if (min(a.k, total) > 0) {
-    auto keep = [&](unsigned long long key) {
+    __syncthreads();
+    // survivors: (key >> shift) >= prefix
+    sweep([&](unsigned long long key) {
       if ((key >> shift) >= prefix && key != 0ull) {
         const int slot = atomicAdd(&s_cnt, 1);
         if (slot < 1024) skey[slot] = key;
       }
-    };
-    if (cached) {
-#pragma unroll
-      for (int u = 0; u < 16; ++u) keep(kc[u]);
-    } else {
-      for (int base = 0; base < total; base += 8 * blockDim.x) {
-        unsigned long long keys[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int i = base + u * blockDim.x + tid;
-          keys[u] = (i < total) ? key_at(i) : 0ull;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) keep(keys[u]);
-      }
-    }
+    });
   }
   __syncthreads();
   // bitonic sort, descending, of the smallest power of two that holds the survivors (the rest of skey is zero)
@@ -739,16 +852,12 @@ __global__ void __launch_bounds__(1024) select_kernel(SelArgs a) {
   }
   if (tid < a.k) {
     const unsigned long long key = skey[tid];
-    float s = -INFINITY;
-    int id = -1;
-    if (key != 0ull) {
-      uint32_t u = (uint32_t)(key >> 32);
-      u = (u & 0x80000000u) ? (u & 0x7fffffffu) : ~u;
-      s = __uint_as_float(u);
-      id = (int)(~(uint32_t)(key & 0xffffffffull));
+    const float s = key != 0ull ? key_score(key) : -INFINITY;
+    const int id = key != 0ull ? (int)(~(uint32_t)(key & 0xffffffffull)) : -1;
+    if (a.top_s != nullptr) {
+      a.top_s[(int64_t)q * a.k + tid] = s;
+      a.top_i[(int64_t)q * a.k + tid] = id;
     }
-    a.top_s[(int64_t)q * a.k + tid] = s;
-    a.top_i[(int64_t)q * a.k + tid] = id;
     if (tid == a.k - 1 && a.kth != nullptr) a.kth[q] = s;
   }
 }
@@ -791,9 +900,8 @@ cudaError_t launch_t(const CUtensorMap& mi, const CUtensorMap& mq, const ScanArg
     if (attr_dev < 64) attr[attr_dev].store(smem, std::memory_order_relaxed);
   }
   const int grid = (int)std::min<int64_t>(args.ntiles, tc::sm_count());
-  kern<<<grid, 32 * (NW + 1), smem, st>>>(mi, mq, args);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_dependent(kern, dim3((unsigned)grid), dim3(32 * (NW + 1)), smem, st, mi, mq, args);
 }
 
 template <int BM, bool PROD>
@@ -908,9 +1016,8 @@ int prepare(const tq_plan* plan, const float* Qcat, int nqp, void* workspace, cu
   for (int i = 0; i < 8; ++i) ba.alpha[i] = plan->ms.alpha[i];
   ba.out = bfrag;
   const int64_t total = (int64_t)c.NT * plan->ms.R * (ks_a(bm) + ks_s(prod)) * 32;
-  bprep_kernel<<<(unsigned)((total * 8 + 255) / 256), 256, 0, st>>>(ba);
   count_launches(1);
-  TQ_CHECK_CUDA(cudaGetLastError(), who);
+  TQ_CHECK_CUDA(launch_dependent(bprep_kernel, dim3((unsigned)((total * 8 + 255) / 256)), dim3(256), 0, st, ba), who);
   return TQ_OK;
 }
 
@@ -957,8 +1064,8 @@ int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8
 }
 
 cudaError_t select_topk(const float* cand_s, const int* cand_i, const int* count, int cap, int m, int id0, int nq, int k,
-                        int merge, float* top_s, int* top_i, float* kth, int* overflow, const int* run_if,
-                        cudaStream_t st) {
+                        int merge, float* top_s, int* top_i, float* kth, int* overflow, const int* run_if, int* clear_count,
+                        int* clear_flag, cudaStream_t st) {
   SelArgs a;
   a.cand_s = cand_s;
   a.cand_i = cand_i;
@@ -973,14 +1080,15 @@ cudaError_t select_topk(const float* cand_s, const int* cand_i, const int* count
   a.kth = kth;
   a.overflow = overflow;
   a.run_if = run_if;
-  select_kernel<<<nq, 1024, 0, st>>>(a);
+  a.clear_count = clear_count;
+  a.clear_flag = clear_flag;
   count_launches(1);
-  return cudaGetLastError();
+  return launch_dependent(select_kernel, dim3((unsigned)nq), dim3(1024), 0, st, a);
 }
 
 cudaError_t select_pairs(const float* cand_s, const int* cand_i, int ld, int m, int nq, int k, float* top_s, int* top_i,
                          cudaStream_t st) {
-  return select_topk(cand_s, cand_i, nullptr, ld, m, 0, nq, k, 0, top_s, top_i, nullptr, nullptr, nullptr, st);
+  return select_topk(cand_s, cand_i, nullptr, ld, m, 0, nq, k, 0, top_s, top_i, nullptr, nullptr, nullptr, nullptr, nullptr, st);
 }
 
 }  // namespace mscan

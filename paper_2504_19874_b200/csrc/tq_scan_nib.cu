@@ -68,8 +68,6 @@ struct PrepArgs {
 // Programmatic dependent launch: a kernel launched with the stream-serialisation attribute may start while its
 // predecessor in the stream still runs; it must pass this wait before touching anything the predecessor
 // writes or reads.  launch_dependents lets the successor's CTAs be scheduled as this grid's CTAs drain.
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Warp `ql` of every block derives the scales of query ql itself (a few thousand loads from L2, the same
 // values in the same order everywhere); block 0 publishes the constants the scan needs.
@@ -102,8 +100,8 @@ __device__ void query_scales(const PrepArgs& a, QScale* sc /* shared, [8] */) {
 
 __global__ void __launch_bounds__(256) nprep_kernel(PrepArgs a) {
   __shared__ QScale sc[8];
-  grid_dependency_wait();   // the rotated queries come from the kernel before; the operand may still be in use
-  grid_launch_dependents();
+  wait_for_predecessor();   // the rotated queries come from the kernel before; the operand may still be in use
+  allow_successor();
   query_scales(a, sc);
   const int KPB = a.tiled ? KPB_TILE : KPB_COL;
   const int total = a.nblocks * KPB * 32;
@@ -233,9 +231,10 @@ scan_nib_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
   constexpr int NT_Q = TILED ? 2 : 1;   // per sign-bit position
   constexpr int STAGE_BYTES = SB * BLOCK_BYTES;
 
+  allow_successor();
   // the switch may be written by the kernel before this one
   if (a.run_if != nullptr) {
-    grid_dependency_wait();
+    wait_for_predecessor();
     if (*a.run_if == 0) return;
   }
 
@@ -304,7 +303,7 @@ scan_nib_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
   }
 
   // ------------------------------------------------------------------ consumers
-  grid_dependency_wait();   // the query-side operand and constants are the previous kernel's output
+  wait_for_predecessor();   // the query-side operand and constants are the previous kernel's output
   {
     const uint4* src = reinterpret_cast<const uint4*>(a.Bfrag);
     uint4* dst = reinterpret_cast<uint4*>(Bs);

@@ -157,6 +157,8 @@ struct StatArgs {
 // Nibble layout: one warp per query, the same reductions in the same order as the register-fed engine's
 // (lane-strided maxima in fp32, the sum of q'' in fp64 folded by xor shuffles).
 __global__ void __launch_bounds__(32) tstats_nib_kernel(StatArgs a) {
+  allow_successor();
+  wait_for_predecessor();   // the queries are its output; what this kernel writes may still be read by it
   const int lane = threadIdx.x;
   const float* q = a.Qcat + (int64_t)blockIdx.x * a.ldq;
   float mx1 = 0.f, mx2 = 0.f;
@@ -187,6 +189,8 @@ __global__ void __launch_bounds__(32) tstats_nib_kernel(StatArgs a) {
 
 __global__ void __launch_bounds__(256) tstats_kernel(StatArgs a) {
   __shared__ double red[4][8];
+  allow_successor();
+  wait_for_predecessor();   // the queries are its output; what this kernel writes may still be read by it
   const float* q = a.Qcat + (int64_t)blockIdx.x * a.ldq;
   double mx1 = 0.0, sm1 = 0.0, mx2 = 0.0, sm2 = 0.0;
   for (int j = threadIdx.x; j < a.d; j += blockDim.x) {
@@ -251,93 +255,89 @@ struct BPrepArgs {
   uint8_t* Bs;
 };
 
-__device__ __forceinline__ int digit_of(long long J, int limb) {
-  int dg = 0;
-  for (int l = 0; l <= limb; ++l) {
-    dg = (int)(((J + 128) & 255) - 128);
-    J = (J - dg) >> 8;
-  }
-  return dg;
-}
+// 2^e as a double, e in the normal range.
+__device__ __forceinline__ double pow2_of(int e) { return __hiloint2double((e + 1023) << 20, 0); }
 
-__global__ void __launch_bounds__(256) tbprep_kernel(BPrepArgs a, int part, int rows) {
+// One thread per 32-bit word of B (four K-bytes) and query: the weights are formed once and leave as a word in each of the
+// three digit rows; a warp writes 128 contiguous bytes of each.  (A thread per 32 K-bytes and digit spent 12.6 us on its own
+// serial chain of fp64 operations, whatever the number of queries; now 2.3 us for 32 queries at d = 1536.)
+__global__ void __launch_bounds__(256) tbprep_kernel(BPrepArgs a, int part, int queries) {
+  allow_successor();
+  wait_for_predecessor();   // the queries are its output; what this kernel writes may still be read by it
   const int nkb = part ? a.g.kbs : a.g.kba;
-  const int64_t total = (int64_t)rows * nkb * 4;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= total) return;
-  const int wl = (int)(tid & 3);
-  const int kb = (int)((tid >> 2) % nkb);
-  const int row = (int)((tid >> 2) / nkb);      // pass * 96 + n
-  const int ql = (row / NCOL) * kQueriesPerPass + (row % NCOL) % kQueriesPerPass, limb = (row % NCOL) / kQueriesPerPass;
-  uint32_t out[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+  if (tid >= (int64_t)queries * nkb * 32) return;
+  const int wl = (int)(tid >> 3) & 3, k = (int)tid & 7;
+  const int kb = (int)((tid >> 5) % nkb), ql = (int)((tid >> 5) / nkb);
+  uint32_t out[LIMBS] = {0u, 0u, 0u};
   if (ql < a.nqg) {
     const float* q = a.Qcat + (int64_t)ql * a.ldq;
-    const QConst c = a.qc[ql];
-    for (int k = 0; k < 8; ++k) {
-      for (int i = 0; i < 4; ++i) {
-        const int bit = 8 * i + k;
-        double W = 0.0;
-        int f;
-        if (!part) {
-          const Slot s = slot_a(a.g, kb, wl, bit);
-          if (s.coord < a.g.d) W = 2.0 * a.alpha[s.term] * (double)q[s.coord];
-          f = c.fa;
-        } else {
-          const int j = 32 * (4 * kb + wl) + bit;
-          if (j < a.g.d) W = 2.0 * (double)q[a.g.dpad + j];
-          f = c.fs;
-        }
-        double Jd = rint(ldexp(W, f - k));
-        if (!(fabs(Jd) <= 8388608.0)) Jd = 0.0;   // non-finite query entries contribute nothing
-        out[k] |= (uint32_t)(digit_of((long long)Jd, limb) & 255) << (8 * i);
+    const double scale = pow2_of((part ? a.qc[ql].fs : a.qc[ql].fa) - k);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int bit = 8 * i + k;
+      double W = 0.0;
+      if (!part) {
+        const Slot s = slot_a(a.g, kb, wl, bit);
+        if (s.coord < a.g.d) W = 2.0 * a.alpha[s.term] * (double)q[s.coord];
+      } else {
+        const int j = 32 * (4 * kb + wl) + bit;
+        if (j < a.g.d) W = 2.0 * (double)q[a.g.dpad + j];
+      }
+      const double Jd = rint(W * scale);
+      int J = fabs(Jd) <= 8388608.0 ? (int)Jd : 0;   // non-finite query entries contribute nothing
+#pragma unroll
+      for (int l = 0; l < LIMBS; ++l) {
+        const int dg = ((J + 128) & 255) - 128;
+        J = (J - dg) >> 8;
+        out[l] |= (uint32_t)(dg & 255) << (8 * i);
       }
     }
   }
-  uint8_t* dst = (part ? a.Bs : a.Ba) + (size_t)row * nkb * KB_BYTES + (size_t)kb * KB_BYTES + wl * 32;
-  *reinterpret_cast<uint4*>(dst) = make_uint4(out[0], out[1], out[2], out[3]);
-  *reinterpret_cast<uint4*>(dst + 16) = make_uint4(out[4], out[5], out[6], out[7]);
+  const int row0 = ql / kQueriesPerPass * NCOL + ql % kQueriesPerPass;   // digit l of the query: row0 + 32 l
+  uint8_t* dst = (part ? a.Bs : a.Ba) + ((size_t)row0 * nkb + kb) * KB_BYTES + wl * 32 + k * 4;
+#pragma unroll
+  for (int l = 0; l < LIMBS; ++l) *reinterpret_cast<uint32_t*>(dst + (size_t)l * kQueriesPerPass * nkb * KB_BYTES) = out[l];
 }
 
 // Nibble layout: one B matrix Bn[pass*96 + n][3 nblk * 128]; k-block 3 b + type of block b.  K-byte kappa of an h or l
 // k-block <-> coordinate kappa of the block; of a sign k-block: register kappa / 4 = 2 word + parity, byte i = kappa % 4
 // <-> coordinate 8 word + 2 i + parity (low nibbles, parity 0, have the value 8 and carry 16 J; high nibbles 128 and J).
-__global__ void __launch_bounds__(256) tbprep_nib_kernel(BPrepArgs a, int rows) {
+// Threads as in tbprep_kernel.
+__global__ void __launch_bounds__(256) tbprep_nib_kernel(BPrepArgs a, int queries) {
+  allow_successor();
+  wait_for_predecessor();   // the queries are its output; what this kernel writes may still be read by it
   const int nkb = a.g.kba;
-  const int64_t total = (int64_t)rows * nkb * 4;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= total) return;
-  const int wl = (int)(tid & 3);
-  const int kb = (int)((tid >> 2) % nkb);
-  const int row = (int)((tid >> 2) / nkb);      // pass * 96 + n
-  const int ql = (row / NCOL) * kQueriesPerPass + (row % NCOL) % kQueriesPerPass, limb = (row % NCOL) / kQueriesPerPass;
+  if (tid >= (int64_t)queries * nkb * 32) return;
+  const int word = (int)tid & 31;               // of the k-block's 32
+  const int kb = (int)((tid >> 5) % nkb), ql = (int)((tid >> 5) / nkb);
   const int b = kb / 3, type = kb % 3;
-  uint32_t out[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+  uint32_t out[LIMBS] = {0u, 0u, 0u};
   if (ql < a.nqg) {
     const float* q = a.Qcat + (int64_t)ql * a.ldq;
     const QConst c = a.qc[ql];
     nib::QScale sc;
     sc.fh = c.fa;
     sc.sq = __hiloint2double(c.pad[1], c.pad[0]);
-    for (int r = 0; r < 8; ++r)
-      for (int i = 0; i < 4; ++i) {
-        const int kappa = 32 * wl + 4 * r + i;
-        int cib, mul = 1;
-        if (type < 2) {
-          cib = kappa;
-        } else {
-          const int reg = kappa >> 2;
-          cib = 8 * (reg >> 1) + 2 * i + (reg & 1);
-          mul = (reg & 1) ? 1 : 16;
-        }
-        const int coord = nib::coord_of_block(a.g.nbi, a.g.idx_rb, a.g.qjl_rb, a.g.d, b, cib);
-        if (coord < 0) continue;
-        const long long J = mul * nib::weight(sc, type, q[(type < 2 ? 0 : a.g.dpad) + coord]);
-        out[r] |= (uint32_t)(nib::digit_of(J, limb) & 255) << (8 * i);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      int cib = 4 * word + i, mul = 1;
+      if (type == 2) {
+        cib = 8 * (word >> 1) + 2 * i + (word & 1);
+        mul = (word & 1) ? 1 : 16;
       }
+      const int coord = nib::coord_of_block(a.g.nbi, a.g.idx_rb, a.g.qjl_rb, a.g.d, b, cib);
+      if (coord < 0) continue;
+      const long long J = mul * nib::weight(sc, type, q[(type < 2 ? 0 : a.g.dpad) + coord]);
+#pragma unroll
+      for (int l = 0; l < LIMBS; ++l) out[l] |= (uint32_t)(nib::digit_of(J, l) & 255) << (8 * i);
+    }
   }
-  uint8_t* dst = a.Ba + (size_t)row * nkb * KB_BYTES + (size_t)kb * KB_BYTES + wl * 32;
-  *reinterpret_cast<uint4*>(dst) = make_uint4(out[0], out[1], out[2], out[3]);
-  *reinterpret_cast<uint4*>(dst + 16) = make_uint4(out[4], out[5], out[6], out[7]);
+  const int row0 = ql / kQueriesPerPass * NCOL + ql % kQueriesPerPass;
+  uint8_t* dst = a.Ba + ((size_t)row0 * nkb + kb) * KB_BYTES + word * 4;
+#pragma unroll
+  for (int l = 0; l < LIMBS; ++l) *reinterpret_cast<uint32_t*>(dst + (size_t)l * kQueriesPerPass * nkb * KB_BYTES) = out[l];
 }
 
 // ------------------------------------------------------------------ scan kernel
@@ -398,7 +398,11 @@ template <int BM, int MODE, bool NIB = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
 scan_tc_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__ CUtensorMap tmBs,
                const __grid_constant__ CUtensorMap tmPa, const __grid_constant__ CUtensorMap tmPs, ScanArgs a) {
-  if (a.run_if != nullptr && *a.run_if == 0) return;
+  allow_successor();
+  if (a.run_if != nullptr) {
+    wait_for_predecessor();   // it may write the switch
+    if (*a.run_if == 0) return;
+  }
 
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -443,6 +447,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__
     if (a.g.kba > 0) tc::tma_prefetch_desc(&tmPa);
     if (a.g.kbs > 0) tc::tma_prefetch_desc(&tmPs);
   }
+  wait_for_predecessor();   // every input may be its output
   if (threadIdx.x < kQueriesPerPass) {
     QConst c = {1.f, 0.f, 1.f, 0.f, 0, 0, {0, 0}};
     if ((int)threadIdx.x < a.nqp) c = a.qc[threadIdx.x];
@@ -811,9 +816,8 @@ cudaError_t launch_t(const CUtensorMap& ma, const CUtensorMap& ms, const CUtenso
     if (attr_dev < 64) attr_devices.fetch_or(1ull << attr_dev, std::memory_order_relaxed);
   }
   const int grid = (int)std::min<int64_t>(args.npairs, tc::sm_count());
-  kern<<<grid, NTHREADS, kSmemBytes, st>>>(ma, ms, pa, ps, args);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_dependent(kern, dim3((unsigned)grid), dim3(NTHREADS), kSmemBytes, st, ma, ms, pa, ps, args);
 }
 
 template <int BM, int MODE, bool NIB, int CTAS>
@@ -830,23 +834,24 @@ cudaError_t launch_wide_c(const CUtensorMap& ma, const CUtensorMap& ms, const CU
   }
   count_launches(1);
   const int64_t ntiles = (args.n + TILE - 1) / TILE;
-  if (CTAS == 1) {
-    kern<<<(int)std::min<int64_t>(ntiles, tc::sm_count()), W_NTHREADS, kWideSmemBytes, st>>>(ma, ms, pa, ps, args);
-    return cudaGetLastError();
-  }
+  if (CTAS == 1)
+    return launch_dependent(kern, dim3((unsigned)std::min<int64_t>(ntiles, tc::sm_count())), dim3(W_NTHREADS), kWideSmemBytes, st, ma, ms, pa,
+                            ps, args);
   const int units = (int)std::min<int64_t>((ntiles + CTAS - 1) / CTAS, tc::sm_count() / CTAS);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(units * CTAS));
   cfg.blockDim = dim3(W_NTHREADS);
   cfg.dynamicSmemBytes = kWideSmemBytes;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = CTAS;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, ma, ms, pa, ps, args);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -924,10 +929,9 @@ int prepare_group(const tq_plan* plan, const float* Qcat, int nqg, void* workspa
   sa.nib = g.nib;
   sa.delta = plan->nb.delta;
   sa.out = qc;
-  if (g.nib) tstats_nib_kernel<<<nqg, 32, 0, st>>>(sa);
-  else tstats_kernel<<<nqg, 256, 0, st>>>(sa);
   count_launches(1);
-  TQ_CHECK_CUDA(cudaGetLastError(), who);
+  TQ_CHECK_CUDA(g.nib ? launch_dependent(tstats_nib_kernel, dim3((unsigned)nqg), dim3(32), 0, st, sa)
+                      : launch_dependent(tstats_kernel, dim3((unsigned)nqg), dim3(256), 0, st, sa), who);
   BPrepArgs ba;
   ba.Qcat = Qcat;
   ba.ldq = ncols;
@@ -937,22 +941,19 @@ int prepare_group(const tq_plan* plan, const float* Qcat, int nqg, void* workspa
   for (int i = 0; i < 8; ++i) ba.alpha[i] = plan->ms.alpha[i];
   ba.Ba = Ba;
   ba.Bs = Bs;
-  const int passes = (nqg + kQueriesPerPass - 1) / kQueriesPerPass;
-  const int rows = passes * NCOL;
+  const int queries = (nqg + kQueriesPerPass - 1) / kQueriesPerPass * kQueriesPerPass;   // absent ones get zero rows
   if (g.nib) {
-    const int64_t total = (int64_t)rows * g.kba * 4;
-    tbprep_nib_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(ba, rows);
+    const int64_t total = (int64_t)queries * g.kba * 32;
     count_launches(1);
-    TQ_CHECK_CUDA(cudaGetLastError(), who);
+    TQ_CHECK_CUDA(launch_dependent(tbprep_nib_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, ba, queries), who);
     return TQ_OK;
   }
   for (int part = 0; part < 2; ++part) {
     const int nkb = part ? g.kbs : g.kba;
     if (nkb == 0) continue;
-    const int64_t total = (int64_t)rows * nkb * 4;
-    tbprep_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(ba, part, rows);
+    const int64_t total = (int64_t)queries * nkb * 32;
     count_launches(1);
-    TQ_CHECK_CUDA(cudaGetLastError(), who);
+    TQ_CHECK_CUDA(launch_dependent(tbprep_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, ba, part, queries), who);
   }
   return TQ_OK;
 }

@@ -97,7 +97,11 @@ template <int BM, int MODE, bool NIB, int CTAS>
 __global__ void __launch_bounds__(W_NTHREADS, 1)
 scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__ CUtensorMap tmBs,
                 const __grid_constant__ CUtensorMap tmPa, const __grid_constant__ CUtensorMap tmPs, ScanArgs a) {
-  if (a.run_if != nullptr && *a.run_if == 0) return;
+  allow_successor();
+  if (a.run_if != nullptr) {
+    wait_for_predecessor();   // it may write the switch
+    if (*a.run_if == 0) return;
+  }
   // B ring of this CTA: a CTA of a pair holds half of every box, so the same shared memory gives twice the stages --
   // the boxes arrive ~2500 cycles after they are requested (all SMs read the same lines of L2 at about the same time),
   // and the number of boxes in flight, not the bytes, sets the rate at which they arrive
@@ -162,6 +166,7 @@ scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant_
     if (a.g.kba > 0) tc::tma_prefetch_desc(&tmPa);
     if (a.g.kbs > 0) tc::tma_prefetch_desc(&tmPs);
   }
+  wait_for_predecessor();   // every input may be its output
   if (threadIdx.x < W_QPP) {
     QConst c = {1.f, 0.f, 1.f, 0.f, 0, 0, {0, 0}};
     if ((int)threadIdx.x < a.nqp) c = a.qc[threadIdx.x];

@@ -1,0 +1,45 @@
+"""The selection kernel at the limits of its two methods: lists around the register limit, ties, a far outlier that leaves all
+other scores in one bin, non-finite scores, empty slots.  Order and ids are exact: descending score, then ascending id."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2504_19874_b200 as tq
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def expected(s, i, k):
+    keep = np.nonzero(i >= 0)[0]
+    order = keep[np.lexsort((i[keep], -s[keep].astype(np.float64)))][:k]
+    out_s, out_i = np.full(k, -np.inf, np.float32), np.full(k, -1, np.int32)
+    out_s[:order.size], out_i[:order.size] = s[order], i[order]
+    return out_s, out_i
+
+
+@pytest.mark.parametrize("m", [1, 31, 1000, 1025, 16384, 16385, 40000])
+@pytest.mark.parametrize("kind", ["normal", "ties", "equal", "outlier", "infinite", "empty slots"])
+def test_selection(m, kind):
+    g = np.random.default_rng(m)
+    nq = 3
+    s = g.standard_normal((nq, m)).astype(np.float32)
+    if kind == "ties":
+        s = np.round(s, 1)
+        s[s == 0] = 0.0
+    elif kind == "equal":
+        s[:] = 0.25
+    elif kind == "outlier":
+        s[:, m // 2] = 1e30
+    elif kind == "infinite":
+        s[0, 0], s[1, m - 1] = np.inf, -np.inf
+    ids = np.stack([g.permutation(m) for _ in range(nq)]).astype(np.int32)
+    if kind == "empty slots":
+        ids[g.random((nq, m)) < 0.9] = -1
+    cs, ci = torch.from_numpy(s).to(DEV), torch.from_numpy(ids).to(DEV)
+    for k in (1, 10, 1024):
+        ts, ti = torch.empty((nq, k), device=DEV), torch.empty((nq, k), dtype=torch.int32, device=DEV)
+        tq.tq_select_topk(cs, ci, k, ts, ti)
+        for q in range(nq):
+            ws, wi = expected(s[q], ids[q], k)
+            assert np.array_equal(ti[q].cpu().numpy(), wi) and np.array_equal(ts[q].cpu().numpy(), ws), (q, k)
