@@ -103,10 +103,8 @@ constexpr int64_t kFilterMinN = 65536;
 constexpr int64_t kDenseRowsMin = 4096;
 constexpr int kGroupQueries = tscan::kQueriesPerPass * tscan::kPassesPerGroup;
 
-// The two engines behind the bit-plane scan: register-fed integer MMA (2 or 4 queries per pass) for few
-// queries, tcgen05 (32 queries per pass, 64 in calls of more than 32 queries) from 7 queries on (measured at d = 1536, b = 4, n = 10^6: a short
-// tcgen05 pass 0.69 ms, register-fed passes 0.24 ms for 1-2 queries and 0.37 ms for 3-4, so 4 + 3 queries
-// already cost more).
+// The two engines behind the bit-plane scan: register-fed integer MMA (2, 4 or 8 queries per pass) for few queries, tcgen05
+// (32 queries per pass, 64 in calls of more than 32 queries) for more.
 struct ScanEngine {
   const tq_plan* plan;
   bool tc;
@@ -123,12 +121,17 @@ ScanEngine pick_engine(const tq_plan* plan, int nq) {
   // nibble layout (measured at n = 10^6): at d = 1536 a tcgen05 pass costs 0.53 ms against 0.28 ms per pass of the
   // eight-query register-fed shape, so it wins from 15 queries on; where that shape does not fit shared memory
   // (d = 3072: 0.84 ms against 0.35 ms per two-query pass) from five queries on
-  const int tc_from = !e.nib ? 7 : nscan::queries_per_pass(plan, 8) == 8 ? 15 : 5;
+  // bit streams: a tcgen05 pass costs the same for any number of queries up to 32; the register-fed eight-query shape, where
+  // its operand fits shared memory, is cheaper up to eight (whole calls of 8 queries, 10^6 rows: d = 1536 mse b = 2 207 against
+  // 301 us, prod b = 3 309 against 440, d = 1024 prod b = 4 336 against 487, d = 200 prod b = 3 93 against 148); two passes of it
+  // are not (9 queries and more).  Where only the four-query shape fits (prod b = 4 and mse b = 4 at d = 1536), 4 + 3 queries
+  // already cost more than a tcgen05 pass.
+  const int tc_from = e.nib ? (nscan::queries_per_pass(plan, 8) == 8 ? 15 : 5) : mscan::queries_per_pass(plan, 8) == 8 ? 9 : 7;
   e.tc = nq >= tc_from && tscan::available(plan);
   e.nib = e.nib && !e.tc;
   e.qpp = e.tc ? tscan::queries_per_pass(nq) : e.nib ? nscan::queries_per_pass(plan, nq) : mscan::queries_per_pass(plan, nq);
   e.dense_rows_pref = 1 << 20;   // n = 10^6: the guarded rescue is one scan + one selection launch per pass
-  e.ws_bytes = e.tc ? tscan::workspace_bytes(plan) : e.nib ? nscan::workspace_bytes(plan) : mscan::workspace_bytes(plan);
+  e.ws_bytes = e.tc ? tscan::workspace_bytes(plan) : e.nib ? nscan::workspace_bytes(plan) : mscan::workspace_bytes(plan, nq);
   return e;
 }
 
@@ -865,7 +868,7 @@ static bool engine_that_fits(const tq_plan* plan, int nq, size_t avail, ScanEngi
   *out = pick_engine(plan, nq);
   if (align_up(out->ws_bytes, 256) <= avail) return true;
   if (!out->tc) return false;
-  *out = pick_engine(plan, std::min(nq, 6));
+  *out = pick_engine(plan, std::min(nq, 4));
   return align_up(out->ws_bytes, 256) <= avail;
 }
 

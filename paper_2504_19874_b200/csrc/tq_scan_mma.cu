@@ -44,7 +44,7 @@ namespace {
 constexpr int LIMBS = 4;                    // signed radix-256 digits per B value
 constexpr int MAX_STAGES = 6;
 constexpr int SMEM_LIMIT = 227 * 1024;
-constexpr size_t kQConstBytes = 256;        // room for the per-query constants of one pass (4 x 48 bytes)
+constexpr size_t kQConstBytes = 256;        // room for the per-query constants of one pass (8 x 32 bytes)
 
 __host__ __device__ constexpr int idx_words(int bm) { return 4 * bm; }
 __host__ __device__ constexpr int der_words(int bm) { return bm == 3 ? 4 : (bm == 4 ? 16 : 0); }
@@ -106,14 +106,15 @@ struct BPrepArgs {
   uint2* out;          // [NT][R][KS][32]
 };
 
-constexpr int kMaxPassQueries = 4;
+constexpr int kMaxPassQueries = 8;
+constexpr int kTiledNT = 3;   // column tiles of the eight-query shape: tile l holds digit l of the eight queries
 
-// Per-query scale and constants.  Every block derives them itself (a few thousand loads from L2),
-// in the same order, so that no separate launch is needed; block 0 publishes them for the scan.
-__device__ void query_constants(const BPrepArgs& a, QConst* sc /* shared, [kMaxPassQueries] */) {
+// Per-query scale and constants of queries [first, last).  Up to four queries every block of bprep_kernel derives them itself
+// (a few thousand loads from L2, in the same order), so that no separate launch is needed; `publish` writes them for the scan.
+__device__ void query_constants(const BPrepArgs& a, QConst* sc /* shared, [kMaxPassQueries] */, int first, int last, bool publish) {
   __shared__ double red[4][8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int ql = 0; ql < a.nq_pass; ++ql) {
+  for (int ql = first; ql < last; ++ql) {
     const float* q = a.Qcat + (int64_t)ql * a.ldq;
     double mx1 = 0.0, sm1 = 0.0, mx2 = 0.0, sm2 = 0.0;
     for (int j = threadIdx.x; j < a.d; j += blockDim.x) {
@@ -160,7 +161,7 @@ __device__ void query_constants(const BPrepArgs& a, QConst* sc /* shared, [kMaxP
       c.cs = (float)(-sm2);
       c.pad[0] = c.pad[1] = 0;
       sc[ql] = c;
-      if (blockIdx.x == 0) a.qc[ql] = c;
+      if (publish) a.qc[ql] = c;
     }
     __syncthreads();
   }
@@ -181,13 +182,27 @@ __device__ __forceinline__ int digit_of(long long J, int limb) {
   return dg;
 }
 
+// The same with a block per query, for the eight-query shape.
+__global__ void __launch_bounds__(256) query_constants_kernel(BPrepArgs a) {
+  __shared__ QConst sc[kMaxPassQueries];
+  allow_successor();
+  wait_for_predecessor();
+  query_constants(a, sc, blockIdx.x, blockIdx.x + 1, true);
+}
+
 // One thread per output byte (8 per uint2 element): the chain of fp64 and index arithmetic behind a digit is
 // long, and this kernel sits in front of every scan call; the 8 bytes meet by a shuffle-OR.
 __global__ void __launch_bounds__(256) bprep_kernel(BPrepArgs a) {
   __shared__ QConst sc[kMaxPassQueries];
   allow_successor();
   wait_for_predecessor();   // the rotated queries are its output; the operand may still be read by it
-  query_constants(a, sc);
+  const bool tiled = a.NT == kTiledNT;
+  if (!tiled) {
+    query_constants(a, sc, 0, a.nq_pass, blockIdx.x == 0);
+  } else {   // query_constants_kernel has written them
+    if ((int)threadIdx.x < a.nq_pass) sc[threadIdx.x] = a.qc[threadIdx.x];
+    __syncthreads();
+  }
   const int ksa = ks_a(a.bm), kss = ks_s(a.prod != 0), KS = ksa + kss;
   const int64_t total = (int64_t)a.NT * a.R * KS * 32;
   const int64_t tid8 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -199,7 +214,7 @@ __global__ void __launch_bounds__(256) bprep_kernel(BPrepArgs a) {
   const int r = (int)((tid >> 5) / KS % a.R);
   const int nt = (int)((tid >> 5) / KS / a.R);
   const int g = lane >> 2, t4 = lane & 3;
-  const int col = nt * 8 + g, ql = col / LIMBS, limb = col % LIMBS;
+  const int col = nt * 8 + g, ql = tiled ? g : col / LIMBS, limb = tiled ? nt : col % LIMBS;
   uint32_t out[2] = {0u, 0u};
   if (ql < a.nq_pass) {
     const float* q = a.Qcat + (int64_t)ql * a.ldq;
@@ -289,7 +304,9 @@ scan_mma_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
   constexpr int STAGE_BYTES = NBLK * VT * 64;
   constexpr int NI = idx_words(BM), WA = a_words(BM);
   constexpr int KSA = ks_a(BM), KSS = ks_s(PROD), KS = KSA + KSS;
-  constexpr int NQP = NT * 8 / LIMBS;              // queries per pass
+  constexpr bool TILED = NT == kTiledNT;           // a query's digits in the column tiles, eight queries
+  constexpr int NQP = TILED ? 8 : NT * 8 / LIMBS;  // queries per pass
+  constexpr int NCH = TILED ? 1 : 2;               // accumulator chains per column tile (three tiles are chains enough)
 
   allow_successor();
   if (a.run_if != nullptr) {
@@ -372,36 +389,41 @@ scan_mma_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
   bool ok = true;
   // Per-row scalars of the epilogue (nu, coef * gamma), requested one tile ahead: with short rows (d = 200: one
   // pipeline step per tile) a request made at the top of its own tile is still in flight when the epilogue needs it.
-  float nu_next[MT], gm_next[MT];
+  constexpr int NRW = TILED ? 2 : 1;   // rows whose estimates this thread forms per tile of 16: g and g + 8, or one of them
+  float nu_next[MT][NRW], gm_next[MT][NRW];
   auto request_scalars = [&](int64_t tile) {
 #pragma unroll
-    for (int m = 0; m < MT; ++m) {
-      const int64_t row = tile * VT + cw * (MT * 16) + m * 16 + g + ((t4 & 1) ? 8 : 0);
-      const bool in = row < a.n;   // (also false for a tile past the last)
-      nu_next[m] = (in && a.norms != nullptr) ? __ldg(a.norms + row) : 1.f;
-      gm_next[m] = (PROD && in) ? __ldg(a.gamma + row) : 0.f;   // multiplied by coef where it is used: no wait here
-    }
+    for (int m = 0; m < MT; ++m)
+#pragma unroll
+      for (int h = 0; h < NRW; ++h) {
+        const int64_t row = tile * VT + cw * (MT * 16) + m * 16 + g + ((TILED ? h != 0 : (t4 & 1) != 0) ? 8 : 0);
+        const bool in = row < a.n;   // (also false for a tile past the last)
+        nu_next[m][h] = (in && a.norms != nullptr) ? __ldg(a.norms + row) : 1.f;
+        gm_next[m][h] = (PROD && in) ? __ldg(a.gamma + row) : 0.f;   // multiplied by coef where it is used: no wait here
+      }
   };
   constexpr bool AHEAD = (NT == 1);   // with two column tiles the longer tile hides the request and the registers cost more
   if (AHEAD) request_scalars(blockIdx.x);
   for (int64_t tile = blockIdx.x; tile < a.ntiles && ok; tile += gridDim.x) {
-    int accA[MT][NT][2][4], accS[MT][NT][2][4];
+    int accA[MT][NT][NCH][4], accS[MT][NT][NCH][4];
 #pragma unroll
     for (int m = 0; m < MT; ++m)
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-        for (int e = 0; e < 2; ++e)
+        for (int e = 0; e < NCH; ++e)
 #pragma unroll
           for (int i = 0; i < 4; ++i) accA[m][nt][e][i] = accS[m][nt][e][i] = 0;
 
-    float nu_pre[MT], gm_pre[MT];
+    float nu_pre[MT][NRW], gm_pre[MT][NRW];
     if (!AHEAD) request_scalars(tile);
 #pragma unroll
-    for (int m = 0; m < MT; ++m) {
-      nu_pre[m] = nu_next[m];
-      gm_pre[m] = gm_next[m];
-    }
+    for (int m = 0; m < MT; ++m)
+#pragma unroll
+      for (int h = 0; h < NRW; ++h) {
+        nu_pre[m][h] = nu_next[m][h];
+        gm_pre[m][h] = gm_next[m][h];
+      }
     if (AHEAD) request_scalars(tile + gridDim.x);
 
     for (int r = 0; r < a.R; ++r) {
@@ -494,7 +516,7 @@ scan_mma_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
             const uint32_t a2 = (k == 7) ? w[m][0][2 * p + 1] : (w[m][0][2 * p + 1] & mk);
             const uint32_t a3 = (k == 7) ? w[m][1][2 * p + 1] : (w[m][1][2 * p + 1] & mk);
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) mma_u8s8(accA[m][nt][k & 1], a0, a1, a2, a3, b[nt].x, b[nt].y);
+            for (int nt = 0; nt < NT; ++nt) mma_u8s8(accA[m][nt][k % NCH], a0, a1, a2, a3, b[nt].x, b[nt].y);
           }
         }
       }
@@ -517,7 +539,7 @@ scan_mma_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
               const uint32_t a2 = (k == 7) ? z[m][0][2 * p + 1] : (z[m][0][2 * p + 1] & mk);
               const uint32_t a3 = (k == 7) ? z[m][1][2 * p + 1] : (z[m][1][2 * p + 1] & mk);
 #pragma unroll
-              for (int nt = 0; nt < NT; ++nt) mma_u8s8(accS[m][nt][k & 1], a0, a1, a2, a3, b[nt].x, b[nt].y);
+              for (int nt = 0; nt < NT; ++nt) mma_u8s8(accS[m][nt][k % NCH], a0, a1, a2, a3, b[nt].x, b[nt].y);
             }
           }
       }
@@ -525,47 +547,68 @@ scan_mma_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
     if (!ok) break;
 
     // ---------------------------------------------------------------- epilogue
-    // Thread (g, t4) holds columns 2 t4, 2 t4 + 1 of rows g and g + 8: two of the four digits of
-    // query t4 / 2.  The digit sums are recombined exactly (T = D0 + 256 D1 + 65536 D2 + ... as a 64-bit
-    // integer, the same T in both engines although their digit sums differ), then everything is fp32: one
-    // rounding of T (2^-24 of sum |W|, three orders below the tolerance) and three FMAs.  The even lane of a
-    // pair finishes row g, the odd lane row g + 8: one 64-bit shuffle hands each the other's half.
+    auto emit = [&](int64_t row, int ql, float est) {
+      if (row >= a.n || ql >= a.nq_pass) return;
+      if (MODE == 0) {
+        if (TQ_DEVICE_CHECK(row >= 0 && row < a.n && row < a.lds, a.status)) a.scores[(int64_t)ql * a.lds + row] = est;
+      } else if (est >= __ldg(a.tau + ql)) {
+        const int slot = atomicAdd(a.count + ql, 1);
+        if (slot < a.cap) {
+          a.cand_s[(int64_t)ql * a.cap + slot] = est;
+          a.cand_i[(int64_t)ql * a.cap + slot] = (int)row;
+        }
+      }
+    };
+    if constexpr (TILED) {
+      // Thread (g, t4) holds all digits of queries 2 t4, 2 t4 + 1 for rows g and g + 8.  The same exact T as below.
 #pragma unroll
-    for (int m = 0; m < MT; ++m) {
-      const int64_t row0 = tile * VT + cw * (MT * 16) + m * 16;
-      const int64_t row = row0 + g + ((t4 & 1) ? 8 : 0);
-      const bool row_ok = row < a.n;
-      const float nu = nu_pre[m], gm = PROD ? a.coef * gm_pre[m] : 0.f;
+      for (int m = 0; m < MT; ++m)
 #pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        auto combine = [&](const int (&acc)[2][4]) -> float {
-          long long mine[2];
+        for (int h = 0; h < 2; ++h) {
+          const int64_t row = tile * VT + cw * (MT * 16) + m * 16 + g + 8 * h;
+          const float nu = nu_pre[m][h], gm = PROD ? a.coef * gm_pre[m][h] : 0.f;
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {   // digits (0, 1) on the even lane, (2, 3) on the odd lane, as one integer
-            const int lo = acc[0][2 * h] + acc[1][2 * h], hi = acc[0][2 * h + 1] + acc[1][2 * h + 1];
-            mine[h] = (long long)hi * 256 + lo;
+          for (int c2 = 0; c2 < 2; ++c2) {
+            auto whole = [&](const int (&acc)[NT][NCH][4]) -> float {
+              const int at = 2 * h + c2;
+              return (float)(((long long)acc[2][0][at] * 256 + acc[1][0][at]) * 256 + acc[0][0][at]);
+            };
+            const QConst c = qcs[2 * t4 + c2];
+            const float av = (BM > 0) ? fmaf(whole(accA[m]), c.sa, c.ca) : 0.f;
+            const float sv = PROD ? fmaf(whole(accS[m]), c.ss, c.cs) : 0.f;
+            emit(row, 2 * t4 + c2, __fmul_rn(nu, fmaf(gm, sv, av)));
           }
-          const long long recv = shfl_xor_ll((t4 & 1) ? mine[0] : mine[1], 1);
-          const long long T = (t4 & 1) ? mine[1] * 65536 + recv : recv * 65536 + mine[0];
-          return (float)T;   // one rounding of the exact integer: the same value in both engines
-        };
-        const float Ta = combine(accA[m][nt]);
-        const float Ts = PROD ? combine(accS[m][nt]) : 0.f;
-        const int ql = nt * 2 + (t4 >> 1);
-        const QConst c = qcs[ql];
-        const float av = (BM > 0) ? fmaf(Ta, c.sa, c.ca) : 0.f;
-        const float sv = PROD ? fmaf(Ts, c.ss, c.cs) : 0.f;
-        const float est = __fmul_rn(nu, fmaf(gm, sv, av));
-        if (row_ok && ql < a.nq_pass) {
-          if (MODE == 0) {
-            if (TQ_DEVICE_CHECK(row >= 0 && row < a.n && row < a.lds, a.status)) a.scores[(int64_t)ql * a.lds + row] = est;
-          } else if (est >= __ldg(a.tau + ql)) {
-            const int slot = atomicAdd(a.count + ql, 1);
-            if (slot < a.cap) {
-              a.cand_s[(int64_t)ql * a.cap + slot] = est;
-              a.cand_i[(int64_t)ql * a.cap + slot] = (int)row;
+        }
+    } else {
+      // Thread (g, t4) holds columns 2 t4, 2 t4 + 1 of rows g and g + 8: two of the four digits of
+      // query t4 / 2.  The digit sums are recombined exactly (T = D0 + 256 D1 + 65536 D2 + ... as a 64-bit
+      // integer, the same T in both engines although their digit sums differ), then everything is fp32: one
+      // rounding of T (2^-24 of sum |W|, three orders below the tolerance) and three FMAs.  The even lane of a
+      // pair finishes row g, the odd lane row g + 8: one 64-bit shuffle hands each the other's half.
+#pragma unroll
+      for (int m = 0; m < MT; ++m) {
+        const int64_t row = tile * VT + cw * (MT * 16) + m * 16 + g + ((t4 & 1) ? 8 : 0);
+        const float nu = nu_pre[m][0], gm = PROD ? a.coef * gm_pre[m][0] : 0.f;
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+          auto combine = [&](const int (&acc)[NCH][4]) -> float {
+            long long mine[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {   // digits (0, 1) on the even lane, (2, 3) on the odd lane, as one integer
+              const int lo = acc[0][2 * h] + acc[NCH - 1][2 * h], hi = acc[0][2 * h + 1] + acc[NCH - 1][2 * h + 1];
+              mine[h] = (long long)hi * 256 + lo;
             }
-          }
+            const long long recv = shfl_xor_ll((t4 & 1) ? mine[0] : mine[1], 1);
+            const long long T = (t4 & 1) ? mine[1] * 65536 + recv : recv * 65536 + mine[0];
+            return (float)T;   // one rounding of the exact integer: the same value in both engines
+          };
+          const float Ta = combine(accA[m][nt]);
+          const float Ts = PROD ? combine(accS[m][nt]) : 0.f;
+          const int ql = nt * 2 + (t4 >> 1);
+          const QConst c = qcs[ql];
+          const float av = (BM > 0) ? fmaf(Ta, c.sa, c.ca) : 0.f;
+          const float sv = PROD ? fmaf(Ts, c.ss, c.cs) : 0.f;
+          emit(row, ql, __fmul_rn(nu, fmaf(gm, sv, av)));
         }
       }
     }
@@ -602,25 +645,55 @@ __device__ __forceinline__ float key_score(unsigned long long key) {
   return __uint_as_float(u);
 }
 
+// Four entries of a query's list, positions base + u * 1024 + tid (0 past its end): the candidates, then the previous best list.
+__device__ __noinline__ void fetch_keys(const SelArgs& a, int q, int m_new, int total, int base, unsigned long long (&key)[4]) {
+  const float* src_s = a.cand_s + (int64_t)q * a.cap;
+  const int* src_i = a.cand_i ? a.cand_i + (int64_t)q * a.cap : nullptr;
+  float s[4];
+  int id[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {   // all loads in flight before the first use
+    const int i = base + u * 1024 + (int)threadIdx.x;
+    s[u] = 0.f;
+    id[u] = -1;
+    if (i < m_new) {
+      s[u] = src_s[i];
+      id[u] = src_i ? src_i[i] : a.id0 + i;
+    } else if (i < total) {
+      s[u] = a.top_s[(int64_t)q * a.k + i - m_new];
+      id[u] = a.top_i[(int64_t)q * a.k + i - m_new];
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) key[u] = id[u] < 0 ? 0ull : make_key(s[u], id[u]);   // a negative id is an empty slot
+}
+
 // One CTA per query: the k largest keys, sorted.
 // Usual case: the scores are counted in kSelBins equal steps between their minimum and maximum; the bin that holds the k-th
 // largest is found by a suffix sum, and everything in it and above is sorted (scores of a search thin out towards the top, so
-// that is hardly more than k).  Three sweeps over the list; lists of up to 16,384 entries stay in registers.  If more than
-// 1024 entries would have to be sorted (ties, a few far outliers) or a score is not finite, a radix select over the key's
-// bytes does the job (up to eight sweeps, each with lane-matching and a histogram of its own: 20 us for 15,616 scores
-// against 15).
+// that is hardly more than k).  Three sweeps over the list; lists of up to kSelCached entries stay in shared memory.  If more
+// than 1024 entries would have to be sorted (ties, a few far outliers) or a score is not finite, a radix select over the key's
+// bytes does the job.
+// Bound: latency -- a chain of some fifteen barriers, and above all the fetch of the kernel's own instructions, which the scan
+// ahead has driven out of the caches.  So the sweeps are short loops: with the list in registers and every sweep unrolled
+// sixteen times the same algorithm took 15 us for 2,441 candidates, a third of it in instruction fetches.
 constexpr int kSelBins = 2048;
+constexpr int kSelCached = 16384;
 __global__ void __launch_bounds__(1024) select_kernel(SelArgs a) {
+  extern __shared__ unsigned long long scache[];   // [kSelCached]
   __shared__ int hist[kSelBins];
   __shared__ unsigned long long s_prefix;
   __shared__ int s_kk, s_done, s_cnt;
   __shared__ unsigned long long skey[1024];
   __shared__ float wmin[32], wmax[32];
   __shared__ int wsum[32];
+  const int q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   allow_successor();
+  if (tid == 0) s_cnt = 0;
+  skey[tid] = 0ull;
+  hist[tid] = hist[tid + 1024] = 0;
   wait_for_predecessor();   // all inputs are outputs of kernels ahead in the stream
   if (a.run_if != nullptr && *a.run_if == 0) return;
-  const int q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (a.clear_count != nullptr && tid == 0) {   // the candidate counters of the pass that follows
     a.clear_count[q] = 0;
     if (q == 0) *a.clear_flag = 0;
@@ -632,71 +705,49 @@ __global__ void __launch_bounds__(1024) select_kernel(SelArgs a) {
     if (a.overflow != nullptr && c > a.cap && tid == 0) atomicExch(a.overflow, 1);
   }
   const int total = m_new + (a.merge ? a.k : 0);
-  const float* src_s = a.cand_s + (int64_t)q * a.cap;
-  const int* src_i = a.cand_i ? a.cand_i + (int64_t)q * a.cap : nullptr;
-  auto key_at = [&](int i) -> unsigned long long {
-    if (i < m_new) {
-      const int id = src_i ? src_i[i] : a.id0 + i;
-      return id < 0 ? 0ull : make_key(src_s[i], id);
-    }
-    const int j = i - m_new;
-    const int id = a.top_i[(int64_t)q * a.k + j];
-    if (id < 0) return 0ull;   // an empty slot of the previous list
-    return make_key(a.top_s[(int64_t)q * a.k + j], id);
-  };
-  // up to 16 keys per thread stay in registers for all rounds (lists up to 16,384 entries)
-  const bool cached = total <= 16 * 1024;
-  unsigned long long kc[16];
-  if (cached) {
-#pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int i = u * 1024 + tid;
-      kc[u] = (i < total) ? key_at(i) : 0ull;
-    }
-  }
-  // f(key) for every entry of the list (0 where there is none), all threads of a warp together
+  const bool cached = total <= kSelCached;
+  const int k_target = min(a.k, total);
+  // f(key) for every entry of the list (0 past its end), all threads of a warp together
   auto sweep = [&](auto&& f) {
     if (cached) {
-#pragma unroll
-      for (int u = 0; u < 16; ++u)
-        if (u * 1024 < total) f(kc[u]);
+#pragma unroll 1
+      for (int i0 = 0; i0 < total; i0 += 1024) f(i0 + tid < total ? scache[i0 + tid] : 0ull);
     } else {
-      // batches of 8 independent loads per thread, then the (convergent) uses
-      for (int base = 0; base < total; base += 8 * 1024) {
-        unsigned long long keys[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int i = base + u * 1024 + tid;
-          keys[u] = (i < total) ? key_at(i) : 0ull;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) f(keys[u]);
+#pragma unroll 1
+      for (int base = 0; base < total; base += 4096) {
+        unsigned long long key[4];
+        fetch_keys(a, q, m_new, total, base, key);
+#pragma unroll 1
+        for (int u = 0; u < 4; ++u) f(u == 0 ? key[0] : u == 1 ? key[1] : u == 2 ? key[2] : key[3]);
       }
     }
   };
-  const int k_target = min(a.k, total);
-  bool sorted_set = false;   // skey holds the survivors
-  if (tid == 0) s_cnt = 0;
-  skey[tid] = 0ull;
-  if (k_target > 0) {
-    // ---- range of the scores
-    float mn = INFINITY, mx = -INFINITY;
-    int odd = 0;
-    sweep([&](unsigned long long key) {
-      if (key != 0ull) {
-        const float v = key_score(key);
+  // ---- range of the scores; the list to shared memory on the way
+  float mn = INFINITY, mx = -INFINITY;
+  int odd = 0;
+#pragma unroll 1
+  for (int base = 0; base < total; base += 4096) {
+    unsigned long long key[4];
+    fetch_keys(a, q, m_new, total, base, key);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = base + u * 1024 + tid;
+      if (cached && i < total) scache[i] = key[u];
+      if (key[u] != 0ull) {
+        const float v = key_score(key[u]);
         odd |= !(fabsf(v) <= FLT_MAX);
         mn = fminf(mn, v);
         mx = fmaxf(mx, v);
       }
-    });
+    }
+  }
+  auto block_range = [&]() {   // over the block, for every thread; the barrier also publishes the list
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     }
     if (lane == 0) { wmin[warp] = mn; wmax[warp] = mx; }
-    for (int b = tid; b < kSelBins; b += 1024) hist[b] = 0;
     odd = __syncthreads_or(odd);
     mn = wmin[lane];
     mx = wmax[lane];
@@ -705,71 +756,62 @@ __global__ void __launch_bounds__(1024) select_kernel(SelArgs a) {
       mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     }
-    const float scale = (float)kSelBins / (mx - mn);
-    if (!odd && mx > mn && scale <= FLT_MAX) {
-      // the bin of a score never decreases with the score: subtraction, product and truncation round monotonically
-      auto bin_of = [&](unsigned long long key) { return min(kSelBins - 1, (int)((key_score(key) - mn) * scale)); };
+  };
+  block_range();
+  bool sorted_set = k_target == 0;   // skey holds the survivors
+  const float scale = (float)kSelBins / (mx - mn);
+  if (!sorted_set && !odd && mx > mn && scale <= FLT_MAX) {
+    // the bin of a score never decreases with the score: subtraction, product and truncation round monotonically
+    const float lowest = mn;
+    auto bin_of = [&](unsigned long long key) { return min(kSelBins - 1, (int)((key_score(key) - lowest) * scale)); };
+    sweep([&](unsigned long long key) {
+      if (key != 0ull) atomicAdd(&hist[bin_of(key)], 1);
+    });
+    __syncthreads();
+    // thread t owns bins B - 1 - 2 t and B - 2 - 2 t: counts from the top by a block-wide prefix sum
+    const int hi = hist[kSelBins - 1 - 2 * tid], lo = hist[kSelBins - 2 - 2 * tid];
+    int incl = hi + lo;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    const int before = __reduce_add_sync(0xffffffffu, lane < warp ? wsum[lane] : 0), all = __reduce_add_sync(0xffffffffu, wsum[lane]);
+    const int above = before + incl - hi - lo;   // entries in higher bins than this thread's
+    if (above < k_target && above + hi + lo >= k_target) {   // the k-th largest is in one of this thread's bins
+      const bool first = above + hi >= k_target;
+      s_kk = kSelBins - (first ? 1 : 2) - 2 * tid;
+      s_done = above + hi + (first ? 0 : lo);                // entries to sort
+    }
+    __syncthreads();
+    const bool few = all < k_target;   // fewer entries than k (empty slots in the list): all of them
+    const int cut = few ? 0 : s_kk;
+    if (a.top_s == nullptr && !few) {
+      // only a lower bound of the k-th score is wanted: the smallest score in the bins from that of the k-th on
+      mn = INFINITY;
       sweep([&](unsigned long long key) {
-        if (key != 0ull) atomicAdd(&hist[bin_of(key)], 1);
+        if (key != 0ull && bin_of(key) >= cut) mn = fminf(mn, key_score(key));
       });
-      __syncthreads();
-      // thread t owns bins B - 1 - 2 t and B - 2 - 2 t: counts from the top by a block-wide prefix sum
-      const int hi = hist[kSelBins - 1 - 2 * tid], lo = hist[kSelBins - 2 - 2 * tid];
-      int incl = hi + lo;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      if (lane == 31) wsum[warp] = incl;
-      __syncthreads();
-      int before = lane < warp ? wsum[lane] : 0, all = wsum[lane];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        before += __shfl_xor_sync(0xffffffffu, before, o);
-        all += __shfl_xor_sync(0xffffffffu, all, o);
-      }
-      const int above = before + incl - hi - lo;   // entries in higher bins than this thread's
-      if (above < k_target && above + hi + lo >= k_target) {   // the k-th largest is in one of this thread's bins
-        const bool first = above + hi >= k_target;
-        s_kk = kSelBins - (first ? 1 : 2) - 2 * tid;
-        s_done = above + hi + (first ? 0 : lo);                // entries to sort
-      }
-      __syncthreads();
-      if (a.top_s == nullptr && all >= k_target) {
-        // only a lower bound of the k-th score is wanted: the smallest score in the bins from that of the k-th on
-        const int cut = s_kk;
-        float low = INFINITY;
-        sweep([&](unsigned long long key) {
-          if (key != 0ull && bin_of(key) >= cut) low = fminf(low, key_score(key));
-        });
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) low = fminf(low, __shfl_xor_sync(0xffffffffu, low, o));
-        if (lane == 0) wmin[warp] = low;
-        __syncthreads();
-        if (warp == 0) {
-          low = wmin[lane];
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) low = fminf(low, __shfl_xor_sync(0xffffffffu, low, o));
-          if (lane == 0) a.kth[q] = low;
-        }
-        return;
-      }
-      const bool few = all < k_target;   // fewer entries than k (empty slots in the list): all of them
-      const int cut = few ? 0 : s_kk;
-      if ((few ? all : s_done) <= 1024) {
-        sweep([&](unsigned long long key) {
-          if (key != 0ull && bin_of(key) >= cut) skey[atomicAdd(&s_cnt, 1)] = key;
-        });
-        sorted_set = true;
-      }
+      __syncthreads();   // wmin has been read
+      block_range();
+      if (tid == 0) a.kth[q] = mn;
+      return;
+    }
+    if ((few ? all : s_done) <= 1024) {
+      sweep([&](unsigned long long key) {
+        if (key != 0ull && bin_of(key) >= cut) skey[atomicAdd(&s_cnt, 1)] = key;
+      });
+      sorted_set = true;
     }
   }
-  if (!sorted_set && k_target > 0) {
+  if (!sorted_set) {
     // ---- radix select over the key's bytes, from the top
     int kk = k_target;
     unsigned long long prefix = 0ull;
     int shift = 56;
+#pragma unroll 1
     for (int round = 0; round < 8; ++round) {
       shift = 56 - 8 * round;
       __syncthreads();
@@ -833,10 +875,34 @@ __global__ void __launch_bounds__(1024) select_kernel(SelArgs a) {
     });
   }
   __syncthreads();
+  const int found = min(s_cnt, 1024);
+  auto put = [&](int rank, unsigned long long key) {
+    const float s = key != 0ull ? key_score(key) : -INFINITY;
+    if (a.top_s != nullptr) {
+      a.top_s[(int64_t)q * a.k + rank] = s;
+      a.top_i[(int64_t)q * a.k + rank] = key != 0ull ? (int)(~(uint32_t)(key & 0xffffffffull)) : -1;
+    }
+    if (rank == a.k - 1 && a.kth != nullptr) a.kth[q] = s;
+  };
+  if (found <= 256) {
+    // a key's rank is the number of larger ones (keys are distinct: they contain the id); four threads count for one key, so
+    // that there is no barrier at all
+    const unsigned long long key = skey[tid >> 2];
+    int rank = 0;
+#pragma unroll 4
+    for (int i = tid & 3; i < found; i += 4) rank += skey[i] > key ? 1 : 0;
+    rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+    rank += __shfl_xor_sync(0xffffffffu, rank, 2);
+    if ((tid & 3) == 0 && (tid >> 2) < found && rank < a.k) put(rank, key);
+    if (tid >= found && tid < a.k) put(tid, 0ull);
+    return;
+  }
   // bitonic sort, descending, of the smallest power of two that holds the survivors (the rest of skey is zero)
-  int sort_n = 32;
-  while (sort_n < min(s_cnt, 1024)) sort_n <<= 1;
+  int sort_n = 512;
+  while (sort_n < found) sort_n <<= 1;
+#pragma unroll 1
   for (int kb = 2; kb <= sort_n; kb <<= 1) {
+#pragma unroll 1
     for (int j = kb >> 1; j > 0; j >>= 1) {
       const int p = tid ^ j;
       if (p > tid && p < sort_n) {
@@ -850,16 +916,7 @@ __global__ void __launch_bounds__(1024) select_kernel(SelArgs a) {
       __syncthreads();
     }
   }
-  if (tid < a.k) {
-    const unsigned long long key = skey[tid];
-    const float s = key != 0ull ? key_score(key) : -INFINITY;
-    const int id = key != 0ull ? (int)(~(uint32_t)(key & 0xffffffffull)) : -1;
-    if (a.top_s != nullptr) {
-      a.top_s[(int64_t)q * a.k + tid] = s;
-      a.top_i[(int64_t)q * a.k + tid] = id;
-    }
-    if (tid == a.k - 1 && a.kth != nullptr) a.kth[q] = s;
-  }
+  if (tid < a.k) put(tid, skey[tid]);
 }
 
 // ------------------------------------------------------------------ host side
@@ -876,7 +933,7 @@ size_t bfrag_bytes(const tq_plan* plan, int NT) {
 bool pick_config(const tq_plan* plan, int NW, int MT, int NT, Config* out) {
   const int nblk = plan->mse_bits + (plan->mode == TQ_PROD ? 1 : 0);
   const size_t stage = (size_t)nblk * (NW * MT * 16) * 64;
-  const size_t fixed = bfrag_bytes(plan, NT) + 1024 /*alignment*/ + 2 * MAX_STAGES * 8 + 16 + 4 * sizeof(QConst);
+  const size_t fixed = bfrag_bytes(plan, NT) + 1024 /*alignment*/ + 2 * MAX_STAGES * 8 + 16 + kMaxPassQueries * sizeof(QConst);
   if (fixed + 2 * stage > (size_t)SMEM_LIMIT) return false;
   int stages = (int)std::min<size_t>((SMEM_LIMIT - fixed) / stage, MAX_STAGES);
   out->NW = NW;
@@ -907,6 +964,11 @@ cudaError_t launch_t(const CUtensorMap& mi, const CUtensorMap& mq, const ScanArg
 template <int BM, bool PROD>
 cudaError_t launch_cfg(const Config& c, bool filter, const CUtensorMap& mi, const CUtensorMap& mq, const ScanArgs& args,
                        cudaStream_t st) {
+  if (c.NT == kTiledNT) {
+    if (c.NW == 16)
+      return filter ? launch_t<BM, PROD, 16, 1, kTiledNT, 1>(mi, mq, args, c.smem, st) : launch_t<BM, PROD, 16, 1, kTiledNT, 0>(mi, mq, args, c.smem, st);
+    return filter ? launch_t<BM, PROD, 8, 1, kTiledNT, 1>(mi, mq, args, c.smem, st) : launch_t<BM, PROD, 8, 1, kTiledNT, 0>(mi, mq, args, c.smem, st);
+  }
   if (c.NW == 16 && c.NT == 1)
     return filter ? launch_t<BM, PROD, 16, 1, 1, 1>(mi, mq, args, c.smem, st) : launch_t<BM, PROD, 16, 1, 1, 0>(mi, mq, args, c.smem, st);
   if (c.NW == 12 && c.NT == 2)
@@ -928,10 +990,13 @@ cudaError_t launch_scan(const tq_plan* plan, const Config& c, bool filter, const
   }
 }
 
-// nq <= 2: one column tile, 16 consumer warps of 16 vectors; nq > 2: two column tiles, 12 (else 8) warps.
-// Falls back to the smallest shape when the B operand leaves no room for two stages.
+// nq <= 2: one column tile, 16 consumer warps of 16 vectors; nq > 2: two column tiles, 12 (else 8) warps; nq > 4: three column
+// tiles (one per digit, the fourth is always zero) for eight queries, 16 (else 8) warps.
+// Falls back to the smaller shapes when the B operand leaves no room for two stages.
 Config config_for(const tq_plan* plan, int nq) {
   Config c{8, 1, 1, 2, 0};
+  if (nq > 4 && pick_config(plan, 16, 1, kTiledNT, &c)) return c;
+  if (nq > 4 && pick_config(plan, 8, 1, kTiledNT, &c)) return c;
   if (nq > 2 && pick_config(plan, 12, 1, 2, &c)) return c;
   if (nq > 2 && pick_config(plan, 8, 1, 2, &c)) return c;
   if (pick_config(plan, 16, 1, 1, &c)) return c;
@@ -983,13 +1048,15 @@ void plan_init(tq_plan* plan) {
   plan->ms.ok = 1;
 }
 
-int queries_per_pass(const tq_plan* plan, int nq) { return config_for(plan, nq).NT * 8 / LIMBS; }
+int queries_per_pass(const tq_plan* plan, int nq) {
+  const int nt = config_for(plan, nq).NT;
+  return nt == kTiledNT ? 8 : nt * 8 / LIMBS;
+}
 
-
-size_t workspace_bytes(const tq_plan* plan) {
+size_t workspace_bytes(const tq_plan* plan, int nq) {
   if (!plan->ms.ok) return 0;
   Config c;
-  const int nt = pick_config(plan, 8, 1, 2, &c) ? 2 : 1;
+  const int nt = std::max(pick_config(plan, 8, 1, 2, &c) ? 2 : 1, config_for(plan, nq).NT);
   return kQConstBytes + (bfrag_bytes(plan, nt) + 255) / 256 * 256;
 }
 
@@ -1016,6 +1083,10 @@ int prepare(const tq_plan* plan, const float* Qcat, int nqp, void* workspace, cu
   for (int i = 0; i < 8; ++i) ba.alpha[i] = plan->ms.alpha[i];
   ba.out = bfrag;
   const int64_t total = (int64_t)c.NT * plan->ms.R * (ks_a(bm) + ks_s(prod)) * 32;
+  if (c.NT == kTiledNT) {
+    count_launches(1);
+    TQ_CHECK_CUDA(launch_dependent(query_constants_kernel, dim3((unsigned)nqp), dim3(256), 0, st, ba), who);
+  }
   count_launches(1);
   TQ_CHECK_CUDA(launch_dependent(bprep_kernel, dim3((unsigned)((total * 8 + 255) / 256)), dim3(256), 0, st, ba), who);
   return TQ_OK;
@@ -1082,8 +1153,22 @@ cudaError_t select_topk(const float* cand_s, const int* cand_i, const int* count
   a.run_if = run_if;
   a.clear_count = clear_count;
   a.clear_flag = clear_flag;
+  // the shared-memory copy of the list: as much as this call can need (none where the list is known to be too long for it)
+  const int64_t most = std::max<int64_t>(count != nullptr ? cap : m, 0) + (merge ? k : 0);
+  const size_t smem = count == nullptr && most > kSelCached ? 0 : (size_t)std::min<int64_t>(most, kSelCached) * sizeof(unsigned long long);
+  if (smem > 24 * 1024) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    static std::atomic<unsigned long long> attr_devices{0};   // devices whose function attribute has been set
+    if (dev >= 64 || !((attr_devices.load(std::memory_order_relaxed) >> dev) & 1ull)) {
+      e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelCached * (int)sizeof(unsigned long long));
+      if (e != cudaSuccess) return e;
+      if (dev < 64) attr_devices.fetch_or(1ull << dev, std::memory_order_relaxed);
+    }
+  }
   count_launches(1);
-  return launch_dependent(select_kernel, dim3((unsigned)nq), dim3(1024), 0, st, a);
+  return launch_dependent(select_kernel, dim3((unsigned)nq), dim3(1024), smem, st, a);
 }
 
 cudaError_t select_pairs(const float* cand_s, const int* cand_i, int ld, int m, int nq, int k, float* top_s, int* top_i,

@@ -9,11 +9,11 @@ namespace mscan {
 // Decides whether the plan's codebook / dimension admit the bit-plane scan and fills plan->ms.
 void plan_init(tq_plan* plan);
 
-// Queries served by one pass over the codes when nq queries remain (2 or 4).
+// Queries served by one pass over the codes when nq queries remain (2, 4 or 8).
 int queries_per_pass(const tq_plan* plan, int nq);
 
-// Bytes of workspace one pass needs: per-query constants + the B operand (query-side matrix).
-size_t workspace_bytes(const tq_plan* plan);
+// Bytes of workspace a pass of a call of nq queries needs: per-query constants + the B operand (query-side matrix).
+size_t workspace_bytes(const tq_plan* plan, int nq);
 
 struct Filter {          // top-k candidate collection for the queries of one pass
   const float* tau;      // [nqp] admission threshold per query (score >= tau is kept)

@@ -77,11 +77,20 @@ __device__ void query_scales(const PrepArgs& a, QScale* sc /* shared, [8] */) {
     const float* q = a.Qcat + (int64_t)warp * a.ldq;
     float mx1 = 0.f, mx2 = 0.f;
     double sm2 = 0.0;
-    for (int j = lane; j < a.d; j += 32) {
-      mx1 = fmaxf(mx1, fabsf(q[j]));
-      const float u = q[a.dpad + j];
-      mx2 = fmaxf(mx2, fabsf(u));
-      if (blockIdx.x == 0) sm2 += (double)u;
+    for (int j0 = lane; j0 < a.d; j0 += 32 * 16) {   // sixteen rounds of loads in flight: one by one this loop took 10 us at d = 1536
+      float v[16], u[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int j = j0 + 32 * i;
+        v[i] = j < a.d ? q[j] : 0.f;
+        u[i] = j < a.d ? q[a.dpad + j] : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        mx1 = fmaxf(mx1, fabsf(v[i]));
+        mx2 = fmaxf(mx2, fabsf(u[i]));
+        if (blockIdx.x == 0) sm2 += (double)u[i];   // (a zero past the end changes nothing)
+      }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
