@@ -340,6 +340,24 @@ __global__ void __launch_bounds__(256) tbprep_nib_kernel(BPrepArgs a, int querie
   for (int l = 0; l < LIMBS; ++l) *reinterpret_cast<uint32_t*>(dst + (size_t)l * kQueriesPerPass * nkb * KB_BYTES) = out[l];
 }
 
+// ------------------------------------------------------------------ epilogue
+// Estimates of one row for 16 queries (constants qc[0 .. 16)) from the three digit sums of the two terms.  The digits are
+// recombined exactly (64-bit integer: the same T as in the register-fed engine), then fp32.  No branch in here, so that the
+// sixteen chains overlap: with the threshold test inside the loop the epilogue ran at 8 cycles per instruction and was half of
+// the many-query scan's time at d = 200.
+template <bool MSE, bool SIGNS>
+__device__ __forceinline__ void estimates16(const uint32_t (&va)[LIMBS][16], const uint32_t (&vs)[LIMBS][16], const QConst* qc, float nu,
+                                            float cg, float (&est)[16]) {
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const float4 c = *reinterpret_cast<const float4*>(qc + i);   // sa, ca, ss, cs
+    float av = 0.f, sv = 0.f;
+    if (MSE) av = fmaf((float)(((long long)(int)va[2][i] * 256 + (int)va[1][i]) * 256 + (int)va[0][i]), c.x, c.y);
+    if (SIGNS) sv = fmaf((float)(((long long)(int)vs[2][i] * 256 + (int)vs[1][i]) * 256 + (int)vs[0][i]), c.z, c.w);
+    est[i] = __fmul_rn(nu, fmaf(cg, sv, av));
+  }
+}
+
 // ------------------------------------------------------------------ scan kernel
 struct ScanArgs {
   int64_t n, npairs;
@@ -733,35 +751,34 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__
           if (a.g.kbs > 0 || NIB) tc::tmem_ld16(taddr + NCOL + l * 32 + h * 16, vs[l]);
         }
         tc::tmem_ld_wait();
+        float est[16];
+        const float cg = __fmul_rn(a.coef, gm);
+        if (a.g.kbs > 0 || NIB) estimates16<(BM > 0), true>(va, vs, qcs + 16 * h, nu, cg, est);
+        else estimates16<(BM > 0), false>(va, vs, qcs + 16 * h, nu, cg, est);
+        if (MODE == 0) {
 #pragma unroll
-        for (int qq = 0; qq < 16; ++qq) {
-          const int ql = h * 16 + qq;
-          if (ql >= a.nqp) break;
-          // digits recombined exactly (64-bit integer: the same T as in the register-fed engine), then fp32
-          const QConst c = qcs[ql];
-          float av = 0.f, sv = 0.f;
-          if (a.g.kba > 0) {
-            const long long T = ((long long)(int)va[2][qq] * 256 + (int)va[1][qq]) * 256 + (int)va[0][qq];
-            av = fmaf((float)T, c.sa, c.ca);
-          }
-          if (a.g.kbs > 0 || NIB) {
-            const long long T = ((long long)(int)vs[2][qq] * 256 + (int)vs[1][qq]) * 256 + (int)vs[0][qq];
-            sv = fmaf((float)T, c.ss, c.cs);
-          }
-          const float est = __fmul_rn(nu, fmaf(__fmul_rn(a.coef, gm), sv, av));
-          if (row_ok && ql < a.nqp) {
-            if (MODE == 0) {
-              if (TQ_DEVICE_CHECK(row >= 0 && row < a.n && row < a.lds, a.status)) a.scores[(int64_t)ql * a.lds + row] = est;
-            } else if (est >= taus[ql]) {
-              const int ls = atomicAdd(&lcnt[ql], 1);
-              if (ls < LBUF) {
-                lbuf[ql * LBUF + ls] = make_uint2(__float_as_uint(est), (uint32_t)row);
-              } else {   // the CTA's buffer is full: straight to the global list
-                const int slot = atomicAdd(a.count + ql, 1);
-                if (slot < a.cap) {
-                  a.cand_s[(int64_t)ql * a.cap + slot] = est;
-                  a.cand_i[(int64_t)ql * a.cap + slot] = (int)row;
-                }
+          for (int qq = 0; qq < 16; ++qq)
+            if (row_ok && h * 16 + qq < a.nqp && TQ_DEVICE_CHECK(row >= 0 && row < a.n && row < a.lds, a.status))
+              a.scores[(int64_t)(h * 16 + qq) * a.lds + row] = est[qq];
+          continue;
+        }
+        uint32_t hits = 0u;
+#pragma unroll
+        for (int qq = 0; qq < 16; ++qq) hits |= est[qq] >= taus[h * 16 + qq] ? 1u << qq : 0u;
+        if (!row_ok) hits = 0u;
+        if (a.nqp < 16 * h + 16) hits &= (1u << (a.nqp - 16 * h)) - 1u;
+        if (hits != 0u) {
+#pragma unroll
+          for (int qq = 0; qq < 16; ++qq) {
+            if (!((hits >> qq) & 1u)) continue;
+            const int ql = h * 16 + qq, ls = atomicAdd(&lcnt[ql], 1);
+            if (ls < LBUF) {
+              lbuf[ql * LBUF + ls] = make_uint2(__float_as_uint(est[qq]), (uint32_t)row);
+            } else {   // the CTA's buffer is full: straight to the global list
+              const int slot = atomicAdd(a.count + ql, 1);
+              if (slot < a.cap) {
+                a.cand_s[(int64_t)ql * a.cap + slot] = est[qq];
+                a.cand_i[(int64_t)ql * a.cap + slot] = (int)row;
               }
             }
           }

@@ -468,35 +468,35 @@ scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant_
         tc::tmem_ld_wait();
         // the last columns are in registers: the next tile's MMAs may start while their estimates are formed
         if (h == nh - 1) release_accumulators();
+        const int q0 = 32 * set + 16 * h;
+        float est[16];
+        const float cg = __fmul_rn(a.coef, gm);
+        if (a.g.kbs > 0 || NIB) estimates16<(BM > 0), true>(va, vs, qcs + q0, nu, cg, est);
+        else estimates16<(BM > 0), false>(va, vs, qcs + q0, nu, cg, est);
+        if (MODE == 0) {
 #pragma unroll
-        for (int qq = 0; qq < 16; ++qq) {
-          const int ql = 32 * set + h * 16 + qq;
-          if (ql >= a.nqp) break;
-          // digits recombined exactly (64-bit integer: the same T as in the register-fed engine), then fp32
-          const QConst c = qcs[ql];
-          float av = 0.f, sv = 0.f;
-          if (a.g.kba > 0) {
-            const long long T = ((long long)(int)va[2][qq] * 256 + (int)va[1][qq]) * 256 + (int)va[0][qq];
-            av = fmaf((float)T, c.sa, c.ca);
-          }
-          if (a.g.kbs > 0 || NIB) {
-            const long long T = ((long long)(int)vs[2][qq] * 256 + (int)vs[1][qq]) * 256 + (int)vs[0][qq];
-            sv = fmaf((float)T, c.ss, c.cs);
-          }
-          const float est = __fmul_rn(nu, fmaf(__fmul_rn(a.coef, gm), sv, av));
-          if (row_ok) {
-            if (MODE == 0) {
-              if (TQ_DEVICE_CHECK(row >= 0 && row < a.n && row < a.lds, a.status)) a.scores[(int64_t)ql * a.lds + row] = est;
-            } else if (est >= taus[ql]) {
-              const int ls = atomicAdd(&lcnt[ql], 1);
-              if (ls < W_LBUF) {
-                lbuf[ql * W_LBUF + ls] = make_uint2(__float_as_uint(est), (uint32_t)row);
-              } else {   // the CTA's buffer is full: straight to the global list
-                const int slot = atomicAdd(a.count + ql, 1);
-                if (slot < a.cap) {
-                  a.cand_s[(int64_t)ql * a.cap + slot] = est;
-                  a.cand_i[(int64_t)ql * a.cap + slot] = (int)row;
-                }
+          for (int qq = 0; qq < 16; ++qq)
+            if (row_ok && q0 + qq < a.nqp && TQ_DEVICE_CHECK(row >= 0 && row < a.n && row < a.lds, a.status))
+              a.scores[(int64_t)(q0 + qq) * a.lds + row] = est[qq];
+          continue;
+        }
+        uint32_t hits = 0u;
+#pragma unroll
+        for (int qq = 0; qq < 16; ++qq) hits |= est[qq] >= taus[q0 + qq] ? 1u << qq : 0u;
+        if (!row_ok) hits = 0u;
+        if (a.nqp < q0 + 16) hits &= (1u << (a.nqp - q0)) - 1u;
+        if (hits != 0u) {
+#pragma unroll
+          for (int qq = 0; qq < 16; ++qq) {
+            if (!((hits >> qq) & 1u)) continue;
+            const int ql = q0 + qq, ls = atomicAdd(&lcnt[ql], 1);
+            if (ls < W_LBUF) {
+              lbuf[ql * W_LBUF + ls] = make_uint2(__float_as_uint(est[qq]), (uint32_t)row);
+            } else {   // the CTA's buffer is full: straight to the global list
+              const int slot = atomicAdd(a.count + ql, 1);
+              if (slot < a.cap) {
+                a.cand_s[(int64_t)ql * a.cap + slot] = est[qq];
+                a.cand_i[(int64_t)ql * a.cap + slot] = (int)row;
               }
             }
           }
