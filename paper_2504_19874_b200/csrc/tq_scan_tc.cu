@@ -358,6 +358,39 @@ __device__ __forceinline__ void estimates16(const uint32_t (&va)[LIMBS][16], con
   }
 }
 
+// est[i], i in a register array and different from lane to lane: four levels of selects.
+__device__ __forceinline__ float pick16(const float (&est)[16], int i) {
+  float a8[8], a4[4];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) a8[j] = (i & 1) ? est[2 * j + 1] : est[2 * j];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) a4[j] = (i & 2) ? a8[2 * j + 1] : a8[2 * j];
+  const float x = (i & 4) ? a4[1] : a4[0], y = (i & 4) ? a4[3] : a4[2];
+  return (i & 8) ? y : x;
+}
+
+// Filter mode: the estimates that reach their query's threshold (bit i of `hits`: query q0 + i) go to the CTA's buffers.  A lane
+// takes its own hits one after the other, all lanes at once: a test per query, each with a body for the few lanes that hit,
+// cost 1,300 cycles per 16 queries where one estimate in 120 hits.
+template <int CAPACITY, class Args>
+__device__ __forceinline__ void append_hits(const Args& a, uint32_t hits, const float (&est)[16], int q0, int64_t row, int* lcnt, uint2* lbuf) {
+  while (hits != 0u) {
+    const int i = __ffs((int)hits) - 1, ql = q0 + i;
+    hits &= hits - 1u;
+    const float e = pick16(est, i);
+    const int ls = atomicAdd(&lcnt[ql], 1);
+    if (ls < CAPACITY) {
+      lbuf[ql * CAPACITY + ls] = make_uint2(__float_as_uint(e), (uint32_t)row);
+    } else {   // the CTA's buffer is full: straight to the global list
+      const int slot = atomicAdd(a.count + ql, 1);
+      if (slot < a.cap) {
+        a.cand_s[(int64_t)ql * a.cap + slot] = e;
+        a.cand_i[(int64_t)ql * a.cap + slot] = (int)row;
+      }
+    }
+  }
+}
+
 // ------------------------------------------------------------------ scan kernel
 struct ScanArgs {
   int64_t n, npairs;
@@ -767,22 +800,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__
         for (int qq = 0; qq < 16; ++qq) hits |= est[qq] >= taus[h * 16 + qq] ? 1u << qq : 0u;
         if (!row_ok) hits = 0u;
         if (a.nqp < 16 * h + 16) hits &= (1u << (a.nqp - 16 * h)) - 1u;
-        if (hits != 0u) {
-#pragma unroll
-          for (int qq = 0; qq < 16; ++qq) {
-            if (!((hits >> qq) & 1u)) continue;
-            const int ql = h * 16 + qq, ls = atomicAdd(&lcnt[ql], 1);
-            if (ls < LBUF) {
-              lbuf[ql * LBUF + ls] = make_uint2(__float_as_uint(est[qq]), (uint32_t)row);
-            } else {   // the CTA's buffer is full: straight to the global list
-              const int slot = atomicAdd(a.count + ql, 1);
-              if (slot < a.cap) {
-                a.cand_s[(int64_t)ql * a.cap + slot] = est[qq];
-                a.cand_i[(int64_t)ql * a.cap + slot] = (int)row;
-              }
-            }
-          }
-        }
+        append_hits<LBUF>(a, hits, est, 16 * h, row, lcnt, lbuf);
       }
       tc::tc_fence_before();
     }

@@ -314,6 +314,24 @@ scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant_
       }
     };
     release_accumulators();
+    // Filter mode: a tile's estimates stay in registers until the next tile's codes are expanded, and are tested while the MMAs
+    // of that tile run (the wait for them is 2,200 cycles at d = 200).
+    float est0[16], est1[16];
+    int64_t kept_row = -1;
+    auto flush_hits = [&]() {
+      if (MODE != 1 || kept_row < 0) return;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float (&e)[16] = h == 0 ? est0 : est1;
+        const int q0 = 32 * set + 16 * h;
+        if (q0 >= a.nqp) break;
+        uint32_t hits = 0u;
+#pragma unroll
+        for (int qq = 0; qq < 16; ++qq) hits |= e[qq] >= taus[q0 + qq] ? 1u << qq : 0u;
+        if (a.nqp < q0 + 16) hits &= (1u << (a.nqp - q0)) - 1u;
+        append_hits<W_LBUF>(a, hits, e, q0, kept_row, lcnt, lbuf);
+      }
+    };
     float nu_next = load_nu(unit * CTAS + rank), gm_next = load_gm(unit * CTAS + rank);
     for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits, ++it) {
       const int64_t tile = rnd * CTAS + rank;
@@ -450,6 +468,8 @@ scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant_
       }
       if (!ok) break;
 
+      flush_hits();   // of the tile before
+      __syncwarp();
       // ---- epilogue: this thread's row, the set's 32 queries
       if (!(ok = tc::mbar_wait(dfull, it & 1u, abort_flag, a.status))) break;
       tc::tc_fence_after();
@@ -457,8 +477,9 @@ scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant_
       // halves of 16 queries; a short last pass: columns of absent queries are not read
       const int nh = min(2, max(0, (a.nqp - 32 * set + 15) >> 4));
       if (nh == 0) release_accumulators();
-#pragma unroll 1
-      for (int h = 0; h < nh; ++h) {   // digit l of query 32 set + 16 h + qq sits in column 96 set + 32 l + 16 h + qq
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (h >= nh) break;   // digit l of query 32 set + 16 h + qq sits in column 96 set + 32 l + 16 h + qq
         uint32_t va[LIMBS][16], vs[LIMBS][16];
 #pragma unroll
         for (int l = 0; l < LIMBS; ++l) {
@@ -469,41 +490,22 @@ scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant_
         // the last columns are in registers: the next tile's MMAs may start while their estimates are formed
         if (h == nh - 1) release_accumulators();
         const int q0 = 32 * set + 16 * h;
-        float est[16];
         const float cg = __fmul_rn(a.coef, gm);
-        if (a.g.kbs > 0 || NIB) estimates16<(BM > 0), true>(va, vs, qcs + q0, nu, cg, est);
-        else estimates16<(BM > 0), false>(va, vs, qcs + q0, nu, cg, est);
+        float (&e)[16] = h == 0 ? est0 : est1;
+        if (a.g.kbs > 0 || NIB) estimates16<(BM > 0), true>(va, vs, qcs + q0, nu, cg, e);
+        else estimates16<(BM > 0), false>(va, vs, qcs + q0, nu, cg, e);
         if (MODE == 0) {
 #pragma unroll
           for (int qq = 0; qq < 16; ++qq)
             if (row_ok && q0 + qq < a.nqp && TQ_DEVICE_CHECK(row >= 0 && row < a.n && row < a.lds, a.status))
-              a.scores[(int64_t)(q0 + qq) * a.lds + row] = est[qq];
-          continue;
-        }
-        uint32_t hits = 0u;
-#pragma unroll
-        for (int qq = 0; qq < 16; ++qq) hits |= est[qq] >= taus[q0 + qq] ? 1u << qq : 0u;
-        if (!row_ok) hits = 0u;
-        if (a.nqp < q0 + 16) hits &= (1u << (a.nqp - q0)) - 1u;
-        if (hits != 0u) {
-#pragma unroll
-          for (int qq = 0; qq < 16; ++qq) {
-            if (!((hits >> qq) & 1u)) continue;
-            const int ql = q0 + qq, ls = atomicAdd(&lcnt[ql], 1);
-            if (ls < W_LBUF) {
-              lbuf[ql * W_LBUF + ls] = make_uint2(__float_as_uint(est[qq]), (uint32_t)row);
-            } else {   // the CTA's buffer is full: straight to the global list
-              const int slot = atomicAdd(a.count + ql, 1);
-              if (slot < a.cap) {
-                a.cand_s[(int64_t)ql * a.cap + slot] = est[qq];
-                a.cand_i[(int64_t)ql * a.cap + slot] = (int)row;
-              }
-            }
-          }
+              a.scores[(int64_t)(q0 + qq) * a.lds + row] = e[qq];
         }
       }
+      if (MODE == 1) kept_row = row_ok ? row : -1;
       tc::tc_fence_before();
     }
+    flush_hits();
+    __syncwarp();
   }
 
   tc::tc_fence_before();
