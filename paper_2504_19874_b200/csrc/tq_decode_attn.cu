@@ -536,10 +536,15 @@ struct AppendArgs {
 // Quant_mse / Quant_prod (Algorithms 1, 2) of one d-vector by one CTA, thread j = rotated coordinate j, with the
 // comparisons the batch quantiser makes: y = Pi x, idx_j = #{i : y_j > t_i nu}, e = y / nu - c[idx],
 // z = sign(S' e), gamma = ||e||.
+// Bound: a chain of latencies (32 CTAs for 8 heads and 2 groups).  The matrices are the plan's: their copies to shared memory
+// start before the wait for the kernel ahead, and the dot products then run at shared-memory latency (with a load from L2 per
+// product the kernel took 12.4 us, 22.7 with cold caches).
 template <typename T>
 __global__ void __launch_bounds__(MAXD) append_kernel(AppendArgs a, const T* __restrict__ K, int64_t ldk,
                                                       const T* __restrict__ V, int64_t ldv) {
-  __shared__ float xs[MAXD], es[MAXD], red[4];
+  extern __shared__ __align__(16) float mats[];   // [d][d] Pi^T, then (TQ_PROD keys) [d][d + 4] S'
+  __shared__ __align__(16) float xs[MAXD], es[MAXD];
+  __shared__ float red[4];
   __shared__ uint32_t words[MAXD * 4 / 32 + 1];
   const int h = blockIdx.x / a.ngroups, gi = blockIdx.x % a.ngroups, isv = blockIdx.y;
   const AppendGroup& g = a.g[gi];
@@ -548,6 +553,21 @@ __global__ void __launch_bounds__(MAXD) append_kernel(AppendArgs a, const T* __r
   const Codebook& cb = isv ? g.v_cb : g.k_cb;
   const bool prod = !isv && g.k_prod;
   const int bm = cb.bits;
+  float* sps = mats + d * d;
+  {
+    const float* bt = isv ? g.v_backt : g.k_backt;
+    const int ncols = isv ? g.v_ncols : g.k_ncols, row4 = d / 4;
+    const uint32_t to = (uint32_t)__cvta_generic_to_shared(mats);
+    for (int i = j; i < d * row4; i += MAXD)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + 16 * i), "l"(bt + (size_t)(i / row4) * ncols + 4 * (i % row4)) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (prod)
+      for (int i = j; i < d * row4; i += MAXD)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + 4 * (d * d + (i / row4) * (d + 4)) + 16 * (i % row4)), "l"(g.k_sp + 4 * i) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  allow_successor();
+  wait_for_predecessor();   // it may write K and V, or read the rows that this kernel writes
   auto block_sum = [&](float v) -> float {   // fixed order: lanes by shuffles, then the warps in turn
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -565,15 +585,22 @@ __global__ void __launch_bounds__(MAXD) append_kernel(AppendArgs a, const T* __r
   }
   xs[j] = x;
   if (j < (int)(sizeof(words) / sizeof(words[0]))) words[j] = 0u;
-  float nu = sqrtf(block_sum(x * x));   // the sync inside also publishes xs and words
+  asm volatile("cp.async.wait_group 1;" ::: "memory");
+  float nu = sqrtf(block_sum(x * x));   // the syncs inside also publish xs, words and the first matrix
   // no norms array: the row is taken as already unit-norm and quantised as it is, like tq_quantize_*
   if ((isv ? g.v_norms : g.k_norms) == nullptr) nu = 1.f;
   const float inv = nu > 0.f ? 1.f / nu : 0.f, vcmp = nu > 0.f ? nu : 1.f;
-  const float* bt = isv ? g.v_backt : g.k_backt;
-  const int ncols = isv ? g.v_ncols : g.k_ncols;
   float y = 0.f;
-  if (j < d)
-    for (int c = 0; c < d; ++c) y = fmaf(bt[(size_t)c * ncols + j], xs[c], y);
+  if (j < d) {
+#pragma unroll 4
+    for (int c = 0; c < d; c += 4) {
+      const float4 x4 = *reinterpret_cast<const float4*>(xs + c);
+      y = fmaf(mats[c * d + j], x4.x, y);
+      y = fmaf(mats[(c + 1) * d + j], x4.y, y);
+      y = fmaf(mats[(c + 2) * d + j], x4.z, y);
+      y = fmaf(mats[(c + 3) * d + j], x4.w, y);
+    }
+  }
   int code = 0;
   for (int t = 0; t < (1 << bm) - 1; ++t) code += (y > cb.t[t] * vcmp) ? 1 : 0;
   if (j < d && bm > 0) {
@@ -584,6 +611,7 @@ __global__ void __launch_bounds__(MAXD) append_kernel(AppendArgs a, const T* __r
   const float e = (j < d && nu > 0.f) ? y * inv - cb.c[code] : 0.f;
   es[j] = e;
   float gamma = 0.f;
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   if (prod) gamma = sqrtf(block_sum(e * e)); else __syncthreads();
   uint8_t* idx_row = (isv ? g.v_idx + (size_t)row * g.v_idx_rb : g.k_idx + (size_t)row * g.k_idx_rb);
   const int idx_rb = isv ? g.v_idx_rb : g.k_idx_rb;
@@ -594,8 +622,15 @@ __global__ void __launch_bounds__(MAXD) append_kernel(AppendArgs a, const T* __r
     if (j == 0) g.k_gamma[row] = gamma;
     float sp = 0.f;
     if (j < d) {
-      const float* srow = g.k_sp + (size_t)j * d;
-      for (int c = 0; c < d; ++c) sp = fmaf(srow[c], es[c], sp);
+      const float* srow = sps + j * (d + 4);
+#pragma unroll 4
+      for (int c = 0; c < d; c += 4) {
+        const float4 s4 = *reinterpret_cast<const float4*>(srow + c), e4 = *reinterpret_cast<const float4*>(es + c);
+        sp = fmaf(s4.x, e4.x, sp);
+        sp = fmaf(s4.y, e4.y, sp);
+        sp = fmaf(s4.z, e4.z, sp);
+        sp = fmaf(s4.w, e4.w, sp);
+      }
     }
     const uint32_t bits = __ballot_sync(0xffffffffu, j < d && sp >= 0.f);
     uint32_t* qrow = reinterpret_cast<uint32_t*>(g.k_qjl + (size_t)row * g.k_qjl_rb);
@@ -846,13 +881,24 @@ extern "C" int tq_attend_decode(const tq_kv_group* groups, int ngroups, int head
   MmaArgs ma;
   size_t mma_smem = 0;
   if (plan_mma(ngroups, d, a, static_cast<char*>(workspace), off, heads, &ma, &mma_smem)) {
+    size_t prep_smem = 0;
+    for (int gi = 0; gi < ngroups; ++gi)
+      prep_smem = std::max(prep_smem, (size_t)d * (a.g[gi].k_prod ? 2 : 1) * a.g[gi].k_dpad * sizeof(float));
+    constexpr int prep_smem_max = MAXD * 2 * MAXD * (int)sizeof(float);
+    TQ_REQUIRE(prep_smem <= (size_t)prep_smem_max, TQ_ERR_UNSUPPORTED, "%s: rotation of %zu bytes", who, prep_smem);
+    static std::atomic<bool> prep_set[16];
+    if (dev >= 16 || !prep_set[dev].load(std::memory_order_relaxed)) {
+      TQ_CHECK_CUDA(cudaFuncSetAttribute(prepare_mma_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, prep_smem_max), who);
+      TQ_CHECK_CUDA(cudaFuncSetAttribute(prepare_mma_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, prep_smem_max), who);
+      if (dev < 16) prep_set[dev].store(true, std::memory_order_relaxed);
+    }
     // all three launches may be scheduled while their predecessor in the stream drains; each orders itself with
     // griddepcontrol.wait before it reads or writes global memory that another kernel touches
     if (q_dtype == TQ_F32)
-      TQ_CHECK_CUDA(launch_dependent(prepare_mma_kernel<float>, dim3((unsigned)(heads * ngroups)), dim3(256), 0, st, a, ma,
+      TQ_CHECK_CUDA(launch_dependent(prepare_mma_kernel<float>, dim3((unsigned)(heads * ngroups)), dim3(256), prep_smem, st, a, ma,
                                  static_cast<const float*>(Q), ldq), who);
     else
-      TQ_CHECK_CUDA(launch_dependent(prepare_mma_kernel<__nv_bfloat16>, dim3((unsigned)(heads * ngroups)), dim3(256), 0, st, a, ma,
+      TQ_CHECK_CUDA(launch_dependent(prepare_mma_kernel<__nv_bfloat16>, dim3((unsigned)(heads * ngroups)), dim3(256), prep_smem, st, a, ma,
                                  static_cast<const __nv_bfloat16*>(Q), ldq), who);
     static std::atomic<size_t> mma_smem_set[16];
     if (dev >= 16 || mma_smem > mma_smem_set[dev].load(std::memory_order_relaxed)) {
@@ -936,12 +982,20 @@ extern "C" int tq_kv_append(const tq_kv_group* groups, int ngroups, int heads, i
                "%s: group %d: the plans belong to another device than the current one (%d)", who, gi, dev);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const dim3 grid((unsigned)(heads * ngroups), 2);
+  const size_t smem = (size_t)(d * d + d * (d + 4)) * sizeof(float);
+  static std::atomic<bool> smem_set[16];   // zero-initialised; written by any thread that launches
+  if (dev >= 16 || !smem_set[dev].load(std::memory_order_relaxed)) {
+    constexpr int smem_max = (MAXD * MAXD + MAXD * (MAXD + 4)) * (int)sizeof(float);
+    TQ_CHECK_CUDA(cudaFuncSetAttribute(append_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max), who);
+    TQ_CHECK_CUDA(cudaFuncSetAttribute(append_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max), who);
+    if (dev < 16) smem_set[dev].store(true, std::memory_order_relaxed);
+  }
   if (kv_dtype == TQ_F32)
-    append_kernel<float><<<grid, MAXD, 0, st>>>(a, static_cast<const float*>(K), ldk, static_cast<const float*>(V), ldv);
+    TQ_CHECK_CUDA(launch_dependent(append_kernel<float>, grid, dim3(MAXD), smem, st, a, static_cast<const float*>(K), ldk,
+                                   static_cast<const float*>(V), ldv), who);
   else
-    append_kernel<__nv_bfloat16><<<grid, MAXD, 0, st>>>(a, static_cast<const __nv_bfloat16*>(K), ldk,
-                                                         static_cast<const __nv_bfloat16*>(V), ldv);
-  TQ_CHECK_CUDA(cudaGetLastError(), who);
+    TQ_CHECK_CUDA(launch_dependent(append_kernel<__nv_bfloat16>, grid, dim3(MAXD), smem, st, a, static_cast<const __nv_bfloat16*>(K), ldk,
+                                   static_cast<const __nv_bfloat16*>(V), ldv), who);
   count_launches(1);
   return TQ_OK;
 }

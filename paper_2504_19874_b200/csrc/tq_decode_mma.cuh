@@ -166,7 +166,8 @@ __device__ __forceinline__ void derive_planes(const uint32_t* raw, uint32_t* der
 // ------------------------------------------------------------------ query preparation for the tensor path
 template <typename T>
 __global__ void __launch_bounds__(256) prepare_mma_kernel(Args a, MmaArgs ma, const T* __restrict__ Q, int64_t ldq) {
-  __shared__ float qs[MAXQ][MAXD];
+  extern __shared__ __align__(16) float rot[];   // [d][nrows] of [Pi ; S], transposed
+  __shared__ __align__(16) float qs[MAXD][MAXQ];
   __shared__ float qr[MAXQ][2 * MAXD];           // q' then q''
   __shared__ int wmax[2][MAXQ];                  // bit patterns of the largest |weight| per term and query
   __shared__ int wdsum[2][MAXQ][4];
@@ -175,9 +176,17 @@ __global__ void __launch_bounds__(256) prepare_mma_kernel(Args a, MmaArgs ma, co
   const GroupDev& g = a.g[gi];
   const MmaGroup& m = ma.m[gi];
   const int d = a.d, tid = threadIdx.x;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the slices' code rows may start to travel
-  // this kernel may itself have been scheduled while the kernel ahead in the stream drains (it may produce Q)
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int nrows = (g.k_prod ? 2 : 1) * g.k_dpad;
+  {   // the rotation (the plan's) to shared memory: ahead of the wait
+    const uint32_t to = (uint32_t)__cvta_generic_to_shared(rot);
+    for (int i = tid; i < d * nrows / 4; i += blockDim.x)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + 16 * i), "l"(g.k_backt + 4 * i) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  // This kernel may itself have been scheduled while the kernel ahead in the stream drains, which may produce Q and, if it is
+  // tq_kv_append, code rows: the partial kernel copies code rows before its own wait, so it may be scheduled only from here on.
+  wait_for_predecessor();
+  allow_successor();
   for (int e = tid; e < MAXQ * d; e += blockDim.x) {
     const int j = e / d, c = e % d;
     float v = 0.f;
@@ -185,22 +194,25 @@ __global__ void __launch_bounds__(256) prepare_mma_kernel(Args a, MmaArgs ma, co
       const int ch = g.k_channels[h * d + c];
       if (TQ_DEVICE_CHECK(ch >= 0 && ch < a.ldq_dbg, a.status)) v = (float)Q[(int64_t)(h * a.qpk + j) * ldq + ch];
     }
-    qs[j][c] = v;
+    qs[c][j] = v;
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   if (tid < 2 * MAXQ) wmax[tid / MAXQ][tid % MAXQ] = 0;
   if (tid < 2 * MAXQ * 4) (&wdsum[0][0][0])[tid] = 0;
   __syncthreads();
-  const int nrows = (g.k_prod ? 2 : 1) * g.k_dpad;
   for (int o = tid; o < 2 * MAXD; o += blockDim.x) {
     const int half = o / MAXD, r = o % MAXD;
     float acc[MAXQ] = {0.f, 0.f, 0.f, 0.f};
     if (r < d && (half == 0 || g.k_prod)) {
-      const float* col = g.k_backt + half * g.k_dpad + r;
-#pragma unroll 32
-      for (int c = 0; c < d; ++c) {   // independent loads: unrolled deep, the kernel is latency-bound
-        const float mm = __ldg(col + (size_t)c * nrows);
-#pragma unroll
-        for (int j = 0; j < MAXQ; ++j) acc[j] = fmaf(mm, qs[j][c], acc[j]);
+      const float* col = rot + half * g.k_dpad + r;
+#pragma unroll 16
+      for (int c = 0; c < d; ++c) {
+        const float mm = col[c * nrows];
+        const float4 q4 = *reinterpret_cast<const float4*>(qs[c]);
+        acc[0] = fmaf(mm, q4.x, acc[0]);
+        acc[1] = fmaf(mm, q4.y, acc[1]);
+        acc[2] = fmaf(mm, q4.z, acc[2]);
+        acc[3] = fmaf(mm, q4.w, acc[3]);
       }
     }
 #pragma unroll
