@@ -216,7 +216,8 @@ bool has_pad_words(int d, int bits, size_t row_bytes) {
 // Few queries: one warp per output column j forms <Rot[j, :], q> for up to 8 queries at a time.  The
 // warp's slice of the matrix row goes to registers first, so that its latency overlaps the staging
 // of the queries in shared memory; each lane sums its products in fp32, the 32 partial sums are
-// added in fp64.  The matrix is read once per 8 queries.
+// added in fp64.  The matrix is read once per 8 queries; its rows are padded with zeros to a multiple of 8 columns, so that
+// they are read 16 bytes at a time at every d (element by element, 123 queries of d = 1863 took 162 us and more).
 constexpr int kRotQ = 8, kRotChunk = 2048;   // 64 KB of queries per chunk (dynamic shared memory)
 constexpr int kRotQPerBlock = 64;            // most queries per CTA (grid.y covers the rest)
 // Queries per CTA: 64 (eight rounds, the matrix is read once for all of them) where that still gives every SM two CTAs, else
@@ -228,15 +229,14 @@ inline int rotate_queries_per_cta(int64_t column_ctas, int nq) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) rotate_queries_kernel(const float* __restrict__ Rot, int nrows, int d,
+__global__ void __launch_bounds__(256) rotate_queries_kernel(const float* __restrict__ Rot, int nrows, int d, int dpad,
                                                              const T* __restrict__ Q, int64_t ldq, int nq,
                                                              float* __restrict__ Qcat, int64_t ldo, int per_cta, int stride) {
   extern __shared__ __align__(16) float qs_raw[];   // [queries of a round][stride]
   auto qs = [&](int qq, int c) -> float* { return qs_raw + qq * stride + c; };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int j = blockIdx.x * 8 + warp;
-  const float* row = Rot + (size_t)min(j, nrows - 1) * d;
-  const bool vec = (d & 3) == 0;   // rows are 16-byte aligned
+  const float* row = Rot + (size_t)min(j, nrows - 1) * dpad;
   const int q_begin = blockIdx.y * per_cta, q_end = min(nq, q_begin + per_cta);
   for (int q0 = q_begin; q0 < q_end; q0 += kRotQ) {
     float acc[kRotQ];
@@ -244,15 +244,13 @@ __global__ void __launch_bounds__(256) rotate_queries_kernel(const float* __rest
     for (int qq = 0; qq < kRotQ; ++qq) acc[qq] = 0.f;
     const int nact = min(kRotQ, q_end - q0);   // queries of this round: the others are neither staged nor summed
     for (int c0 = 0; c0 < d; c0 += kRotChunk) {
-      const int len = min(kRotChunk, d - c0);
+      const int len = min(kRotChunk, dpad - c0);   // the matrix and the staged queries hold zeros in the columns past d
       float4 r[kRotChunk / 128];
-      if (vec) {
-        const float4* row4 = reinterpret_cast<const float4*>(row + c0);
+      const float4* row4 = reinterpret_cast<const float4*>(row + c0);
 #pragma unroll
-        for (int i = 0; i < kRotChunk / 128; ++i) {
-          const int c4 = lane + 32 * i;
-          r[i] = (4 * c4 < len) ? __ldg(row4 + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+      for (int i = 0; i < kRotChunk / 128; ++i) {
+        const int c4 = lane + 32 * i;
+        r[i] = (4 * c4 < len) ? __ldg(row4 + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
       if (q0 == q_begin && c0 == 0) {   // the first piece of the matrix (the plan's) is on its way
         wait_for_predecessor();         // it may write the queries
@@ -262,35 +260,24 @@ __global__ void __launch_bounds__(256) rotate_queries_kernel(const float* __rest
       for (int e = threadIdx.x; e < nact * (stride / 4); e += blockDim.x) {
         const int qq = e / (stride / 4), c = 4 * (e % (stride / 4));
         float v[4] = {0.f, 0.f, 0.f, 0.f};
-        if (q0 + qq < q_end && c < len) {
-          const T* src = Q + (int64_t)(q0 + qq) * ldq + c0 + c;
+        const T* src = Q + (int64_t)(q0 + qq) * ldq + c0 + c;
 #pragma unroll
-          for (int t = 0; t < 4; ++t)
-            if (c + t < len) v[t] = scan::to_f32<T>(src[t]);
-        }
+        for (int t = 0; t < 4; ++t)
+          if (c0 + c + t < d) v[t] = scan::to_f32<T>(src[t]);
         *reinterpret_cast<float4*>(qs(qq, c)) = make_float4(v[0], v[1], v[2], v[3]);
       }
       __syncthreads();
-      if (vec) {
 #pragma unroll
-        for (int i = 0; i < kRotChunk / 128; ++i) {
-          const int c4 = lane + 32 * i;
-          if (4 * c4 < len) {
+      for (int i = 0; i < kRotChunk / 128; ++i) {
+        const int c4 = lane + 32 * i;
+        if (4 * c4 < len) {
 #pragma unroll
-            for (int qq = 0; qq < kRotQ; ++qq) {
-              if (qq < nact) {
-                const float4 v = *reinterpret_cast<const float4*>(qs(qq, 4 * c4));
-                acc[qq] = fmaf(r[i].x, v.x, fmaf(r[i].y, v.y, fmaf(r[i].z, v.z, fmaf(r[i].w, v.w, acc[qq]))));
-              }
+          for (int qq = 0; qq < kRotQ; ++qq) {
+            if (qq < nact) {
+              const float4 v = *reinterpret_cast<const float4*>(qs(qq, 4 * c4));
+              acc[qq] = fmaf(r[i].x, v.x, fmaf(r[i].y, v.y, fmaf(r[i].z, v.z, fmaf(r[i].w, v.w, acc[qq]))));
             }
           }
-        }
-      } else {
-        for (int c = lane; c < len; c += 32) {
-          const float rv = __ldg(row + c0 + c);
-#pragma unroll
-          for (int qq = 0; qq < kRotQ; ++qq)
-            if (qq < nact) acc[qq] = fmaf(rv, *qs(qq, c), acc[qq]);
         }
       }
     }
@@ -311,10 +298,10 @@ __global__ void __launch_bounds__(256) rotate_queries_kernel(const float* __rest
 // 16-byte loads), a CTA of four warps 32 rows, and the queries are read once per 32 output columns instead of once
 // per 8.  Three CTAs per SM hide each other's staging.
 constexpr int kRmRows = 8, kRmWarps = 4, kRmRowsPerBlock = kRmWarps * kRmRows;
-constexpr int kRotManyFrom = 64;   // queries from which the blocked kernel is used (d a multiple of 4)
+constexpr int kRotManyFrom = 64;   // queries from which the blocked kernel is used
 
 template <typename T>
-__global__ void __launch_bounds__(32 * kRmWarps) rotate_many_kernel(const float* __restrict__ Rot, int nrows, int d,
+__global__ void __launch_bounds__(32 * kRmWarps) rotate_many_kernel(const float* __restrict__ Rot, int nrows, int d, int dpad,
                                                                     const T* __restrict__ Q, int64_t ldq, int nq,
                                                                     float* __restrict__ Qcat, int64_t ldo, int per_cta, int stride) {
   extern __shared__ __align__(16) float qs_raw[];   // [queries of a round][stride]
@@ -332,7 +319,7 @@ __global__ void __launch_bounds__(32 * kRmWarps) rotate_many_kernel(const float*
       for (int qq = 0; qq < kRotQ; ++qq) acc[rr][qq] = 0.f;
     const int nact = min(kRotQ, q_end - q0);
     for (int c0 = 0; c0 < d; c0 += kRotChunk) {
-      const int len = min(kRotChunk, d - c0);
+      const int len = min(kRotChunk, dpad - c0);   // the matrix and the staged queries hold zeros in the columns past d
       __syncthreads();
       for (int e = threadIdx.x; e < nact * (stride / 4); e += blockDim.x) {
         const int qq = e / (stride / 4), c = 4 * (e % (stride / 4));
@@ -340,7 +327,7 @@ __global__ void __launch_bounds__(32 * kRmWarps) rotate_many_kernel(const float*
         const T* src = Q + (int64_t)(q0 + qq) * ldq + c0 + c;
         float v[4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) v[t] = scan::to_f32<T>(src[t]);   // d is a multiple of 4: whole groups of four
+        for (int t = 0; t < 4; ++t) v[t] = c0 + c + t < d ? scan::to_f32<T>(src[t]) : 0.f;
         *reinterpret_cast<float4*>(qs(qq, c)) = make_float4(v[0], v[1], v[2], v[3]);
       }
       __syncthreads();
@@ -351,7 +338,7 @@ __global__ void __launch_bounds__(32 * kRmWarps) rotate_many_kernel(const float*
         float4 r[kRmRows];
 #pragma unroll
         for (int rr = 0; rr < kRmRows; ++rr)
-          r[rr] = __ldg(reinterpret_cast<const float4*>(Rot + (size_t)min(j0 + rr, nrows - 1) * d + c0) + c4);
+          r[rr] = __ldg(reinterpret_cast<const float4*>(Rot + (size_t)min(j0 + rr, nrows - 1) * dpad + c0) + c4);
 #pragma unroll
         for (int qq = 0; qq < kRotQ; ++qq) {
           if (qq < nact) {
@@ -396,7 +383,7 @@ template <typename T>
 cudaError_t launch_rotate_queries(const tq_plan* plan, const T* Q, int64_t ldq, int nq, float* Qcat, cudaStream_t st) {
   const int ncols = plan->ncat * plan->dpad;
   constexpr int smem_max = kRotQ * kRotChunk * (int)sizeof(float);
-  const int stride = std::min(round_up(plan->d, 4), kRotChunk), smem = std::min(nq, kRotQ) * stride * (int)sizeof(float);
+  const int stride = std::min(plan->dpad, kRotChunk), smem = std::min(nq, kRotQ) * stride * (int)sizeof(float);
   // function attributes are per device: remember the devices this launcher has prepared
   static std::atomic<unsigned long long> attr_devices{0};   // written by any thread that launches
   int attr_dev = 0;
@@ -406,7 +393,7 @@ cudaError_t launch_rotate_queries(const tq_plan* plan, const T* Q, int64_t ldq, 
     if (e != cudaSuccess) return e;
     if (attr_dev < 64) attr_devices.fetch_or(1ull << attr_dev, std::memory_order_relaxed);
   }
-  if (nq >= kRotManyFrom && (plan->d & 3) == 0) {
+  if (nq >= kRotManyFrom) {
     static std::atomic<unsigned long long> many_devices{0};
     if (attr_dev >= 64 || !((many_devices.load(std::memory_order_relaxed) >> attr_dev) & 1ull)) {
       cudaError_t e = cudaFuncSetAttribute(rotate_many_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
@@ -416,13 +403,13 @@ cudaError_t launch_rotate_queries(const tq_plan* plan, const T* Q, int64_t ldq, 
     const int cols = (ncols + kRmRowsPerBlock - 1) / kRmRowsPerBlock, per = rotate_queries_per_cta(cols, nq);
     const dim3 grid((unsigned)cols, (unsigned)((nq + per - 1) / per));
     count_launches(1);
-    return launch_dependent(rotate_many_kernel<T>, grid, dim3(32 * kRmWarps), smem, st, plan->dRotCat, ncols, plan->d, Q, ldq, nq, Qcat,
+    return launch_dependent(rotate_many_kernel<T>, grid, dim3(32 * kRmWarps), smem, st, plan->dRotCat, ncols, plan->d, plan->dpad, Q, ldq, nq, Qcat,
                             (int64_t)ncols, per, stride);
   }
   const int cols = (ncols + 7) / 8, per = rotate_queries_per_cta(cols, nq);
   const dim3 grid((unsigned)cols, (unsigned)((nq + per - 1) / per));
   count_launches(1);
-  return launch_dependent(rotate_queries_kernel<T>, grid, dim3(256), smem, st, plan->dRotCat, ncols, plan->d, Q, ldq, nq, Qcat, (int64_t)ncols,
+  return launch_dependent(rotate_queries_kernel<T>, grid, dim3(256), smem, st, plan->dRotCat, ncols, plan->d, plan->dpad, Q, ldq, nq, Qcat, (int64_t)ncols,
                           per, stride);
 }
 
@@ -567,15 +554,15 @@ extern "C" int tq_plan_create(int d, int bits, int mode, const float* Pi, const 
   PLAN_CUDA(cudaGetDevice(&p->device), "cudaGetDevice");
   PLAN_CUDA(cudaMalloc(&p->dPi, dd * sizeof(float)), "cudaMalloc Pi");
   PLAN_CUDA(cudaMemcpy(p->dPi, Pi, dd * sizeof(float), cudaMemcpyHostToDevice), "copy Pi");
-  std::vector<float> rot((size_t)ncols * d, 0.f), back((size_t)d * ncols, 0.f);
+  std::vector<float> rot((size_t)ncols * p->dpad, 0.f), back((size_t)d * ncols, 0.f);
   for (int i = 0; i < d; ++i) {
-    std::memcpy(&rot[(size_t)i * d], Pi + (size_t)i * d, d * sizeof(float));
+    std::memcpy(&rot[(size_t)i * p->dpad], Pi + (size_t)i * d, d * sizeof(float));
     for (int j = 0; j < d; ++j) back[(size_t)j * ncols + i] = Pi[(size_t)i * d + j];
   }
   float* dS = nullptr;
   if (mode == TQ_PROD) {
     for (int i = 0; i < d; ++i) {
-      std::memcpy(&rot[(size_t)(p->dpad + i) * d], S + (size_t)i * d, d * sizeof(float));
+      std::memcpy(&rot[(size_t)(p->dpad + i) * p->dpad], S + (size_t)i * d, d * sizeof(float));
       for (int j = 0; j < d; ++j) back[(size_t)j * ncols + p->dpad + i] = S[(size_t)i * d + j];
     }
     PLAN_CUDA(cudaMalloc(&dS, dd * sizeof(float)), "cudaMalloc S");

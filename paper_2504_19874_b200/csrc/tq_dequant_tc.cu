@@ -605,7 +605,7 @@ cudaError_t plan_init(tq_plan* plan, const float* Pi, const float* S) {
     if (e == cudaSuccess) e = cudaMalloc(lo, count * 2);
     if (e != cudaSuccess) return e;
     // dRotCat: rows of Pi, then (from row dpad) rows of S
-    transpose_limbs_kernel<<<grid, block>>>(plan->dRotCat + (which == 0 ? 0 : (size_t)plan->dpad * d), d, d,
+    transpose_limbs_kernel<<<grid, block>>>(plan->dRotCat + (which == 0 ? 0 : (size_t)plan->dpad * plan->dpad), d, plan->dpad,
                                             (float)std::ldexp(1.0, which == 0 ? eP : eS), *hi, *lo, m.pitch);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -109,7 +109,7 @@ struct tq_plan {
   tq::Codebook cb;
   float* dPi;      // [d, d]            y = Pi x            (rows of Pi)
   float* dSp;      // [d, d]            S' = S Pi^T         (TQ_PROD)
-  float* dRotCat;  // [ncat*dpad, d]    rows: Pi (padded to dpad rows) then S     (query preparation)
+  float* dRotCat;  // [ncat*dpad, dpad] rows: Pi (padded to dpad rows) then S, zeros in the padding (query preparation)
   float* dBackT;   // [d, ncat*dpad]    row j: [ Pi[:, j] | S[:, j] ]             (dequantisation)
   int ncat;        // 1 (mse) or 2 (prod): halves of the virtual K axis [ c[idx] | coef*gamma*z ]
   // tensor-core quantisation path (d >= 128)
