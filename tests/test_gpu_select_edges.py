@@ -18,8 +18,8 @@ def expected(s, i, k):
     return out_s, out_i
 
 
-@pytest.mark.parametrize("m", [1, 31, 1000, 1025, 16384, 16385, 40000])
-@pytest.mark.parametrize("kind", ["normal", "ties", "equal", "outlier", "infinite", "empty slots"])
+@pytest.mark.parametrize("m", [1, 31, 1000, 1025, 4096, 4097, 16384, 16385, 40000])
+@pytest.mark.parametrize("kind", ["normal", "ties", "equal", "outlier", "infinite", "empty slots", "crowded"])
 def test_selection(m, kind):
     g = np.random.default_rng(m)
     nq = 3
@@ -33,11 +33,13 @@ def test_selection(m, kind):
         s[:, m // 2] = 1e30
     elif kind == "infinite":
         s[0, 0], s[1, m - 1] = np.inf, -np.inf
+    elif kind == "crowded":   # the largest scores meet in few threads, so that the threads' maxima say little about them
+        s[:, np.arange(m) % 1024 < 40] += 10.0
     ids = np.stack([g.permutation(m) for _ in range(nq)]).astype(np.int32)
     if kind == "empty slots":
         ids[g.random((nq, m)) < 0.9] = -1
     cs, ci = torch.from_numpy(s).to(DEV), torch.from_numpy(ids).to(DEV)
-    for k in (1, 10, 1024):
+    for k in (1, 10, 256, 257, 1024):
         ts, ti = torch.empty((nq, k), device=DEV), torch.empty((nq, k), dtype=torch.int32, device=DEV)
         tq.tq_select_topk(cs, ci, k, ts, ti)
         for q in range(nq):
