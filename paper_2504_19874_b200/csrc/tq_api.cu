@@ -584,10 +584,9 @@ extern "C" int tq_plan_create(int d, int bits, int mode, const float* Pi, const 
   PLAN_CUDA(cudaMalloc(&p->d_status, sizeof(int)), "cudaMalloc status");
   PLAN_CUDA(cudaMemset(p->d_status, 0, sizeof(int)), "clear status");
   if (tc::supported(d)) {
-    p->tc_bn = tc::pick_bn(d);
-    PLAN_CUDA(tc::build_matrix_limbs(p->dPi, d, d, p->dpad, p->tc_bn, &p->pi_limbs), "bf16 limbs of Pi");
+    PLAN_CUDA(tc::build_matrix_limbs(p->dPi, d, d, p->dpad, &p->pi_limbs), "bf16 limbs of Pi");
     if (mode == TQ_PROD)
-      PLAN_CUDA(tc::build_matrix_limbs(p->dSp, d, d, p->dpad, p->tc_bn, &p->sp_limbs), "bf16 limbs of S'");
+      PLAN_CUDA(tc::build_matrix_limbs(p->dSp, d, d, p->dpad, &p->sp_limbs), "bf16 limbs of S'");
     p->tc_ok = 1;
   }
   PLAN_CUDA(sq::plan_init(p), "transpose of S'");

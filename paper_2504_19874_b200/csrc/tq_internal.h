@@ -85,13 +85,12 @@ cudaError_t launch_dependent(void (*kern)(KArgs...), dim3 grid, dim3 block, size
 }
 #endif
 
+constexpr int kBoxes = 4;
 struct MatrixLimbs {
   __nv_bfloat16* hi;
   __nv_bfloat16* lo;
-  alignas(64) CUtensorMap map_hi;
-  alignas(64) CUtensorMap map_lo;
-  alignas(64) CUtensorMap map_hi_half;   // boxes of half as many rows: what one CTA of a pair loads
-  alignas(64) CUtensorMap map_lo_half;
+  alignas(64) CUtensorMap map_hi[kBoxes];   // box i: 32 (i + 1) rows, what one CTA of a tile loads
+  alignas(64) CUtensorMap map_lo[kBoxes];
 };
 
 }  // namespace tq
@@ -114,7 +113,6 @@ struct tq_plan {
   int ncat;        // 1 (mse) or 2 (prod): halves of the virtual K axis [ c[idx] | coef*gamma*z ]
   // tensor-core quantisation path (d >= 128)
   int tc_ok;       // 1 when the limbs / TMA descriptors below are built
-  int tc_bn;       // N extent of its MMA tile
   tq::MatrixLimbs pi_limbs;   // Pi
   tq::MatrixLimbs sp_limbs;   // S' (TQ_PROD)
   // bit-plane scan on the integer tensor path (d >= 128, antisymmetric codebook)

@@ -8,8 +8,9 @@
 // ~1e-7 on a rotated coordinate of a unit vector at d = 1536 -- far inside the 1e-5 window in
 // which a nearest-centroid decision may legitimately differ from exact arithmetic.
 //
-// Two forms of the GEMM kernel: one CTA per 128 x 256 tile, and (the usual one at d > 128) a pair of CTAs of one
-// cluster per 256 x 256 tile (tcgen05 cta_group::2), which halves what every SM reads of B from shared memory.
+// Two forms of the GEMM kernel: one CTA per tile of 128 rows, and (the usual one at d > 128) a pair of CTAs of one
+// cluster per tile of 256 rows (tcgen05 cta_group::2), which halves what every SM reads of B from shared memory.  The
+// tiles are up to 256 columns wide; few rows take narrower ones, so that every SM has one (pick_tile).
 #include <atomic>
 #include <cstdlib>
 #include <algorithm>
@@ -26,21 +27,25 @@ namespace {
 constexpr int BM = 128;          // rows of X per tile = TMEM lanes
 constexpr int BK = 64;           // bf16 elements per 128-byte swizzled row
 constexpr int UMMA_K = 16;
-constexpr int EPS = 4;           // epilogue warps per TMEM lane group: each takes 1/EPS of the tile's columns
-constexpr int NSPLIT = 2;        // warps that prepare the next block's operand limbs beside the GEMM (see SplitTask)
-constexpr int NTHREADS = 32 * (2 + 4 * EPS + NSPLIT);   // warp 0: TMA, warp 1: MMA + TMEM owner, the epilogue warps, the split warps
+constexpr int NSPLIT = 2;        // spare warps beside the GEMM: the next block's operand limbs (see SplitTask), gamma (MODE 2)
 
 // CTAS = 2: two CTAs of a cluster share one 256-row tile (tcgen05 cta_group::2).  Each loads its own 128 rows of A and
 // its own half of B's rows, so a k-block costs each SM 64 KB of shared-memory writes instead of 96 and its MMAs read
 // half of B from the partner: the shared-memory bandwidth that caps the one-CTA kernel (158 bytes per clock wanted,
 // 128 available) drops to 104.
+struct Tile { int bn, ctas; };   // columns of a tile, CTAs that share it
+
 template <int BN, int CTAS>
 struct Cfg {
+  // epilogue warps per TMEM lane group: each takes 1/kEps of the tile's columns, 64 (32 where the tile is the whole row)
+  static constexpr int kEps = CTAS == 1 && BN == 128 ? 4 : BN / 64;
+  static constexpr int kThreads = 32 * (2 + 4 * kEps + NSPLIT);             // warp 0: TMA, warp 1: MMA + TMEM owner, epilogue, spare
   static constexpr int kBRows = BN / CTAS;                                  // rows of B this CTA loads
   static constexpr int kStageBytes = 2 * BM * BK * 2 + 2 * kBRows * BK * 2; // A hi/lo + B hi/lo
-  static constexpr int kStages = CTAS == 2 ? 3 : ((BN == 256) ? 2 : (BN == 128 ? 3 : 4));
-  static constexpr int kTmemCols = 2 * BN;                                  // two accumulators
-  static constexpr int kStoreBytes = 4 * EPS * 2048;   // MODE 1: one [32 rows x 64 B] box per epilogue warp, staged for a TMA store
+  static constexpr int kStages = CTAS == 2 ? (BN == 128 ? 4 : 3) : (BN == 128 ? 3 : 4);
+  static constexpr int kAccCols = BN == 192 ? 256 : BN;                     // TMEM columns from one accumulator to the next
+  static constexpr int kTmemCols = 2 * kAccCols;                            // two accumulators
+  static constexpr int kStoreBytes = 4 * kEps * 2048;  // MODE 1: one [32 rows x 64 B] box per epilogue warp, staged for a TMA store
   static constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 512 /*barriers, centroids*/ + kStoreBytes;
 };
 
@@ -56,7 +61,9 @@ struct GemmArgs {
   const CUtensorMap* store_e1;   // host pointers to the TMA store maps of E1 / E2 (box 32 rows x 32 columns, 64-byte swizzle);
   const CUtensorMap* store_e2;   // the launcher passes them on as kernel arguments
   int64_t ldE;
-  float* gpart;          // MODE 1: [EPS * tiles_n][Mpad] partial sums of e^2 (one per epilogue warp's columns)
+  float* gpart;          // MODE 1: [parts][Mpad] partial sums of e^2, one per epilogue warp's columns; MODE 2: gamma from them
+  float* gamma;          // MODE 2
+  int parts;
   int64_t Mpad;
   const float* nu;       // MODE 1: per-row norm (row with nu == 0 has residual 0); nullable
   // TQ_LAYOUT_NIBBLE (BITS = 3 with MODE 1, and MODE 2): the codes of 32 coordinates are four words of the combined
@@ -205,15 +212,24 @@ __device__ __forceinline__ void split_rows(const T* __restrict__ X, int64_t ldx,
       return;
     }
   }
+  // Other rows: a lane adds its squares over j = lane, lane + 32, ... with sixteen loads in flight (one load at a time took
+  // 11.7 us for 1,001 rows of 3,072 bf16), then converts eight neighbouring elements at a time (one 16-byte load where bf16 rows
+  // are aligned).
+  const bool vec8 = sizeof(T) == 2 && (ldx & 7) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+  auto value = [](T v) -> float {
+    if constexpr (sizeof(T) == 4) return v; else return __bfloat162float(v);
+  };
   for (int64_t r = warp; r < n; r += nwarps) {
     const T* row = X + r * ldx;
     float inv = 1.f;
     if (NORMALIZE) {
       float s = 0.f;
-      for (int j = lane; j < d; j += 32) {
-        float v;
-        if constexpr (sizeof(T) == 4) v = row[j]; else v = __bfloat162float(row[j]);
-        s = fmaf(v, v, s);
+      for (int j0 = lane; j0 < d; j0 += 512) {
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = j0 + 32 * i < d ? value(row[j0 + 32 * i]) : 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) s = fmaf(v[i], v[i], s);
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -221,24 +237,29 @@ __device__ __forceinline__ void split_rows(const T* __restrict__ X, int64_t ldx,
       inv = (nu > 0.f) ? 1.f / nu : 0.f;
       if (lane == 0 && norms != nullptr) norms[r] = nu;
     }
+#pragma unroll 2
     for (int j0 = lane * 8; j0 < dpad; j0 += 256) {
+      float u[8];
+      if (vec8 && j0 + 8 <= d) {
+        const uint4 raw = *reinterpret_cast<const uint4*>(row + j0);
+        const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          u[2 * p] = __uint_as_float(w[p] << 16);
+          u[2 * p + 1] = __uint_as_float(w[p] & 0xffff0000u);
+        }
+      } else {
+#pragma unroll
+        for (int p = 0; p < 8; ++p) u[p] = j0 + p < d ? value(row[j0 + p]) : 0.f;
+      }
       uint32_t h[4], l[4];
 #pragma unroll
       for (int p = 0; p < 4; ++p) {
-        float u[2];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int j = j0 + 2 * p + q;
-          float v = 0.f;
-          if (j < d) {
-            if constexpr (sizeof(T) == 4) v = row[j]; else v = __bfloat162float(row[j]);
-          }
-          u[q] = v * inv;
-        }
-        const float h0 = __bfloat162float(__float2bfloat16_rn(u[0]));
-        const float h1 = __bfloat162float(__float2bfloat16_rn(u[1]));
+        const float u0 = u[2 * p] * inv, u1 = u[2 * p + 1] * inv;
+        const float h0 = __bfloat162float(__float2bfloat16_rn(u0));
+        const float h1 = __bfloat162float(__float2bfloat16_rn(u1));
         h[p] = pack_bf16x2(h0, h1);
-        l[p] = pack_bf16x2(u[0] - h0, u[1] - h1);
+        l[p] = pack_bf16x2(u0 - h0, u1 - h1);
       }
       *reinterpret_cast<uint4*>(L1 + r * dpad + j0) = make_uint4(h[0], h[1], h[2], h[3]);
       *reinterpret_cast<uint4*>(L2 + r * dpad + j0) = make_uint4(l[0], l[1], l[2], l[3]);
@@ -250,17 +271,20 @@ template <typename T, bool NORMALIZE>
 __global__ void __launch_bounds__(256) split_rows_kernel(const T* __restrict__ X, int64_t ldx, int64_t n, int d, int dpad,
                                                          __nv_bfloat16* __restrict__ L1, __nv_bfloat16* __restrict__ L2,
                                                          float* __restrict__ norms) {
+  allow_successor();        // (every kernel behind waits for this one, and so for those ahead of it, before it writes or reads)
+  wait_for_predecessor();   // it may write X, or read the limb buffers
   split_rows<T, NORMALIZE>(X, ldx, n, d, dpad, L1, L2, norms, (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5),
                            (int64_t)gridDim.x * (blockDim.x >> 5), threadIdx.x & 31);
 }
 
 // MODE 0: idx.  MODE 1: idx + residual limbs + partial ||e||^2.  MODE 2: sign bits.
 template <int BN, int MODE, int BITS, int CTAS>
-__global__ void __launch_bounds__(NTHREADS, 1)
+__global__ void __launch_bounds__(Cfg<BN, CTAS>::kThreads, 1)
 quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmA2,
                      const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2,
                      const __grid_constant__ CUtensorMap tmE1, const __grid_constant__ CUtensorMap tmE2, GemmArgs a) {
   using C = Cfg<BN, CTAS>;
+  constexpr int EPS = C::kEps;
   const int rank = CTAS == 2 ? (int)cluster_ctarank() : 0;   // CTA of the pair; rank 0 issues the MMAs
   const int64_t unit = blockIdx.x / CTAS, nunits = gridDim.x / CTAS;   // a unit = one CTA or one pair
   extern __shared__ unsigned char smem_raw[];
@@ -307,6 +331,8 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
   else __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  wait_for_predecessor();   // the operands are outputs of the kernel ahead; the outputs may be inputs of it
+  allow_successor();        // (only now: a scan's successor may start reading the codes, see nscan::run)
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -357,7 +383,7 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
         const uint32_t acc = (uint32_t)(it & 1), acc_phase = (uint32_t)((it >> 1) & 1);
         if (!(ok = mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, a.status))) break;
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * BN;
+        const uint32_t d_tmem = tmem_base + acc * C::kAccCols;
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!(ok = mbar_wait(&full[stage], phase, abort_flag, a.status))) break;
           tc_fence_after();
@@ -394,7 +420,23 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
     }
     __syncwarp();
   } else if (warp >= 2 + 4 * EPS) {
-    // ------------------------------------------------------------ operand limbs of the next block of rows
+    // ------------------------------------------------------------ spare warps
+    if (MODE == 2) {   // gamma = ||e|| from the rotate launch's partial sums, in the order of the columns
+      // (eight rows of a lane at a time: with one, the loads' latency made this the longest part of the kernel at d = 128)
+      const int64_t step = (int64_t)gridDim.x * NSPLIT * 32;
+      for (int64_t r = ((int64_t)blockIdx.x * NSPLIT + (warp - 2 - 4 * EPS)) * 32 + lane; r < a.M; r += 8 * step) {
+        float g2[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+        for (int t = 0; t < a.parts; ++t) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) g2[i] += r + i * step < a.M ? __ldcg(a.gpart + (int64_t)t * a.Mpad + r + i * step) : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (r + i * step < a.M) a.gamma[r + i * step] = sqrtf(g2[i]);
+      }
+    }
+    // operand limbs of the next block of rows
     const GemmArgs::SplitTask& t = a.split;
     if (t.rows > 0) {
       const int64_t sw = (int64_t)blockIdx.x * NSPLIT + (warp - 2 - 4 * EPS), nsw = (int64_t)gridDim.x * NSPLIT;
@@ -432,7 +474,7 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
         const int col0 = n0 + c * 32;
         if (col0 >= a.N) break;   // uniform across the CTA: nothing but zero padding beyond
         uint32_t v[32];
-        tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + acc * BN + c * 32, v);
+        tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + acc * C::kAccCols + c * 32, v);
         tmem_ld_wait();
         if (MODE == 2) {
           uint32_t word = 0;
@@ -548,7 +590,7 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
         if (CTAS == 2) mbar_arrive_leader(&tempty[acc]);
         else mbar_arrive(&tempty[acc]);
       }
-      if (MODE == 1 && row_ok && TQ_DEVICE_CHECK(row < a.Mpad && tn < a.tiles_n, a.status))
+      if (MODE == 1 && row_ok && EPS * tn + half < a.parts && TQ_DEVICE_CHECK(row < a.Mpad && tn < a.tiles_n, a.status))
         a.gpart[(int64_t)(EPS * tn + half) * a.Mpad + row] = gsum;
       // pad words past the last tile's columns (rows whose stride exceeds the tiles' coverage)
       if (a.nibble && tn == a.tiles_n - 1 && half == EPS - 1 && row_ok) {
@@ -580,17 +622,6 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
     if (CTAS == 2) tmem_dealloc_pair(tmem_base, C::kTmemCols);
     else tmem_dealloc(tmem_base, C::kTmemCols);
   }
-}
-
-// ---------------------------------------------------------------- operand splitting
-// gamma = sqrt(sum over column tiles of the partial sums), in tile order (deterministic).
-__global__ void gamma_finish_kernel(const float* __restrict__ gpart, int64_t Mpad, int tiles_n, int64_t rows,
-                                    float* __restrict__ gamma) {
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= rows) return;
-  float s = 0.f;
-  for (int t = 0; t < tiles_n; ++t) s += gpart[(int64_t)t * Mpad + r];
-  gamma[r] = sqrtf(s);
 }
 
 // ---------------------------------------------------------------- host side
@@ -715,22 +746,20 @@ cudaError_t launch_gemm_t(const CUtensorMap& a1, const CUtensorMap& a2, const CU
   // the store maps of the residual limbs (MODE 1); any valid map otherwise
   const CUtensorMap& e1 = args.store_e1 ? *args.store_e1 : a1;
   const CUtensorMap& e2 = args.store_e2 ? *args.store_e2 : a2;
-  if (CTAS == 1) {
-    kern<<<units, NTHREADS, C::kSmemBytes, st>>>(a1, a2, b1, b2, e1, e2, args);
-    return cudaGetLastError();
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(units * CTAS));
-  cfg.blockDim = dim3(NTHREADS);
+  cfg.blockDim = dim3(C::kThreads);
   cfg.dynamicSmemBytes = C::kSmemBytes;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CTAS;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = CTAS;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = CTAS == 1 ? 1 : 2;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a1, a2, b1, b2, e1, e2, args);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -751,22 +780,27 @@ cudaError_t launch_gemm_bits(int bits, const CUtensorMap& a1, const CUtensorMap&
   }
 }
 
-// ctas = 2: CTA pairs (only with 256-column tiles); b1, b2 are then the maps with half-height boxes.
 template <int MODE>
-cudaError_t launch_gemm(int bn, int ctas, int bits, const CUtensorMap& a1, const CUtensorMap& a2, const CUtensorMap& b1,
-                        const CUtensorMap& b2, const GemmArgs& args, cudaStream_t st) {
-  if (bn == 256 && ctas == 2) return launch_gemm_bits<256, MODE, 2>(bits, a1, a2, b1, b2, args, st);
-  if (bn == 256) return launch_gemm_bits<256, MODE, 1>(bits, a1, a2, b1, b2, args, st);
-  return launch_gemm_bits<128, MODE, 1>(bits, a1, a2, b1, b2, args, st);
+cudaError_t launch_gemm(const Tile& t, int bits, const CUtensorMap& a1, const CUtensorMap& a2, const MatrixLimbs& b,
+                        const GemmArgs& args, cudaStream_t st) {
+  const int box = t.bn / t.ctas / 32 - 1;   // maps by the rows of B that a CTA loads
+  const CUtensorMap &b1 = b.map_hi[box], &b2 = b.map_lo[box];
+  if (t.ctas == 1) {
+    if (t.bn == 128) return launch_gemm_bits<128, MODE, 1>(bits, a1, a2, b1, b2, args, st);
+    return launch_gemm_bits<64, MODE, 1>(bits, a1, a2, b1, b2, args, st);
+  }
+  switch (t.bn) {
+    case 128: return launch_gemm_bits<128, MODE, 2>(bits, a1, a2, b1, b2, args, st);
+    case 192: return launch_gemm_bits<192, MODE, 2>(bits, a1, a2, b1, b2, args, st);
+    default: return launch_gemm_bits<256, MODE, 2>(bits, a1, a2, b1, b2, args, st);
+  }
 }
 
 }  // namespace
 
-int pick_bn(int d) { return d > 128 ? 256 : 128; }
-
 bool supported(int d) { return d >= 128 && encode_fn() != nullptr; }
 
-cudaError_t build_matrix_limbs(const float* dM, int rows, int d, int dpad, int bn, MatrixLimbs* out) {
+cudaError_t build_matrix_limbs(const float* dM, int rows, int d, int dpad, MatrixLimbs* out) {
   out->hi = out->lo = nullptr;
   const size_t bytes = (size_t)rows * dpad * sizeof(__nv_bfloat16);
   cudaError_t e = cudaMalloc(&out->hi, bytes);
@@ -777,9 +811,9 @@ cudaError_t build_matrix_limbs(const float* dM, int rows, int d, int dpad, int b
   split_rows_kernel<float, false><<<blocks, 256>>>(dM, d, rows, d, dpad, out->hi, out->lo, nullptr);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (!make_map(&out->map_hi, out->hi, rows, d, dpad, bn) || !make_map(&out->map_lo, out->lo, rows, d, dpad, bn) ||
-      !make_map(&out->map_hi_half, out->hi, rows, d, dpad, bn / 2) || !make_map(&out->map_lo_half, out->lo, rows, d, dpad, bn / 2))
-    return cudaErrorInvalidValue;
+  for (int i = 0; i < kBoxes; ++i)
+    if (!make_map(&out->map_hi[i], out->hi, rows, d, dpad, 32 * (i + 1)) || !make_map(&out->map_lo[i], out->lo, rows, d, dpad, 32 * (i + 1)))
+      return cudaErrorInvalidValue;
   return cudaSuccess;
 }
 
@@ -798,17 +832,44 @@ bool pair_tiles_enabled() {
   return on;
 }
 
+// Tile of a block of rows: the one with the least waves x time.  Every output is the same sum in the same order on all of them,
+// so the codes do not depend on it.  Time of a k-block of 64 in units of 10 ns, all SMs busy (d = 768 to 3072): 62 for 128 x 64
+// on one CTA, and on a pair 68, 93 and 120 for 256 x 128, 192 and 256 (the rule takes a little more for the narrow ones: under
+// the power limit of a long call they lose 5 to 20 %).  The wider the tile, the fewer operand bytes per MMA, so 256 columns win
+// wherever there are waves enough, and narrower tiles where a wave would leave SMs idle (TQ_PROD, us: d = 3072, 1,000 rows: 145,
+// 113 and 129 with 128, 192 and 256 columns; 50,000 rows: 4,287, 3,963 and 3,813; d = 1536, 128 rows: 42 with 64 columns, 62
+// with 256).  d <= 128: one tile is the whole row.  *time: waves x time.
+Tile pick_tile(int64_t rows, int d, int64_t* time = nullptr) {
+  if (d <= 128) return {128, 1};
+  static constexpr struct { Tile t; int time; } kChoices[] = {{{256, 2}, 120}, {{192, 2}, 96}, {{128, 2}, 72}, {{64, 1}, 64}};
+  Tile best = {64, 1};
+  int64_t least = INT64_MAX;
+  for (const auto& c : kChoices) {
+    if (c.t.ctas == 2 && !pair_tiles_enabled()) continue;
+    const int64_t tiles = ((rows + BM * c.t.ctas - 1) / (BM * c.t.ctas)) * ((d + c.t.bn - 1) / c.t.bn);
+    const int units = sm_count() / c.t.ctas;
+    const int64_t cost = (tiles + units - 1) / units * c.time;
+    if (cost < least) {
+      least = cost;
+      best = c.t;
+    }
+  }
+  if (time != nullptr) *time = least;
+  return best;
+}
+
+// Partial sums of e^2 per row: room for four per 256 columns.
+int gamma_parts(int d) { return 4 * ((d + 255) / 256); }
+
 size_t scratch_bytes_per_row(const tq_plan* plan) {
-  const int tiles_n = (plan->d + plan->tc_bn - 1) / plan->tc_bn;
   size_t per = (size_t)plan->dpad * 2 * 2 + sizeof(float);                            // X limbs + nu
-  if (plan->mode == TQ_PROD) per += (size_t)plan->dpad * 2 * 2 + (size_t)tiles_n * 4 * EPS;  // E limbs + partial sums (EPS per column tile)
+  if (plan->mode == TQ_PROD) per += (size_t)plan->dpad * 2 * 2 + (size_t)gamma_parts(plan->d) * sizeof(float);  // E limbs + partial sums
   return per;
 }
 
 int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t ldx, uint8_t* idx, uint8_t* qjl,
              float* gamma, float* norms, void* scratch, size_t scratch_bytes, cudaStream_t st, const char* who) {
-  const int d = plan->d, dpad = plan->dpad, bn = plan->tc_bn;
-  const int tiles_n = (d + bn - 1) / bn;
+  const int d = plan->d, dpad = plan->dpad;
   const bool prod = plan->mode == TQ_PROD;
   const size_t per_row = scratch_bytes_per_row(plan);
   int64_t R = (int64_t)(scratch_bytes / per_row) / BM * BM;
@@ -823,7 +884,15 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
   // loses (d = 1536: 22.1 against 21.5 ms, d = 3072 alike), so its project launch carries no such task any more; at
   // d = 1024 and below the spare warps are the critical path for both.
   const bool overlap = !prod && d >= 1536;
-  const bool pingpong = overlap && !prod && n > R / 2 / BM * BM && R / 2 >= BM;
+  // A call that fits one block is cut in two for this where the half of the preparation that it hides (at 6 TB/s) takes longer
+  // than the waves that it adds and a launch (5 us): 300 rows of d = 1536 in two halves took 94 us, 20 in one.
+  auto halves_pay = [&] {
+    int64_t one = 0, half = 0;
+    pick_tile(R, d, &one);
+    pick_tile(R / 2 / BM * BM, d, &half);
+    return 0.01 * (double)((d + BK - 1) / BK) * (double)(2 * half - one) + 5.0 < 0.5 * (double)n * d * (x_dtype == TQ_F32 ? 8 : 6) / 6e6;
+  };
+  const bool pingpong = overlap && n > R / 2 / BM * BM && R / 2 >= BM && (n > R || halves_pay());
   const int64_t Rbuf = R;   // rows the carved buffers hold in all
   if (pingpong) R = R / 2 / BM * BM;
   // carve the scratch (every part is a multiple of 256 bytes because Rbuf is a multiple of 128)
@@ -835,7 +904,7 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
   if (prod) {
     EL1 = reinterpret_cast<__nv_bfloat16*>(p); p += (size_t)Rbuf * dpad * 2;
     EL2 = reinterpret_cast<__nv_bfloat16*>(p); p += (size_t)Rbuf * dpad * 2;
-    gpart = reinterpret_cast<float*>(p); p += (size_t)Rbuf * tiles_n * 4 * EPS;
+    gpart = reinterpret_cast<float*>(p); p += (size_t)Rbuf * gamma_parts(d) * sizeof(float);
   }
   // limb buffers of block number b
   auto limbs1 = [&](int64_t b) { return XL1 + (pingpong && (b & 1) ? (size_t)R * dpad : 0); };
@@ -847,19 +916,20 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
     float* nu_out = norms ? norms + r0 : nullptr;
     const int blocks = (int)std::min<int64_t>((rows + 7) / 8, (int64_t)sm_count() * 8);
     __nv_bfloat16 *L1 = limbs1(r0 / R), *L2 = limbs2(r0 / R);
-    if (norms) {
-      if (x_dtype == TQ_F32)
-        split_rows_kernel<float, true><<<blocks, 256, 0, s>>>(static_cast<const float*>(Xc), ldx, rows, d, dpad, L1, L2, nu_out);
-      else
-        split_rows_kernel<__nv_bfloat16, true><<<blocks, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(Xc), ldx, rows, d, dpad, L1, L2, nu_out);
-    } else {
-      if (x_dtype == TQ_F32)
-        split_rows_kernel<float, false><<<blocks, 256, 0, s>>>(static_cast<const float*>(Xc), ldx, rows, d, dpad, L1, L2, nullptr);
-      else
-        split_rows_kernel<__nv_bfloat16, false><<<blocks, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(Xc), ldx, rows, d, dpad, L1, L2, nullptr);
-    }
+    // A grid of more than one wave is launched plainly: as a programmatic dependent its first blocks settle wherever the kernel
+    // ahead drains first, and the uneven rest costs more than the launch gap saves (200,000 rows of d = 200: 135 us a call, 123
+    // plain).
+    auto go = [&](auto kern, auto* x) -> cudaError_t {
+      if (blocks <= 2 * sm_count()) return launch_dependent(kern, dim3((unsigned)blocks), dim3(256), 0, s, x, ldx, rows, d, dpad, L1, L2, nu_out);
+      kern<<<blocks, 256, 0, s>>>(x, ldx, rows, d, dpad, L1, L2, nu_out);
+      return cudaGetLastError();
+    };
+    const float* xf = static_cast<const float*>(Xc);
+    const __nv_bfloat16* xb = static_cast<const __nv_bfloat16*>(Xc);
+    const cudaError_t e = x_dtype == TQ_F32 ? (norms ? go(split_rows_kernel<float, true>, xf) : go(split_rows_kernel<float, false>, xf))
+                                            : (norms ? go(split_rows_kernel<__nv_bfloat16, true>, xb) : go(split_rows_kernel<__nv_bfloat16, false>, xb));
     count_launches(1);
-    return cudaGetLastError();
+    return e;
   };
   for (int64_t r0 = 0; r0 < n; r0 += R) {
     const int64_t rows = std::min(R, n - r0);
@@ -888,10 +958,9 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
     g.M = rows;
     g.N = d;
     g.K = d;
-    // CTA pairs on 256-row tiles where the tile is 256 columns wide and the block has more rows than one CTA's tile
-    const int ctas = (bn == 256 && pair_tiles_enabled() && rows > BM) ? 2 : 1;
-    g.tiles_m = (int)((rows + BM * ctas - 1) / (BM * ctas));
-    g.tiles_n = tiles_n;
+    const Tile tile = pick_tile(rows, d);
+    g.tiles_m = (int)((rows + BM * tile.ctas - 1) / (BM * tile.ctas));
+    g.tiles_n = (d + tile.bn - 1) / tile.bn;
     g.cb = plan->cb;
     g.out = idx ? idx + (size_t)r0 * plan->idx_row_bytes : nullptr;
     g.out_rb = plan->idx_row_bytes;
@@ -907,6 +976,8 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
       g.store_e2 = &sE2;
     }
     g.gpart = gpart;
+    g.gamma = gamma ? gamma + r0 : nullptr;
+    g.parts = d <= 128 ? 4 : (d + 63) / 64;   // per epilogue warp: 32 columns of a tile that is the whole row, else 64
     g.Mpad = R;
     g.nu = nu_out;
     g.split.rows = 0;
@@ -919,25 +990,18 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
     // 2. y = Pi u, idx (+ residual limbs and partial norms)
     if (!prod) {
       if (pingpong && r0 + R < n) next_block_task(g);
-      TQ_CHECK_CUDA(launch_gemm<0>(bn, ctas, plan->mse_bits, mA1, mA2, ctas == 2 ? plan->pi_limbs.map_hi_half : plan->pi_limbs.map_hi,
-                                   ctas == 2 ? plan->pi_limbs.map_lo_half : plan->pi_limbs.map_lo, g, st), who);
+      TQ_CHECK_CUDA(launch_gemm<0>(tile, plan->mse_bits, mA1, mA2, plan->pi_limbs, g, st), who);
       continue;
     }
-    TQ_CHECK_CUDA(launch_gemm<1>(bn, ctas, plan->mse_bits, mA1, mA2, ctas == 2 ? plan->pi_limbs.map_hi_half : plan->pi_limbs.map_hi,
-                                 ctas == 2 ? plan->pi_limbs.map_lo_half : plan->pi_limbs.map_lo, g, st), who);
-    // 3. gamma = ||e||
-    gamma_finish_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(gpart, R, EPS * tiles_n, rows, gamma + r0);
-    count_launches(1);
-    TQ_CHECK_CUDA(cudaGetLastError(), who);
-    // 4. qjl = sign(S' e)
+    TQ_CHECK_CUDA(launch_gemm<1>(tile, plan->mse_bits, mA1, mA2, plan->pi_limbs, g, st), who);
+    // 3. qjl = sign(S' e), gamma = ||e||
     CUtensorMap mE1, mE2;
     TQ_REQUIRE(make_map(&mE1, EL1, rows, d, dpad, BM) && make_map(&mE2, EL2, rows, d, dpad, BM), TQ_ERR_CUDA,
                "%s: cuTensorMapEncodeTiled failed", who);
     g.out = qjl + (size_t)r0 * plan->qjl_row_bytes;
     g.out_rb = plan->qjl_row_bytes;
     if (overlap && r0 + R < n) next_block_task(g);   // the limbs of X are free by now
-    TQ_CHECK_CUDA(launch_gemm<2>(bn, ctas, 1, mE1, mE2, ctas == 2 ? plan->sp_limbs.map_hi_half : plan->sp_limbs.map_hi,
-                                 ctas == 2 ? plan->sp_limbs.map_lo_half : plan->sp_limbs.map_lo, g, st), who);
+    TQ_CHECK_CUDA(launch_gemm<2>(tile, 1, mE1, mE2, plan->sp_limbs, g, st), who);
   }
   return TQ_OK;
 }

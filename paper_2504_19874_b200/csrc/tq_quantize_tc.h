@@ -8,10 +8,9 @@
 namespace tq {
 namespace tc {
 
-int pick_bn(int d);            // N extent of one MMA tile for this dimension
 bool supported(int d);         // d large enough for the tensor path and the driver offers tensor maps
 
-cudaError_t build_matrix_limbs(const float* dM, int rows, int d, int dpad, int bn, MatrixLimbs* out);
+cudaError_t build_matrix_limbs(const float* dM, int rows, int d, int dpad, MatrixLimbs* out);
 void free_matrix_limbs(MatrixLimbs* m);
 
 size_t scratch_bytes_per_row(const tq_plan* plan);
