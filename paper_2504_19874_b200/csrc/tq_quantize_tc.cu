@@ -72,12 +72,12 @@ struct GemmArgs {
   int nibble;
   // Operand preparation of the NEXT block of rows (nu = ||x||, u = x / nu, bf16 limbs of u), done by NSPLIT spare
   // warps of every CTA while this launch's GEMM runs: the GEMM is bound by the tensor pipe and shared memory, the
-  // preparation by HBM and a little issue bandwidth, so it hides completely.  Only the project launch (MODE 2)
-  // carries one: its own A operand is the residual, so the limb buffers of X are free to be rewritten.
+  // preparation by HBM and a little issue bandwidth.  The rotate launch of TQ_MSE plans (MODE 0) carries one where it pays,
+  // see quantize().
   struct SplitTask {
-    const void* X;       // first row of the next block
+    const float* X;      // first row of the next block
     int64_t ldx, rows;   // rows == 0: nothing to do
-    int d, dpad, is_f32, normalize;
+    int d, dpad, normalize;
     __nv_bfloat16* L1;
     __nv_bfloat16* L2;
     float* norms;        // nullable
@@ -198,13 +198,17 @@ __device__ __forceinline__ void split_rows_vec(const float* __restrict__ X, int6
   }
 }
 
+__host__ __device__ __forceinline__ bool vec_rows(const float* X, int64_t ldx, int d, int dpad) {
+  return (d & 3) == 0 && (ldx & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0 && dpad == d;
+}
+
 // One warp per row: nu = ||x|| (optional), u = x / nu, u = hi + lo in bf16.  Rows warp, warp + nwarps, ...
 template <typename T, bool NORMALIZE>
 __device__ __forceinline__ void split_rows(const T* __restrict__ X, int64_t ldx, int64_t n, int d, int dpad,
                                            __nv_bfloat16* __restrict__ L1, __nv_bfloat16* __restrict__ L2,
                                            float* __restrict__ norms, int64_t warp, int64_t nwarps, int lane) {
   if constexpr (sizeof(T) == 4) {
-    if ((d & 3) == 0 && (ldx & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0 && dpad == d) {
+    if (vec_rows(X, ldx, d, dpad)) {
       if (d <= 256) split_rows_vec<NORMALIZE, 2>(X, ldx, n, d, dpad, L1, L2, norms, warp, nwarps, lane);
       else if (d <= 512) split_rows_vec<NORMALIZE, 4>(X, ldx, n, d, dpad, L1, L2, norms, warp, nwarps, lane);
       else if (d <= 1024) split_rows_vec<NORMALIZE, 8>(X, ldx, n, d, dpad, L1, L2, norms, warp, nwarps, lane);
@@ -440,15 +444,8 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
     const GemmArgs::SplitTask& t = a.split;
     if (t.rows > 0) {
       const int64_t sw = (int64_t)blockIdx.x * NSPLIT + (warp - 2 - 4 * EPS), nsw = (int64_t)gridDim.x * NSPLIT;
-      if (t.is_f32) {
-        const float* X = static_cast<const float*>(t.X);
-        if (t.normalize) split_rows<float, true>(X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
-        else split_rows<float, false>(X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
-      } else {
-        const __nv_bfloat16* X = static_cast<const __nv_bfloat16*>(t.X);
-        if (t.normalize) split_rows<__nv_bfloat16, true>(X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
-        else split_rows<__nv_bfloat16, false>(X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
-      }
+      if (t.normalize) split_rows<float, true>(t.X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
+      else split_rows<float, false>(t.X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
     }
   } else {
     // ------------------------------------------------------------ epilogue (4 x EPS warps: 4 TMEM lane groups x EPS column parts)
@@ -883,14 +880,16 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
   // Measured per 10^6 rows with the CTA-pair GEMMs: TQ_MSE d = 1536 10.1 ms with them against 10.6 without; TQ_PROD
   // loses (d = 1536: 22.1 against 21.5 ms, d = 3072 alike), so its project launch carries no such task any more; at
   // d = 1024 and below the spare warps are the critical path for both.
-  const bool overlap = !prod && d >= 1536;
+  // Rows of bf16 or off the 16-byte grid are the critical path at every d (11,734 bf16 rows of d = 1536: 167 us and more with
+  // the spare warps, 136 with a launch of their own).
+  const bool overlap = !prod && d >= 1536 && x_dtype == TQ_F32 && vec_rows(static_cast<const float*>(X), ldx, d, dpad);
   // A call that fits one block is cut in two for this where the half of the preparation that it hides (at 6 TB/s) takes longer
   // than the waves that it adds and a launch (5 us): 300 rows of d = 1536 in two halves took 94 us, 20 in one.
   auto halves_pay = [&] {
     int64_t one = 0, half = 0;
     pick_tile(R, d, &one);
     pick_tile(R / 2 / BM * BM, d, &half);
-    return 0.01 * (double)((d + BK - 1) / BK) * (double)(2 * half - one) + 5.0 < 0.5 * (double)n * d * (x_dtype == TQ_F32 ? 8 : 6) / 6e6;
+    return 0.01 * (double)((d + BK - 1) / BK) * (double)(2 * half - one) + 5.0 < 0.5 * (double)n * d * 8 / 6e6;
   };
   const bool pingpong = overlap && n > R / 2 / BM * BM && R / 2 >= BM && (n > R || halves_pay());
   const int64_t Rbuf = R;   // rows the carved buffers hold in all
@@ -939,12 +938,11 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
     if (r0 == 0 || !overlap || (!prod && !pingpong)) TQ_CHECK_CUDA(launch_split(r0, st), who);
     __nv_bfloat16 *XLc1 = limbs1(r0 / R), *XLc2 = limbs2(r0 / R);
     auto next_block_task = [&](GemmArgs& ga) {
-      ga.split.X = static_cast<const char*>(X) + (size_t)(r0 + R) * ldx * xsz;
+      ga.split.X = static_cast<const float*>(X) + (r0 + R) * ldx;
       ga.split.ldx = ldx;
       ga.split.rows = std::min(R, n - (r0 + R));
       ga.split.d = d;
       ga.split.dpad = dpad;
-      ga.split.is_f32 = x_dtype == TQ_F32 ? 1 : 0;
       ga.split.normalize = norms ? 1 : 0;
       ga.split.L1 = limbs1(r0 / R + 1);
       ga.split.L2 = limbs2(r0 / R + 1);
