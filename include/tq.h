@@ -392,7 +392,9 @@ size_t tq_entropy_workspace_bytes(int64_t n);
 /* Byte offset of every row's stream: row_offsets[i] for i < n, and row_offsets[n] = total bytes of the packed
  * array (read it back to size the output of tq_entropy_pack).
  *   lengths  host, 2^b_m code lengths (from tq_entropy_lengths or the caller's own; must satisfy Kraft's inequality)
- *   idx      device, n canonical rows;  row_offsets device out, n + 1 values;  workspace device, 256-byte aligned */
+ *   idx      device, n canonical rows, at any address here and in tq_entropy_pack (rows off the 4-byte grid are read byte by byte)
+ *   row_offsets device out, n + 1 values, 8-byte aligned;  workspace device, 4-byte aligned
+ * Errors: TQ_ERR_ALIGNMENT for any other workspace or row_offsets, and the usual argument checks. */
 int tq_entropy_measure(const tq_plan* plan, const uint8_t* lengths, int64_t n, const uint8_t* idx,
                        uint64_t* row_offsets, void* workspace, size_t workspace_bytes, void* stream);
 /* Writes the rows' streams at their offsets.  out: device, 4-byte aligned, out_bytes >= row_offsets[n]; if it is

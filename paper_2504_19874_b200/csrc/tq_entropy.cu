@@ -63,14 +63,22 @@ __device__ __forceinline__ uint32_t spread1(uint32_t x) {
   return (x & 0x01010101u) | ((x & 0x02020202u) << 3);
 }
 
-// Coordinates 8 g .. 8 g + 7 of a packed row as eight nibbles (row: 4-byte aligned, row_words words; whole groups of the row
-// lie inside it because its stride covers ceil(d BITS / 8) bytes rounded up to words).
-template <int BITS>
-__device__ __forceinline__ uint32_t nibbles(const uint32_t* __restrict__ row, int row_words, int g) {
-  if (BITS == 4) return __ldg(row + g);
+// Word w of a packed row.  BYTES: the rows are not 4-byte aligned (a slice of a larger buffer) and are read byte by byte.
+template <bool BYTES>
+__device__ __forceinline__ uint32_t row_word(const uint8_t* __restrict__ row, int w) {
+  if (!BYTES) return __ldg(reinterpret_cast<const uint32_t*>(row) + w);
+  const uint8_t* b = row + 4 * w;
+  return (uint32_t)__ldg(b) | ((uint32_t)__ldg(b + 1) << 8) | ((uint32_t)__ldg(b + 2) << 16) | ((uint32_t)__ldg(b + 3) << 24);
+}
+
+// Coordinates 8 g .. 8 g + 7 of a packed row of row_words words as eight nibbles (whole groups of the row lie inside it because
+// its stride covers ceil(d BITS / 8) bytes rounded up to words).
+template <int BITS, bool BYTES>
+__device__ __forceinline__ uint32_t nibbles(const uint8_t* __restrict__ row, int row_words, int g) {
+  if (BITS == 4) return row_word<BYTES>(row, g);
   const int bit = 8 * BITS * g, w = bit >> 5, sh = bit & 31;
-  const uint32_t x = __ldg(row + w);
-  if (BITS == 3) return spread3(__funnelshift_r(x, sh > 8 && w + 1 < row_words ? __ldg(row + w + 1) : 0u, sh) & 0x00ffffffu);
+  const uint32_t x = row_word<BYTES>(row, w);
+  if (BITS == 3) return spread3(__funnelshift_r(x, sh > 8 && w + 1 < row_words ? row_word<BYTES>(row, w + 1) : 0u, sh) & 0x00ffffffu);
   return BITS == 2 ? spread2((x >> sh) & 0xffffu) : spread1((x >> sh) & 0xffu);
 }
 
@@ -91,7 +99,7 @@ __device__ __forceinline__ uint32_t code_bits(const Code& c, uint32_t x, uint32_
 }
 
 // Row sizes in bytes (multiples of 4) and the total of each CTA's 8 R rows.
-template <int BITS>
+template <int BITS, bool BYTES>
 __global__ void __launch_bounds__(256) measure_kernel(Args a, int R, uint32_t* __restrict__ sizes, uint64_t* __restrict__ totals) {
   __shared__ uint32_t warp_tot[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -101,14 +109,14 @@ __global__ void __launch_bounds__(256) measure_kernel(Args a, int R, uint32_t* _
   for (int r = 0; r < R; ++r) {
     const int64_t row = ((int64_t)blockIdx.x * R + r) * 8 + warp;
     if (row >= a.n) break;
-    const uint32_t* p = reinterpret_cast<const uint32_t*>(a.idx + (size_t)row * a.idx_rb);
+    const uint8_t* p = a.idx + (size_t)row * a.idx_rb;
     uint32_t bits = 0;
     for (int g0 = 0; g0 < groups; g0 += 256) {   // eight loads per lane in flight
       uint32_t x[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int g = g0 + 32 * i + lane;
-        x[i] = g < groups ? nibbles<BITS>(p, row_words, g) : 0u;
+        x[i] = g < groups ? nibbles<BITS, BYTES>(p, row_words, g) : 0u;
       }
 #pragma unroll
       for (int i = 0; i < 8; ++i)
@@ -205,7 +213,7 @@ __global__ void __launch_bounds__(1024) offsets_kernel(const uint32_t* __restric
 // that appended to a 64-bit buffer and flushed it word by word took 1,560 instructions per row of 1536 coordinates, because
 // some lane flushed at every step.
 constexpr int kPackWarps = 8;
-template <int BITS, bool LONG>   // LONG: eight code words may take more than 64 bits (a code word of more than 8)
+template <int BITS, bool LONG, bool BYTES>   // LONG: eight code words may take more than 64 bits (a code word of more than 8)
 __global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(Args a, const uint64_t* __restrict__ offsets, uint8_t* __restrict__ out,
                                                                size_t out_bytes, int image_words, int* status) {
   extern __shared__ uint32_t pack_smem[];
@@ -229,15 +237,15 @@ __global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(Args a, const uin
       continue;
     }
     const int words = min((int)((off_end - off) / 4), image_words);
-    const uint32_t* p = reinterpret_cast<const uint32_t*>(a.idx + (size_t)row * a.idx_rb);
+    const uint8_t* p = a.idx + (size_t)row * a.idx_rb;
     for (int w = lane; w < words; w += 32) image[w] = 0u;
     __syncwarp();
     int base = 0;   // stream bits before this sweep's groups
-    uint32_t next = lane < groups ? nibbles<BITS>(p, row_words, lane) : 0u;
+    uint32_t next = lane < groups ? nibbles<BITS, BYTES>(p, row_words, lane) : 0u;
     for (int g0 = 0; g0 < groups; g0 += 32) {
       const int g = g0 + lane;
       const uint32_t x = next;
-      if (g + 32 < groups) next = nibbles<BITS>(p, row_words, g + 32);   // requested one sweep ahead
+      if (g + 32 < groups) next = nibbles<BITS, BYTES>(p, row_words, g + 32);   // requested one sweep ahead
       unsigned long long half[2];   // four code words each, at most 48 bits
       int len[2];
 #pragma unroll
@@ -379,6 +387,22 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_kernel(Args a, int K, c
   for (; ow < row_words; ++ow) dst[ow] = checked_word(ow);
 }
 
+bool by_bytes(const void* idx) { return (reinterpret_cast<uintptr_t>(idx) & 3) != 0; }
+
+using MeasureFn = void (*)(Args, int, uint32_t*, uint64_t*);
+MeasureFn measure_for(int bits, bool bytes) {
+  static constexpr MeasureFn fns[4][2] = {{measure_kernel<1, false>, measure_kernel<1, true>}, {measure_kernel<2, false>, measure_kernel<2, true>},
+                                          {measure_kernel<3, false>, measure_kernel<3, true>}, {measure_kernel<4, false>, measure_kernel<4, true>}};
+  return fns[bits - 1][bytes];
+}
+
+using PackFn = void (*)(Args, const uint64_t*, uint8_t*, size_t, int, int*);
+template <bool LONG, bool BYTES>
+PackFn pack_for(int bits) {
+  static constexpr PackFn fns[4] = {pack_kernel<1, LONG, BYTES>, pack_kernel<2, LONG, BYTES>, pack_kernel<3, LONG, BYTES>, pack_kernel<4, LONG, BYTES>};
+  return fns[bits - 1];
+}
+
 int make_code(const tq_plan* plan, const uint8_t* lengths, Code* c, const char* who) {
   const int L = 1 << plan->mse_bits;
   std::memset(c, 0, sizeof(*c));
@@ -454,10 +478,11 @@ extern "C" int tq_entropy_lengths(int d, int bits, const float* centroids, uint8
   return TQ_OK;
 }
 
-// Row sizes (4 bytes each), then the totals of groups of at least eight rows (8 bytes each).
+// Row sizes (4 bytes each), then the totals of groups of at least eight rows (8 bytes each, with room to start them on an 8-byte
+// boundary of a workspace that has only a 4-byte one).
 static size_t sizes_bytes(int64_t n) { return (size_t)((n * 4 + 255) / 256 * 256); }
 extern "C" size_t tq_entropy_workspace_bytes(int64_t n) {
-  return n > 0 ? sizes_bytes(n) + (size_t)(((n + 7) / 8 * 8 + 255) / 256 * 256) : 0;
+  return n > 0 ? sizes_bytes(n) + (size_t)(((n + 7) / 8 * 8 + 4 + 255) / 256 * 256) : 0;
 }
 
 extern "C" int tq_entropy_measure(const tq_plan* plan, const uint8_t* lengths, int64_t n, const uint8_t* idx, uint64_t* row_offsets,
@@ -469,12 +494,14 @@ extern "C" int tq_entropy_measure(const tq_plan* plan, const uint8_t* lengths, i
   TQ_REQUIRE(row_offsets != nullptr && (n == 0 || idx != nullptr), TQ_ERR_INVALID_ARG, "%s: NULL argument", who);
   TQ_REQUIRE(workspace_bytes >= tq_entropy_workspace_bytes(n) && (n == 0 || workspace != nullptr), TQ_ERR_WORKSPACE,
              "%s: workspace of %zu bytes, %zu needed", who, workspace_bytes, tq_entropy_workspace_bytes(n));
+  TQ_REQUIRE((n == 0 || (reinterpret_cast<uintptr_t>(workspace) & 3) == 0) && (reinterpret_cast<uintptr_t>(row_offsets) & 7) == 0, TQ_ERR_ALIGNMENT,
+             "%s: workspace / row_offsets is misaligned", who);
   entropy::Args a;
   if ((rc = entropy::make_code(plan, lengths, &a.code, who))) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   a.n = n; a.d = plan->d; a.idx = idx; a.idx_rb = plan->idx_row_bytes;
   uint32_t* sizes = static_cast<uint32_t*>(workspace);
-  uint64_t* totals = reinterpret_cast<uint64_t*>(static_cast<char*>(workspace) + sizes_bytes(n));
+  uint64_t* totals = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(workspace) + sizes_bytes(n) + 7) & ~(uintptr_t)7);
   // eight rows per warp once that still fills the chip four times over
   const int R = n >= 8 * 8 * 4 * 148 ? 8 : 1;
   const int64_t groups = (n + 8 * R - 1) / (8 * R);
@@ -482,12 +509,7 @@ extern "C" int tq_entropy_measure(const tq_plan* plan, const uint8_t* lengths, i
   // average (0.27 GB from L2); from there on one launch turns the totals into prefix sums first
   const int prefixed = n > ((int64_t)1 << 21) ? 1 : 0;
   if (n > 0) {
-    switch (a.code.bits) {
-      case 1: entropy::measure_kernel<1><<<(unsigned)groups, 256, 0, st>>>(a, R, sizes, totals); break;
-      case 2: entropy::measure_kernel<2><<<(unsigned)groups, 256, 0, st>>>(a, R, sizes, totals); break;
-      case 3: entropy::measure_kernel<3><<<(unsigned)groups, 256, 0, st>>>(a, R, sizes, totals); break;
-      default: entropy::measure_kernel<4><<<(unsigned)groups, 256, 0, st>>>(a, R, sizes, totals); break;
-    }
+    entropy::measure_for(a.code.bits, entropy::by_bytes(idx))<<<(unsigned)groups, 256, 0, st>>>(a, R, sizes, totals);
     TQ_CHECK_CUDA(cudaGetLastError(), who);
     if (prefixed) {
       entropy::prefix_totals_kernel<<<1, 1024, 0, st>>>(totals, groups);
@@ -517,11 +539,9 @@ extern "C" int tq_entropy_pack(const tq_plan* plan, const uint8_t* lengths, int6
   const size_t smem = (256 * 32 + (size_t)entropy::kPackWarps * (image_words + 4)) * sizeof(uint32_t);
   const int per_sm = std::max(1, std::min(8, (int)(228 * 1024 / (smem + 1024))));
   const int64_t ctas = std::min<int64_t>((n + entropy::kPackWarps - 1) / entropy::kPackWarps, (int64_t)tc::sm_count() * per_sm);
-  const bool wide = a.code.maxlen > 8;
-  const auto kernel = a.code.bits == 1   ? (wide ? entropy::pack_kernel<1, true> : entropy::pack_kernel<1, false>)
-                      : a.code.bits == 2 ? (wide ? entropy::pack_kernel<2, true> : entropy::pack_kernel<2, false>)
-                      : a.code.bits == 3 ? (wide ? entropy::pack_kernel<3, true> : entropy::pack_kernel<3, false>)
-                                         : (wide ? entropy::pack_kernel<4, true> : entropy::pack_kernel<4, false>);
+  const bool wide = a.code.maxlen > 8, bytes = entropy::by_bytes(idx);
+  const auto kernel = wide ? (bytes ? entropy::pack_for<true, true>(a.code.bits) : entropy::pack_for<true, false>(a.code.bits))
+                           : (bytes ? entropy::pack_for<false, true>(a.code.bits) : entropy::pack_for<false, false>(a.code.bits));
   if (smem > 48 * 1024) TQ_CHECK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), who);
   kernel<<<(unsigned)ctas, 32 * entropy::kPackWarps, smem, st>>>(a, row_offsets, out, out_bytes, image_words, plan->d_status);
   count_launches(1);

@@ -65,3 +65,26 @@ def test_offsets_of_many_rows(n):
     back = torch.full_like(idx, 0xEE)
     tq.tq_entropy_unpack(su.plan, lengths, n, packed, offsets, back)
     assert torch.equal(back, idx)
+
+
+@pytest.mark.parametrize("bits,lengths", [(1, [1, 1]), (2, [1, 2, 3, 3]), (3, [3] * 8), (4, DEEP)])
+def test_rows_at_any_address(bits, lengths):
+    """Index rows inside a larger buffer, off the 4-byte grid, and a workspace on no more than that grid: the same stream."""
+    d, n = 203, 77
+    su = P.Setup(d, bits, tq.TQ_MSE)
+    lengths = np.array(lengths, dtype=np.uint8)
+    _, idx = random_rows(su.plan, d, bits, n, bits)
+    want, want_offsets = tq.tq_entropy_pack(su.plan, lengths, n, idx)
+    for shift in (1, 2, 3, 4):
+        buf = torch.full((idx.numel() + 8,), 0xA5, dtype=torch.uint8, device=DEV)
+        moved = buf[shift:shift + idx.numel()].view(n, -1)
+        moved.copy_(idx)
+        packed, offsets = tq.tq_entropy_pack(su.plan, lengths, n, moved)
+        tq.tq_plan_status(su.plan)
+        assert torch.equal(packed, want) and torch.equal(offsets, want_offsets)
+    need = tq.lib().tq_entropy_workspace_bytes(n)
+    ws, offsets = torch.empty(need + 8, dtype=torch.uint8, device=DEV), torch.zeros(n + 1, dtype=torch.int64, device=DEV)
+    measure = lambda shift, at: tq.lib().tq_entropy_measure(su.plan.handle, lengths.ctypes.data, n, idx.data_ptr(), offsets.data_ptr() + at,  # noqa: E731
+                                                            ws.data_ptr() + shift, need, torch.cuda.current_stream().cuda_stream)
+    assert measure(4, 0) == 0 and torch.equal(offsets, want_offsets)
+    assert measure(2, 0) == 3 and measure(0, 4) == 3          # TQ_ERR_ALIGNMENT, nothing launched
