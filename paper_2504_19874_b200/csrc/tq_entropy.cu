@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(256) measure_kernel(Args a, int R, uint32_t* _
   __shared__ uint32_t warp_tot[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int groups = (a.d + 7) / 8, row_words = (int)(a.idx_rb / 4);
-  const int absent = 8 * groups - a.d;   // coordinates of the last group past the row's end: index 0 (pad bits are 0)
+  const int absent = 8 * groups - a.d;   // coordinates of the last group past the row's end: whatever they hold counts as index 0
   uint32_t tot = 0;
   for (int r = 0; r < R; ++r) {
     const int64_t row = ((int64_t)blockIdx.x * R + r) * 8 + warp;
@@ -117,6 +117,7 @@ __global__ void __launch_bounds__(256) measure_kernel(Args a, int R, uint32_t* _
       for (int i = 0; i < 8; ++i) {
         const int g = g0 + 32 * i + lane;
         x[i] = g < groups ? nibbles<BITS, BYTES>(p, row_words, g) : 0u;
+        if (g == groups - 1) x[i] &= 0xffffffffu >> (4 * absent);
       }
 #pragma unroll
       for (int i = 0; i < 8; ++i)

@@ -88,3 +88,19 @@ def test_rows_at_any_address(bits, lengths):
                                                             ws.data_ptr() + shift, need, torch.cuda.current_stream().cuda_stream)
     assert measure(4, 0) == 0 and torch.equal(offsets, want_offsets)
     assert measure(2, 0) == 3 and measure(0, 4) == 3          # TQ_ERR_ALIGNMENT, nothing launched
+
+
+@pytest.mark.parametrize("d,bits,lengths", [(131, 4, LONG), (203, 3, [1, 2, 3, 4, 5, 6, 7, 7]), (9, 1, [1, 2]), (1537, 2, [3, 1, 2, 3])])
+def test_bits_past_the_last_coordinate_do_not_count(d, bits, lengths):
+    su = P.Setup(d, bits, tq.TQ_MSE)
+    lengths = np.array(lengths, dtype=np.uint8)
+    for n in (5, 200):
+        _, idx = random_rows(su.plan, d, bits, n, n)
+        want, want_offsets = tq.tq_entropy_pack(su.plan, lengths, n, idx)
+        used = torch.zeros(idx.shape[1] * 8, dtype=torch.bool)
+        used[:d * bits] = True
+        pad = torch.from_numpy(np.packbits(~used.numpy(), bitorder="little")).to(DEV)
+        for fill in (0xFF, 0x55):
+            packed, offsets = tq.tq_entropy_pack(su.plan, lengths, n, idx | (pad & fill))
+            tq.tq_plan_status(su.plan)
+            assert torch.equal(offsets, want_offsets) and torch.equal(packed, want)
