@@ -397,8 +397,8 @@ size_t tq_entropy_workspace_bytes(int64_t n);
  * Errors: TQ_ERR_ALIGNMENT for any other workspace or row_offsets, and the usual argument checks. */
 int tq_entropy_measure(const tq_plan* plan, const uint8_t* lengths, int64_t n, const uint8_t* idx,
                        uint64_t* row_offsets, void* workspace, size_t workspace_bytes, void* stream);
-/* Writes the rows' streams at their offsets.  out: device, 4-byte aligned, out_bytes >= row_offsets[n]; if it is
- * smaller the rows that do not fit are skipped and the next tq_plan_status(plan) reports an error. */
+/* Writes the rows' streams at their offsets and zeros to every other byte of out.  out: device, 4-byte aligned, out_bytes >=
+ * row_offsets[n]; if it is smaller the rows that do not fit are skipped and the next tq_plan_status(plan) reports an error. */
 int tq_entropy_pack(const tq_plan* plan, const uint8_t* lengths, int64_t n, const uint8_t* idx,
                     const uint64_t* row_offsets, uint8_t* out, size_t out_bytes, void* stream);
 /* The inverse: n canonical idx rows (pad bits zero) from the packed streams. */

@@ -233,11 +233,13 @@ __global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(Args a, const uin
   const int groups = (a.d + 7) / 8, row_words = (int)(a.idx_rb / 4);
   for (int64_t row = (int64_t)blockIdx.x * kPackWarps + warp; row < a.n; row += (int64_t)gridDim.x * kPackWarps) {
     const uint64_t off = offsets[row], off_end = offsets[row + 1];
-    if (off_end > out_bytes) {   // the caller's buffer is smaller than the measured total
+    if (off > off_end || off_end > out_bytes) {   // the caller's buffer is smaller than the measured total
       if (lane == 0) atomicExch(status, TQ_ERR_WORKSPACE);
+      for (uint64_t b = off + lane; b < out_bytes && b < off_end; b += 32) out[b] = 0;
       continue;
     }
-    const int words = min((int)((off_end - off) / 4), image_words);
+    const uint64_t slot = (off_end - off) / 4;   // as many words as the stream has, unless the caller spaced the rows out
+    const int words = (int)min(slot, (uint64_t)image_words);
     const uint8_t* p = a.idx + (size_t)row * a.idx_rb;
     for (int w = lane; w < words; w += 32) image[w] = 0u;
     __syncwarp();
@@ -295,8 +297,19 @@ __global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(Args a, const uin
     __syncwarp();
     uint32_t* dst = reinterpret_cast<uint32_t*>(out + off);
     for (int w = lane; w < words; w += 32) dst[w] = image[w];
+    for (uint64_t w = words + lane; w < slot; w += 32) dst[w] = 0u;
     __syncwarp();
   }
+  // What lies before the first stream and after the last one is zero too.
+  auto clear = [&](uint64_t begin, uint64_t end) {   // begin on a word boundary
+    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t b = begin + 4 * t; b + 4 <= end; b += 4 * step) *reinterpret_cast<uint32_t*>(out + b) = 0u;
+    const uint64_t rest = begin + (end - begin) / 4 * 4 + t;
+    if (rest < end) out[rest] = 0;
+  };
+  const uint64_t first = offsets[0], last = offsets[a.n];
+  if (first > 0) clear(0, min(first, (uint64_t)out_bytes));
+  if (last < out_bytes) clear(last, out_bytes);
 }
 
 // One thread per row.  Look-up on the next K = 10 bits (12 where a code word is longer than 10; always 12 measured 322 us: the

@@ -104,3 +104,36 @@ def test_bits_past_the_last_coordinate_do_not_count(d, bits, lengths):
             packed, offsets = tq.tq_entropy_pack(su.plan, lengths, n, idx | (pad & fill))
             tq.tq_plan_status(su.plan)
             assert torch.equal(offsets, want_offsets) and torch.equal(packed, want)
+
+
+def test_bytes_of_the_output_that_hold_no_stream_are_zero():
+    """A longer buffer, rows that the caller spaced out, and a buffer that is too small: nothing old shines through."""
+    d, bits, n = 203, 3, 67
+    su = P.Setup(d, bits, tq.TQ_MSE)
+    lengths = np.array([1, 2, 3, 4, 5, 6, 7, 7], dtype=np.uint8)
+    _, idx = random_rows(su.plan, d, bits, n, 4)
+    packed, offsets = tq.tq_entropy_pack(su.plan, lengths, n, idx)
+    streams, off = packed.cpu().numpy(), offsets.cpu().numpy()
+
+    def pack(at, size):
+        out = torch.full((size,), 0xFF, dtype=torch.uint8, device=DEV)
+        at = torch.from_numpy(at).to(DEV)
+        assert tq.lib().tq_entropy_pack(su.plan.handle, lengths.ctypes.data, n, idx.data_ptr(), at.data_ptr(), out.data_ptr(), size,
+                                        torch.cuda.current_stream().cuda_stream) == 0
+        return out.cpu().numpy()
+
+    for spare in (0, 1, 6, 4099):
+        got = pack(off, streams.size + spare)
+        assert np.array_equal(got[:streams.size], streams) and not got[streams.size:].any()
+    spaced = np.arange(n + 1, dtype=np.int64) * 200 + 16               # 200 > the longest stream of this code
+    want = np.zeros(int(spaced[n]) + 5, dtype=np.uint8)
+    for r in range(n):
+        want[spaced[r]:spaced[r] + off[r + 1] - off[r]] = streams[off[r]:off[r + 1]]
+    assert np.array_equal(pack(spaced, want.size), want)
+    tq.tq_plan_status(su.plan)
+    size = int(off[n // 2]) + 7                                         # row n / 2 does not fit
+    want = np.zeros(size, dtype=np.uint8)
+    want[:off[n // 2]] = streams[:off[n // 2]]
+    assert np.array_equal(pack(off, size), want)
+    with pytest.raises(tq.TqError):
+        tq.tq_plan_status(su.plan)
