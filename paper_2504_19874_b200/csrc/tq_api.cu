@@ -438,9 +438,11 @@ cudaError_t launch_scan_few(const scan::ScanArgs& base, int nq, cudaStream_t st)
     cudaError_t e = cudaSuccess;
     const size_t smem = per_query * tile;
 #define TQ_SCAN_LAUNCH(NQ)                                                                                  \
-  e = cudaFuncSetAttribute(scan::scan_few_kernel<BITS, NQ, PROD>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                           (int)smem);                                                                      \
-  if (e == cudaSuccess) scan::scan_few_kernel<BITS, NQ, PROD><<<(unsigned)blocks, 256, smem, st>>>(a);
+  {                                                                                                         \
+    static std::atomic<unsigned long long> smem_devices{0};                                                 \
+    e = allow_largest_smem(reinterpret_cast<const void*>(scan::scan_few_kernel<BITS, NQ, PROD>), smem_devices); \
+    if (e == cudaSuccess) scan::scan_few_kernel<BITS, NQ, PROD><<<(unsigned)blocks, 256, smem, st>>>(a);    \
+  }
     switch (tile) {
       case 8: TQ_SCAN_LAUNCH(8) break;
       case 4: TQ_SCAN_LAUNCH(4) break;

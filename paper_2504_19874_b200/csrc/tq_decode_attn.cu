@@ -871,11 +871,8 @@ extern "C" int tq_attend_decode(const tq_kv_group* groups, int ngroups, int head
   TQ_REQUIRE(dev == groups[0].plan_k->device, TQ_ERR_INVALID_ARG, "%s: the plans belong to device %d, current device is %d", who,
              groups[0].plan_k->device, dev);
   const size_t merge_smem = (size_t)d * d * sizeof(float);
-  static std::atomic<size_t> merge_smem_set[16];
-  if (dev >= 16 || merge_smem > merge_smem_set[dev].load(std::memory_order_relaxed)) {
-    TQ_CHECK_CUDA(cudaFuncSetAttribute(merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)merge_smem), who);
-    if (dev < 16) merge_smem_set[dev].store(merge_smem, std::memory_order_relaxed);
-  }
+  static std::atomic<unsigned long long> merge_devices{0};
+  TQ_CHECK_CUDA(allow_largest_smem(reinterpret_cast<const void*>(merge_kernel), merge_devices), who);
   // ---- the tensor path: antisymmetric codebooks (every Lloyd-Max codebook of the library is) and a slice that fits
   //      in shared memory; otherwise the table-lookup kernel
   MmaArgs ma;
@@ -900,12 +897,13 @@ extern "C" int tq_attend_decode(const tq_kv_group* groups, int ngroups, int head
     else
       TQ_CHECK_CUDA(launch_dependent(prepare_mma_kernel<__nv_bfloat16>, dim3((unsigned)(heads * ngroups)), dim3(256), prep_smem, st, a, ma,
                                  static_cast<const __nv_bfloat16*>(Q), ldq), who);
-    static std::atomic<size_t> mma_smem_set[16];
-    if (dev >= 16 || mma_smem > mma_smem_set[dev].load(std::memory_order_relaxed)) {
-      TQ_CHECK_CUDA(cudaFuncSetAttribute(partial_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mma_smem), who);
+    static std::atomic<unsigned long long> partial_devices{0};
+    static std::atomic<bool> carveout_set[16];
+    TQ_CHECK_CUDA(allow_largest_smem(reinterpret_cast<const void*>(partial_mma_kernel), partial_devices), who);
+    if (dev >= 16 || !carveout_set[dev].load(std::memory_order_relaxed)) {
       // several CTAs per SM hide the latencies of the kernel's short phases: ask for the largest shared-memory carve-out
       TQ_CHECK_CUDA(cudaFuncSetAttribute(partial_mma_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared), who);
-      if (dev < 16) mma_smem_set[dev].store(mma_smem, std::memory_order_relaxed);
+      if (dev < 16) carveout_set[dev].store(true, std::memory_order_relaxed);
     }
     TQ_CHECK_CUDA(launch_dependent(partial_mma_kernel, dim3((unsigned)(heads * nslices)), dim3(NT), mma_smem, st, a, ma), who);
     TQ_CHECK_CUDA(launch_dependent(merge_kernel, dim3((unsigned)(heads * ngroups)), dim3(MERGE_NT), merge_smem, st, a, out, ldo), who);
@@ -920,11 +918,8 @@ extern "C" int tq_attend_decode(const tq_kv_group* groups, int ngroups, int head
   const size_t smem = (size_t)a.region0 * sizeof(float4) + (size_t)ngroups * SLICE * sizeof(float4) + kbytes + vbytes +
                       MAXG * 16 * sizeof(float) + (NT / 32 + 1) * MAXQ * sizeof(float);
   TQ_REQUIRE(smem <= 220 * 1024, TQ_ERR_UNSUPPORTED, "%s: %zu bytes of shared memory needed (too many wide groups)", who, smem);
-  static std::atomic<size_t> smem_set[16];   // zero-initialised; written by any thread that launches
-  if (dev >= 16 || smem > smem_set[dev].load(std::memory_order_relaxed)) {
-    TQ_CHECK_CUDA(cudaFuncSetAttribute(partial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), who);
-    if (dev < 16) smem_set[dev].store(smem, std::memory_order_relaxed);
-  }
+  static std::atomic<unsigned long long> table_devices{0};
+  TQ_CHECK_CUDA(allow_largest_smem(reinterpret_cast<const void*>(partial_kernel), table_devices), who);
   partial_kernel<<<(unsigned)(heads * nslices), NT, smem, st>>>(a);
   TQ_CHECK_CUDA(cudaGetLastError(), who);
   merge_kernel<<<heads * ngroups, MERGE_NT, merge_smem, st>>>(a, out, ldo);

@@ -556,7 +556,9 @@ extern "C" int tq_entropy_pack(const tq_plan* plan, const uint8_t* lengths, int6
   const bool wide = a.code.maxlen > 8, bytes = entropy::by_bytes(idx);
   const auto kernel = wide ? (bytes ? entropy::pack_for<true, true>(a.code.bits) : entropy::pack_for<true, false>(a.code.bits))
                            : (bytes ? entropy::pack_for<false, true>(a.code.bits) : entropy::pack_for<false, false>(a.code.bits));
-  if (smem > 48 * 1024) TQ_CHECK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), who);
+  static std::atomic<unsigned long long> smem_devices[16];   // per instantiation
+  if (smem > 48 * 1024)
+    TQ_CHECK_CUDA(allow_largest_smem(reinterpret_cast<const void*>(kernel), smem_devices[a.code.bits - 1 + 4 * wide + 8 * bytes]), who);
   kernel<<<(unsigned)ctas, 32 * entropy::kPackWarps, smem, st>>>(a, row_offsets, out, out_bytes, image_words, plan->d_status);
   count_launches(1);
   TQ_CHECK_CUDA(cudaGetLastError(), who);

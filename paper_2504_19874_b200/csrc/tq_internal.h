@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <atomic>
 #include <cstdarg>
 #include <cstdint>
 #include <cstdio>
@@ -84,6 +85,22 @@ cudaError_t launch_dependent(void (*kern)(KArgs...), dim3 grid, dim3 block, size
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 #endif
+
+// Lets a kernel be launched with as much dynamic shared memory as a block of the current device may have.  Once per device
+// (`devices`: one word of bits per kernel), and always to the same value: the attribute is the kernel's, and a thread that set it
+// to the size of its own call would make another thread's larger launch fail.
+inline cudaError_t allow_largest_smem(const void* kern, std::atomic<unsigned long long>& devices) {
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 64 && ((devices.load(std::memory_order_relaxed) >> dev) & 1ull)) return cudaSuccess;
+  cudaFuncAttributes own;
+  if ((e = cudaFuncGetAttributes(&own, kern)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)own.sharedSizeBytes);
+  if (e == cudaSuccess && dev < 64) devices.fetch_or(1ull << dev, std::memory_order_relaxed);
+  return e;
+}
 
 constexpr int kBoxes = 4;
 struct MatrixLimbs {

@@ -983,15 +983,9 @@ bool pick_config(const tq_plan* plan, int NW, int MT, int NT, Config* out) {
 template <int BM, bool PROD, int NW, int MT, int NT, int MODE>
 cudaError_t launch_t(const CUtensorMap& mi, const CUtensorMap& mq, const ScanArgs& args, size_t smem, cudaStream_t st) {
   auto kern = scan_mma_kernel<BM, PROD, NW, MT, NT, MODE>;
-  // function attributes are per device: the largest size set so far, per device
-  static std::atomic<size_t> attr[64];   // zero-initialised; written by any thread that launches
-  int attr_dev = 0;
-  if (cudaGetDevice(&attr_dev) != cudaSuccess) return cudaErrorInvalidDevice;
-  if (attr_dev >= 64 || smem > attr[attr_dev].load(std::memory_order_relaxed)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (attr_dev < 64) attr[attr_dev].store(smem, std::memory_order_relaxed);
-  }
+  static std::atomic<unsigned long long> smem_devices{0};
+  const cudaError_t e = allow_largest_smem(reinterpret_cast<const void*>(kern), smem_devices);
+  if (e != cudaSuccess) return e;
   const int grid = (int)std::min<int64_t>(args.ntiles, tc::sm_count());
   count_launches(1);
   return launch_dependent(kern, dim3((unsigned)grid), dim3(32 * (NW + 1)), smem, st, mi, mq, args);

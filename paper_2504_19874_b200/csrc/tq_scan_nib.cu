@@ -597,7 +597,8 @@ template <int TILED, int MODE, int SB>
 cudaError_t launch_t(const CUtensorMap& mi, const CUtensorMap& mq, const ScanArgs& args, size_t smem, bool dependent,
                      cudaStream_t st) {
   auto kern = scan_nib_kernel<TILED, MODE, SB>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static std::atomic<unsigned long long> smem_devices{0};
+  cudaError_t e = allow_largest_smem(reinterpret_cast<const void*>(kern), smem_devices);
   if (e != cudaSuccess) return e;
   const int grid = (int)std::min<int64_t>(args.ntiles, tc::sm_count());
   if (dependent) e = launch_dependent(kern, dim3(grid), dim3(32 * (NW + 1)), smem, st, mi, mq, args);
