@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(256) measure_kernel(Args a, int R, uint32_t* _
   __shared__ uint32_t warp_tot[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int groups = (a.d + 7) / 8, row_words = (int)(a.idx_rb / 4);
-  const int absent = 8 * groups - a.d;   // coordinates of the last group past the row's end: whatever they hold counts as index 0
+  const int absent = 8 * groups - a.d;   // coordinates of the last group past the row's end: taken off again, whatever they hold
   uint32_t tot = 0;
   for (int r = 0; r < R; ++r) {
     const int64_t row = ((int64_t)blockIdx.x * R + r) * 8 + warp;
@@ -117,7 +117,6 @@ __global__ void __launch_bounds__(256) measure_kernel(Args a, int R, uint32_t* _
       for (int i = 0; i < 8; ++i) {
         const int g = g0 + 32 * i + lane;
         x[i] = g < groups ? nibbles<BITS, BYTES>(p, row_words, g) : 0u;
-        if (g == groups - 1) x[i] &= 0xffffffffu >> (4 * absent);
       }
 #pragma unroll
       for (int i = 0; i < 8; ++i)
@@ -125,7 +124,10 @@ __global__ void __launch_bounds__(256) measure_kernel(Args a, int R, uint32_t* _
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) bits += __shfl_xor_sync(0xffffffffu, bits, o);
-    bits -= (uint32_t)absent * a.code.len[0];
+    if (absent > 0) {   // their nibbles moved to the bottom, index 0 above them
+      const uint32_t tail = nibbles<BITS, BYTES>(p, row_words, groups - 1) >> (4 * (8 - absent));
+      bits -= code_bits<BITS>(a.code, tail, 0u) - (uint32_t)(8 - absent) * a.code.len[0];
+    }
     const uint32_t bytes = (bits + 31) / 32 * 4;
     if (lane == 0) sizes[row] = bytes;
     tot += bytes;
@@ -238,8 +240,8 @@ __global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(Args a, const uin
       for (uint64_t b = off + lane; b < out_bytes && b < off_end; b += 32) out[b] = 0;
       continue;
     }
-    const uint64_t slot = (off_end - off) / 4;   // as many words as the stream has, unless the caller spaced the rows out
-    const int words = (int)min(slot, (uint64_t)image_words);
+    const uint64_t slot = (off_end - off) / 4;
+    const int words = slot > (uint64_t)image_words ? image_words : (int)slot;
     const uint8_t* p = a.idx + (size_t)row * a.idx_rb;
     for (int w = lane; w < words; w += 32) image[w] = 0u;
     __syncwarp();
@@ -297,7 +299,8 @@ __global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(Args a, const uin
     __syncwarp();
     uint32_t* dst = reinterpret_cast<uint32_t*>(out + off);
     for (int w = lane; w < words; w += 32) dst[w] = image[w];
-    for (uint64_t w = words + lane; w < slot; w += 32) dst[w] = 0u;
+    if (slot > (uint64_t)image_words)   // the caller spaced the rows out
+      for (uint64_t w = words + lane; w < slot; w += 32) dst[w] = 0u;
     __syncwarp();
   }
   // What lies before the first stream and after the last one is zero too.
