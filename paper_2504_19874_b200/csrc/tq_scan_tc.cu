@@ -777,6 +777,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {   // 16 queries per half: digit l of query 16 h + qq sits in column 32 l + 16 h + qq
         if (h * 16 >= a.nqp) break;   // a short last pass: columns of absent queries are not read
+        __syncwarp();                 // lanes leave the first half's stores and hits one by one; the TMEM load takes whole warps
         uint32_t va[LIMBS][16], vs[LIMBS][16];
 #pragma unroll
         for (int l = 0; l < LIMBS; ++l) {
@@ -802,6 +803,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__
         if (a.nqp < 16 * h + 16) hits &= (1u << (a.nqp - 16 * h)) - 1u;
         append_hits<LBUF>(a, hits, est, 16 * h, row, lcnt, lbuf);
       }
+      __syncwarp();
       tc::tc_fence_before();
     }
   }

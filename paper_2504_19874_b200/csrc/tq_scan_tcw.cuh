@@ -480,6 +480,7 @@ scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant_
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         if (h >= nh) break;   // digit l of query 32 set + 16 h + qq sits in column 96 set + 32 l + 16 h + qq
+        if (MODE == 0) __syncwarp();   // lanes leave the first half's stores one by one; the TMEM load takes whole warps
         uint32_t va[LIMBS][16], vs[LIMBS][16];
 #pragma unroll
         for (int l = 0; l < LIMBS; ++l) {

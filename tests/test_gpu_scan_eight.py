@@ -39,3 +39,21 @@ def test_filter_pass():
         ts, ti = su.topk(Q[:nq].contiguous(), n, *codes, k)
         order = torch.sort(sc[:nq], dim=1, descending=True, stable=True)
         assert torch.equal(ts, order.values[:, :k]) and torch.equal(ti.long(), order.indices[:, :k])
+
+
+@pytest.mark.parametrize("nq", [9, 16, 17, 32, 33, 64])
+def test_filter_pass_whose_lanes_hit_unequally(nq):
+    """Every seventh row is close to all queries, so that a lane of the tensor-core scans has up to sixteen hits at once and its
+    neighbours none."""
+    su = P.Setup(136, 2, tq.TQ_MSE)
+    g = torch.Generator(device="cpu").manual_seed(nq)
+    n = 70_003
+    X, Q = torch.randn((n, 136), generator=g), torch.randn((nq, 136), generator=g) + 2.0
+    X[::7] += 2.0
+    codes = su.quantize(X.to(DEV))
+    sc = su.score(Q.to(DEV), n, *codes)
+    order = torch.sort(sc, dim=1, descending=True, stable=True)
+    for k in (1, 1024):
+        ts, ti = su.topk(Q.to(DEV), n, *codes, k)
+        tq.tq_plan_status(su.plan)
+        assert torch.equal(ts, order.values[:, :k]) and torch.equal(ti.long(), order.indices[:, :k])
