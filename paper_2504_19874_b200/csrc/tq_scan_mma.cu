@@ -921,12 +921,12 @@ __global__ void __launch_bounds__(1024) select_kernel(SelArgs a) {
     if (rank == a.k - 1 && a.kth != nullptr) a.kth[q] = s;
   };
   if (found <= 256) {
-    // a key's rank is the number of larger ones (keys are distinct: they contain the id); four threads count for one key, so
-    // that there is no barrier at all
+    // a key's rank is the number of larger ones (and of equal ones before it: an id may have been given twice); four threads
+    // count for one key, so that there is no barrier at all
     const unsigned long long key = skey[tid >> 2];
     int rank = 0;
 #pragma unroll 4
-    for (int i = tid & 3; i < found; i += 4) rank += skey[i] > key ? 1 : 0;
+    for (int i = tid & 3; i < found; i += 4) rank += skey[i] > key || (skey[i] == key && i < (tid >> 2)) ? 1 : 0;
     rank += __shfl_xor_sync(0xffffffffu, rank, 1);
     rank += __shfl_xor_sync(0xffffffffu, rank, 2);
     if ((tid & 3) == 0 && (tid >> 2) < found && rank < a.k) put(rank, key);

@@ -45,3 +45,18 @@ def test_selection(m, kind):
         for q in range(nq):
             ws, wi = expected(s[q], ids[q], k)
             assert np.array_equal(ti[q].cpu().numpy(), wi) and np.array_equal(ts[q].cpu().numpy(), ws), (q, k)
+
+
+@pytest.mark.parametrize("m", [6, 300, 2000, 5000])
+def test_the_same_pair_given_twice(m):
+    """Shards that overlap hand in a (score, id) pair twice: every output slot is written, both copies in place."""
+    g = np.random.default_rng(m)
+    s, ids = np.repeat(g.standard_normal(m // 2).astype(np.float32), 2), np.repeat(g.permutation(m // 2).astype(np.int32), 2)
+    shuffle = g.permutation(m)
+    s, ids = s[shuffle], ids[shuffle]
+    cs, ci = torch.from_numpy(s[None]).to(DEV), torch.from_numpy(ids[None]).to(DEV)
+    for k in (1, 6, 100, 256, 1000):
+        ts, ti = torch.full((1, k), -77.0, device=DEV), torch.full((1, k), -77, dtype=torch.int32, device=DEV)
+        tq.tq_select_topk(cs, ci, k, ts, ti)
+        ws, wi = expected(s, ids, k)
+        assert np.array_equal(ti[0].cpu().numpy(), wi) and np.array_equal(ts[0].cpu().numpy(), ws)
