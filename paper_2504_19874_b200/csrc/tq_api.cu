@@ -148,12 +148,12 @@ int engine_prepare(const ScanEngine& e, const float* Qcat, int q0, int nq, void*
 
 int engine_run(const ScanEngine& e, int q0, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma,
                const float* norms, float* scores, int64_t lds, const mscan::Filter* filter, const int* run_if, const void* ws,
-               cudaStream_t st, const char* who) {
-  if (e.nib) return nscan::run(e.plan, nqp, n, idx, qjl, gamma, norms, scores, lds, filter, run_if, ws, true, st, who);
+               cudaStream_t st, const char* who, int64_t step = 1) {
+  if (e.nib) return nscan::run(e.plan, nqp, n, idx, qjl, gamma, norms, scores, lds, filter, run_if, ws, true, st, who, step);
   if (e.tc)
     return tscan::run_pass(e.plan, (q0 % kGroupQueries) / tscan::kQueriesPerPass, nqp, n, idx, qjl, gamma, norms, scores, lds,
-                           filter, run_if, ws, st, who);
-  return mscan::run(e.plan, nqp, n, idx, qjl, gamma, norms, scores, lds, filter, run_if, ws, st, who);
+                           filter, run_if, ws, st, who, step);
+  return mscan::run(e.plan, nqp, n, idx, qjl, gamma, norms, scores, lds, filter, run_if, ws, st, who, step);
 }
 
 size_t ms_score_fixed(const tq_plan* plan, int nq) { return qcat_bytes(plan, nq) + align_up(pick_engine(plan, nq).ws_bytes, 256); }
@@ -988,7 +988,7 @@ extern "C" int tq_score_prepared(const tq_plan* plan, const void* prepared, int 
   return TQ_OK;
 }
 
-// Top-k through the tensor-path scan.  Large n: a pilot pass over the first rows gives, per query,
+// Top-k through the tensor-path scan.  Large n: a pilot pass over a sample of the rows gives, per query,
 // the k-th best score among them -- a lower bound on the final k-th score -- and the full pass
 // keeps only (score, id) pairs at or above it; a final selection sorts the survivors.  Should a
 // candidate list overflow (massive ties, adversarial order) a device-side flag switches on a
@@ -1020,12 +1020,16 @@ static int topk_ms(const tq_plan* plan, const float* Qcat, int nq, int64_t n, co
     const bool use_filter = n >= kFilterMinN && dense_rows >= std::min<int64_t>(n, eng.dense_rows_pref);
     const int* guard = nullptr;
     if (use_filter) {
-      // pilot rows: about 8192 candidates are then expected from the full pass (n k / m), well inside the lists' 32,768 (the
-      // k-th best of the pilot varies by 1 / sqrt(k)) and what the final selection keeps in registers; a larger pilot costs a
-      // longer pilot scan and selection
-      int64_t m = std::max<int64_t>(round_up64((int64_t)((double)n * k / 8192.0), 256), 4096);
+      // Pilot rows m: the full pass then has n / m times as many candidates as the pilot has scores down to the threshold, which
+      // are k where it meets the k-th best exactly.  That number varies like a sum of k exponentials, so that at k = 1 the count
+      // is four times the expected one in one query of 55, and one overflow of a list of 32,768 has all rows scored again for
+      // the whole pass (k = 1, 64 queries, 34 * 10^6 rows, 8,192 expected: 28.3 ms instead of 5.5).  m = n (k + 8) / 8192 expects
+      // 910 at k = 1 and 7,585 at k = 100; a larger pilot costs a longer pilot scan and selection.
+      // The rows are spread over the whole index: the first ones say nothing about the others where an index is stored by topic
+      // or time (1,000 clusters in turn, 8 queries, k = 10, 10^6 rows: 607 us from the first 4,096 rows, 84 when shuffled).
+      int64_t m = std::max<int64_t>(round_up64((int64_t)((double)n * (k + 8) / 8192.0), 256), 4096);
       m = std::min<int64_t>(m, std::min<int64_t>(dense_rows / 256 * 256, n));
-      if ((rc = engine_run(eng, q0, nqp, m, idx, qjl, gamma, norms, dense, m, nullptr, nullptr, msw, st, who))) return rc;
+      if ((rc = engine_run(eng, q0, nqp, m, idx, qjl, gamma, norms, dense, m, nullptr, nullptr, msw, st, who, n / m))) return rc;
       TQ_CHECK_CUDA(mscan::select_topk(dense, nullptr, nullptr, (int)m, (int)m, 0, nqp, k, 0, nullptr, nullptr, tau, nullptr, nullptr, count, overflow, st), who);
       mscan::Filter f{tau, count, cand_s, cand_i, kCandCap};
       if ((rc = engine_run(eng, q0, nqp, n, idx, qjl, gamma, norms, nullptr, 0, &f, nullptr, msw, st, who))) return rc;

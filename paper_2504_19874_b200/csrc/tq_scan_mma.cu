@@ -267,6 +267,7 @@ struct ScanArgs {
   int nq_pass;
   const float* gamma;
   const float* norms;      // nullable
+  int64_t step;            // rows of the arrays from one vector to the next
   float coef;
   float* scores;           // dense: row q of this pass at scores + q*lds
   int64_t lds;
@@ -398,8 +399,8 @@ scan_mma_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
       for (int h = 0; h < NRW; ++h) {
         const int64_t row = tile * VT + cw * (MT * 16) + m * 16 + g + ((TILED ? h != 0 : (t4 & 1) != 0) ? 8 : 0);
         const bool in = row < a.n;   // (also false for a tile past the last)
-        nu_next[m][h] = (in && a.norms != nullptr) ? __ldg(a.norms + row) : 1.f;
-        gm_next[m][h] = (PROD && in) ? __ldg(a.gamma + row) : 0.f;   // multiplied by coef where it is used: no wait here
+        nu_next[m][h] = (in && a.norms != nullptr) ? __ldg(a.norms + row * a.step) : 1.f;
+        gm_next[m][h] = (PROD && in) ? __ldg(a.gamma + row * a.step) : 0.f;   // multiplied by coef where it is used: no wait here
       }
   };
   constexpr bool AHEAD = (NT == 1);   // with two column tiles the longer tile hides the request and the registers cost more
@@ -1127,17 +1128,17 @@ int prepare(const tq_plan* plan, const float* Qcat, int nqp, void* workspace, cu
 
 int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma,
         const float* norms, float* scores, int64_t lds, const Filter* filter, const int* run_if, const void* workspace,
-        cudaStream_t st, const char* who) {
+        cudaStream_t st, const char* who, int64_t step) {
   const Config c = config_for(plan, nqp);
   const bool prod = plan->mode == TQ_PROD;
   const int bm = plan->mse_bits;
   const int VT = c.NW * c.MT * 16;
   CUtensorMap mi, mq;
   if (bm > 0)
-    TQ_REQUIRE(tc::make_byte_map(&mi, idx, (uint64_t)n, plan->idx_row_bytes, plan->idx_row_bytes, 64, VT), TQ_ERR_CUDA,
+    TQ_REQUIRE(tc::make_byte_map(&mi, idx, (uint64_t)n, plan->idx_row_bytes, plan->idx_row_bytes * step, 64, VT), TQ_ERR_CUDA,
                "%s: cuTensorMapEncodeTiled failed (idx)", who);
   if (prod)
-    TQ_REQUIRE(tc::make_byte_map(&mq, qjl, (uint64_t)n, plan->qjl_row_bytes, plan->qjl_row_bytes, 64, VT), TQ_ERR_CUDA,
+    TQ_REQUIRE(tc::make_byte_map(&mq, qjl, (uint64_t)n, plan->qjl_row_bytes, plan->qjl_row_bytes * step, 64, VT), TQ_ERR_CUDA,
                "%s: cuTensorMapEncodeTiled failed (qjl)", who);
   if (bm == 0) mi = mq;
   if (!prod) mq = mi;
@@ -1153,6 +1154,7 @@ int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8
   sa.nq_pass = nqp;
   sa.gamma = gamma;
   sa.norms = norms;
+  sa.step = step;
   sa.coef = plan->coef;
   sa.scores = scores;
   sa.lds = lds;

@@ -29,10 +29,11 @@ int prepare(const tq_plan* plan, const float* Qcat, int nqp, void* workspace, cu
 
 // One pass over vectors [0, n) with the operand prepared in `workspace`: dense estimates into
 // scores[nqp, lds], or, with a filter, only the (score, row) pairs it admits.  When run_if is not null
-// the kernel returns at once if *run_if == 0 (device-side switch, read at launch).
+// the kernel returns at once if *run_if == 0 (device-side switch, read at launch).  step > 1: vector i of the pass is row i step
+// of the arrays (a sample of the database).
 int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma,
         const float* norms, float* scores, int64_t lds, const Filter* filter, const int* run_if, const void* workspace,
-        cudaStream_t st, const char* who);
+        cudaStream_t st, const char* who, int64_t step = 1);
 
 // The k best (score desc, id asc) per query out of `count[q]` (clamped to cap) candidate pairs, or, when
 // cand_i is nullptr, out of the dense row cand_s[q*cap .. +m) with ids id0 + position.  Optionally merges

@@ -184,6 +184,7 @@ struct ScanArgs {
   int nq_pass;
   const float* gamma;
   const float* norms;      // nullable
+  int64_t step;            // rows of the arrays from one vector to the next
   float coef;
   float* scores;
   int64_t lds;
@@ -348,8 +349,8 @@ scan_nib_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int64_t row = rt + cw * 16 + g + 8 * h;
-      nu_pre[h] = (row < row_end && a.norms != nullptr) ? ldg_now(a.norms + row) : 1.f;
-      gm_pre[h] = (row < row_end) ? ldg_now(a.gamma + row) : 0.f;
+      nu_pre[h] = (row < row_end && a.norms != nullptr) ? ldg_now(a.norms + row * a.step) : 1.f;
+      gm_pre[h] = (row < row_end) ? ldg_now(a.gamma + row * a.step) : 0.f;
     }
 
     for (int s = 0; s < a.nsteps; ++s) {
@@ -691,14 +692,14 @@ int prepare(const tq_plan* plan, const float* Qcat, int nqp, void* workspace, cu
 
 int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma,
         const float* norms, float* scores, int64_t lds, const mscan::Filter* filter, const int* run_if,
-        const void* workspace, bool codes_final, cudaStream_t st, const char* who) {
+        const void* workspace, bool codes_final, cudaStream_t st, const char* who, int64_t step) {
   const bool tiled = queries_per_pass(plan, nqp) == 8;
   Config c;
   TQ_REQUIRE(pick_config(plan, tiled, &c), TQ_ERR_UNSUPPORTED, "%s: no shared-memory configuration for d=%d", who, plan->d);
   CUtensorMap mi, mq;
-  TQ_REQUIRE(tc::make_byte_map(&mi, idx, (uint64_t)n, plan->idx_row_bytes, plan->idx_row_bytes, 64, VT), TQ_ERR_CUDA,
+  TQ_REQUIRE(tc::make_byte_map(&mi, idx, (uint64_t)n, plan->idx_row_bytes, plan->idx_row_bytes * step, 64, VT), TQ_ERR_CUDA,
              "%s: cuTensorMapEncodeTiled failed (idx)", who);
-  TQ_REQUIRE(tc::make_byte_map(&mq, qjl, (uint64_t)n, plan->qjl_row_bytes, plan->qjl_row_bytes, 64, VT), TQ_ERR_CUDA,
+  TQ_REQUIRE(tc::make_byte_map(&mq, qjl, (uint64_t)n, plan->qjl_row_bytes, plan->qjl_row_bytes * step, 64, VT), TQ_ERR_CUDA,
              "%s: cuTensorMapEncodeTiled failed (qjl)", who);
   ScanArgs sa;
   sa.n = n;
@@ -714,6 +715,7 @@ int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8
   sa.nq_pass = nqp;
   sa.gamma = gamma;
   sa.norms = norms;
+  sa.step = step;
   sa.coef = plan->coef;
   sa.scores = scores;
   sa.lds = lds;

@@ -26,7 +26,7 @@ int prepare(const tq_plan* plan, const float* Qcat, int nqp, void* workspace, cu
 // call began and the scan may start copying them while that kernel still runs (programmatic dependent launch).
 int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma,
         const float* norms, float* scores, int64_t lds, const mscan::Filter* filter, const int* run_if,
-        const void* workspace, bool codes_final, cudaStream_t st, const char* who);
+        const void* workspace, bool codes_final, cudaStream_t st, const char* who, int64_t step = 1);
 
 // Rewrites n rows of (idx, qjl) in place from one layout into the other (an exact permutation of the bits).
 int convert(const tq_plan* plan, int64_t n, uint8_t* idx, uint8_t* qjl, int to_layout, cudaStream_t st, const char* who);

@@ -404,6 +404,7 @@ struct ScanArgs {
   size_t qjl_rb;
   const float* gamma;
   const float* norms;
+  int64_t step;            // rows of the arrays from one vector to the next
   float coef;
   float* scores;
   int64_t lds;
@@ -610,11 +611,11 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__
     // the row's scalars are requested one pair ahead, so that their latency hides behind a pair's k-blocks
     auto load_nu = [&](int64_t pr) -> float {
       const int64_t rw = pr * (2 * TILE) + t * TILE + r;
-      return (pr < a.npairs && rw < a.n && a.norms != nullptr) ? __ldg(a.norms + rw) : 1.f;
+      return (pr < a.npairs && rw < a.n && a.norms != nullptr) ? __ldg(a.norms + rw * a.step) : 1.f;
     };
     auto load_gm = [&](int64_t pr) -> float {
       const int64_t rw = pr * (2 * TILE) + t * TILE + r;
-      return (pr < a.npairs && rw < a.n && (a.g.kbs > 0 || NIB)) ? __ldg(a.gamma + rw) : 0.f;   // times coef where it is used, so that nothing waits for the load here
+      return (pr < a.npairs && rw < a.n && (a.g.kbs > 0 || NIB)) ? __ldg(a.gamma + rw * a.step) : 0.f;   // times coef where it is used, so that nothing waits for the load here
     };
     float nu_next = load_nu(blockIdx.x), gm_next = load_gm(blockIdx.x);
     for (int64_t pair = blockIdx.x; pair < a.npairs && ok; pair += gridDim.x, ++it) {
@@ -997,7 +998,7 @@ int prepare_group(const tq_plan* plan, const float* Qcat, int nqg, void* workspa
 
 int run_pass(const tq_plan* plan, int pass, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma,
              const float* norms, float* scores, int64_t lds, const mscan::Filter* filter, const int* run_if,
-             const void* workspace, cudaStream_t st, const char* who) {
+             const void* workspace, cudaStream_t st, const char* who, int64_t step) {
   const Geo g = make_geo(plan);
   const QConst* qc = static_cast<const QConst*>(workspace);
   const uint8_t* Ba = static_cast<const uint8_t*>(workspace) + kConstBytes;
@@ -1030,15 +1031,15 @@ int run_pass(const tq_plan* plan, int pass, int nqp, int64_t n, const uint8_t* i
   CUtensorMap pa, ps;
   const int gb = g.nib ? 64 : group_bytes(g.bm);
   if (g.nib) {
-    TQ_REQUIRE(tc::make_byte_map(&pa, idx, (uint64_t)n, plan->idx_row_bytes, plan->idx_row_bytes, 64, prows, 64) &&
-                   tc::make_byte_map(&ps, qjl, (uint64_t)n, plan->qjl_row_bytes, plan->qjl_row_bytes, 64, prows, 64),
+    TQ_REQUIRE(tc::make_byte_map(&pa, idx, (uint64_t)n, plan->idx_row_bytes, plan->idx_row_bytes * step, 64, prows, 64) &&
+                   tc::make_byte_map(&ps, qjl, (uint64_t)n, plan->qjl_row_bytes, plan->qjl_row_bytes * step, 64, prows, 64),
                TQ_ERR_CUDA, "%s: cuTensorMapEncodeTiled failed (code rows)", who);
   } else if (g.kba > 0)
-    TQ_REQUIRE(tc::make_byte_map(&pa, idx, (uint64_t)n, plan->idx_row_bytes, plan->idx_row_bytes, gb, prows,
+    TQ_REQUIRE(tc::make_byte_map(&pa, idx, (uint64_t)n, plan->idx_row_bytes, plan->idx_row_bytes * step, gb, prows,
                                  gb == 64 ? 64 : gb == 32 ? 32 : 0),
                TQ_ERR_CUDA, "%s: cuTensorMapEncodeTiled failed (idx rows)", who);
   if (!g.nib && g.kbs > 0)
-    TQ_REQUIRE(tc::make_byte_map(&ps, qjl, (uint64_t)n, plan->qjl_row_bytes, plan->qjl_row_bytes, 64, prows, 64), TQ_ERR_CUDA,
+    TQ_REQUIRE(tc::make_byte_map(&ps, qjl, (uint64_t)n, plan->qjl_row_bytes, plan->qjl_row_bytes * step, 64, prows, 64), TQ_ERR_CUDA,
                "%s: cuTensorMapEncodeTiled failed (qjl rows)", who);
   if (!g.nib && g.kba == 0) pa = ps;
   if (!g.nib && g.kbs == 0) ps = pa;
@@ -1056,6 +1057,7 @@ int run_pass(const tq_plan* plan, int pass, int nqp, int64_t n, const uint8_t* i
   a.qjl_rb = plan->qjl_row_bytes;
   a.gamma = gamma;
   a.norms = norms;
+  a.step = step;
   a.coef = plan->coef;
   a.scores = scores;
   a.lds = lds;

@@ -24,10 +24,10 @@ int prepare_group(const tq_plan* plan, const float* Qcat, int nqg, void* workspa
 
 // One pass of up to 32 queries (pass index `pass` inside the prepared group), or of 33 to 64 queries (the queries of
 // passes `pass` and `pass + 1`, `pass` even), over vectors [0, n): dense estimates into scores[nqp, lds] or the pairs
-// admitted by the filter.  run_if as in mscan::run.
+// admitted by the filter.  run_if and step as in mscan::run.
 int run_pass(const tq_plan* plan, int pass, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma,
              const float* norms, float* scores, int64_t lds, const mscan::Filter* filter, const int* run_if,
-             const void* workspace, cudaStream_t st, const char* who);
+             const void* workspace, cudaStream_t st, const char* who, int64_t step = 1);
 
 }  // namespace tscan
 }  // namespace tq

@@ -291,11 +291,11 @@ scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant_
     uint32_t it = 0;
     auto load_nu = [&](int64_t tl) -> float {
       const int64_t rw = tl * TILE + r;
-      return (rw < a.n && a.norms != nullptr) ? __ldg(a.norms + rw) : 1.f;
+      return (rw < a.n && a.norms != nullptr) ? __ldg(a.norms + rw * a.step) : 1.f;
     };
     auto load_gm = [&](int64_t tl) -> float {
       const int64_t rw = tl * TILE + r;
-      return (rw < a.n && (a.g.kbs > 0 || NIB)) ? __ldg(a.gamma + rw) : 0.f;   // times coef where it is used, so that nothing waits for the load here
+      return (rw < a.n && (a.g.kbs > 0 || NIB)) ? __ldg(a.gamma + rw * a.step) : 0.f;   // times coef where it is used, so that nothing waits for the load here
     };
     // zeroes this thread's columns of both accumulators and tells the issuers (before the first tile, and in every
     // epilogue as soon as the columns have been read into registers)

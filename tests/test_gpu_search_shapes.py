@@ -54,3 +54,26 @@ def test_one_row_far_above_the_others(nq, k):
     for norm in (1e4, 1e6):
         codes[3][:: N // 8] = norm                    # (row 0 is in any sample of the rows)
         check(su, Q, codes, k, plain)
+
+
+@pytest.mark.parametrize("bits,mode,layout,nq", [(2, tq.TQ_MSE, None, 1), (2, tq.TQ_MSE, None, 8), (2, tq.TQ_MSE, None, 24), (2, tq.TQ_MSE, None, 64),
+                                                 (4, tq.TQ_PROD, tq.TQ_LAYOUT_NIBBLE, 2), (4, tq.TQ_PROD, tq.TQ_LAYOUT_NIBBLE, 8)])
+def test_rows_in_the_order_of_their_clusters(bits, mode, layout, nq):
+    su = P.Setup(D, bits, mode, layout=layout)
+    clusters, g = 1000, torch.Generator(device=DEV).manual_seed(1000)
+    centres = torch.randn((clusters, D), generator=g, device=DEV)
+    X = centres.repeat_interleave(N // clusters, dim=0) + torch.randn((N, D), generator=g, device=DEV)
+    codes = su.quantize(X)
+    shuffle = torch.randperm(N, generator=g, device=DEV)
+    Q = centres[torch.randint(500, 1000, (nq,), generator=torch.Generator().manual_seed(5))] + torch.randn((nq, D), generator=g, device=DEV)
+    for k in (10, 100):
+        plain = search(su, Q, N, [None if t is None else t[shuffle].contiguous() for t in codes], k)[2]
+        check(su, Q, codes, k, plain)
+
+
+def test_the_nearest_of_very_many_rows():
+    n = 34_000_000                                    # 8,192 candidates per score of the pilot once meant a list of 32,768 at times
+    su = P.Setup(128, 1, tq.TQ_MSE)
+    codes = random_codes(su, n, 2)
+    Q = torch.randn((64, 128), generator=torch.Generator().manual_seed(3)).to(DEV)
+    assert search(su, Q, n, codes, 1)[2] < 2.0 * search(su, Q, n, codes, 10)[2]
