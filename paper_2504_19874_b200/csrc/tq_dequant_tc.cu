@@ -69,8 +69,10 @@ struct Args {
   int bits;                         // b_m; 0: no centroid term
   int nibble;                       // TQ_LAYOUT_NIBBLE
   uint32_t tab[4][4];               // bytes of the fp16 limbs of the codebook: hi low byte, hi high byte, lo low, lo high; 16 entries each
-  float gscale;                     // coef 2^(eP + ec - eS): weight of the z accumulators per unit of gamma
-  float oscale;                     // 2^-(eP + ec)
+  // Weights of the accumulators, powers of two but for coef.  They are applied as the accumulators are drained, so that the sums
+  // are in the units of the result and any norm and gamma of an fp32 result's range may multiply them.
+  float oscale;                     // 2^-(eP + ec): centroid term
+  float gscale;                     // coef 2^-eS: sign term, per unit of gamma
   float* out;
   int64_t ldo;
   int tma_store;                    // Xhat rows are 16-byte aligned: boxes leave by TMA
@@ -428,7 +430,7 @@ dequant_kernel(const __grid_constant__ CUtensorMap tmP1, const __grid_constant__
         ++it;
         if (!(ok = mbar_wait(&tfull[acc], acc_phase, abort_flag, a.status))) break;
         tc_fence_after();
-        const float s = drained_term == 0 ? 1.f : g;
+        const float s = drained_term == 0 ? a.oscale : g;
         const uint32_t base = tmem_base + ((uint32_t)(lg * 32) << 16) + acc * BN + part * NC;
 #pragma unroll
         for (int q = 0; q < NC / 16; ++q) {
@@ -447,7 +449,7 @@ dequant_kernel(const __grid_constant__ CUtensorMap tmP1, const __grid_constant__
       }
       if (!ok) break;
       if (split > 1) break;   // one tile per CTA: the sums of the cluster meet below
-      store_sums<NC>(a, tmO, r, a.oscale * nu, row0, col0, buf, lane);
+      store_sums<NC>(a, tmO, r, nu, row0, col0, buf, lane);
     }
     if constexpr (CTAS == 1) {
       if (split > 1) {
@@ -485,7 +487,7 @@ dequant_kernel(const __grid_constant__ CUtensorMap tmP1, const __grid_constant__
         }
         __syncwarp();
         const float nu = (a.norms != nullptr && row < a.n) ? __ldg(a.norms + row) : 1.f;
-        store_sums<NC>(a, tmO, r, a.oscale * nu, row0, (int)(unit % a.tiles_n) * BN + (w >> 2) * NC, buf, lane);
+        store_sums<NC>(a, tmO, r, nu, row0, (int)(unit % a.tiles_n) * BN + (w >> 2) * NC, buf, lane);
         if (lane == 0) tma_store_wait_all();
         __syncwarp();
       }
@@ -584,9 +586,9 @@ cudaError_t plan_init(tq_plan* plan, const float* Pi, const float* S) {
   const double pmax = max_abs(Pi), smax = S ? max_abs(S) : 0.0;
   if (!std::isfinite(pmax) || !std::isfinite(smax)) return cudaSuccess;   // the CUDA-core path carries such values through
   const int eP = limb_exponent(pmax), eS = limb_exponent(smax), ec = limb_exponent(cmax);
-  for (int e : {eP, eS, ec, eP + ec, eP + ec - eS})
+  for (int e : {eP, eS, ec, eP + ec})
     if (e > 100 || e < -100) return cudaSuccess;
-  m.gscale = (float)std::ldexp(1.0, eP + ec - eS) * plan->coef;
+  m.gscale = (float)std::ldexp(1.0, -eS) * plan->coef;
   m.oscale = (float)std::ldexp(1.0, -(eP + ec));
   for (int p = 0; p < 4; ++p)
     for (int q = 0; q < 4; ++q) m.tab[p][q] = 0u;

@@ -155,7 +155,7 @@ struct tq_plan {
     __half *p_hi, *p_lo, *s_hi, *s_lo; // fp16 limbs of Pi^T and S^T, scaled by powers of two
     alignas(64) CUtensorMap map_p_hi, map_p_lo, map_s_hi, map_s_lo;
     uint32_t tab[4][4];                // bytes of the codebook's limbs: hi low / high byte, lo low / high byte, 16 entries each
-    float gscale, oscale;              // weight of the sign term per unit of gamma; scale of the result
+    float gscale, oscale;              // weights of the accumulated sign term (per unit of gamma) and centroid term
   } dq;
   // one-launch quantiser for short vectors (d = 32, 64, 96)
   struct {

@@ -42,3 +42,24 @@ def test_reconstruction_at_tile_edges(d, bits, mode, layout, n, pad):
     tq.tq_dequantize(su.plan, n, codes[0], codes[1], codes[2], None, again)
     tq.tq_plan_status(su.plan)
     assert torch.allclose(again * codes[3][:, None], out[:, :d], rtol=1e-6, atol=0)
+
+
+@pytest.mark.parametrize("n", [40, 3000])                       # both tiles
+@pytest.mark.parametrize("bits,mode", [(3, tq.TQ_MSE), (3, tq.TQ_PROD)])
+def test_norms_and_residual_norms_of_any_size(bits, mode, n):
+    """Scaling a row's norm or its gamma scales the row: to 1e-6 of it where the result is a normal number (a quotient of two
+    fp32 results of the same sums errs by three roundings, 3 x 2^-24), also at 1e-34 and at 1e30."""
+    d = 256
+    su = P.Setup(d, bits, mode)
+    X = torch.randn((n, d), generator=torch.Generator().manual_seed(n)).to(DEV)
+    idx, qjl, gamma, _ = su.quantize(X)
+    ones = torch.ones(n, device=DEV)
+    base = su.dequantize(n, idx, qjl, gamma, ones).double()
+    for nu in (1e-34, 1e-30, 1e-20, 1e20, 1e30):
+        out = su.dequantize(n, idx, qjl, gamma, ones * nu).double()
+        assert ((out - base * float(np.float32(nu))).norm(dim=1) <= 1e-6 * (base * nu).norm(dim=1)).all(), nu
+    if mode == tq.TQ_PROD:
+        sign = su.dequantize(n, idx, qjl, ones * 2.0 ** 40, None).double()        # the centroid term is 2^-40 of this
+        for g in (2.0 ** 60, 2.0 ** 100):
+            out = su.dequantize(n, idx, qjl, ones * g, None).double()
+            assert ((out - sign * (g / 2.0 ** 40)).norm(dim=1) <= 1e-6 * out.norm(dim=1)).all(), g
