@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads) small_quantize_kernel(Args a
   float* bs = xs + RT * S;                 // [D][D]   Pi^T
   float* ss = bs + D * D;                  // [D][D]   S'^T (PROD)
   float* vs = bs + (PROD ? 2 : 1) * D * D; // [RT]     nu as the comparisons take it (1 for a zero row)
-  float* is = vs + RT;                     // [RT]     1 / nu (0 for a zero row)
+  float* is = vs + RT;                     // [RT]     1 / nu (-1 for a zero row; 0 where the norm has overflowed)
   const int tid = threadIdx.x, lane = tid & 31;
   const int tx = tid % TX, ty = tid / TX, t8 = lane & 7;
   const int64_t row0 = (int64_t)blockIdx.x * RT;
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads) small_quantize_kernel(Args a
     if ((tid & 3) == 0) {
       if (a.norms != nullptr && row0 + r < a.n) a.norms[row0 + r] = nu;
       vs[r] = nu > 0.f ? nu : 1.f;
-      is[r] = nu > 0.f ? 1.f / nu : 0.f;
+      is[r] = nu > 0.f ? 1.f / nu : -1.f;
     }
   }
   if (PROD) asm volatile("cp.async.wait_group 1;" ::: "memory");
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads) small_quantize_kernel(Args a
         if (PROD) cent = above ? a.cb.c[t + 1] : cent;
       }
       four |= (uint32_t)code << (BITS * c);
-      if (PROD) e[c] = inv > 0.f ? fmaf(y, inv, -cent) : 0.f;
+      if (PROD) e[c] = inv >= 0.f ? fmaf(y, inv, -cent) : 0.f;
     }
     if (BITS > 0) {
       int which;
