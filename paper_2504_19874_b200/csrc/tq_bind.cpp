@@ -249,7 +249,7 @@ TQ_FN(softmax, 4) {   // s1, s2, scale, W
   });
 }
 
-// ---- channel groups of a compressed KV layer: a sequence of dicts
+// ---- channel groups of a compressed KV layer: a sequence of dicts (or of other mappings, which are copied into dicts)
 enum { kPlanK, kPlanV, kKIdx, kKQjl, kKGamma, kKNorms, kVIdx, kVNorms, kKChan, kVChan, kKeys };
 PyObject* keys[kKeys];
 PyObject* handle_name;
@@ -257,6 +257,10 @@ PyObject* handle_name;
 struct Groups {
   tq_kv_group g[TQ_MAX_KV_GROUPS];
   int n;
+  PyObject* copies[TQ_MAX_KV_GROUPS] = {};   // they keep the tensors until the call has returned
+  ~Groups() {
+    for (PyObject* c : copies) Py_XDECREF(c);
+  }
 };
 
 PyObject* item(PyObject* dict, int key, bool needed) {
@@ -295,7 +299,10 @@ void kv_groups(PyObject* seq, Groups* out) {
   out->n = (int)n;
   for (Py_ssize_t i = 0; i < n && i < TQ_MAX_KV_GROUPS; ++i) {   // more groups than that: the library rejects the count
     PyObject* d = PySequence_Fast_GET_ITEM(fast, i);
-    if (!PyDict_Check(d)) fail("groups must be a sequence of dicts");
+    if (!PyDict_Check(d)) {
+      d = out->copies[i] = PyDict_New();
+      if (d == nullptr || PyDict_Update(d, PySequence_Fast_GET_ITEM(fast, i)) != 0) throw Failed();
+    }
     tq_kv_group& g = out->g[i];
     g.plan_k = group_plan(d, kPlanK);
     g.plan_v = group_plan(d, kPlanV);
