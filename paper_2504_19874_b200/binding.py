@@ -71,7 +71,8 @@ _SIGNATURES = {
 
 
 class KvGroup(ctypes.Structure):
-    """struct tq_kv_group of include/tq.h (one channel group of a compressed KV layer)."""
+    """struct tq_kv_group of include/tq.h (one channel group of a compressed KV layer), for programs that call
+    lib().tq_attend_decode / tq_kv_append themselves; the functions below take mappings."""
     _fields_ = [(name, c_void_p) for name in ("plan_k", "plan_v", "k_idx", "k_qjl", "k_gamma", "k_norms", "v_idx", "v_norms",
                                               "k_channels", "v_channels")]
 

@@ -416,8 +416,6 @@ cudaError_t launch_rotate_queries(const tq_plan* plan, const T* Q, int64_t ldq, 
 // Q' = Q Pi^T and Q'' = Q S^T side by side: Qcat[nq, ncat*dpad].
 cudaError_t prepare_queries(const tq_plan* plan, const void* Q, int q_dtype, int nq, int64_t ldq, float* Qcat,
                             cudaStream_t st) {
-  const int ncols = plan->ncat * plan->dpad;
-  (void)ncols;
   // Both kernels add the same products in the same order, so that a query's rotated form (and hence its
   // estimates) does not depend on how many other queries came with it.
   if (q_dtype == TQ_F32) return launch_rotate_queries(plan, static_cast<const float*>(Q), ldq, nq, Qcat, st);

@@ -440,12 +440,13 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
           if (r + i * step < a.M) a.gamma[r + i * step] = sqrtf(g2[i]);
       }
     }
-    // operand limbs of the next block of rows
-    const GemmArgs::SplitTask& t = a.split;
-    if (t.rows > 0) {
-      const int64_t sw = (int64_t)blockIdx.x * NSPLIT + (warp - 2 - 4 * EPS), nsw = (int64_t)gridDim.x * NSPLIT;
-      if (t.normalize) split_rows<float, true>(t.X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
-      else split_rows<float, false>(t.X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
+    if constexpr (MODE == 0) {   // operand limbs of the next block of rows
+      const GemmArgs::SplitTask& t = a.split;
+      if (t.rows > 0) {
+        const int64_t sw = (int64_t)blockIdx.x * NSPLIT + (warp - 2 - 4 * EPS), nsw = (int64_t)gridDim.x * NSPLIT;
+        if (t.normalize) split_rows<float, true>(t.X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
+        else split_rows<float, false>(t.X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
+      }
     }
   } else {
     // ------------------------------------------------------------ epilogue (4 x EPS warps: 4 TMEM lane groups x EPS column parts)
@@ -872,14 +873,13 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
   int64_t R = (int64_t)(scratch_bytes / per_row) / BM * BM;
   R = std::min<int64_t>(R, round_up64(n, BM));
   TQ_REQUIRE(R >= BM, TQ_ERR_WORKSPACE, "%s: scratch of %zu bytes cannot hold one block of %d rows", who, scratch_bytes, BM);
-  // The operand limbs of block i + 1 are prepared by spare warps of a GEMM launch of block i.  TQ_PROD: the project
-  // launch (its A operand is the residual, the limbs of X are free by then), one set of limb buffers.  TQ_MSE: the
-  // rotate launch itself, so the scratch is used as two half-size sets written and read in turn (when the data
-  // spans more than one block and each half still holds a tile).
+  // TQ_MSE: the operand limbs of block i + 1 may be prepared by spare warps of the rotate launch of block i; the scratch is then
+  // used as two half-size sets written and read in turn (when the data spans more than one block and each half still holds a
+  // tile).
   // Two warps per CTA keep up only while the GEMM gives them time: its work per row grows with d^2, theirs with d.
-  // Measured per 10^6 rows with the CTA-pair GEMMs: TQ_MSE d = 1536 10.1 ms with them against 10.6 without; TQ_PROD
-  // loses (d = 1536: 22.1 against 21.5 ms, d = 3072 alike), so its project launch carries no such task any more; at
-  // d = 1024 and below the spare warps are the critical path for both.
+  // Measured per 10^6 rows with the CTA-pair GEMMs: TQ_MSE d = 1536 10.1 ms with them against 10.6 without; beside the project
+  // launch of TQ_PROD they lost (d = 1536: 22.1 against 21.5 ms, d = 3072 alike), so it has none; at d = 1024 and below the
+  // spare warps were the critical path for both.
   // Rows of bf16 or off the 16-byte grid are the critical path at every d (11,734 bf16 rows of d = 1536: 167 us and more with
   // the spare warps, 136 with a launch of their own).
   const bool overlap = !prod && d >= 1536 && x_dtype == TQ_F32 && vec_rows(static_cast<const float*>(X), ldx, d, dpad);
@@ -933,9 +933,8 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
   for (int64_t r0 = 0; r0 < n; r0 += R) {
     const int64_t rows = std::min(R, n - r0);
     float* nu_out = norms ? norms + r0 : nullptr;
-    // 1. nu, u = x / nu, bf16 limbs of u: by a launch of its own for the first block (and for TQ_MSE plans), by the
-    //    spare warps of the previous block's project launch otherwise
-    if (r0 == 0 || !overlap || (!prod && !pingpong)) TQ_CHECK_CUDA(launch_split(r0, st), who);
+    // 1. nu, u = x / nu, bf16 limbs of u: by a launch of its own, or by the spare warps of the previous block's rotate launch
+    if (r0 == 0 || !pingpong) TQ_CHECK_CUDA(launch_split(r0, st), who);
     __nv_bfloat16 *XLc1 = limbs1(r0 / R), *XLc2 = limbs2(r0 / R);
     auto next_block_task = [&](GemmArgs& ga) {
       ga.split.X = static_cast<const float*>(X) + (r0 + R) * ldx;
@@ -998,7 +997,6 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
                "%s: cuTensorMapEncodeTiled failed", who);
     g.out = qjl + (size_t)r0 * plan->qjl_row_bytes;
     g.out_rb = plan->qjl_row_bytes;
-    if (overlap && r0 + R < n) next_block_task(g);   // the limbs of X are free by now
     TQ_CHECK_CUDA(launch_gemm<2>(tile, 1, mE1, mE2, plan->sp_limbs, g, st), who);
   }
   return TQ_OK;
