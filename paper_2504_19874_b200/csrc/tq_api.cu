@@ -164,7 +164,7 @@ size_t ms_topk_fixed(const tq_plan* plan, int nq) {
 template <typename T>
 cudaError_t launch_row_norm(const T* X, int64_t ld, int64_t n, int d, float* out, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  const int64_t blocks = std::min<int64_t>((n + 7) / 8, 148 * 16);
+  const int64_t blocks = std::min<int64_t>((n + 7) / 8, tc::sm_count() * 16);
   scan::row_norm_kernel<T><<<(unsigned)blocks, 256, 0, st>>>(X, ld, n, d, out);
   count_launches(1);
   return cudaGetLastError();
@@ -224,7 +224,7 @@ constexpr int kRotQPerBlock = 64;            // most queries per CTA (grid.y cov
 // fewer rounds in more CTAs: 64 queries of d = 128 took four CTAs 33 us for eight rounds each, 32 CTAs take 3.4 us.
 inline int rotate_queries_per_cta(int64_t column_ctas, int nq) {
   int per = kRotQPerBlock;
-  while (per > kRotQ && column_ctas * ((nq + per - 1) / per) < 2 * 148) per /= 2;
+  while (per > kRotQ && column_ctas * ((nq + per - 1) / per) < 2 * tc::sm_count()) per /= 2;
   return per;
 }
 
@@ -428,7 +428,7 @@ cudaError_t launch_scan_few(const scan::ScanArgs& base, int nq, cudaStream_t st)
   int tile = 8;
   while (tile > 1 && per_query * tile > 200 * 1024) tile >>= 1;
   if (per_query * tile > 220 * 1024) return cudaErrorInvalidConfiguration;
-  const int64_t blocks = std::min<int64_t>((base.n + 255) / 256, 148 * 2);
+  const int64_t blocks = std::min<int64_t>((base.n + 255) / 256, tc::sm_count() * 2);
   for (int q0 = 0; q0 < nq; q0 += tile) {
     scan::ScanArgs a = base;
     a.q0 = q0;

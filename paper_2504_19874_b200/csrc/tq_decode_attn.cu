@@ -405,14 +405,14 @@ __global__ void __launch_bounds__(MERGE_NT, 2) merge_kernel(Args a, float* __res
   const int h = blockIdx.x / a.ngroups, gi = blockIdx.x % a.ngroups;
   const int ncoord = a.ngroups * a.d, d = a.d, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const GroupDev& g = a.g[gi];
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  allow_successor();
   {
     const float4* src = reinterpret_cast<const float4*>(g.v_pi);
     float4* dst = reinterpret_cast<float4*>(pis);
     for (int i = tid; i < d * d / 4; i += MERGE_NT) dst[i] = __ldg(src + i);
     if (tid < d) chan[tid] = g.v_channels[h * d + tid];
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // the slices' partial results come from the kernel before
+  wait_for_predecessor();   // the slices' partial results come from the kernel before
   const float4* ml4 = reinterpret_cast<const float4*>(a.part_ml + (size_t)h * a.nslices * 2 * MAXQ);   // [slice][max, sum]
   // Everything this thread needs from the partial kernel for the first MERGE_NT slices is requested at once -- its
   // slice's maximum and sum, and the first MERGE_PF partial sums of its coordinate -- so that the reductions below

@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(NT, 4) partial_mma_kernel(Args a, MmaArgs ma) 
   const int ntok = (int)min((int64_t)SLICE, a.tokens - t0);
   const int64_t row0 = (int64_t)h * a.head_stride + t0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g8 = lane >> 2, kq = lane & 3;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  allow_successor();
 
   // ---- 0) the slice's code rows and scalars are contiguous in global memory: one flat copy each, dealt to the warps.
   //         They are inputs of the call; the wait for the kernel ahead (the query-side operand) comes only after the
@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(NT, 4) partial_mma_kernel(Args a, MmaArgs ma) 
       }
     }
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // the query-side operand is the previous kernel's output
+  wait_for_predecessor();   // the query-side operand is the previous kernel's output
   {
     const uint4* src = ma.bfrag + (size_t)h * ma.kw * 32;
     uint4* bs = reinterpret_cast<uint4*>(smem_raw + ma.bs_off);

@@ -531,7 +531,7 @@ extern "C" int tq_entropy_measure(const tq_plan* plan, const uint8_t* lengths, i
   uint32_t* sizes = static_cast<uint32_t*>(workspace);
   uint64_t* totals = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(workspace) + sizes_bytes(n) + 7) & ~(uintptr_t)7);
   // eight rows per warp once that still fills the chip four times over
-  const int R = n >= 8 * 8 * 4 * 148 ? 8 : 1;
+  const int R = n >= (int64_t)8 * 8 * 4 * tc::sm_count() ? 8 : 1;
   const int64_t groups = (n + 8 * R - 1) / (8 * R);
   // CTA j of offsets_kernel adds up the j 1024 / (8 R) totals before it: 2^21 rows make 2,048 CTAs read 16,384 totals on
   // average (0.27 GB from L2); from there on one launch turns the totals into prefix sums first

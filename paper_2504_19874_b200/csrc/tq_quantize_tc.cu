@@ -805,7 +805,7 @@ cudaError_t build_matrix_limbs(const float* dM, int rows, int d, int dpad, Matri
   if (e != cudaSuccess) return e;
   e = cudaMalloc(&out->lo, bytes);
   if (e != cudaSuccess) return e;
-  const int blocks = std::min((rows + 7) / 8, 148 * 8);
+  const int blocks = std::min((rows + 7) / 8, sm_count() * 8);
   split_rows_kernel<float, false><<<blocks, 256>>>(dM, d, rows, d, dpad, out->hi, out->lo, nullptr);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;

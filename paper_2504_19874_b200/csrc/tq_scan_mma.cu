@@ -617,8 +617,7 @@ scan_mma_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
 }
 
 // ------------------------------------------------------------------ top-k selection
-// One CTA per query: MSD radix select (8-bit digits) on the 64-bit key (ordered score, ~id) for the
-// k-th best element, then a bitonic sort of the k survivors.  Keys are distinct because ids are.
+// 64-bit keys (ordered score, ~id): the order of the keys is that of the results.  select_kernel below says how they are chosen.
 struct SelArgs {
   const float* cand_s;
   const int* cand_i;      // nullptr: dense row, id = id0 + position

@@ -65,10 +65,6 @@ struct PrepArgs {
   uint2* out;          // [nblocks][KPB][32], k-steps 2j and 2j + 1 of a lane side by side
 };
 
-// Programmatic dependent launch: a kernel launched with the stream-serialisation attribute may start while its
-// predecessor in the stream still runs; it must pass this wait before touching anything the predecessor
-// writes or reads.  launch_dependents lets the successor's CTAs be scheduled as this grid's CTAs drain.
-
 // Warp `ql` of every block derives the scales of query ql itself (a few thousand loads from L2, the same
 // values in the same order everywhere); block 0 publishes the constants the scan needs.
 __device__ void query_scales(const PrepArgs& a, QScale* sc /* shared, [8] */) {
