@@ -14,8 +14,9 @@
 //   pack      one warp per row: code words are looked up two at a time, a lane joins the eight of its group, a warp scan of the
 //             lengths places them in a shared-memory image of the row (atomic OR), which leaves in one coalesced sweep
 //   unpack    one thread per row: a look-up on the next 10 (12) stream bits gives as many whole symbols as they hold
-// Bound by instruction issue, not by memory.  Measured at n = 100,000, d = 1536, b = 4 (76.8 MB of indices), before -> now:
-// measure 121 -> 33 us, offsets 83 (one CTA) -> 3, clearing the output 13 -> 0, pack 396 -> 112, unpack 471 -> 150.
+// Bound by instruction issue (pack: 71 % of the slots) and, in unpack (54 %), by the latency of a thread's chain of look-ups; not by
+// memory.  Measured at n = 100,000, d = 1536, b = 4 (76.8 MB of indices), before -> now: measure 121 -> 34 us, offsets 83 (one
+// CTA) -> 4, clearing the output 13 -> 1, pack 396 -> 113, unpack 471 -> 154.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
