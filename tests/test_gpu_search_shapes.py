@@ -77,3 +77,21 @@ def test_the_nearest_of_very_many_rows():
     codes = random_codes(su, n, 2)
     Q = torch.randn((64, 128), generator=torch.Generator().manual_seed(3)).to(DEV)
     assert search(su, Q, n, codes, 1)[2] < 2.0 * search(su, Q, n, codes, 10)[2]
+
+
+@pytest.mark.parametrize("nq", [1, 8, 24, 40])
+@pytest.mark.parametrize("good", [4, 15])
+def test_a_sample_that_misses_the_best_rows(nq, good):
+    """The sample is every 16th row here (66,049 rows, 4,096 of them).  The `good` rows that follow each of these score far higher,
+    so that the threshold admits them all: 16,512 candidates, more than a CTA's own list holds, or 61,921, more than the global
+    lists hold, which is the rescue pass."""
+    n, d, k = 66_049, 136, 64
+    su = P.Setup(d, 2, tq.TQ_MSE)
+    g = torch.Generator().manual_seed(nq)
+    X, Q = torch.randn((n, d), generator=g) + 2.0, torch.randn((nq, d), generator=g) + 2.0
+    at = torch.arange(n) % 16
+    X[~((at >= 1) & (at <= good))] *= 0.01
+    codes = su.quantize(X.to(DEV))
+    ts, ti, _ = search(su, Q.to(DEV), n, codes, k)
+    order = torch.sort(su.score(Q.to(DEV), n, *codes), dim=1, descending=True, stable=True)
+    assert torch.equal(ts, order.values[:, :k]) and torch.equal(ti.long(), order.indices[:, :k])
