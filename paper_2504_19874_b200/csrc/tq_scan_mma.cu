@@ -720,9 +720,9 @@ __global__ void __launch_bounds__(1024) select_kernel(SelArgs a) {
       for (int i0 = 0; i0 < total; i0 += 1024) f(i0 + tid < total ? scache[i0 + tid] : 0ull);
     } else {
 #pragma unroll 1
-      for (int base = 0; base < total; base += 8192) {   // eight loads in flight per thread: one SM reads the list
-        unsigned long long key[8];
-        fetch_keys(a, q, m_new, total, base, key);
+      for (unsigned base = 0; base < (unsigned)total; base += 8192) {   // eight loads in flight per thread: one SM reads the list
+        unsigned long long key[8];   // (unsigned: past the end of a list of nearly 2^31 entries the count must not turn negative)
+        fetch_keys(a, q, m_new, total, (int)base, key);
 #pragma unroll
         for (int u = 0; u < 8; ++u) f(key[u]);
       }

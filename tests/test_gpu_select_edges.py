@@ -60,3 +60,17 @@ def test_the_same_pair_given_twice(m):
         tq.tq_select_topk(cs, ci, k, ts, ti)
         ws, wi = expected(s, ids, k)
         assert np.array_equal(ti[0].cpu().numpy(), wi) and np.array_equal(ts[0].cpu().numpy(), ws)
+
+
+def test_the_longest_list():
+    """2^31 - 1 candidates: positions and the loop that counts them end at the largest 32-bit integer."""
+    m, k = 2**31 - 1, 10
+    if torch.cuda.mem_get_info()[0] < 24e9:
+        pytest.skip("needs 17 GB of device memory")
+    s, ids = torch.empty((1, m), device=DEV), torch.arange(m, dtype=torch.int32, device=DEV)[None]
+    s.uniform_(0.0, 1.0)
+    at = torch.tensor([m - 1, 0, m - 8192, 5, 8191, m // 2, m - 2, 2**30, 8192, m - 1025], device=DEV)
+    s[0, at] = torch.arange(20, 10, -1, device=DEV, dtype=torch.float32)
+    ts, ti = torch.empty((1, k), device=DEV), torch.empty((1, k), dtype=torch.int32, device=DEV)
+    tq.tq_select_topk(s, ids, k, ts, ti)
+    assert torch.equal(ti[0].long(), at) and ts[0].tolist() == list(range(20, 10, -1))
