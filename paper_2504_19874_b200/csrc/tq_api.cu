@@ -161,6 +161,37 @@ size_t ms_topk_fixed(const tq_plan* plan, int nq) {
   return ms_score_fixed(plan, nq) + 1024 /* tau, count, overflow */ + (size_t)pick_engine(plan, nq).qpp * kCandCap * 8;
 }
 
+// Top-k of more than kScreenFrom queries over at least kFilterMinN vectors: bounds of the estimates from one fp16 pass per 256
+// queries, exact estimates only for the rows that the bounds leave (tq_screen_tc.cu).
+constexpr int kScreenFrom = 192;
+bool screens(const tq_plan* plan, int nq, int64_t n) { return nq > kScreenFrom && n >= kFilterMinN && pick_engine(plan, nq).tc; }
+// Workspace of a screened pass, between the exact engine's operand and the dense score buffer.
+struct ScreenSpace {
+  size_t operand, tau, kth, count, left, flag, left_s, left_i, cand_s, cand_i, total;   // byte offsets
+};
+ScreenSpace screen_space(const tq_plan* plan) {
+  ScreenSpace s;
+  constexpr size_t Q = screen::kQueries;
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    const size_t here = at;
+    at += align_up(bytes, 256);
+    return here;
+  };
+  s.operand = take(screen::workspace_bytes(plan));
+  s.tau = take(Q * 4);
+  s.kth = take(Q * 4);
+  s.count = take(Q * 4);
+  s.left = take(Q * 4);
+  s.flag = take(4);
+  s.left_s = take(Q * screen::kSurvivors * 4);
+  s.left_i = take(Q * screen::kSurvivors * 4);
+  s.cand_s = take(Q * kCandCap * 4);
+  s.cand_i = take(Q * kCandCap * 4);
+  s.total = at;
+  return s;
+}
+
 template <typename T>
 cudaError_t launch_row_norm(const T* X, int64_t ld, int64_t n, int d, float* out, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
@@ -717,7 +748,7 @@ extern "C" size_t tq_workspace_bytes(const tq_plan* plan, int op, int64_t n, int
       return plan->ms.ok ? ms_score_fixed(plan, nq) : qcat_bytes(plan, nq);
     case TQ_OP_TOPK:
       if (plan->ms.ok)
-        return ms_topk_fixed(plan, nq) +
+        return ms_topk_fixed(plan, nq) + (screens(plan, nq, n) ? screen_space(plan).total : 0) +
                align_up((size_t)pick_engine(plan, nq).qpp *
                             std::max<int64_t>(std::min<int64_t>(n, pick_engine(plan, nq).dense_rows_pref), kDenseRowsMin) * sizeof(float),
                         256);
@@ -986,6 +1017,78 @@ extern "C" int tq_score_prepared(const tq_plan* plan, const void* prepared, int 
   return TQ_OK;
 }
 
+// Pilot rows m of a search for the k best of n: the pass over all rows then has n / m times as many candidates as the pilot has
+// scores down to the threshold, which are k where it meets the k-th best exactly.  That number varies like a sum of k
+// exponentials, so that at k = 1 the count is four times the expected one in one query of 55, and one overflow of a list of 32,768
+// has all rows scored again for the whole pass (k = 1, 64 queries, 34 * 10^6 rows, 8,192 expected: 28.3 ms instead of 5.5).
+// m = n (k + 8) / 8192 expects 910 at k = 1 and 7,585 at k = 100; a larger pilot costs a longer pilot scan and selection.
+static int64_t pilot_rows(int64_t n, int k, int64_t most) {
+  const int64_t m = std::max<int64_t>(round_up64((int64_t)((double)n * (k + 8) / 8192.0), 256), 4096);
+  return std::min<int64_t>(m, std::min<int64_t>(most / 256 * 256, n));
+}
+
+// Dense block flow over the queries of one pass: the whole job for small n, the guarded rescue of a filtered search otherwise.
+static int topk_dense(const ScanEngine& eng, int q0, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma,
+                      const float* norms, int k, float* ts, int32_t* ti, float* dense, int64_t dense_floats, const int* guard, void* msw,
+                      cudaStream_t st, const char* who) {
+  int rc;
+  const size_t xrb = eng.plan->idx_row_bytes, qrb = eng.plan->qjl_row_bytes;
+  int64_t block = std::min<int64_t>(dense_floats / eng.qpp, n);
+  if (block < n) block = block / 256 * 256;
+  for (int64_t v0 = 0; v0 < n; v0 += block) {
+    const int64_t cn = std::min(block, n - v0);
+    if ((rc = engine_run(eng, q0, nqp, cn, idx ? idx + (size_t)v0 * xrb : nullptr, qjl ? qjl + (size_t)v0 * qrb : nullptr,
+                         gamma ? gamma + v0 : nullptr, norms ? norms + v0 : nullptr, dense, block, nullptr, guard, msw, st, who)))
+      return rc;
+    TQ_CHECK_CUDA(mscan::select_topk(dense, nullptr, nullptr, (int)block, (int)cn, (int)v0, nqp, k, v0 > 0 ? 1 : 0, ts, ti,
+                                     nullptr, nullptr, guard, nullptr, nullptr, st), who);
+  }
+  return TQ_OK;
+}
+
+// Top-k of many queries by screening: per 256 queries lower bounds of a sample's estimates give a threshold that k rows reach, the
+// rows whose upper bounds reach it are listed, and those whose upper bounds reach the list's k-th lower bound are scored exactly.
+static int topk_screened(const ScanEngine& eng, const float* Qcat, int nq, int64_t n, const uint8_t* idx, const uint8_t* qjl,
+                         const float* gamma, const float* norms, int k, float* top_scores, int32_t* top_ids, char* ws, size_t ws_bytes,
+                         cudaStream_t st, const char* who) {
+  int rc;
+  const tq_plan* plan = eng.plan;
+  const ScreenSpace sp = screen_space(plan);
+  void* msw = ws;
+  char* p = ws + align_up(eng.ws_bytes, 256);
+  auto at = [&](size_t offset) { return static_cast<void*>(p + offset); };
+  float *tau = (float*)at(sp.tau), *kth = (float*)at(sp.kth), *cand_s = (float*)at(sp.cand_s), *left_s = (float*)at(sp.left_s);
+  int *count = (int*)at(sp.count), *left = (int*)at(sp.left), *flag = (int*)at(sp.flag), *cand_i = (int*)at(sp.cand_i),
+      *left_i = (int*)at(sp.left_i);
+  void* operand = at(sp.operand);
+  float* dense = (float*)at(sp.total);
+  const int64_t dense_floats = (int64_t)((ws + ws_bytes - reinterpret_cast<char*>(dense)) / sizeof(float));
+  const int64_t m = pilot_rows(n, k, dense_floats / screen::kQueries);
+  static_assert(screen::kQueries == kGroupQueries, "one exact operand per screened pass");
+  for (int q0 = 0; q0 < nq; q0 += screen::kQueries) {
+    const int nqp = std::min(screen::kQueries, nq - q0);
+    float* ts = top_scores + (size_t)q0 * k;
+    int32_t* ti = top_ids + (size_t)q0 * k;
+    if ((rc = engine_prepare(eng, Qcat, q0, nq, msw, st, who))) return rc;
+    if ((rc = screen::prepare(plan, Qcat + (size_t)q0 * plan->ncat * plan->dpad, nqp, operand, st, who))) return rc;
+    if ((rc = screen::run(plan, nqp, m, idx, qjl, gamma, norms, dense, m, nullptr, nullptr, nullptr, nullptr, 0, operand, st, who, n / m)))
+      return rc;
+    TQ_CHECK_CUDA(mscan::select_topk(dense, nullptr, nullptr, (int)m, (int)m, 0, nqp, k, 0, nullptr, nullptr, tau, nullptr, nullptr, count, flag, st), who);
+    if ((rc = screen::run(plan, nqp, n, idx, qjl, gamma, norms, nullptr, 0, tau, count, cand_s, cand_i, kCandCap, operand, st, who, 1)))
+      return rc;
+    TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count, kCandCap, 0, 0, nqp, k, 0, nullptr, nullptr, kth, flag, nullptr, nullptr, nullptr, st), who);
+    if ((rc = tscan::rescore(plan, nqp, idx, qjl, gamma, norms, msw, screen::query_terms(plan, operand), kth, count, cand_s, cand_i, kCandCap,
+                             left_s, left_i, left, flag, st, who)))
+      return rc;
+    TQ_CHECK_CUDA(mscan::select_topk(left_s, left_i, left, screen::kSurvivors, 0, 0, nqp, k, 0, ts, ti, nullptr, nullptr, nullptr, nullptr, nullptr, st), who);
+    for (int s = 0; s < nqp; s += eng.qpp)
+      if ((rc = topk_dense(eng, q0 + s, std::min(eng.qpp, nqp - s), n, idx, qjl, gamma, norms, k, ts + (size_t)s * k, ti + (size_t)s * k, dense,
+                           dense_floats, flag, msw, st, who)))
+        return rc;
+  }
+  return TQ_OK;
+}
+
 // Top-k through the tensor-path scan.  Large n: a pilot pass over a sample of the rows gives, per query,
 // the k-th best score among them -- a lower bound on the final k-th score -- and the full pass
 // keeps only (score, id) pairs at or above it; a final selection sorts the survivors.  Should a
@@ -996,6 +1099,10 @@ static int topk_ms(const tq_plan* plan, const float* Qcat, int nq, int64_t n, co
                    size_t ws_bytes, cudaStream_t st, const char* who) {
   int rc;
   const ScanEngine eng = pick_engine(plan, nq);
+  // (a workspace of the documented minimum has no room for the lists of 256 queries)
+  if (screens(plan, nq, n) &&
+      ws_bytes >= align_up(eng.ws_bytes, 256) + screen_space(plan).total + (size_t)kDenseRowsMin * screen::kQueries * sizeof(float))
+    return topk_screened(eng, Qcat, nq, n, idx, qjl, gamma, norms, k, top_scores, top_ids, ws, ws_bytes, st, who);
   void* msw = ws;
   char* p = ws + align_up(eng.ws_bytes, 256);
   float* tau = reinterpret_cast<float*>(p);          // [qpp] (qpp <= 64: 256 bytes)
@@ -1008,7 +1115,6 @@ static int topk_ms(const tq_plan* plan, const float* Qcat, int nq, int64_t n, co
   float* dense = reinterpret_cast<float*>(p);
   const int64_t dense_floats = (int64_t)((ws + ws_bytes - p) / sizeof(float));
   const int qpp = eng.qpp;
-  const size_t xrb = plan->idx_row_bytes, qrb = plan->qjl_row_bytes;
   for (int q0 = 0; q0 < nq; q0 += qpp) {
     const int nqp = std::min(qpp, nq - q0);
     float* ts = top_scores + (size_t)q0 * k;
@@ -1018,15 +1124,9 @@ static int topk_ms(const tq_plan* plan, const float* Qcat, int nq, int64_t n, co
     const bool use_filter = n >= kFilterMinN && dense_rows >= std::min<int64_t>(n, eng.dense_rows_pref);
     const int* guard = nullptr;
     if (use_filter) {
-      // Pilot rows m: the full pass then has n / m times as many candidates as the pilot has scores down to the threshold, which
-      // are k where it meets the k-th best exactly.  That number varies like a sum of k exponentials, so that at k = 1 the count
-      // is four times the expected one in one query of 55, and one overflow of a list of 32,768 has all rows scored again for
-      // the whole pass (k = 1, 64 queries, 34 * 10^6 rows, 8,192 expected: 28.3 ms instead of 5.5).  m = n (k + 8) / 8192 expects
-      // 910 at k = 1 and 7,585 at k = 100; a larger pilot costs a longer pilot scan and selection.
       // The rows are spread over the whole index: the first ones say nothing about the others where an index is stored by topic
       // or time (1,000 clusters in turn, 8 queries, k = 10, 10^6 rows: 607 us from the first 4,096 rows, 84 when shuffled).
-      int64_t m = std::max<int64_t>(round_up64((int64_t)((double)n * (k + 8) / 8192.0), 256), 4096);
-      m = std::min<int64_t>(m, std::min<int64_t>(dense_rows / 256 * 256, n));
+      const int64_t m = pilot_rows(n, k, dense_rows);
       if ((rc = engine_run(eng, q0, nqp, m, idx, qjl, gamma, norms, dense, m, nullptr, nullptr, msw, st, who, n / m))) return rc;
       TQ_CHECK_CUDA(mscan::select_topk(dense, nullptr, nullptr, (int)m, (int)m, 0, nqp, k, 0, nullptr, nullptr, tau, nullptr, nullptr, count, overflow, st), who);
       mscan::Filter f{tau, count, cand_s, cand_i, kCandCap};
@@ -1034,17 +1134,7 @@ static int topk_ms(const tq_plan* plan, const float* Qcat, int nq, int64_t n, co
       TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count, kCandCap, 0, 0, nqp, k, 0, ts, ti, nullptr, overflow, nullptr, nullptr, nullptr, st), who);
       guard = overflow;
     }
-    // dense block flow: the whole job for small n, the guarded rescue otherwise
-    int64_t block = std::min<int64_t>(dense_rows, n);
-    if (block < n) block = block / 256 * 256;
-    for (int64_t v0 = 0; v0 < n; v0 += block) {
-      const int64_t cn = std::min(block, n - v0);
-      if ((rc = engine_run(eng, q0, nqp, cn, idx ? idx + (size_t)v0 * xrb : nullptr, qjl ? qjl + (size_t)v0 * qrb : nullptr,
-                           gamma ? gamma + v0 : nullptr, norms ? norms + v0 : nullptr, dense, block, nullptr, guard, msw, st, who)))
-        return rc;
-      TQ_CHECK_CUDA(mscan::select_topk(dense, nullptr, nullptr, (int)block, (int)cn, (int)v0, nqp, k, v0 > 0 ? 1 : 0, ts, ti,
-                                       nullptr, nullptr, guard, nullptr, nullptr, st), who);
-    }
+    if ((rc = topk_dense(eng, q0, nqp, n, idx, qjl, gamma, norms, k, ts, ti, dense, dense_floats, guard, msw, st, who))) return rc;
   }
   return TQ_OK;
 }

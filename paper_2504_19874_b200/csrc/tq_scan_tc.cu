@@ -45,6 +45,7 @@
 #include "tq_nib_common.cuh"
 #include "tq_quantize_tc.h"
 #include "tq_scan_tc.h"
+#include "tq_screen_tc.h"
 #include "tq_tc.cuh"
 
 namespace tq {
@@ -141,6 +142,18 @@ __device__ inline Slot slot_a(const Geo& g, int kb, int wl, int bit) {
     return {P / 4, P % 4};
   }
   return {8 * (2 * kb + wl - 2) + bit / 4, 4 + (bit & 3)};
+}
+
+// The parity word of 32 three-bit codes, and the 3-subset parities of eight four-bit codes.
+__device__ __forceinline__ uint32_t parity3(uint32_t w0, uint32_t w1, uint32_t w2) {
+  const uint32_t p0 = w0 ^ __funnelshift_r(w0, w1, 1) ^ __funnelshift_r(w0, w1, 2);
+  const uint32_t p1 = w1 ^ __funnelshift_r(w1, w2, 1) ^ __funnelshift_r(w1, w2, 2);
+  const uint32_t p2 = w2 ^ (w2 >> 1) ^ (w2 >> 2);
+  return (p0 & 0x49249249u) | (p1 & 0x92492492u) | (p2 & 0x24924924u);
+}
+__device__ __forceinline__ uint32_t parities4(uint32_t x) {
+  const uint32_t M = 0x11111111u, s1 = x >> 1, s2 = x >> 2, s3 = x >> 3;
+  return ((x ^ s1 ^ s2) & M) | (((x ^ s1 ^ s3) & M) << 1) | (((x ^ s2 ^ s3) & M) << 2) | (((s1 ^ s2 ^ s3) & M) << 3);
 }
 
 // ------------------------------------------------------------------ per-query constants
@@ -652,17 +665,10 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__
         if (f >= nkb_total) return true;
         if (f < a.g.kba) {
           if (BM == 3) {
-            const uint32_t p0 = w[0] ^ __funnelshift_r(w[0], w[1], 1) ^ __funnelshift_r(w[0], w[1], 2);
-            const uint32_t p1 = w[1] ^ __funnelshift_r(w[1], w[2], 1) ^ __funnelshift_r(w[1], w[2], 2);
-            const uint32_t p2 = w[2] ^ (w[2] >> 1) ^ (w[2] >> 2);
-            w[3] = (p0 & 0x49249249u) | (p1 & 0x92492492u) | (p2 & 0x24924924u);
+            w[3] = parity3(w[0], w[1], w[2]);
           } else if (BM == 4) {
-            const uint32_t M = 0x11111111u;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-              const uint32_t x = w[i], s1 = x >> 1, s2 = x >> 2, s3 = x >> 3;
-              w[2 + i] = ((x ^ s1 ^ s2) & M) | (((x ^ s1 ^ s3) & M) << 1) | (((x ^ s2 ^ s3) & M) << 2) | (((s1 ^ s2 ^ s3) & M) << 3);
-            }
+            w[2] = parities4(w[0]);
+            w[3] = parities4(w[1]);
           }
         }
         // the row's 128 A bytes of this k-block: register 4 c + e = (word c / 2, bit 4 (c % 2) + e of every byte)
@@ -830,6 +836,142 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__
           a.cand_i[(int64_t)ql * a.cap + slot] = (int)e.y;
         }
       }
+    }
+  }
+}
+
+// ------------------------------------------------------------------ exact estimates of single rows
+// For the rows that a screening pass leaves: the same digit sums as the scan kernels, hence the same estimates, by byte dot
+// products on CUDA cores over the digit rows of B that the scan kernels read.
+struct RescoreArgs {
+  Geo g;
+  uint32_t hi_a, hi_b, lo_a, lo_b;
+  const QConst* qc;
+  const uint8_t* Ba;
+  const uint8_t* Bs;
+  const uint8_t* idx;
+  const uint8_t* qjl;
+  const float* gamma;
+  const float* norms;
+  float coef;
+  const screen::QueryTerms* terms;
+  const float* kth;        // lower bound of the k-th best estimate
+  const int* count;        // candidates: (lower bound, row)
+  const float* cand_s;
+  const int* cand_i;
+  int cap;
+  float* out_s;            // [queries][kSurvivors]
+  int* out_i;
+  int* out_count;
+  int* overflow;
+};
+
+__device__ __forceinline__ int dp4a_us(uint32_t a, uint32_t b, int c) {
+  int d;
+  asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+__device__ __forceinline__ int dp4a_ss(uint32_t a, uint32_t b, int c) {
+  int d;
+  asm("dp4a.s32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+
+// One CTA per query: candidates whose upper bound reaches the k-th lower bound, then a warp per row; lane = 32-bit word of a k-block.
+// Bound: latency of the gathers (the list's rows lie anywhere in the index); some 130 of 1,600 candidates are left for k = 100.
+constexpr int kRescoreThreads = 256;
+__global__ void __launch_bounds__(kRescoreThreads) rescore_kernel(const __grid_constant__ RescoreArgs a) {
+  __shared__ int ids[screen::kSurvivors];
+  __shared__ int s_n;
+  allow_successor();
+  if (threadIdx.x == 0) s_n = 0;
+  __syncthreads();
+  wait_for_predecessor();   // the lists are its output
+  const int q = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool signs = a.g.kbs > 0 || a.g.nib;
+  const int m = min(a.count[q], a.cap);
+  const float kth = a.kth[q], err = a.terms[q].err, unscale = a.terms[q].unscale;
+  for (int i = threadIdx.x; i < m; i += kRescoreThreads) {
+    const int id = a.cand_i[(int64_t)q * a.cap + i];
+    const screen::RowTerms t = screen::row_terms(a.norms ? __ldg(a.norms + id) : 1.f, signs ? __ldg(a.gamma + id) : 0.f);
+    const float high = a.cand_s[(int64_t)q * a.cap + i] + 2.f * t.rho * err * unscale;
+    if (!(high < kth)) {
+      const int s = atomicAdd(&s_n, 1);
+      if (s < screen::kSurvivors) ids[s] = id;
+    }
+  }
+  __syncthreads();
+  const int n = min(s_n, screen::kSurvivors);
+  if (threadIdx.x == 0) {
+    a.out_count[q] = n;
+    if (s_n > screen::kSurvivors) atomicExch(a.overflow, 1);
+  }
+  const QConst c = a.qc[q];
+  const int row0 = q / kQueriesPerPass * NCOL + q % kQueriesPerPass;
+  const size_t pa = (size_t)a.g.kba * KB_BYTES, psn = (size_t)a.g.kbs * KB_BYTES;
+  const uint8_t* ba = a.Ba + (size_t)row0 * pa + 4 * lane;
+  const uint8_t* bs = a.Bs + (size_t)row0 * psn + 4 * lane;
+  const uint32_t mask = 0x01010101u << (((lane >> 2) & 1) * 4 + (lane & 3));   // of register `lane` of a k-block of the bit streams
+  for (int s = warp; s < n; s += kRescoreThreads / 32) {
+    const int64_t row = ids[s];
+    int va[LIMBS] = {0, 0, 0}, vs[LIMBS] = {0, 0, 0};
+    const uint32_t* iw = reinterpret_cast<const uint32_t*>(a.idx + (size_t)row * a.g.idx_rb);
+    const uint32_t* qw = reinterpret_cast<const uint32_t*>(a.qjl + (size_t)row * a.g.qjl_rb);
+    if (a.g.nib) {
+      for (int b = 0; b < a.g.nblk; ++b) {
+        const bool second = b >= a.g.nbi;
+        const int word = 16 * (second ? b - a.g.nbi : b) + (lane >> 1);
+        const uint32_t x = word < (second ? a.g.wq : a.g.widx) ? __ldg((second ? qw : iw) + word) : 0u;
+        const uint32_t sl = (x & 0x77777777u) >> ((lane & 1) * 16);
+        const uint32_t h = prmt(a.hi_a, a.hi_b, sl), l = prmt(a.lo_a, a.lo_b, sl), z = x & ((lane & 1) ? 0x80808080u : 0x08080808u);
+        const uint8_t* bb = ba + (size_t)(3 * b) * KB_BYTES;
+#pragma unroll
+        for (int g = 0; g < LIMBS; ++g) {
+          const uint8_t* bd = bb + (size_t)g * kQueriesPerPass * pa;
+          va[g] = dp4a_ss(h, __ldg(reinterpret_cast<const uint32_t*>(bd)), va[g]);
+          va[g] = dp4a_us(l, __ldg(reinterpret_cast<const uint32_t*>(bd + KB_BYTES)), va[g]);
+          vs[g] = dp4a_us(z, __ldg(reinterpret_cast<const uint32_t*>(bd + 2 * KB_BYTES)), vs[g]);
+        }
+      }
+    } else {
+      const int wl = lane >> 3;   // the register's word of the k-block
+      auto word = [&](const uint32_t* w, int i, int words) -> uint32_t { return i < words ? __ldg(w + i) : 0u; };
+      for (int kb = 0; kb < a.g.kba; ++kb) {
+        uint32_t x;
+        if (a.g.bm <= 2) {
+          x = word(iw, 4 * kb + wl, a.g.widx);
+        } else if (a.g.bm == 3) {
+          const uint32_t w0 = word(iw, 3 * kb, a.g.widx), w1 = word(iw, 3 * kb + 1, a.g.widx), w2 = word(iw, 3 * kb + 2, a.g.widx);
+          x = wl == 0 ? w0 : wl == 1 ? w1 : wl == 2 ? w2 : parity3(w0, w1, w2);
+        } else {
+          const uint32_t w = word(iw, 2 * kb + (wl & 1), a.g.widx);
+          x = wl < 2 ? w : parities4(w);
+        }
+        x &= mask;
+#pragma unroll
+        for (int g = 0; g < LIMBS; ++g)
+          va[g] = dp4a_us(x, __ldg(reinterpret_cast<const uint32_t*>(ba + (size_t)g * kQueriesPerPass * pa + (size_t)kb * KB_BYTES)), va[g]);
+      }
+      for (int kb = 0; kb < a.g.kbs; ++kb) {
+        const uint32_t x = word(qw, 4 * kb + wl, a.g.wq) & mask;
+#pragma unroll
+        for (int g = 0; g < LIMBS; ++g)
+          vs[g] = dp4a_us(x, __ldg(reinterpret_cast<const uint32_t*>(bs + (size_t)g * kQueriesPerPass * psn + (size_t)kb * KB_BYTES)), vs[g]);
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < LIMBS; ++g) {
+      va[g] = __reduce_add_sync(0xffffffffu, va[g]);
+      vs[g] = __reduce_add_sync(0xffffffffu, vs[g]);
+    }
+    if (lane == 0) {   // the operations of estimates16
+      float av = 0.f, sv = 0.f;
+      if (a.g.bm > 0) av = fmaf((float)(((long long)va[2] * 256 + va[1]) * 256 + va[0]), c.sa, c.ca);
+      if (signs) sv = fmaf((float)(((long long)vs[2] * 256 + vs[1]) * 256 + vs[0]), c.ss, c.cs);
+      const float nu = a.norms != nullptr ? __ldg(a.norms + row) : 1.f, cg = __fmul_rn(a.coef, signs ? __ldg(a.gamma + row) : 0.f);
+      const float e = __fmul_rn(nu, fmaf(cg, sv, av));
+      a.out_s[(int64_t)q * screen::kSurvivors + s] = e;
+      a.out_i[(int64_t)q * screen::kSurvivors + s] = isnan(e) ? -1 : (int)row;   // a negative id is an empty slot
     }
   }
 }
@@ -1070,6 +1212,35 @@ int run_pass(const tq_plan* plan, int pass, int nqp, int64_t n, const uint8_t* i
   a.status = plan->d_status;
   if (wide) TQ_CHECK_CUDA(filter ? launch_wide<1>(g.bm, pairs, ma, ms, pa, ps, a, st) : launch_wide<0>(g.bm, pairs, ma, ms, pa, ps, a, st), who);
   else TQ_CHECK_CUDA(filter ? launch_bm<1>(g.bm, ma, ms, pa, ps, a, st) : launch_bm<0>(g.bm, ma, ms, pa, ps, a, st), who);
+  return TQ_OK;
+}
+
+int rescore(const tq_plan* plan, int nqp, const uint8_t* idx, const uint8_t* qjl, const float* gamma, const float* norms,
+            const void* workspace, const screen::QueryTerms* terms, const float* kth, const int* count, const float* cand_s,
+            const int* cand_i, int cap, float* out_s, int* out_i, int* out_count, int* overflow, cudaStream_t st, const char* who) {
+  RescoreArgs a;
+  a.g = make_geo(plan);
+  a.hi_a = plan->nb.hi_a; a.hi_b = plan->nb.hi_b; a.lo_a = plan->nb.lo_a; a.lo_b = plan->nb.lo_b;
+  a.qc = static_cast<const QConst*>(workspace);
+  a.Ba = static_cast<const uint8_t*>(workspace) + kConstBytes;
+  a.Bs = a.Ba + b_bytes(a.g, 0);
+  a.idx = idx;
+  a.qjl = qjl;
+  a.gamma = gamma;
+  a.norms = norms;
+  a.coef = plan->coef;
+  a.terms = terms;
+  a.kth = kth;
+  a.count = count;
+  a.cand_s = cand_s;
+  a.cand_i = cand_i;
+  a.cap = cap;
+  a.out_s = out_s;
+  a.out_i = out_i;
+  a.out_count = out_count;
+  a.overflow = overflow;
+  count_launches(1);
+  TQ_CHECK_CUDA(launch_dependent(rescore_kernel, dim3((unsigned)nqp), dim3(kRescoreThreads), 0, st, a), who);
   return TQ_OK;
 }
 

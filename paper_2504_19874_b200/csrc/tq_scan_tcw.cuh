@@ -364,17 +364,10 @@ scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant_
       auto emit = [&](uint32_t (&w)[4], int f) -> bool {
         if (f < a.g.kba) {
           if (BM == 3) {
-            const uint32_t p0 = w[0] ^ __funnelshift_r(w[0], w[1], 1) ^ __funnelshift_r(w[0], w[1], 2);
-            const uint32_t p1 = w[1] ^ __funnelshift_r(w[1], w[2], 1) ^ __funnelshift_r(w[1], w[2], 2);
-            const uint32_t p2 = w[2] ^ (w[2] >> 1) ^ (w[2] >> 2);
-            w[3] = (p0 & 0x49249249u) | (p1 & 0x92492492u) | (p2 & 0x24924924u);
+            w[3] = parity3(w[0], w[1], w[2]);
           } else if (BM == 4) {
-            const uint32_t M = 0x11111111u;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-              const uint32_t x = w[i], s1 = x >> 1, s2 = x >> 2, s3 = x >> 3;
-              w[2 + i] = ((x ^ s1 ^ s2) & M) | (((x ^ s1 ^ s3) & M) << 1) | (((x ^ s2 ^ s3) & M) << 2) | (((s1 ^ s2 ^ s3) & M) << 3);
-            }
+            w[2] = parities4(w[0]);
+            w[3] = parities4(w[1]);
           }
         }
         // register 4 c + e2 = (word c / 2, bit 4 (c % 2) + e2 of every byte)

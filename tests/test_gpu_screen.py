@@ -1,0 +1,58 @@
+"""Top-k of many queries: bounds from one fp16 pass decide which rows are scored, so the results are those of sorting the dense
+estimates, bit for bit."""
+import pytest
+import torch
+
+import paper_2504_19874_b200 as tq
+from tests import parity as P
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+NIB = tq.TQ_LAYOUT_NIBBLE
+
+
+def check(su, Q, n, codes, k):
+    nq = Q.shape[0]
+    ts, ti = torch.empty((nq, k), device=DEV), torch.empty((nq, k), dtype=torch.int32, device=DEV)
+    ws = torch.empty(tq.tq_workspace_bytes(su.plan, tq.TQ_OP_TOPK, n, nq, k), dtype=torch.uint8, device=DEV)
+    tq.tq_topk(su.plan, Q, n, *codes, k, ts, ti, ws)
+    tq.tq_plan_status(su.plan)
+    order = torch.sort(su.score(Q, n, *codes), dim=1, descending=True, stable=True)
+    assert torch.equal(ts, order.values[:, :k]) and torch.equal(ti.long(), order.indices[:, :k])
+
+
+# one to four bits with and without signs; d at the edges of K steps (16), k-blocks (64), row groups (128, 256) and of the nibble
+# layout's blocks; n and nq at the edges of the row tiles (256) and of the halves and passes (128, 256)
+@pytest.mark.parametrize("d,bits,mode,layout", [
+    (128, 1, tq.TQ_MSE, None), (257, 1, tq.TQ_PROD, None), (200, 2, tq.TQ_MSE, None), (384, 2, tq.TQ_PROD, None), (200, 3, tq.TQ_PROD, None),
+    (136, 3, tq.TQ_MSE, None), (130, 4, tq.TQ_MSE, None), (768, 4, tq.TQ_PROD, None), (200, 4, tq.TQ_PROD, NIB), (1000, 4, tq.TQ_PROD, NIB),
+    (1536, 4, tq.TQ_PROD, NIB), (3072, 2, tq.TQ_PROD, None)])
+@pytest.mark.parametrize("n,nq,k", [(65_536, 193, 100), (65_793, 513, 1)])
+def test_screened_search_is_the_dense_one(d, bits, mode, layout, n, nq, k):
+    su = P.Setup(d, bits, mode, layout=layout)
+    g = torch.Generator(device=DEV).manual_seed(d + nq)
+    X, Q = torch.randn((n, d), generator=g, device=DEV) + 0.3, torch.randn((nq, d), generator=g, device=DEV) + 0.3
+    check(su, Q, n, su.quantize(X), k)
+
+
+def test_rows_and_queries_that_the_bounds_do_not_cover():
+    """Norms and gammas outside what the fp16 operands hold, a query of zeros, one of very large and one of very small entries, and
+    rows that are all alike (more candidates than the lists hold: every row is scored)."""
+    n, d, nq, k = 65_600, 200, 200, 10
+    su = P.Setup(d, 3, tq.TQ_PROD)
+    g = torch.Generator(device=DEV).manual_seed(1)
+    X, Q = torch.randn((n, d), generator=g, device=DEV), torch.randn((nq, d), generator=g, device=DEV)
+    idx, qjl, gamma, norms = su.quantize(X)
+    norms[::1000] = 0.0
+    norms[7::5000] = 1e-30
+    norms[11::20000] = 1e27
+    norms[13::20000] = -3.0
+    gamma[17::5000] = 1e-7
+    gamma[19::20000] = 1e6
+    gamma[23::20000] = -2.0
+    Q[3] = 0.0
+    Q[5] *= 1e15
+    Q[9] *= 1e-25
+    check(su, Q, n, (idx, qjl, gamma, norms), k)
+    same = su.quantize(X[:1].expand(n, d).contiguous())
+    check(su, Q[:195], n, same, k)
