@@ -165,9 +165,11 @@ size_t ms_topk_fixed(const tq_plan* plan, int nq) {
 // queries, exact estimates only for the rows that the bounds leave (tq_screen_tc.cu).
 constexpr int kScreenFrom = 192;
 bool screens(const tq_plan* plan, int nq, int64_t n) { return nq > kScreenFrom && n >= kFilterMinN && pick_engine(plan, nq).tc; }
+// A query's list: 2,048 candidates are expected at most (screen_samples), and two CTAs of the selection fit an SM.
+constexpr int kScreenCap = 8192;
 // Workspace of a screened pass, between the exact engine's operand and the dense score buffer.
 struct ScreenSpace {
-  size_t operand, tau, kth, count, left, flag, left_s, left_i, cand_s, cand_i, total;   // byte offsets
+  size_t operand, tau, kth, count, count1, left, flag, left_s, left_i, cand_s, cand_i, total;   // byte offsets
 };
 ScreenSpace screen_space(const tq_plan* plan) {
   ScreenSpace s;
@@ -182,12 +184,13 @@ ScreenSpace screen_space(const tq_plan* plan) {
   s.tau = take(Q * 4);
   s.kth = take(Q * 4);
   s.count = take(Q * 4);
+  s.count1 = take(Q * 4);
   s.left = take(Q * 4);
-  s.flag = take(4);
+  s.flag = take(8);
   s.left_s = take(Q * screen::kSurvivors * 4);
   s.left_i = take(Q * screen::kSurvivors * 4);
-  s.cand_s = take(Q * kCandCap * 4);
-  s.cand_i = take(Q * kCandCap * 4);
+  s.cand_s = take(Q * kScreenCap * 4);
+  s.cand_i = take(Q * kScreenCap * 4);
   s.total = at;
   return s;
 }
@@ -1046,8 +1049,32 @@ static int topk_dense(const ScanEngine& eng, int q0, int nqp, int64_t n, const u
   return TQ_OK;
 }
 
-// Top-k of many queries by screening: per 256 queries lower bounds of a sample's estimates give a threshold that k rows reach, the
-// rows whose upper bounds reach it are listed, and those whose upper bounds reach the list's k-th lower bound are scored exactly.
+// Samples of a screened search: `dense` rows whose lower bounds are written out give a threshold that k rows reach, `first` rows (0:
+// none) are filtered with it and give the threshold of the pass over all rows.  That one then keeps k n / first candidates: a hit
+// costs its warp as much as testing 30 estimates, and with one sample of 13,312 of 10^6 rows (one hit in 132) the pass took
+// 939 us instead of 130.
+// The rows written out are among the first sample's, so that at least k of that one reach the threshold.
+struct ScreenSamples {
+  int64_t dense, dense_step, first, first_step;
+};
+static ScreenSamples screen_samples(int64_t n, int k, int64_t most) {
+  const double expect = 2048.0 / (k + 8);   // rows per sampled row that make a list of 2,048
+  const double dense0 = std::max(4096.0, 16.0 * (k + 8));
+  double first = std::max(std::sqrt((double)n * dense0), n / expect), dense = std::max(dense0, first / expect);
+  ScreenSamples s;
+  if ((double)n <= 16.0 * dense0 && n / dense0 <= expect) {
+    first = 0.0;
+    dense = dense0;
+  }
+  s.first = std::min<int64_t>(round_up64((int64_t)first, 256), n);
+  s.dense = std::min<int64_t>(round_up64((int64_t)dense, 256), std::min<int64_t>(most / 256 * 256, s.first > 0 ? s.first : n));
+  s.first_step = s.first > 0 ? n / s.first : 1;
+  s.dense_step = s.first > 0 ? s.first_step * (s.first / s.dense) : n / s.dense;
+  return s;
+}
+
+// Top-k of many queries by screening: lower bounds of samples' estimates give a threshold that k rows reach, the rows whose upper
+// bounds reach it are listed, and those whose upper bounds reach the list's k-th lower bound are scored exactly.
 static int topk_screened(const ScanEngine& eng, const float* Qcat, int nq, int64_t n, const uint8_t* idx, const uint8_t* qjl,
                          const float* gamma, const float* norms, int k, float* top_scores, int32_t* top_ids, char* ws, size_t ws_bytes,
                          cudaStream_t st, const char* who) {
@@ -1058,12 +1085,12 @@ static int topk_screened(const ScanEngine& eng, const float* Qcat, int nq, int64
   char* p = ws + align_up(eng.ws_bytes, 256);
   auto at = [&](size_t offset) { return static_cast<void*>(p + offset); };
   float *tau = (float*)at(sp.tau), *kth = (float*)at(sp.kth), *cand_s = (float*)at(sp.cand_s), *left_s = (float*)at(sp.left_s);
-  int *count = (int*)at(sp.count), *left = (int*)at(sp.left), *flag = (int*)at(sp.flag), *cand_i = (int*)at(sp.cand_i),
-      *left_i = (int*)at(sp.left_i);
+  int *count = (int*)at(sp.count), *count1 = (int*)at(sp.count1), *left = (int*)at(sp.left), *flag = (int*)at(sp.flag),
+      *cand_i = (int*)at(sp.cand_i), *left_i = (int*)at(sp.left_i);
   void* operand = at(sp.operand);
   float* dense = (float*)at(sp.total);
   const int64_t dense_floats = (int64_t)((ws + ws_bytes - reinterpret_cast<char*>(dense)) / sizeof(float));
-  const int64_t m = pilot_rows(n, k, dense_floats / screen::kQueries);
+  const ScreenSamples sm = screen_samples(n, k, dense_floats / screen::kQueries);
   static_assert(screen::kQueries == kGroupQueries, "one exact operand per screened pass");
   for (int q0 = 0; q0 < nq; q0 += screen::kQueries) {
     const int nqp = std::min(screen::kQueries, nq - q0);
@@ -1071,13 +1098,22 @@ static int topk_screened(const ScanEngine& eng, const float* Qcat, int nq, int64
     int32_t* ti = top_ids + (size_t)q0 * k;
     if ((rc = engine_prepare(eng, Qcat, q0, nq, msw, st, who))) return rc;
     if ((rc = screen::prepare(plan, Qcat + (size_t)q0 * plan->ncat * plan->dpad, nqp, operand, st, who))) return rc;
-    if ((rc = screen::run(plan, nqp, m, idx, qjl, gamma, norms, dense, m, nullptr, nullptr, nullptr, nullptr, 0, operand, st, who, n / m)))
+    auto filter = [&](int64_t rows, int64_t step, int* counts) {
+      return screen::run(plan, nqp, rows, idx, qjl, gamma, norms, nullptr, 0, tau, counts, cand_s, cand_i, kScreenCap, operand, st, who, step);
+    };
+    int* unused = flag + 1;
+    if ((rc = screen::run(plan, nqp, sm.dense, idx, qjl, gamma, norms, dense, sm.dense, nullptr, nullptr, nullptr, nullptr, 0, operand, st, who,
+                          sm.dense_step)))
       return rc;
-    TQ_CHECK_CUDA(mscan::select_topk(dense, nullptr, nullptr, (int)m, (int)m, 0, nqp, k, 0, nullptr, nullptr, tau, nullptr, nullptr, count, flag, st), who);
-    if ((rc = screen::run(plan, nqp, n, idx, qjl, gamma, norms, nullptr, 0, tau, count, cand_s, cand_i, kCandCap, operand, st, who, 1)))
-      return rc;
-    TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count, kCandCap, 0, 0, nqp, k, 0, nullptr, nullptr, kth, flag, nullptr, nullptr, nullptr, st), who);
-    if ((rc = tscan::rescore(plan, nqp, idx, qjl, gamma, norms, msw, screen::query_terms(plan, operand), kth, count, cand_s, cand_i, kCandCap,
+    TQ_CHECK_CUDA(mscan::select_topk(dense, nullptr, nullptr, (int)sm.dense, (int)sm.dense, 0, nqp, k, 0, nullptr, nullptr, tau, nullptr, nullptr,
+                                     sm.first > 0 ? count1 : count, sm.first > 0 ? unused : flag, st), who);
+    if (sm.first > 0) {   // (a list that is too short here still gives a threshold that k rows reach)
+      if ((rc = filter(sm.first, sm.first_step, count1))) return rc;
+      TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count1, kScreenCap, 0, 0, nqp, k, 0, nullptr, nullptr, tau, nullptr, nullptr, count, flag, st), who);
+    }
+    if ((rc = filter(n, 1, count))) return rc;
+    TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count, kScreenCap, 0, 0, nqp, k, 0, nullptr, nullptr, kth, flag, nullptr, nullptr, nullptr, st), who);
+    if ((rc = tscan::rescore(plan, nqp, idx, qjl, gamma, norms, msw, screen::query_terms(plan, operand), kth, count, cand_s, cand_i, kScreenCap,
                              left_s, left_i, left, flag, st, who)))
       return rc;
     TQ_CHECK_CUDA(mscan::select_topk(left_s, left_i, left, screen::kSurvivors, 0, 0, nqp, k, 0, ts, ti, nullptr, nullptr, nullptr, nullptr, nullptr, st), who);

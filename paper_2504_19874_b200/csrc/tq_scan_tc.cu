@@ -879,8 +879,8 @@ __device__ __forceinline__ int dp4a_ss(uint32_t a, uint32_t b, int c) {
 
 // One CTA per query: candidates whose upper bound reaches the k-th lower bound, then a warp per row; lane = 32-bit word of a k-block.
 // Bound: latency of the gathers (the list's rows lie anywhere in the index); some 130 of 1,600 candidates are left for k = 100.
-constexpr int kRescoreThreads = 256;
-__global__ void __launch_bounds__(kRescoreThreads) rescore_kernel(const __grid_constant__ RescoreArgs a) {
+constexpr int kRescoreThreads = 512;
+__global__ void __launch_bounds__(kRescoreThreads, 2) rescore_kernel(const __grid_constant__ RescoreArgs a) {
   __shared__ int ids[screen::kSurvivors];
   __shared__ int s_n;
   allow_successor();
