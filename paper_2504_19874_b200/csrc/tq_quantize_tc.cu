@@ -12,9 +12,11 @@
 // cluster per tile of 256 rows (tcgen05 cta_group::2), which halves what every SM reads of B from shared memory.  The
 // tiles are up to 256 columns wide; few rows take narrower ones, so that every SM has one (pick_tile).
 #include <atomic>
+#include <cfloat>
 #include <cstdlib>
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "tq_quantize_tc.h"
 #include "tq_tc.cuh"
@@ -46,6 +48,10 @@ struct Cfg {
   static constexpr int kAccCols = BN == 192 ? 256 : BN;                     // TMEM columns from one accumulator to the next
   static constexpr int kTmemCols = 2 * kAccCols;                            // two accumulators
   static constexpr int kStoreBytes = 4 * kEps * 2048;  // MODE 1: one [32 rows x 64 B] box per epilogue warp, staged for a TMA store
+  // bf16 rows have one limb: smaller stages, more of them in the same bytes
+  static constexpr int kStageBytes1 = kStageBytes - BM * BK * 2;
+  static constexpr int kStages1 = kStages * kStageBytes / kStageBytes1;
+  static_assert((2 * kStages1 + 4) * 8 + 8 <= 192, "barriers");
   static constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 512 /*barriers, centroids*/ + kStoreBytes;
 };
 
@@ -65,7 +71,8 @@ struct GemmArgs {
   float* gamma;          // MODE 2
   int parts;
   int64_t Mpad;
-  const float* nu;       // MODE 1: per-row norm (row with nu == 0 has residual 0); nullable
+  const float* nu;       // per-row norm (MODE 1: a row with nu == 0 has residual 0; one_limb: see RowScale); nullable
+  int one_limb;          // MODE 0, 1: the rows came in bf16, A is one limb of x 2^-e: two MMA passes, the accumulators are scaled
   // TQ_LAYOUT_NIBBLE (BITS = 3 with MODE 1, and MODE 2): the codes of 32 coordinates are four words of the combined
   // row [idx row | qjl row], nibble = index | sign << 3.  MODE 1 writes them with the sign bits clear, MODE 2 ORs
   // the sign bits in.
@@ -87,6 +94,18 @@ struct GemmArgs {
   size_t nib_idx_rb, nib_qjl_rb;
   int* status;
 };
+
+// Rows of bf16 enter the rotation as they are but for a power of two, exactly: A = x down with |A| in [1, 2), and y = back * acc.
+// (u = x / nu takes two limbs, that is a third MMA pass and half again the preparation: 1,001 rows of d = 3072, prod b = 2, took
+// 118 us, 96 with one limb.)  A zero row, and one whose norm is not finite, becomes what x times 0 is.
+struct RowScale {
+  float down, back;
+};
+__device__ __forceinline__ RowScale row_scale(float nu) {
+  if (!(nu > 0.f) || !(nu <= FLT_MAX)) return {0.f, 0.f};
+  const float down = ldexpf(1.f, -max(-126, min(126, ilogbf(nu))));
+  return {down, 1.f / (nu * down)};
+}
 
 // Bit i of the low byte of x at bit 4 i + 3.
 __device__ __forceinline__ uint32_t spread_to_nibble_tops(uint32_t x) {
@@ -203,35 +222,28 @@ __host__ __device__ __forceinline__ bool vec_rows(const float* X, int64_t ldx, i
 }
 
 // One warp per row: nu = ||x|| (optional), u = x / nu, u = hi + lo in bf16.  Rows warp, warp + nwarps, ...
-template <typename T, bool NORMALIZE>
-__device__ __forceinline__ void split_rows(const T* __restrict__ X, int64_t ldx, int64_t n, int d, int dpad,
+template <bool NORMALIZE>
+__device__ __forceinline__ void split_rows(const float* __restrict__ X, int64_t ldx, int64_t n, int d, int dpad,
                                            __nv_bfloat16* __restrict__ L1, __nv_bfloat16* __restrict__ L2,
                                            float* __restrict__ norms, int64_t warp, int64_t nwarps, int lane) {
-  if constexpr (sizeof(T) == 4) {
-    if (vec_rows(X, ldx, d, dpad)) {
-      if (d <= 256) split_rows_vec<NORMALIZE, 2>(X, ldx, n, d, dpad, L1, L2, norms, warp, nwarps, lane);
-      else if (d <= 512) split_rows_vec<NORMALIZE, 4>(X, ldx, n, d, dpad, L1, L2, norms, warp, nwarps, lane);
-      else if (d <= 1024) split_rows_vec<NORMALIZE, 8>(X, ldx, n, d, dpad, L1, L2, norms, warp, nwarps, lane);
-      else split_rows_vec<NORMALIZE, 16>(X, ldx, n, d, dpad, L1, L2, norms, warp, nwarps, lane);
-      return;
-    }
+  if (vec_rows(X, ldx, d, dpad)) {
+    if (d <= 256) split_rows_vec<NORMALIZE, 2>(X, ldx, n, d, dpad, L1, L2, norms, warp, nwarps, lane);
+    else if (d <= 512) split_rows_vec<NORMALIZE, 4>(X, ldx, n, d, dpad, L1, L2, norms, warp, nwarps, lane);
+    else if (d <= 1024) split_rows_vec<NORMALIZE, 8>(X, ldx, n, d, dpad, L1, L2, norms, warp, nwarps, lane);
+    else split_rows_vec<NORMALIZE, 16>(X, ldx, n, d, dpad, L1, L2, norms, warp, nwarps, lane);
+    return;
   }
-  // Other rows: a lane adds its squares over j = lane, lane + 32, ... with sixteen loads in flight (one load at a time took
-  // 11.7 us for 1,001 rows of 3,072 bf16), then converts eight neighbouring elements at a time (one 16-byte load where bf16 rows
-  // are aligned).
-  const bool vec8 = sizeof(T) == 2 && (ldx & 7) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
-  auto value = [](T v) -> float {
-    if constexpr (sizeof(T) == 4) return v; else return __bfloat162float(v);
-  };
+  // Other rows: a lane adds its squares over j = lane, lane + 32, ... with sixteen loads in flight, then converts eight
+  // neighbouring elements at a time.
   for (int64_t r = warp; r < n; r += nwarps) {
-    const T* row = X + r * ldx;
+    const float* row = X + r * ldx;
     float inv = 1.f;
     if (NORMALIZE) {
       float s = 0.f;
       for (int j0 = lane; j0 < d; j0 += 512) {
         float v[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = j0 + 32 * i < d ? value(row[j0 + 32 * i]) : 0.f;
+        for (int i = 0; i < 16; ++i) v[i] = j0 + 32 * i < d ? row[j0 + 32 * i] : 0.f;
 #pragma unroll
         for (int i = 0; i < 16; ++i) s = fmaf(v[i], v[i], s);
       }
@@ -244,18 +256,8 @@ __device__ __forceinline__ void split_rows(const T* __restrict__ X, int64_t ldx,
 #pragma unroll 2
     for (int j0 = lane * 8; j0 < dpad; j0 += 256) {
       float u[8];
-      if (vec8 && j0 + 8 <= d) {
-        const uint4 raw = *reinterpret_cast<const uint4*>(row + j0);
-        const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-          u[2 * p] = __uint_as_float(w[p] << 16);
-          u[2 * p + 1] = __uint_as_float(w[p] & 0xffff0000u);
-        }
-      } else {
-#pragma unroll
-        for (int p = 0; p < 8; ++p) u[p] = j0 + p < d ? value(row[j0 + p]) : 0.f;
-      }
+      for (int p = 0; p < 8; ++p) u[p] = j0 + p < d ? row[j0 + p] : 0.f;
       uint32_t h[4], l[4];
 #pragma unroll
       for (int p = 0; p < 4; ++p) {
@@ -271,14 +273,82 @@ __device__ __forceinline__ void split_rows(const T* __restrict__ X, int64_t ldx,
   }
 }
 
-template <typename T, bool NORMALIZE>
-__global__ void __launch_bounds__(256) split_rows_kernel(const T* __restrict__ X, int64_t ldx, int64_t n, int d, int dpad,
+template <bool NORMALIZE>
+__global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict__ X, int64_t ldx, int64_t n, int d, int dpad,
                                                          __nv_bfloat16* __restrict__ L1, __nv_bfloat16* __restrict__ L2,
                                                          float* __restrict__ norms) {
   allow_successor();        // (every kernel behind waits for this one, and so for those ahead of it, before it writes or reads)
   wait_for_predecessor();   // it may write X, or read the limb buffers
-  split_rows<T, NORMALIZE>(X, ldx, n, d, dpad, L1, L2, norms, (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5),
-                           (int64_t)gridDim.x * (blockDim.x >> 5), threadIdx.x & 31);
+  split_rows<NORMALIZE>(X, ldx, n, d, dpad, L1, L2, norms, (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5),
+                        (int64_t)gridDim.x * (blockDim.x >> 5), threadIdx.x & 31);
+}
+
+// Rows of bf16, one warp per row: nu = ||x|| (optional) and the row's only limb.  Bound: HBM, 4 bytes per element (6 with the two
+// limbs of x / nu).  Rows of at most 256 NV elements stay in registers between the two, all their loads in flight at once; longer
+// rows are read a second time.  VEC: 16-byte loads (rows on the 16-byte grid).
+template <int NV, bool VEC>
+__global__ void __launch_bounds__(256) scale_rows_kernel(const __nv_bfloat16* __restrict__ X, int64_t ldx, int64_t n, int d, int dpad,
+                                                         __nv_bfloat16* __restrict__ L1, float* __restrict__ norms) {
+  allow_successor();
+  wait_for_predecessor();   // it may write X, or read the limb buffer
+  const int lane = threadIdx.x & 31;
+  const int nseg = (dpad + 256 * NV - 1) / (256 * NV);
+  for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n; r += (int64_t)gridDim.x * (blockDim.x >> 5)) {
+    const __nv_bfloat16* row = X + r * ldx;
+    uint4 v[NV];
+    auto load_seg = [&](int seg) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const int j = (seg * NV + i) * 256 + lane * 8;
+        if (VEC && j + 8 <= d) {
+          v[i] = __ldg(reinterpret_cast<const uint4*>(row + j));
+        } else {
+          uint32_t w[4];
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            const uint32_t lo = j + 2 * p < d ? __bfloat16_as_ushort(row[j + 2 * p]) : 0u;
+            const uint32_t hi = j + 2 * p + 1 < d ? __bfloat16_as_ushort(row[j + 2 * p + 1]) : 0u;
+            w[p] = lo | (hi << 16);
+          }
+          v[i] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+      }
+    };
+    auto low = [](uint32_t w) { return __uint_as_float(w << 16); };
+    auto high = [](uint32_t w) { return __uint_as_float(w & 0xffff0000u); };
+    float down = 1.f;
+    load_seg(0);
+    if (norms != nullptr) {
+      float s = 0.f;
+      for (int seg = 0; seg < nseg; ++seg) {
+        if (seg > 0) load_seg(seg);
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+          const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+          for (int p = 0; p < 4; ++p) s = fmaf(low(w[p]), low(w[p]), fmaf(high(w[p]), high(w[p]), s));
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      const float nu = sqrtf(s);
+      down = row_scale(nu).down;
+      if (lane == 0) norms[r] = nu;
+    }
+    for (int seg = 0; seg < nseg; ++seg) {
+      if (nseg > 1 && (seg > 0 || norms != nullptr)) load_seg(seg);   // registers hold the last segment read
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const int j = (seg * NV + i) * 256 + lane * 8;
+        if (j >= dpad) continue;
+        const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+        uint32_t o[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) o[p] = pack_bf16x2(low(w[p]) * down, high(w[p]) * down);
+        *reinterpret_cast<uint4*>(L1 + r * dpad + j) = make_uint4(o[0], o[1], o[2], o[3]);
+      }
+    }
+  }
 }
 
 // MODE 0: idx.  MODE 1: idx + residual limbs + partial ||e||^2.  MODE 2: sign bits.
@@ -293,16 +363,19 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
   const int64_t unit = blockIdx.x / CTAS, nunits = gridDim.x / CTAS;   // a unit = one CTA or one pair
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const bool one = MODE != 2 && a.one_limb != 0;                       // A has one limb
+  const int stages = one ? C::kStages1 : C::kStages, stage_bytes = one ? C::kStageBytes1 : C::kStageBytes;
+  const int b_off = one ? BM * BK * 2 : 2 * BM * BK * 2;               // B's limbs in a stage
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kStages * C::kStageBytes);
-  uint64_t* full = bars;                    // [kStages]  TMA -> MMA
-  uint64_t* empty = bars + C::kStages;      // [kStages]  MMA -> TMA
-  uint64_t* tfull = bars + 2 * C::kStages;  // [2]        MMA -> epilogue
+  uint64_t* full = bars;                    // [stages]   TMA -> MMA
+  uint64_t* empty = bars + stages;          // [stages]   MMA -> TMA
+  uint64_t* tfull = bars + 2 * stages;      // [2]        MMA -> epilogue
   uint64_t* tempty = tfull + 2;             // [2]        epilogue -> MMA
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   // the centroids in shared memory: indexed by the code they are one wavefront per load, where the same index into
   // the kernel's constant arguments is replayed once per distinct code of the warp
-  float* cs = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(bars) + 128);   // [16]
+  float* cs = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(bars) + 192);   // [16]
   unsigned char* stg = reinterpret_cast<unsigned char*>(bars) + 512;                    // [4 EPS][2048], 512-byte aligned
   if (MODE == 1 && threadIdx.x < 16) cs[threadIdx.x] = a.cb.c[threadIdx.x];
 
@@ -311,7 +384,7 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
   const int64_t num_tiles = (int64_t)a.tiles_m * a.tiles_n;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < C::kStages; ++s) {
+    for (int s = 0; s < stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -348,22 +421,22 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
         const int m0 = ((int)(t / a.tiles_n) * CTAS + rank) * BM, n0 = (int)(t % a.tiles_n) * BN + rank * C::kBRows;
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!(ok = mbar_wait(&empty[stage], phase ^ 1u, abort_flag, a.status))) break;
-          unsigned char* sa = smem + stage * C::kStageBytes;
+          unsigned char* sa = smem + stage * stage_bytes;
           if (CTAS == 2) {
             // both CTAs' bytes are counted on the leader's barrier, which the leader arms for both
-            if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * C::kStageBytes);
+            if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * stage_bytes);
             tma_load_2d_pair(sa, &tmA1, &full[stage], kb * BK, m0);
-            tma_load_2d_pair(sa + BM * BK * 2, &tmA2, &full[stage], kb * BK, m0);
-            tma_load_2d_pair(sa + 2 * BM * BK * 2, &tmB1, &full[stage], kb * BK, n0);
-            tma_load_2d_pair(sa + 2 * BM * BK * 2 + C::kBRows * BK * 2, &tmB2, &full[stage], kb * BK, n0);
+            if (!one) tma_load_2d_pair(sa + BM * BK * 2, &tmA2, &full[stage], kb * BK, m0);
+            tma_load_2d_pair(sa + b_off, &tmB1, &full[stage], kb * BK, n0);
+            tma_load_2d_pair(sa + b_off + C::kBRows * BK * 2, &tmB2, &full[stage], kb * BK, n0);
           } else {
-            mbar_arrive_expect_tx(&full[stage], C::kStageBytes);
+            mbar_arrive_expect_tx(&full[stage], stage_bytes);
             tma_load_2d(sa, &tmA1, &full[stage], kb * BK, m0);
-            tma_load_2d(sa + BM * BK * 2, &tmA2, &full[stage], kb * BK, m0);
-            tma_load_2d(sa + 2 * BM * BK * 2, &tmB1, &full[stage], kb * BK, n0);
-            tma_load_2d(sa + 2 * BM * BK * 2 + BN * BK * 2, &tmB2, &full[stage], kb * BK, n0);
+            if (!one) tma_load_2d(sa + BM * BK * 2, &tmA2, &full[stage], kb * BK, m0);
+            tma_load_2d(sa + b_off, &tmB1, &full[stage], kb * BK, n0);
+            tma_load_2d(sa + b_off + BN * BK * 2, &tmB2, &full[stage], kb * BK, n0);
           }
-          if (++stage == C::kStages) {
+          if (++stage == stages) {
             stage = 0;
             phase ^= 1u;
           }
@@ -391,27 +464,27 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!(ok = mbar_wait(&full[stage], phase, abort_flag, a.status))) break;
           tc_fence_after();
-          const uint32_t sa = smem_u32(smem + stage * C::kStageBytes);
+          const uint32_t sa = smem_u32(smem + stage * stage_bytes);
           const uint64_t a1 = smem_desc_sw128(sa), a2 = smem_desc_sw128(sa + BM * BK * 2);
-          const uint64_t b1 = smem_desc_sw128(sa + 2 * BM * BK * 2);
-          const uint64_t b2 = smem_desc_sw128(sa + 2 * BM * BK * 2 + C::kBRows * BK * 2);
+          const uint64_t b1 = smem_desc_sw128(sa + b_off);
+          const uint64_t b2 = smem_desc_sw128(sa + b_off + C::kBRows * BK * 2);
 #pragma unroll
           for (int k = 0; k < BK / UMMA_K; ++k) {
             const uint64_t off = (uint64_t)((k * UMMA_K * 2) >> 4);   // 32 bytes per K step
             if (CTAS == 2) {
               umma_bf16_pair(d_tmem, a1 + off, b2 + off, idesc, (kb | k) != 0 ? 1u : 0u);   // hi * lo
-              umma_bf16_pair(d_tmem, a2 + off, b1 + off, idesc, 1u);                        // lo * hi
+              if (!one) umma_bf16_pair(d_tmem, a2 + off, b1 + off, idesc, 1u);              // lo * hi
               umma_bf16_pair(d_tmem, a1 + off, b1 + off, idesc, 1u);                        // hi * hi
             } else {
               umma_bf16(d_tmem, a1 + off, b2 + off, idesc, (kb | k) != 0 ? 1u : 0u);
-              umma_bf16(d_tmem, a2 + off, b1 + off, idesc, 1u);
+              if (!one) umma_bf16(d_tmem, a2 + off, b1 + off, idesc, 1u);
               umma_bf16(d_tmem, a1 + off, b1 + off, idesc, 1u);
             }
           }
           // frees the stage (in both CTAs of a pair) once these MMAs have read it
           if (CTAS == 2) umma_commit_pair(&empty[stage]);
           else umma_commit(&empty[stage]);
-          if (++stage == C::kStages) {
+          if (++stage == stages) {
             stage = 0;
             phase ^= 1u;
           }
@@ -444,8 +517,8 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
       const GemmArgs::SplitTask& t = a.split;
       if (t.rows > 0) {
         const int64_t sw = (int64_t)blockIdx.x * NSPLIT + (warp - 2 - 4 * EPS), nsw = (int64_t)gridDim.x * NSPLIT;
-        if (t.normalize) split_rows<float, true>(t.X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
-        else split_rows<float, false>(t.X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
+        if (t.normalize) split_rows<true>(t.X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
+        else split_rows<false>(t.X, t.ldx, t.rows, t.d, t.dpad, t.L1, t.L2, t.norms, sw, nsw, lane);
       }
     }
   } else {
@@ -463,7 +536,12 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
       tc_fence_after();
       const bool row_ok = row < a.M;
       bool zero_row = false;
-      if (MODE == 1 && a.nu != nullptr && row_ok) zero_row = (__ldg(a.nu + row) == 0.f);
+      float back = 1.f;
+      if (MODE != 2 && a.nu != nullptr && row_ok) {
+        const float nu = __ldg(a.nu + row);
+        zero_row = nu == 0.f;
+        if (one) back = row_scale(nu).back;
+      }
       float gsum = 0.f;
       uint32_t* out_row = reinterpret_cast<uint32_t*>(a.out + (size_t)(row_ok ? row : 0) * a.out_rb);
       const size_t row_words = a.out_rb / 4;
@@ -510,7 +588,7 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
               const int i = 2 * i2 + q;
-              const float y = __uint_as_float(v[i]);
+              const float y = __uint_as_float(v[i]) * back;
               const bool col_ok = (col0 + i < a.N);
               int code = 0;
 #pragma unroll
@@ -806,7 +884,7 @@ cudaError_t build_matrix_limbs(const float* dM, int rows, int d, int dpad, Matri
   e = cudaMalloc(&out->lo, bytes);
   if (e != cudaSuccess) return e;
   const int blocks = std::min((rows + 7) / 8, sm_count() * 8);
-  split_rows_kernel<float, false><<<blocks, 256>>>(dM, d, rows, d, dpad, out->hi, out->lo, nullptr);
+  split_rows_kernel<false><<<blocks, 256>>>(dM, d, rows, d, dpad, out->hi, out->lo, nullptr);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   for (int i = 0; i < kBoxes; ++i)
@@ -918,15 +996,24 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
     // A grid of more than one wave is launched plainly: as a programmatic dependent its first blocks settle wherever the kernel
     // ahead drains first, and the uneven rest costs more than the launch gap saves (200,000 rows of d = 200: 135 us a call, 123
     // plain).
-    auto go = [&](auto kern, auto* x) -> cudaError_t {
-      if (blocks <= 2 * sm_count()) return launch_dependent(kern, dim3((unsigned)blocks), dim3(256), 0, s, x, ldx, rows, d, dpad, L1, L2, nu_out);
-      kern<<<blocks, 256, 0, s>>>(x, ldx, rows, d, dpad, L1, L2, nu_out);
+    auto go = [&](auto kern, auto... args) -> cudaError_t {
+      if (blocks <= 2 * sm_count()) return launch_dependent(kern, dim3((unsigned)blocks), dim3(256), 0, s, args...);
+      kern<<<blocks, 256, 0, s>>>(args...);
       return cudaGetLastError();
     };
-    const float* xf = static_cast<const float*>(Xc);
-    const __nv_bfloat16* xb = static_cast<const __nv_bfloat16*>(Xc);
-    const cudaError_t e = x_dtype == TQ_F32 ? (norms ? go(split_rows_kernel<float, true>, xf) : go(split_rows_kernel<float, false>, xf))
-                                            : (norms ? go(split_rows_kernel<__nv_bfloat16, true>, xb) : go(split_rows_kernel<__nv_bfloat16, false>, xb));
+    cudaError_t e;
+    if (x_dtype == TQ_F32) {
+      const float* x = static_cast<const float*>(Xc);
+      e = norms ? go(split_rows_kernel<true>, x, ldx, rows, d, dpad, L1, L2, nu_out) : go(split_rows_kernel<false>, x, ldx, rows, d, dpad, L1, L2, nu_out);
+    } else {
+      const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(Xc);
+      const bool vec = ldx % 8 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
+      auto pick = [&](auto nv) {
+        constexpr int NV = decltype(nv)::value;
+        return vec ? go(scale_rows_kernel<NV, true>, x, ldx, rows, d, dpad, L1, nu_out) : go(scale_rows_kernel<NV, false>, x, ldx, rows, d, dpad, L1, nu_out);
+      };
+      e = d <= 256 ? pick(std::integral_constant<int, 1>()) : d <= 1024 ? pick(std::integral_constant<int, 4>()) : pick(std::integral_constant<int, 12>());
+    }
     count_launches(1);
     return e;
   };
@@ -977,6 +1064,7 @@ int quantize(const tq_plan* plan, const void* X, int x_dtype, int64_t n, int64_t
     g.parts = d <= 128 ? 4 : (d + 63) / 64;   // per epilogue warp: 32 columns of a tile that is the whole row, else 64
     g.Mpad = R;
     g.nu = nu_out;
+    g.one_limb = x_dtype == TQ_F32 ? 0 : 1;
     g.split.rows = 0;
     g.nibble = (plan->layout == TQ_LAYOUT_NIBBLE) ? 1 : 0;
     g.nib_idx = idx ? idx + (size_t)r0 * plan->idx_row_bytes : nullptr;

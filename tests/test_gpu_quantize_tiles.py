@@ -44,3 +44,27 @@ def test_codes_do_not_depend_on_the_number_of_rows(d, n, mode, bits, nibble, dty
     for part, full in zip(quantize(plan, Y[:, :d], mode), whole):
         if dtype == torch.bfloat16 or d % 4:
             assert torch.equal(part, full[:300])
+
+
+@pytest.mark.parametrize("d,n", [(129, 70), (384, 300), (3072, 130), (5000, 40)])
+@pytest.mark.parametrize("mode,bits", [(tq.TQ_PROD, 3), (tq.TQ_MSE, 2)])
+def test_bf16_rows_at_any_scale(d, n, mode, bits):
+    """Rows enter the rotation scaled by a power of two: codes are those of the same rows at another power of two, bit for bit, and rows
+    of zeros, of a norm that overflows or of a NaN are coded as the fp32 rows are."""
+    prod = mode == tq.TQ_PROD
+    cent, _ = tq.tq_codebook(d, bits - 1 if prod else bits)
+    plan = tq.Plan(d, bits, mode, tq.tq_rotation(d, 5), tq.tq_rotation(d, 6, tq.TQ_GAUSSIAN) if prod else None, cent)
+    X = torch.randn((n, d), generator=torch.Generator(device=DEV).manual_seed(d), device=DEV).bfloat16()
+    base = quantize(plan, X, mode)
+    for e in (-50, 40):                                # squares stay inside fp32
+        out = quantize(plan, X * 2.0 ** e, mode)
+        for a, b in zip(out[:-1], base[:-1]):
+            assert torch.equal(a, b), e
+        assert torch.equal(out[-1], base[-1] * 2.0 ** e)
+    X[3] = 0.0
+    X[5, 7] = 1e30
+    X[7, 2] = float("nan")
+    X[9] = 1e-30
+    for a, b in zip(quantize(plan, X, mode)[:-1], quantize(plan, X.float(), mode)[:-1]):
+        for r in (3, 5, 7, 9):
+            assert torch.equal(a[r], b[r]) or (a.dtype == torch.float32 and torch.isnan(a[r]) and torch.isnan(b[r])), r
