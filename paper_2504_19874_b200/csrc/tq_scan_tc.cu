@@ -156,57 +156,34 @@ __device__ __forceinline__ uint32_t parities4(uint32_t x) {
   return ((x ^ s1 ^ s2) & M) | (((x ^ s1 ^ s3) & M) << 1) | (((x ^ s2 ^ s3) & M) << 2) | (((s1 ^ s2 ^ s3) & M) << 3);
 }
 
-// ------------------------------------------------------------------ per-query constants
-struct StatArgs {
+// ------------------------------------------------------------------ per-query constants and B matrices
+// Ba[pass*96 + n][kba*128], Bs[pass*96 + n][kbs*128], n = 32 * digit + (query in pass); K-major int8.
+// Byte kappa of a k-block = (2 wl + k / 4) * 16 + (k % 4) * 4 + i  <->  bit 8 i + k of word wl: the order in
+// which the transform threads lay out their registers.
+// Nibble layout: one B matrix Bn[pass*96 + n][3 nblk * 128]; k-block 3 b + type of block b.  K-byte kappa of an h or l
+// k-block <-> coordinate kappa of the block; of a sign k-block: register kappa / 4 = 2 word + parity, byte i = kappa % 4
+// <-> coordinate 8 word + 2 i + parity (low nibbles, parity 0, have the value 8 and carry 16 J; high nibbles 128 and J).
+struct OperandArgs {
   const float* Qcat;
   int64_t ldq;
-  int d, dpad, prod;
-  double amax, csum;
-  int nib;          // nibble layout: the scales and constants of the table-lookup form
-  double delta;
-  QConst* out;
+  int nqg, dpad, prod;
+  Geo g;
+  double alpha[8], amax, csum;
+  double delta;     // nibble layout: step of the centroid table
+  QConst* qc;
+  uint8_t* Ba;
+  uint8_t* Bs;
 };
 
-// Nibble layout: one warp per query, the same reductions in the same order as the register-fed engine's
-// (lane-strided maxima in fp32, the sum of q'' in fp64 folded by xor shuffles).
-__global__ void __launch_bounds__(32) tstats_nib_kernel(StatArgs a) {
-  allow_successor();
-  wait_for_predecessor();   // the queries are its output; what this kernel writes may still be read by it
-  const int lane = threadIdx.x;
-  const float* q = a.Qcat + (int64_t)blockIdx.x * a.ldq;
-  float mx1 = 0.f, mx2 = 0.f;
-  double sm2 = 0.0;
-  for (int j = lane; j < a.d; j += 32) {
-    mx1 = fmaxf(mx1, fabsf(q[j]));
-    const float u = q[a.dpad + j];
-    mx2 = fmaxf(mx2, fabsf(u));
-    sm2 += (double)u;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
-    mx2 = fmaxf(mx2, __shfl_xor_sync(0xffffffffu, mx2, o));
-    sm2 += __shfl_xor_sync(0xffffffffu, sm2, o);
-  }
-  if (lane == 0) {
-    const nib::QScale s = nib::make_scale(mx1, mx2);
-    const nib::QConst n = nib::make_const(s, a.delta, sm2);
-    QConst c;
-    c.sa = n.sa; c.ca = 0.f; c.ss = n.ss; c.cs = n.cs;
-    c.fa = s.fh; c.fs = 0;
-    // the real scale of the sign-bit weights travels in the two spare words
-    c.pad[0] = __double2loint(s.sq); c.pad[1] = __double2hiint(s.sq);
-    a.out[blockIdx.x] = c;
-  }
-}
+// 2^e as a double, e in the normal range.
+__device__ __forceinline__ double pow2_of(int e) { return __hiloint2double((e + 1023) << 20, 0); }
 
-__global__ void __launch_bounds__(256) tstats_kernel(StatArgs a) {
+// Maxima and sums of a rotated query, all threads of a CTA of 256.
+__device__ __forceinline__ QConst query_constants(const OperandArgs& a, const float* q) {
   __shared__ double red[4][8];
-  allow_successor();
-  wait_for_predecessor();   // the queries are its output; what this kernel writes may still be read by it
-  const float* q = a.Qcat + (int64_t)blockIdx.x * a.ldq;
+  __shared__ QConst shared_c;
   double mx1 = 0.0, sm1 = 0.0, mx2 = 0.0, sm2 = 0.0;
-  for (int j = threadIdx.x; j < a.d; j += blockDim.x) {
+  for (int j = threadIdx.x; j < a.g.d; j += 256) {
     const double v = (double)q[j];
     mx1 = fmax(mx1, fabs(v));
     sm1 += v;
@@ -249,108 +226,116 @@ __global__ void __launch_bounds__(256) tstats_kernel(StatArgs a) {
     c.ca = (float)(a.csum * sm1);
     c.cs = (float)(-sm2);
     c.pad[0] = c.pad[1] = 0;
-    a.out[blockIdx.x] = c;
+    shared_c = c;
   }
+  __syncthreads();
+  return shared_c;
 }
 
-// ------------------------------------------------------------------ B matrices
-// Ba[pass*96 + n][kba*128], Bs[pass*96 + n][kbs*128], n = 32 * digit + (query in pass); K-major int8.
-// Byte kappa of a k-block = (2 wl + k / 4) * 16 + (k % 4) * 4 + i  <->  bit 8 i + k of word wl: the order in
-// which the transform threads lay out their registers.
-struct BPrepArgs {
-  const float* Qcat;
-  int64_t ldq;
-  const QConst* qc;
-  int nqg;
-  Geo g;
-  double alpha[8];
-  uint8_t* Ba;
-  uint8_t* Bs;
-};
+// Nibble layout: one warp, the same reductions in the same order as the register-fed engine's (lane-strided maxima in fp32, the
+// sum of q'' in fp64 folded by xor shuffles).
+__device__ __forceinline__ QConst query_constants_nib(const OperandArgs& a, const float* q) {
+  __shared__ QConst shared_c;
+  const int lane = threadIdx.x;
+  if (threadIdx.x < 32) {
+    float mx1 = 0.f, mx2 = 0.f;
+    double sm2 = 0.0;
+#pragma unroll 8
+    for (int j = lane; j < a.g.d; j += 32) {
+      mx1 = fmaxf(mx1, fabsf(q[j]));
+      const float u = q[a.dpad + j];
+      mx2 = fmaxf(mx2, fabsf(u));
+      sm2 += (double)u;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
+      mx2 = fmaxf(mx2, __shfl_xor_sync(0xffffffffu, mx2, o));
+      sm2 += __shfl_xor_sync(0xffffffffu, sm2, o);
+    }
+    if (lane == 0) {
+      const nib::QScale s = nib::make_scale(mx1, mx2);
+      const nib::QConst n = nib::make_const(s, a.delta, sm2);
+      QConst c;
+      c.sa = n.sa; c.ca = 0.f; c.ss = n.ss; c.cs = n.cs;
+      c.fa = s.fh; c.fs = 0;
+      // the real scale of the sign-bit weights travels in the two spare words
+      c.pad[0] = __double2loint(s.sq); c.pad[1] = __double2hiint(s.sq);
+      shared_c = c;
+    }
+  }
+  __syncthreads();
+  return shared_c;
+}
 
-// 2^e as a double, e in the normal range.
-__device__ __forceinline__ double pow2_of(int e) { return __hiloint2double((e + 1023) << 20, 0); }
-
-// One thread per 32-bit word of B (four K-bytes) and query: the weights are formed once and leave as a word in each of the
-// three digit rows; a warp writes 128 contiguous bytes of each.  (A thread per 32 K-bytes and digit spent 12.6 us on its own
-// serial chain of fp64 operations, whatever the number of queries; now 2.3 us for 32 queries at d = 1536.)
-__global__ void __launch_bounds__(256) tbprep_kernel(BPrepArgs a, int part, int queries) {
+// One launch for constants and operand: CTA (query, share of the operand's words).  Every share forms the query's constants again,
+// which is cheaper than a launch of their own (3 us each: two or three fewer per call, 64 queries against 4,096 rows of d = 128: 15.5 -> 13.8 us).  A thread
+// takes a 32-bit word of B (four K-bytes): its weights are formed once and leave as a word in each of the three digit rows; a
+// warp writes 128 contiguous bytes of each.
+template <bool NIB>
+__global__ void __launch_bounds__(256) toperand_kernel(const __grid_constant__ OperandArgs a) {
   allow_successor();
   wait_for_predecessor();   // the queries are its output; what this kernel writes may still be read by it
-  const int nkb = part ? a.g.kbs : a.g.kba;
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= (int64_t)queries * nkb * 32) return;
-  const int wl = (int)(tid >> 3) & 3, k = (int)tid & 7;
-  const int kb = (int)((tid >> 5) % nkb), ql = (int)((tid >> 5) / nkb);
-  uint32_t out[LIMBS] = {0u, 0u, 0u};
-  if (ql < a.nqg) {
-    const float* q = a.Qcat + (int64_t)ql * a.ldq;
-    const double scale = pow2_of((part ? a.qc[ql].fs : a.qc[ql].fa) - k);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int bit = 8 * i + k;
-      double W = 0.0;
-      if (!part) {
-        const Slot s = slot_a(a.g, kb, wl, bit);
-        if (s.coord < a.g.d) W = 2.0 * a.alpha[s.term] * (double)q[s.coord];
-      } else {
-        const int j = 32 * (4 * kb + wl) + bit;
-        if (j < a.g.d) W = 2.0 * (double)q[a.g.dpad + j];
-      }
-      const double Jd = rint(W * scale);
-      int J = fabs(Jd) <= 8388608.0 ? (int)Jd : 0;   // non-finite query entries contribute nothing
-#pragma unroll
-      for (int l = 0; l < LIMBS; ++l) {
-        const int dg = ((J + 128) & 255) - 128;
-        J = (J - dg) >> 8;
-        out[l] |= (uint32_t)(dg & 255) << (8 * i);
-      }
-    }
+  const int ql = blockIdx.x;
+  const bool present = ql < a.nqg;   // absent queries of the last pass get zero rows
+  const float* q = a.Qcat + (int64_t)(present ? ql : 0) * a.ldq;
+  QConst c = {};
+  if (present) {
+    c = NIB ? query_constants_nib(a, q) : query_constants(a, q);
+    if (blockIdx.y == 0 && threadIdx.x == 0) a.qc[ql] = c;
   }
   const int row0 = ql / kQueriesPerPass * NCOL + ql % kQueriesPerPass;   // digit l of the query: row0 + 32 l
-  uint8_t* dst = (part ? a.Bs : a.Ba) + ((size_t)row0 * nkb + kb) * KB_BYTES + wl * 32 + k * 4;
+  for (int i = blockIdx.y * 256 + threadIdx.x; i < (a.g.kba + a.g.kbs) * 32; i += gridDim.y * 256) {
+    const bool part = i >= a.g.kba * 32;   // bit streams: the sign part
+    const int nkb = part ? a.g.kbs : a.g.kba;
+    const int at = part ? i - a.g.kba * 32 : i, kb = at >> 5, word = at & 31;
+    uint32_t out[LIMBS] = {0u, 0u, 0u};
+    if (present && NIB) {
+      const int b = kb / 3, type = kb % 3;
+      nib::QScale sc;
+      sc.fh = c.fa;
+      sc.sq = __hiloint2double(c.pad[1], c.pad[0]);
 #pragma unroll
-  for (int l = 0; l < LIMBS; ++l) *reinterpret_cast<uint32_t*>(dst + (size_t)l * kQueriesPerPass * nkb * KB_BYTES) = out[l];
-}
-
-// Nibble layout: one B matrix Bn[pass*96 + n][3 nblk * 128]; k-block 3 b + type of block b.  K-byte kappa of an h or l
-// k-block <-> coordinate kappa of the block; of a sign k-block: register kappa / 4 = 2 word + parity, byte i = kappa % 4
-// <-> coordinate 8 word + 2 i + parity (low nibbles, parity 0, have the value 8 and carry 16 J; high nibbles 128 and J).
-// Threads as in tbprep_kernel.
-__global__ void __launch_bounds__(256) tbprep_nib_kernel(BPrepArgs a, int queries) {
-  allow_successor();
-  wait_for_predecessor();   // the queries are its output; what this kernel writes may still be read by it
-  const int nkb = a.g.kba;
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= (int64_t)queries * nkb * 32) return;
-  const int word = (int)tid & 31;               // of the k-block's 32
-  const int kb = (int)((tid >> 5) % nkb), ql = (int)((tid >> 5) / nkb);
-  const int b = kb / 3, type = kb % 3;
-  uint32_t out[LIMBS] = {0u, 0u, 0u};
-  if (ql < a.nqg) {
-    const float* q = a.Qcat + (int64_t)ql * a.ldq;
-    const QConst c = a.qc[ql];
-    nib::QScale sc;
-    sc.fh = c.fa;
-    sc.sq = __hiloint2double(c.pad[1], c.pad[0]);
+      for (int i4 = 0; i4 < 4; ++i4) {
+        int cib = 4 * word + i4, mul = 1;
+        if (type == 2) {
+          cib = 8 * (word >> 1) + 2 * i4 + (word & 1);
+          mul = (word & 1) ? 1 : 16;
+        }
+        const int coord = nib::coord_of_block(a.g.nbi, a.g.idx_rb, a.g.qjl_rb, a.g.d, b, cib);
+        if (coord < 0) continue;
+        const long long J = mul * nib::weight(sc, type, q[(type < 2 ? 0 : a.dpad) + coord]);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      int cib = 4 * word + i, mul = 1;
-      if (type == 2) {
-        cib = 8 * (word >> 1) + 2 * i + (word & 1);
-        mul = (word & 1) ? 1 : 16;
+        for (int l = 0; l < LIMBS; ++l) out[l] |= (uint32_t)(nib::digit_of(J, l) & 255) << (8 * i4);
       }
-      const int coord = nib::coord_of_block(a.g.nbi, a.g.idx_rb, a.g.qjl_rb, a.g.d, b, cib);
-      if (coord < 0) continue;
-      const long long J = mul * nib::weight(sc, type, q[(type < 2 ? 0 : a.g.dpad) + coord]);
+    } else if (present) {
+      const int wl = word >> 3, k = word & 7;
+      const double scale = pow2_of((part ? c.fs : c.fa) - k);
 #pragma unroll
-      for (int l = 0; l < LIMBS; ++l) out[l] |= (uint32_t)(nib::digit_of(J, l) & 255) << (8 * i);
+      for (int i4 = 0; i4 < 4; ++i4) {
+        const int bit = 8 * i4 + k;
+        double W = 0.0;
+        if (!part) {
+          const Slot s = slot_a(a.g, kb, wl, bit);
+          if (s.coord < a.g.d) W = 2.0 * a.alpha[s.term] * (double)q[s.coord];
+        } else {
+          const int j = 32 * (4 * kb + wl) + bit;
+          if (j < a.g.d) W = 2.0 * (double)q[a.dpad + j];
+        }
+        const double Jd = rint(W * scale);
+        int J = fabs(Jd) <= 8388608.0 ? (int)Jd : 0;   // non-finite query entries contribute nothing
+#pragma unroll
+        for (int l = 0; l < LIMBS; ++l) {
+          const int dg = ((J + 128) & 255) - 128;
+          J = (J - dg) >> 8;
+          out[l] |= (uint32_t)(dg & 255) << (8 * i4);
+        }
+      }
     }
-  }
-  const int row0 = ql / kQueriesPerPass * NCOL + ql % kQueriesPerPass;
-  uint8_t* dst = a.Ba + ((size_t)row0 * nkb + kb) * KB_BYTES + word * 4;
+    uint8_t* dst = (part ? a.Bs : a.Ba) + ((size_t)row0 * nkb + kb) * KB_BYTES + word * 4;
 #pragma unroll
-  for (int l = 0; l < LIMBS; ++l) *reinterpret_cast<uint32_t*>(dst + (size_t)l * kQueriesPerPass * nkb * KB_BYTES) = out[l];
+    for (int l = 0; l < LIMBS; ++l) *reinterpret_cast<uint32_t*>(dst + (size_t)l * kQueriesPerPass * nkb * KB_BYTES) = out[l];
+  }
 }
 
 // ------------------------------------------------------------------ epilogue
@@ -1098,43 +1083,28 @@ int prepare_group(const tq_plan* plan, const float* Qcat, int nqg, void* workspa
   QConst* qc = static_cast<QConst*>(workspace);
   uint8_t* Ba = static_cast<uint8_t*>(workspace) + kConstBytes;
   uint8_t* Bs = Ba + b_bytes(g, 0);
-  StatArgs sa;
-  sa.Qcat = Qcat;
-  sa.ldq = ncols;
-  sa.d = plan->d;
-  sa.dpad = plan->dpad;
-  sa.prod = plan->mode == TQ_PROD ? 1 : 0;
-  sa.amax = plan->ms.amax;
-  sa.csum = plan->ms.csum;
-  sa.nib = g.nib;
-  sa.delta = plan->nb.delta;
-  sa.out = qc;
-  count_launches(1);
-  TQ_CHECK_CUDA(g.nib ? launch_dependent(tstats_nib_kernel, dim3((unsigned)nqg), dim3(32), 0, st, sa)
-                      : launch_dependent(tstats_kernel, dim3((unsigned)nqg), dim3(256), 0, st, sa), who);
-  BPrepArgs ba;
-  ba.Qcat = Qcat;
-  ba.ldq = ncols;
-  ba.qc = qc;
-  ba.nqg = nqg;
-  ba.g = g;
-  for (int i = 0; i < 8; ++i) ba.alpha[i] = plan->ms.alpha[i];
-  ba.Ba = Ba;
-  ba.Bs = Bs;
+  OperandArgs a;
+  a.Qcat = Qcat;
+  a.ldq = ncols;
+  a.nqg = nqg;
+  a.dpad = plan->dpad;
+  a.prod = plan->mode == TQ_PROD ? 1 : 0;
+  a.g = g;
+  for (int i = 0; i < 8; ++i) a.alpha[i] = plan->ms.alpha[i];
+  a.amax = plan->ms.amax;
+  a.csum = plan->ms.csum;
+  a.delta = plan->nb.delta;
+  a.qc = qc;
+  a.Ba = Ba;
+  a.Bs = Bs;
   const int queries = (nqg + kQueriesPerPass - 1) / kQueriesPerPass * kQueriesPerPass;   // absent ones get zero rows
-  if (g.nib) {
-    const int64_t total = (int64_t)queries * g.kba * 32;
-    count_launches(1);
-    TQ_CHECK_CUDA(launch_dependent(tbprep_nib_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, ba, queries), who);
-    return TQ_OK;
-  }
-  for (int part = 0; part < 2; ++part) {
-    const int nkb = part ? g.kbs : g.kba;
-    if (nkb == 0) continue;
-    const int64_t total = (int64_t)queries * nkb * 32;
-    count_launches(1);
-    TQ_CHECK_CUDA(launch_dependent(tbprep_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, ba, part, queries), who);
-  }
+  const int words = (g.kba + g.kbs) * 32;
+  // shares of an operand: one round of 256 words each, fewer rounds than that only where the queries fill the chip
+  const int shares = std::max(1, std::min((words + 255) / 256, 4 * tc::sm_count() / queries));
+  count_launches(1);
+  const dim3 grid((unsigned)queries, (unsigned)shares);
+  TQ_CHECK_CUDA(g.nib ? launch_dependent(toperand_kernel<true>, grid, dim3(256), 0, st, a)
+                      : launch_dependent(toperand_kernel<false>, grid, dim3(256), 0, st, a), who);
   return TQ_OK;
 }
 
