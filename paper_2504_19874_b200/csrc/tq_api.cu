@@ -161,10 +161,13 @@ size_t ms_topk_fixed(const tq_plan* plan, int nq) {
   return ms_score_fixed(plan, nq) + 1024 /* tau, count, overflow */ + (size_t)pick_engine(plan, nq).qpp * kCandCap * 8;
 }
 
-// Top-k of more than kScreenFrom queries over at least kFilterMinN vectors: bounds of the estimates from one fp16 pass per 256
-// queries, exact estimates only for the rows that the bounds leave (tq_screen_tc.cu).
-constexpr int kScreenFrom = 192;
-bool screens(const tq_plan* plan, int nq, int64_t n) { return nq > kScreenFrom && n >= kFilterMinN && pick_engine(plan, nq).tc; }
+// Top-k of kScreenFrom queries or more over at least kFilterMinN vectors: bounds of the estimates from one fp16 pass per 256 queries,
+// exact estimates only for the rows that the bounds leave (tq_screen_tc.cu).  The line lies where the exact engine needs a second
+// pass of 64 queries (us, exact / screened, n = 10^6: d = 200 prod b = 3, 64 queries 353 / 308, 130 795 / 303, 256 1,365 / 426;
+// d = 1536 prod b = 4 nibble 797 / 1,163, 2,082 / 1,215, 3,013 / 1,583; d = 3072 prod b = 2 1,368 / 2,755, 3,422 / 2,798,
+// 5,293 / 3,611; n = 65,536: d = 200 84 / 107, 161 / 95, 259 / 148; d = 1536 mse b = 2 115 / 190, 248 / 161, 405 / 297).
+constexpr int kScreenFrom = 65;
+bool screens(const tq_plan* plan, int nq, int64_t n) { return nq >= kScreenFrom && n >= kFilterMinN && pick_engine(plan, nq).tc; }
 // A query's list: 2,048 candidates are expected at most (screen_samples), and two CTAs of the selection fit an SM.
 constexpr int kScreenCap = 8192;
 // Workspace of a screened pass, between the exact engine's operand and the dense score buffer.
@@ -193,6 +196,15 @@ ScreenSpace screen_space(const tq_plan* plan) {
   s.cand_i = take(Q * kScreenCap * 4);
   s.total = at;
   return s;
+}
+// Bytes behind the rotated queries that a screened call needs, and those with which its rescue takes few launches.
+size_t screen_least(const tq_plan* plan) {
+  return align_up(tscan::workspace_bytes(plan), 256) + screen_space(plan).total + (size_t)kDenseRowsMin * screen::kQueries * sizeof(float);
+}
+size_t screen_pref(const tq_plan* plan, int nq, int64_t n) {
+  const ScanEngine e = pick_engine(plan, nq);
+  const size_t rescue = (size_t)e.qpp * std::min<int64_t>(n, e.dense_rows_pref), samples = (size_t)screen::kQueries * 16384;
+  return align_up(e.ws_bytes, 256) + screen_space(plan).total + align_up(std::max(rescue, samples) * sizeof(float), 256);
 }
 
 template <typename T>
@@ -751,10 +763,11 @@ extern "C" size_t tq_workspace_bytes(const tq_plan* plan, int op, int64_t n, int
       return plan->ms.ok ? ms_score_fixed(plan, nq) : qcat_bytes(plan, nq);
     case TQ_OP_TOPK:
       if (plan->ms.ok)
-        return ms_topk_fixed(plan, nq) + (screens(plan, nq, n) ? screen_space(plan).total : 0) +
-               align_up((size_t)pick_engine(plan, nq).qpp *
-                            std::max<int64_t>(std::min<int64_t>(n, pick_engine(plan, nq).dense_rows_pref), kDenseRowsMin) * sizeof(float),
-                        256);
+        return std::max(screens(plan, nq, n) ? qcat_bytes(plan, nq) + screen_pref(plan, nq, n) : 0,
+                        ms_topk_fixed(plan, nq) + align_up((size_t)pick_engine(plan, nq).qpp *
+                                                               std::max<int64_t>(std::min<int64_t>(n, pick_engine(plan, nq).dense_rows_pref), kDenseRowsMin) *
+                                                               sizeof(float),
+                                                           256));
       return qcat_bytes(plan, nq) + align_up((size_t)nq * std::min<int64_t>(n, kTopkBlockPref) * sizeof(float), 256);
     case TQ_OP_WSUM: {
       const size_t ncols = (size_t)plan->ncat * plan->dpad;
@@ -1059,7 +1072,7 @@ struct ScreenSamples {
 };
 static ScreenSamples screen_samples(int64_t n, int k, int64_t most) {
   const double expect = 2048.0 / (k + 8);   // rows per sampled row that make a list of 2,048
-  const double dense0 = std::max(4096.0, 16.0 * (k + 8));
+  const double dense0 = std::max(4096.0, std::min(160.0 * (k + 8), std::max(16384.0, 16.0 * (k + 8))));
   double first = std::max(std::sqrt((double)n * dense0), n / expect), dense = std::max(dense0, first / expect);
   ScreenSamples s;
   if ((double)n <= 16.0 * dense0 && n / dense0 <= expect) {
@@ -1092,6 +1105,7 @@ static int topk_screened(const ScanEngine& eng, const float* Qcat, int nq, int64
   const int64_t dense_floats = (int64_t)((ws + ws_bytes - reinterpret_cast<char*>(dense)) / sizeof(float));
   const ScreenSamples sm = screen_samples(n, k, dense_floats / screen::kQueries);
   static_assert(screen::kQueries == kGroupQueries, "one exact operand per screened pass");
+  const screen::QueryTerms* terms = screen::query_terms(plan, operand);
   for (int q0 = 0; q0 < nq; q0 += screen::kQueries) {
     const int nqp = std::min(screen::kQueries, nq - q0);
     float* ts = top_scores + (size_t)q0 * k;
@@ -1112,8 +1126,8 @@ static int topk_screened(const ScanEngine& eng, const float* Qcat, int nq, int64
       TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count1, kScreenCap, 0, 0, nqp, k, 0, nullptr, nullptr, tau, nullptr, nullptr, count, flag, st), who);
     }
     if ((rc = filter(n, 1, count))) return rc;
-    TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count, kScreenCap, 0, 0, nqp, k, 0, nullptr, nullptr, kth, flag, nullptr, nullptr, nullptr, st), who);
-    if ((rc = tscan::rescore(plan, nqp, idx, qjl, gamma, norms, msw, screen::query_terms(plan, operand), kth, count, cand_s, cand_i, kScreenCap,
+    TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count, kScreenCap, 0, 0, nqp, k, 0, nullptr, nullptr, kth, flag, nullptr, left, unused, st), who);
+    if ((rc = tscan::rescore(plan, nqp, idx, qjl, gamma, norms, msw, terms, kth, count, cand_s, cand_i, kScreenCap,
                              left_s, left_i, left, flag, st, who)))
       return rc;
     TQ_CHECK_CUDA(mscan::select_topk(left_s, left_i, left, screen::kSurvivors, 0, 0, nqp, k, 0, ts, ti, nullptr, nullptr, nullptr, nullptr, nullptr, st), who);
@@ -1134,11 +1148,10 @@ static int topk_ms(const tq_plan* plan, const float* Qcat, int nq, int64_t n, co
                    const float* gamma, const float* norms, int k, float* top_scores, int32_t* top_ids, char* ws,
                    size_t ws_bytes, cudaStream_t st, const char* who) {
   int rc;
+  // (a workspace of the documented minimum has no room for the lists)
+  if (screens(plan, nq, n) && ws_bytes >= screen_least(plan))
+    return topk_screened(pick_engine(plan, nq), Qcat, nq, n, idx, qjl, gamma, norms, k, top_scores, top_ids, ws, ws_bytes, st, who);
   const ScanEngine eng = pick_engine(plan, nq);
-  // (a workspace of the documented minimum has no room for the lists of 256 queries)
-  if (screens(plan, nq, n) &&
-      ws_bytes >= align_up(eng.ws_bytes, 256) + screen_space(plan).total + (size_t)kDenseRowsMin * screen::kQueries * sizeof(float))
-    return topk_screened(eng, Qcat, nq, n, idx, qjl, gamma, norms, k, top_scores, top_ids, ws, ws_bytes, st, who);
   void* msw = ws;
   char* p = ws + align_up(eng.ws_bytes, 256);
   float* tau = reinterpret_cast<float*>(p);          // [qpp] (qpp <= 64: 256 bytes)

@@ -862,12 +862,13 @@ __device__ __forceinline__ int dp4a_ss(uint32_t a, uint32_t b, int c) {
   return d;
 }
 
-// One CTA per query: candidates whose upper bound reaches the k-th lower bound, then a warp per row; lane = 32-bit word of a k-block.
+// CTA (query, share of its list): candidates whose upper bound reaches the k-th lower bound, then a warp per row; lane = 32-bit word
+// of a k-block.
 // Bound: latency of the gathers (the list's rows lie anywhere in the index); some 130 of 1,600 candidates are left for k = 100.
 constexpr int kRescoreThreads = 512;
 __global__ void __launch_bounds__(kRescoreThreads, 2) rescore_kernel(const __grid_constant__ RescoreArgs a) {
   __shared__ int ids[screen::kSurvivors];
-  __shared__ int s_n;
+  __shared__ int s_n, s_base;
   allow_successor();
   if (threadIdx.x == 0) s_n = 0;
   __syncthreads();
@@ -876,21 +877,40 @@ __global__ void __launch_bounds__(kRescoreThreads, 2) rescore_kernel(const __gri
   const bool signs = a.g.kbs > 0 || a.g.nib;
   const int m = min(a.count[q], a.cap);
   const float kth = a.kth[q], err = a.terms[q].err, unscale = a.terms[q].unscale;
-  for (int i = threadIdx.x; i < m; i += kRescoreThreads) {
-    const int id = a.cand_i[(int64_t)q * a.cap + i];
-    const screen::RowTerms t = screen::row_terms(a.norms ? __ldg(a.norms + id) : 1.f, signs ? __ldg(a.gamma + id) : 0.f);
-    const float high = a.cand_s[(int64_t)q * a.cap + i] + 2.f * t.rho * err * unscale;
-    if (!(high < kth)) {
-      const int s = atomicAdd(&s_n, 1);
-      if (s < screen::kSurvivors) ids[s] = id;
+  // four candidates of a thread at a time: the loads of their scalars are a chain of two round trips
+  const int stride = kRescoreThreads * (int)gridDim.y;
+  for (int i0 = blockIdx.y * kRescoreThreads + threadIdx.x; i0 < m; i0 += 4 * stride) {
+    int id[4];
+    float low[4], nu[4], gm[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = min(i0 + u * stride, m - 1);
+      id[u] = a.cand_i[(int64_t)q * a.cap + i];
+      low[u] = a.cand_s[(int64_t)q * a.cap + i];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      nu[u] = a.norms ? __ldg(a.norms + id[u]) : 1.f;
+      gm[u] = signs ? __ldg(a.gamma + id[u]) : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float high = low[u] + 2.f * screen::row_terms(nu[u], gm[u]).rho * err * unscale;
+      if (i0 + u * stride < m && !(high < kth)) {
+        const int s = atomicAdd(&s_n, 1);
+        if (s < screen::kSurvivors) ids[s] = id[u];
+      }
     }
   }
   __syncthreads();
-  const int n = min(s_n, screen::kSurvivors);
+  int n = min(s_n, screen::kSurvivors);
   if (threadIdx.x == 0) {
-    a.out_count[q] = n;
-    if (s_n > screen::kSurvivors) atomicExch(a.overflow, 1);
+    s_base = atomicAdd(a.out_count + q, n);
+    if (s_n > screen::kSurvivors || s_base + n > screen::kSurvivors) atomicExch(a.overflow, 1);
   }
+  __syncthreads();
+  const int base = s_base;
+  n = min(n, screen::kSurvivors - base);
   const QConst c = a.qc[q];
   const int row0 = q / kQueriesPerPass * NCOL + q % kQueriesPerPass;
   const size_t pa = (size_t)a.g.kba * KB_BYTES, psn = (size_t)a.g.kbs * KB_BYTES;
@@ -955,8 +975,8 @@ __global__ void __launch_bounds__(kRescoreThreads, 2) rescore_kernel(const __gri
       if (signs) sv = fmaf((float)(((long long)vs[2] * 256 + vs[1]) * 256 + vs[0]), c.ss, c.cs);
       const float nu = a.norms != nullptr ? __ldg(a.norms + row) : 1.f, cg = __fmul_rn(a.coef, signs ? __ldg(a.gamma + row) : 0.f);
       const float e = __fmul_rn(nu, fmaf(cg, sv, av));
-      a.out_s[(int64_t)q * screen::kSurvivors + s] = e;
-      a.out_i[(int64_t)q * screen::kSurvivors + s] = isnan(e) ? -1 : (int)row;   // a negative id is an empty slot
+      a.out_s[(int64_t)q * screen::kSurvivors + base + s] = e;
+      a.out_i[(int64_t)q * screen::kSurvivors + base + s] = isnan(e) ? -1 : (int)row;   // a negative id is an empty slot
     }
   }
 }
@@ -1210,7 +1230,7 @@ int rescore(const tq_plan* plan, int nqp, const uint8_t* idx, const uint8_t* qjl
   a.out_count = out_count;
   a.overflow = overflow;
   count_launches(1);
-  TQ_CHECK_CUDA(launch_dependent(rescore_kernel, dim3((unsigned)nqp), dim3(kRescoreThreads), 0, st, a), who);
+  TQ_CHECK_CUDA(launch_dependent(rescore_kernel, dim3((unsigned)nqp, (unsigned)std::max(1, std::min(8, 2 * tc::sm_count() / nqp))), dim3(kRescoreThreads), 0, st, a), who);
   return TQ_OK;
 }
 

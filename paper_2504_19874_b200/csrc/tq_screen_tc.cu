@@ -11,16 +11,17 @@
 // k best; the few that are left (about k + k / 3 of 10^6 rows) are scored again by the exact integers (tscan::rescore), so the
 // results are the bits that the exact engine returns for every row.
 //
-// CTA pair (cta_group::2, M = 256 rows, 128 per CTA), persistent over row tiles, 640 threads per CTA:
-//   warp 0        TMA producer: per k-block (64 coordinates) the CTA's 64 + 64 rows of the query operand, per row group the packed rows
-//   warps 1..2    MMA issuers of the leader: issuer h owns the accumulator of queries [128 h, 128 h + 128).  The two run
-//                 unsynchronised over the same A slots, so that one half's MMAs fill the tensor pipe while the other half's
-//                 accumulator is read
-//   warps 4..11   expansion (thread = row): packed codes -> fp16 by byte permutes over the codebook's bytes -> tcgen05.st into the A
-//                 slots in TMEM (an A operand in shared memory would bring that to 128 B per clock, all an SM has)
-//   warps 12..19  epilogue: half (warp - 12) / 4, thread = row: one FMA chain and a maximum per estimate, the hits one by one
-// TMEM: two accumulators of 128 columns, eight A slots of 32.  The ring of eight slots is shared by A (TMEM) and B (shared memory):
-// one commit per issuer and k-block frees both.  All waits are bounded.
+// CTA pair (cta_group::2, M = 256 rows, 128 per CTA; N = 256 queries, or 128), persistent over row tiles, 896 threads per CTA:
+//   warp 0        TMA producer of the query operand: per k-block (64 coordinates) the CTA's half of its rows
+//   warp 1        MMA issuer (of the leader)
+//   warp 2        TMA producer of the packed rows
+//   warps 4..11   expansion (thread = row): packed codes -> fp16 by byte permutes over the codebook's bytes -> the stage's A tile; two
+//                 sets of four warps take the k-blocks in turn
+//   warps 12..27  epilogue (thread = row, a quarter of the queries): one FMA chain per pair of estimates, the hits one by one
+// Five stages of 32 KB (A and half of B), two accumulators of 256 columns (all of TMEM), so that a tile is read while the next one's
+// MMAs run.  The single-lane roles are chains of dependent instructions at six cycles each: with some sixty of them per k-block the
+// issuer was the longest part of the kernel, hence one barrier for both operands and nothing in its loop that can be outside.
+// All waits are bounded.
 #include <algorithm>
 #include <atomic>
 #include <cfloat>
@@ -30,7 +31,6 @@
 
 #include "tq_nib_common.cuh"
 #include "tq_quantize_tc.h"
-#include "tq_scan_tc.h"
 #include "tq_screen_tc.h"
 #include "tq_tc.cuh"
 
@@ -42,18 +42,17 @@ namespace {
 using namespace tq::tc;
 
 constexpr int TILE = 128;                   // rows per CTA = TMEM lanes
-constexpr int HALF = 128;                   // queries per accumulator
-constexpr int SLOTS = 8;                    // ring of k-blocks
-constexpr int BTILE = 64 * 128;             // one half's rows of a k-block in one CTA: 64 queries x 64 fp16
-constexpr int PSTAGES = 4, PTILE = TILE * 64;
-constexpr int ACOL0 = 2 * HALF;             // first TMEM column of the A slots
+constexpr int STAGES = 5;                   // ring of k-blocks
+constexpr int ATILE = TILE * 128, BTILE = kQueries / 2 * 128;   // bytes of a k-block in one CTA: 128 rows, 128 queries x 64 fp16
+constexpr int STAGE = ATILE + BTILE;
+constexpr int PSTAGES = 3, PTILE = TILE * 64;
 constexpr int TMEM_COLS = 512;
 constexpr int NEXP0 = 4, NEPI0 = 12;        // first expansion and epilogue warp
-constexpr int NTHREADS = 32 * 20;
-constexpr int LBUF = 24;                    // candidates per query a CTA collects before it appends them
-static_assert(ACOL0 + SLOTS * 32 <= TMEM_COLS, "TMEM columns");
-constexpr size_t kSmemBytes = 1024 + (size_t)SLOTS * 2 * BTILE + PSTAGES * PTILE + 512 +
-                              kQueries * (sizeof(float2) + sizeof(float) + sizeof(int) + LBUF * sizeof(uint2));
+constexpr int NEPI = 16;                    // epilogue warps
+constexpr int NTHREADS = 32 * (NEPI0 + NEPI);
+constexpr int LBUF = 16;                    // candidates per query a CTA collects before it appends them
+constexpr size_t kSmemBytes = 1024 + (size_t)STAGES * STAGE + PSTAGES * PTILE + 512 +
+                              kQueries * (sizeof(float4) / 2 + sizeof(float) + sizeof(int) + LBUF * sizeof(uint2));
 static_assert(kSmemBytes <= 227 * 1024, "shared memory");
 
 // k-blocks of 64 coordinates: those of the centroid term, then those of the sign term; nibble layout: per 64-byte block of the
@@ -105,29 +104,14 @@ __device__ __forceinline__ Element element_of(const Geo& g, int f, int c, int e)
 }
 
 // ------------------------------------------------------------------ query operand and error constants
-struct PrepArgs {
-  const float* Qcat;
-  int64_t ldq;
-  int dpad, nq, prod;
-  Geo g;
-  float cscale;        // 2^ec: the codebook's largest entry times this is in [1, 2)
-  int ec;
-  float cmax, dcmax;   // largest |c16|, largest |c16 - c 2^ec|
-  float coef;
-  int planes;          // fixed-point weights per coordinate of the exact engine's bit streams
-  float amax2;         // 2 max |Walsh coefficient|
-  float delta;         // step of the nibble layout's 16-bit centroid table
-  __half* B;           // [kQueries][64 kblocks]
-  QueryTerms* terms;
-};
-
-__device__ __forceinline__ float block_sum(float v, float* red) {
+template <typename T>
+__device__ __forceinline__ T block_sum(T v, T* red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   __syncthreads();
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  float s = 0.f;
+  T s = 0;
   for (int w = 0; w < 8; ++w) s += red[w];
   return s;
 }
@@ -141,6 +125,66 @@ __device__ __forceinline__ float block_max(float v, float* red) {
   for (int w = 0; w < 8; ++w) s = fmaxf(s, red[w]);
   return s;
 }
+
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+  uint32_t d;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+  return d;
+}
+// Eight 3-bit codes (low 24 bits) as eight nibbles.
+__device__ __forceinline__ uint32_t spread3(uint32_t x) {
+  x = (x & 0x00000fffu) | ((x & 0x00fff000u) << 4);
+  x = (x & 0x003f003fu) | ((x & 0x0fc00fc0u) << 2);
+  return (x & 0x07070707u) | ((x & 0x38383838u) << 1);
+}
+
+// The exact engine's weights are whole numbers: what rounding them can do to the centroid term of an estimate and to its sign term
+// (per unit of gamma), for a query with maxima mx1, mx2 and sum |q'| = l1.
+struct EngineRounding {
+  int nib, d, planes;   // planes: weights per coordinate of the bit streams
+  float amax2;          // 2 max |Walsh coefficient|
+  float delta;          // step of the nibble layout's 16-bit centroid table
+  float coef;
+};
+__device__ __forceinline__ float2 engine_error(const EngineRounding& r, float mx1, float mx2, float l1) {
+  if (r.nib) {
+    const nib::QScale s = nib::make_scale(mx1, mx2);
+    // half a unit of the weights of h (at most 128) and of l (at most 255) per coordinate, half a unit of the 16-bit centroid
+    return make_float2((float)r.d * 192.f * r.delta * (float)ldexp(1.0, 8 - s.fh) + l1 * r.delta, (float)r.d * (float)(1.0 / s.sq) * r.coef);
+  }
+  // a weight of bit k of a byte is rounded to 2^(k - f): 255 / 8 half units per weight and byte on average
+  auto unit = [](float wmax) {
+    if (!(wmax > 0.f)) return 0.f;
+    int e;
+    frexpf(wmax, &e);
+    return ldexpf(1.f, e - 22);
+  };
+  return make_float2((float)(r.d * r.planes + 64) * 16.f * unit(r.amax2 * mx1 * 1.0001f), (float)(r.d + 64) * 16.f * unit(2.f * mx2 * 1.0001f) * r.coef);
+}
+EngineRounding engine_rounding(const tq_plan* plan) {
+  EngineRounding r;
+  r.nib = plan->layout == TQ_LAYOUT_NIBBLE ? 1 : 0;
+  r.d = plan->d;
+  r.planes = plan->mse_bits == 3 ? 4 : plan->mse_bits == 4 ? 8 : plan->mse_bits;
+  r.amax2 = (float)(2.0 * plan->ms.amax);
+  r.delta = (float)plan->nb.delta;
+  r.coef = plan->coef;
+  return r;
+}
+
+struct PrepArgs {
+  const float* Qcat;
+  int64_t ldq;
+  int dpad, nq, prod;
+  Geo g;
+  float cscale;        // 2^ec: the codebook's largest entry times this is in [1, 2)
+  int ec;
+  float cmax, dcmax;   // largest |c16|, largest |c16 - c 2^ec|
+  float coef;
+  EngineRounding engine;
+  __half* B;           // [kQueries][64 kblocks]
+  QueryTerms* terms;
+};
 
 // One CTA per query: the fp16 operand row in the order of the k-blocks, the error constant.
 __global__ void __launch_bounds__(256) screen_prep_kernel(PrepArgs a) {
@@ -211,24 +255,9 @@ __global__ void __launch_bounds__(256) screen_prep_kernel(PrepArgs a) {
   const float adds = (float)(4 * a.g.kblocks() + 8) * 4.76837158e-7f;
   e1 += adds * l1 * a.cmax + l2 * 2.98023224e-8f;          // gamma below fp16's normal range: 2^-25 absolute
   e2 = e2 * 1.001f + l2 * 4.8828125e-4f + adds * l2;       // gamma to 11 bits
-  // The exact engine's weights are whole numbers: what rounding them can do to an estimate.
-  if (a.g.nib) {
-    const nib::QScale s = nib::make_scale(mx1, mx2);
-    // half a unit of the weights of h (at most 128) and of l (at most 255) per coordinate, half a unit of the 16-bit centroid
-    const float unit = a.delta * scale;
-    e1 += (float)d * 192.f * unit * (float)ldexp(1.0, 8 - s.fh) + l1 * a.cscale * a.delta;
-    e2 += (float)d * (float)(1.0 / s.sq) * a.coef * scale;
-  } else {
-    // a weight of bit k of a byte is rounded to 2^(k - f): 255 / 8 half units per weight and byte on average
-    auto unit = [](float wmax) {
-      if (!(wmax > 0.f)) return 0.f;
-      int e;
-      frexpf(wmax, &e);
-      return ldexpf(1.f, e - 22);
-    };
-    e1 += (float)(d * a.planes + 64) * 16.f * unit(a.amax2 * mx1 * 1.0001f) * scale;
-    e2 += (float)(d + 64) * 16.f * unit(2.f * mx2 * 1.0001f) * a.coef * scale;
-  }
+  const float2 engine = engine_error(a.engine, mx1, mx2, l1 / sa);
+  e1 += engine.x * scale;
+  e2 += engine.y * scale;
   // one constant for both terms, one per cent for the roundings of these sums and of the few fp32 operations behind the accumulator
   a.terms[q] = {fmaxf(e1, e2) * 1.01f + 1e-30f, 1.f / scale};
 }
@@ -240,7 +269,7 @@ struct ScanArgs {
   int ngroups;
   uint32_t tab[4];         // bytes of the codebook in fp16: low bytes of entries 0..3, 4..7, high bytes alike; two bits: entries 0, 1 and 2, 3;
                            // four bits: of the eight positive entries; one bit: tab[0] = the pair of positive entries
-  int nqp, nhalf;
+  int nqp, ncols;          // queries, MMA columns (128 or 256)
   const QueryTerms* terms;
   const float* gamma;
   const float* norms;
@@ -296,17 +325,6 @@ __device__ __forceinline__ int k_steps(const Geo& g, int f) {
   return min(4, (g.d - 64 * kb + 15) >> 4);
 }
 
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
-  uint32_t d;
-  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
-  return d;
-}
-// Eight 3-bit codes (low 24 bits) as eight nibbles.
-__device__ __forceinline__ uint32_t spread3(uint32_t x) {
-  x = (x & 0x00000fffu) | ((x & 0x00fff000u) << 4);
-  x = (x & 0x003f003fu) | ((x & 0x0fc00fc0u) << 2);
-  return (x & 0x07070707u) | ((x & 0x38383838u) << 1);
-}
 // Eight selectors (nibbles 0..7) -> eight fp16 centroids in natural order.
 __device__ __forceinline__ void centroids8(const uint32_t (&tab)[4], uint32_t sel, uint32_t* v) {
 #pragma unroll
@@ -338,10 +356,16 @@ __device__ __forceinline__ void centroids16_two(const uint32_t (&tab)[4], uint32
     v[2 * s + 1] = prmt(tab[0], tab[1], sel >> 16);
   }
 }
-// 32 bits: bit b and bit b + 16 as the signs (1: positive) of the pair in word b; `neg` holds the pair, negative.
-__device__ __forceinline__ void signs32(uint32_t neg, uint32_t w, uint32_t* v) {
-#pragma unroll
-  for (int b = 0; b < 16; ++b) v[b] = neg ^ ((w << (15 - b)) & 0x80008000u);
+// Two columns at a time: v = acc nu + (rho E - tau), e = (E, E', -tau, -tau').
+__device__ __forceinline__ void test_pair(float& v0, float& v1, float nu, float rho, const float4& e) {
+  asm("{\n\t.reg .b64 a, b, c, d;\n\t"
+      "mov.b64 a, {%3, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+      "fma.rn.f32x2 c, a, b, c;\n\t"
+      "mov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %2};\n\t"
+      "fma.rn.f32x2 d, a, b, c;\n\t"
+      "mov.b64 {%0, %1}, d;\n\t}"
+      : "+f"(v0), "+f"(v1)
+      : "f"(nu), "f"(rho), "f"(e.x), "f"(e.y), "f"(e.z), "f"(e.w));
 }
 
 template <int BM, bool NIB, int MODE>
@@ -353,20 +377,19 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
   const int64_t unit = blockIdx.x / 2, nunits = gridDim.x / 2;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  unsigned char* bring = smem;                                      // [SLOTS][2 halves][64 rows x 128 B]
-  unsigned char* pring = smem + SLOTS * 2 * BTILE;
+  unsigned char* pring = smem + STAGES * STAGE;
   uint64_t* bars = reinterpret_cast<uint64_t*>(pring + PSTAGES * PTILE);
-  uint64_t* afull = bars;                 // [SLOTS]  k-block stored by its set's four warps of both CTAs -> MMA (the leader's)
-  uint64_t* bfull = afull + SLOTS;        // [SLOTS]  TMA -> MMA (the leader's)
-  uint64_t* empty = bfull + SLOTS;        // [SLOTS]  both issuers' MMAs of the k-block complete
-  uint64_t* pfull = empty + SLOTS;        // [PSTAGES]  TMA (packed rows) -> the owning set
-  uint64_t* pempty = pfull + PSTAGES;     // [PSTAGES]  the owning set -> TMA
+  uint64_t* full = bars;                  // [STAGES]  TMA, and A stored by its set's four warps of both CTAs -> MMA (the leader's)
+  uint64_t* empty = full + STAGES;        // [STAGES]  the k-block's MMAs complete
+  uint64_t* pfull = empty + STAGES;       // [PSTAGES]  TMA (packed rows) -> expansion
+  uint64_t* pempty = pfull + PSTAGES;     // [PSTAGES]  expansion -> TMA
   uint64_t* dfull = pempty + PSTAGES;     // [2]  accumulator complete -> epilogue
-  uint64_t* dfree = dfull + 2;            // [2]  accumulator read -> its issuer (the leader's)
+  uint64_t* dfree = dfull + 2;            // [2]  accumulator read -> issuer (the leader's)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(dfree + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float2* et = reinterpret_cast<float2*>(reinterpret_cast<unsigned char*>(bars) + 512);   // [256] (error constant, -threshold), scaled
-  float* unscale = reinterpret_cast<float*>(et + kQueries);
+  // [128] of two queries each: error constants, then thresholds, negative; scaled like the accumulators
+  float4* et = reinterpret_cast<float4*>(reinterpret_cast<unsigned char*>(bars) + 512);
+  float* unscale = reinterpret_cast<float*>(et + kQueries / 2);
   int* lcnt = reinterpret_cast<int*>(unscale + kQueries);
   uint2* lbuf = reinterpret_cast<uint2*>(lcnt + kQueries);          // [256][LBUF] (lower bound, row)
 
@@ -375,18 +398,17 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
   const int64_t nrounds = (a.n + 2 * TILE - 1) / (2 * TILE);
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < SLOTS; ++s) {
-      mbar_init(&afull[s], 8);
-      mbar_init(&bfull[s], 1);
-      mbar_init(&empty[s], a.nhalf);
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(&full[s], 8 + 1);
+      mbar_init(&empty[s], 1);
     }
     for (int s = 0; s < PSTAGES; ++s) {
       mbar_init(&pfull[s], 1);
-      mbar_init(&pempty[s], 4);
+      mbar_init(&pempty[s], 8);
     }
-    for (int h = 0; h < 2; ++h) {
-      mbar_init(&dfull[h], 1);
-      mbar_init(&dfree[h], 8);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&dfull[i], 1);
+      mbar_init(&dfree[i], 2 * NEPI);
     }
     *abort_flag = 0;
     fence_barrier_init();
@@ -404,7 +426,9 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
       v = make_float2(t.err, MODE == 1 ? -a.tau[q] / t.unscale : 0.f);   // the scale is a power of two
       un = t.unscale;
     }
-    et[q] = v;
+    float* pair = reinterpret_cast<float*>(et + (q >> 1)) + (q & 1);
+    pair[0] = v.x;
+    pair[2] = v.y;
     unscale[q] = un;
     lcnt[q] = 0;
   }
@@ -414,86 +438,88 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp == 0) {
-    // ---------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      uint32_t kt = 0, gc = 0, pgc = 0;   // k-blocks and row groups reached, row groups requested
-      bool ok = true;
-      int64_t prnd = unit;
-      int pgi = 0;
-      auto load_rows = [&]() {
-        const RowGroup rg = row_group<BM, NIB>(a.g, pgi);
-        const uint32_t pst = pgc % PSTAGES;
-        mbar_arrive_expect_tx(&pfull[pst], (uint32_t)(TILE * rg.bytes));
-        tma_load_2d(pring + pst * PTILE, rg.from_qjl ? &tmPs : &tmPa, &pfull[pst], rg.x, (int)((prnd * 2 + rank) * TILE));
-        ++pgc;
-        if (++pgi == ngroups) {
-          pgi = 0;
-          prnd += nunits;
-        }
-      };
-      for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits) {   // rows past the last one read zeros
-        for (int gi = 0; gi < ngroups && ok; ++gi, ++gc) {
-          const RowGroup rg = row_group<BM, NIB>(a.g, gi);
-          while (pgc <= gc) {   // this group's rows at the latest now
-            if (!(ok = mbar_wait(&pempty[pgc % PSTAGES], ((pgc / PSTAGES) & 1u) ^ 1u, abort_flag, a.status))) break;
-            load_rows();
-          }
-          if (!ok) break;
-          for (int j = 0; j < rg.cnt; ++j, ++kt) {
-            if (prnd < nrounds && mbar_test_wait(&pempty[pgc % PSTAGES], ((pgc / PSTAGES) & 1u) ^ 1u)) load_rows();
-            const uint32_t slot = kt % SLOTS;
-            if (!(ok = mbar_wait(&empty[slot], ((kt / SLOTS) & 1u) ^ 1u, abort_flag, a.status))) break;
-            if (rank == 0) mbar_arrive_expect_tx(&bfull[slot], 2u * BTILE * (uint32_t)a.nhalf);
-            for (int h = 0; h < a.nhalf; ++h)
-              tma_load_2d_pair(bring + (slot * 2 + h) * BTILE, &tmB, &bfull[slot], (rg.f0 + j) * 64, h * HALF + rank * 64);
+  if (warp < NEXP0) {
+    if (warp == 0) {
+      // ---------------------------------------------------------------- query operand
+      if (lane == 0) {
+        uint32_t st = 0, ph = 1;
+        bool ok = true;
+        for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits) {
+          for (int f = 0; f < nkb; ++f) {
+            if (!(ok = mbar_wait(&empty[st], ph, abort_flag, a.status))) break;
+            if (rank == 0) mbar_arrive_expect_tx(&full[st], 128u * (uint32_t)a.ncols);
+            tma_load_2d_pair(smem + st * STAGE + ATILE, &tmB, &full[st], f * 64, rank * (a.ncols / 2));   // this CTA's half of the queries
+            if (++st == STAGES) {
+              st = 0;
+              ph ^= 1u;
+            }
           }
         }
+        if (!ok) {
+          for (int i = 0; i < 2000; ++i) __nanosleep(1000);   // let copies in flight land
+        }
       }
-      if (!ok) {
-        for (int i = 0; i < 2000; ++i) __nanosleep(1000);   // let copies in flight land
-      }
-    }
-    __syncwarp();
-  } else if (warp <= 2) {
-    // ---------------------------------------------------------------- MMA issuer of half warp - 1
-    const int h = warp - 1;
-    if (lane == 0 && rank == 0 && h < a.nhalf) {
-      // fp16 x fp16 -> fp32, K-major
-      constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(HALF >> 3) << 17) | ((uint32_t)((2 * TILE) >> 4) << 24);
-      const uint64_t bdesc0 = smem_desc_sw128(smem_u32(bring + h * BTILE));
-      const uint32_t d_tmem = tmem_base + (uint32_t)(h * HALF);
-      bool ok = true;
-      uint32_t kt = 0, it = 0;
-      for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits, ++it) {
-        if (!(ok = mbar_wait(&dfree[h], (it & 1u) ^ 1u, abort_flag, a.status))) break;
-        tc_fence_after();
-        for (int f = 0; f < nkb; ++f, ++kt) {
-          const uint32_t slot = kt % SLOTS, ph = (kt / SLOTS) & 1u;
-          if (!(ok = mbar_wait(&bfull[slot], ph, abort_flag, a.status))) break;
-          if (!(ok = mbar_wait(&afull[slot], ph, abort_flag, a.status))) break;
+      __syncwarp();
+    } else if (warp == 1) {
+      // ---------------------------------------------------------------- MMA issuer
+      if (lane == 0 && rank == 0) {
+        // fp16 x fp16 -> fp32, both K-major
+        const uint32_t idesc = (1u << 4) | ((uint32_t)(a.ncols >> 3) << 17) | ((uint32_t)((2 * TILE) >> 4) << 24);
+        const uint64_t adesc0 = smem_desc_sw128(smem_u32(smem)), bdesc0 = smem_desc_sw128(smem_u32(smem + ATILE));
+        const int last = NIB ? 4 : k_steps<NIB>(a.g, (a.g.kba > 0 ? a.g.kba : a.g.kbs) - 1);   // K steps of a part's last k-block
+        const int end0 = a.g.kba - 1, end1 = nkb - 1;
+        bool ok = true;
+        uint32_t st = 0, ph = 0, it = 0;
+        for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits, ++it) {
+          const uint32_t d = it & 1u, d_tmem = tmem_base + d * 256u;
+          if (!(ok = mbar_wait(&dfree[d], ((it >> 1) & 1u) ^ 1u, abort_flag, a.status))) break;
           tc_fence_after();
-          const uint64_t bdesc = bdesc0 + (uint64_t)(slot * ((2 * BTILE) >> 4));
-          const uint32_t a_tmem = tmem_base + (uint32_t)(ACOL0 + slot * 32);
-          const int steps = k_steps<NIB>(a.g, f);
-          for (int s = 0; s < steps; ++s)
-            asm volatile(
-                "{\n\t.reg .pred p;\n\t"
-                "setp.ne.b32 p, %4, 0;\n\t"
-                "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-                ::"r"(d_tmem), "r"(a_tmem + 8 * s), "l"(bdesc + 2 * s), "r"(idesc), "r"((uint32_t)(f | s))
-                : "memory");
-          umma_commit_pair(&empty[slot]);
+          for (int f = 0; f < nkb; ++f) {
+            const uint64_t off = (uint64_t)(st * (STAGE >> 4));
+            const uint64_t adesc = adesc0 + off, bdesc = bdesc0 + off;
+            const int steps = NIB || (f != end0 && f != end1) ? 4 : last;
+            if (!(ok = mbar_wait(&full[st], ph, abort_flag, a.status))) break;
+            tc_fence_after();
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+              if (s < steps) umma_bf16_pair(d_tmem, adesc + 2 * s, bdesc + 2 * s, idesc, s != 0 || f != 0 ? 1u : 0u);
+            umma_commit_pair(&empty[st]);
+            if (++st == STAGES) {
+              st = 0;
+              ph ^= 1u;
+            }
+          }
+          if (ok) umma_commit_pair(&dfull[d]);
         }
-        if (ok) umma_commit_pair(&dfull[h]);
       }
+      __syncwarp();
+    } else if (warp == 2) {
+      // ---------------------------------------------------------------- packed rows
+      if (lane == 0) {
+        uint32_t pst = 0, ph = 1;
+        bool ok = true;
+        for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits) {   // rows past the last one read zeros
+          for (int gi = 0; gi < ngroups; ++gi) {
+            const RowGroup rg = row_group<BM, NIB>(a.g, gi);
+            if (!(ok = mbar_wait(&pempty[pst], ph, abort_flag, a.status))) break;
+            mbar_arrive_expect_tx(&pfull[pst], (uint32_t)(TILE * rg.bytes));
+            tma_load_2d(pring + pst * PTILE, rg.from_qjl ? &tmPs : &tmPa, &pfull[pst], rg.x, (int)((rnd * 2 + rank) * TILE));
+            if (++pst == PSTAGES) {
+              pst = 0;
+              ph ^= 1u;
+            }
+          }
+        }
+        if (!ok) {
+          for (int i = 0; i < 2000; ++i) __nanosleep(1000);
+        }
+      }
+      __syncwarp();
     }
-    __syncwarp();
   } else if (warp >= NEXP0 && warp < NEPI0) {
-    // ---------------------------------------------------------------- expansion: thread = row; a set takes every second row group
+    // ---------------------------------------------------------------- expansion: thread = row; the sets take the k-blocks in turn
     const int set = (warp - NEXP0) >> 2, quad = warp & 3;
     const int r = quad * 32 + lane;
-    const uint32_t a_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)ACOL0;
     bool ok = true;
     uint32_t it = 0;
     auto load_gamma = [&](int64_t tl) -> float {
@@ -508,20 +534,21 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
       const uint32_t g16 = (uint32_t)__half_as_ushort(__float2half_rn(row_terms(1.f, gm).gamma));
       const uint32_t neg = (g16 | (g16 << 16)) ^ 0x80008000u;
       const uint32_t kt0 = it * (uint32_t)nkb;
-      // The slot was last read by the MMAs of k-block kt - SLOTS.  (A parity wait must not be two completions behind: the set's
-      // previous store is at most five k-blocks back, and k-blocks complete in order.)
-      auto store_a = [&](const uint32_t (&v)[32], uint32_t kt) -> bool {
-        const uint32_t slot = kt % SLOTS;
-        if (!mbar_wait(&empty[slot], ((kt / SLOTS) & 1u) ^ 1u, abort_flag, a.status)) return false;
-        tc_fence_after();
-        tmem_st32(a_addr + slot * 32, v);
-        tmem_st_wait();
-        tc_fence_before();
+      // The stage was last read by the MMAs of k-block kt - STAGES.  (A parity wait must not be two completions behind: the set's
+      // previous store is two k-blocks back, and k-blocks complete in order.)  The tensor core of this SM reads what these threads
+      // write, in a pair too: the proxy fence orders the writes, the arrival only tells the leader's issuer.
+      auto fill = [&](uint32_t kt, auto&& pieces) {
+        const uint32_t st = kt % STAGES;
+        if (!(ok = mbar_wait(&empty[st], ((kt / STAGES) & 1u) ^ 1u, abort_flag, a.status))) return;
+        unsigned char* dst = smem + st * STAGE + r * 128;
+        // 16-byte piece p of the row, 128-byte swizzle
+        pieces([&](int p, const uint32_t* v) { *reinterpret_cast<uint4*>(dst + ((p ^ (r & 7)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]); });
+        fence_proxy_async();
         __syncwarp();
-        if (lane == 0) mbar_arrive_leader(&afull[slot]);
-        return true;
+        if (lane == 0) mbar_arrive_leader(&full[st]);
       };
-      for (int gi = (set + (int)((it * (uint32_t)ngroups) & 1u)) & 1; gi < ngroups && ok; gi += 2) {
+      auto mine = [&](uint32_t kt) { return (int)(kt & 1u) == set; };
+      for (int gi = 0; gi < ngroups && ok; ++gi) {
         const RowGroup rg = row_group<BM, NIB>(a.g, gi);
         const uint32_t gc = it * (uint32_t)ngroups + (uint32_t)gi, pst = gc % PSTAGES;
         if (!(ok = mbar_wait(&pfull[pst], (gc / PSTAGES) & 1u, abort_flag, a.status))) break;
@@ -552,63 +579,87 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
         __syncwarp();
         if (lane == 0) mbar_arrive(&pempty[pst]);
         const uint32_t kt = kt0 + (uint32_t)rg.f0;
-        uint32_t v[32];
         if (NIB) {
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
+            if (ok && mine(kt + 2 * half))
+              fill(kt + 2 * half, [&](auto&& put) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) centroids8(a.tab, w[8 * half + j] & 0x77777777u, v + 4 * j);
-            ok = ok && store_a(v, kt + 2 * half);
+                for (int j = 0; j < 8; ++j) {
+                  uint32_t v[4];
+                  centroids8(a.tab, w[8 * half + j] & 0x77777777u, v);
+                  put(j, v);
+                }
+              });
+            if (ok && mine(kt + 2 * half + 1))
+              fill(kt + 2 * half + 1, [&](auto&& put) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
+                for (int j = 0; j < 8; ++j) {
+                  uint32_t v[4];
 #pragma unroll
-              for (int p = 0; p < 4; ++p) v[4 * j + p] = neg ^ ((w[8 * half + j] << (12 - 4 * p)) & 0x80008000u);
-            ok = ok && store_a(v, kt + 2 * half + 1);
+                  for (int p = 0; p < 4; ++p) v[p] = neg ^ ((w[8 * half + j] << (12 - 4 * p)) & 0x80008000u);
+                  put(j, v);
+                }
+              });
           }
-        } else if (BM == 0 || rg.sign) {
+        } else if (BM <= 1 || rg.sign) {
+          const uint32_t pair = BM == 1 && !rg.sign ? a.tab[0] ^ 0x80008000u : neg;
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            if (j < rg.cnt) {
-              signs32(neg, w[2 * j], v);
-              signs32(neg, w[2 * j + 1], v + 16);
-              ok = ok && store_a(v, kt + j);
-            }
+            if (ok && j < rg.cnt && mine(kt + j))
+              fill(kt + j, [&](auto&& put) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {   // bits b and b + 16 of a word are a pair
+                  uint32_t v[4];
+#pragma unroll
+                  for (int p = 0; p < 4; ++p) v[p] = pair ^ ((w[2 * j + (i >> 2)] << (15 - 4 * (i & 3) - p)) & 0x80008000u);
+                  put(i, v);
+                }
+              });
           }
         } else {
 #pragma unroll
           for (int j = 0; j < a_group_kb(BM); ++j) {
-            if (j < rg.cnt) {
-              if (BM == 1) {
-                signs32(a.tab[0] ^ 0x80008000u, w[2 * j], v);
-                signs32(a.tab[0] ^ 0x80008000u, w[2 * j + 1], v + 16);
-              } else if (BM == 2) {
+            if (ok && j < rg.cnt && mine(kt + j))
+              fill(kt + j, [&](auto&& put) {
+                if (BM == 2) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) centroids16_two(a.tab, w[4 * j + i], v + 8 * i);
-              } else if (BM == 3) {
+                  for (int i = 0; i < 4; ++i) {
+                    uint32_t v[8];
+                    centroids16_two(a.tab, w[4 * j + i], v);
+                    put(2 * i, v);
+                    put(2 * i + 1, v + 4);
+                  }
+                } else if (BM == 3) {
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {   // 32 codes in three words
-                  const uint32_t *x = w + 6 * j + 3 * i;
-                  centroids8(a.tab, spread3(x[0] & 0xffffffu), v + 16 * i);
-                  centroids8(a.tab, spread3(__funnelshift_r(x[0], x[1], 24) & 0xffffffu), v + 16 * i + 4);
-                  centroids8(a.tab, spread3(__funnelshift_r(x[1], x[2], 16) & 0xffffffu), v + 16 * i + 8);
-                  centroids8(a.tab, spread3(x[2] >> 8), v + 16 * i + 12);
+                  for (int i = 0; i < 2; ++i) {   // 32 codes in three words
+                    const uint32_t* x = w + 6 * j + 3 * i;
+                    const uint32_t sel[4] = {x[0], __funnelshift_r(x[0], x[1], 24), __funnelshift_r(x[1], x[2], 16), x[2] >> 8};
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                      uint32_t v[4];
+                      centroids8(a.tab, spread3(sel[p] & 0xffffffu), v);
+                      put(4 * i + p, v);
+                    }
+                  }
+                } else {
+#pragma unroll
+                  for (int i = 0; i < 8; ++i) {
+                    uint32_t v[4];
+                    centroids8_wide(a.tab, w[8 * j + i], v);
+                    put(i, v);
+                  }
                 }
-              } else {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) centroids8_wide(a.tab, w[8 * j + i], v + 4 * i);
-              }
-              ok = ok && store_a(v, kt + j);
-            }
+              });
           }
         }
       }
     }
     __syncwarp();
-  } else if (warp >= NEPI0 && (warp - NEPI0) / 4 < a.nhalf) {
-    // ---------------------------------------------------------------- epilogue: thread = row, the half's 128 queries
+  } else {
+    // ---------------------------------------------------------------- epilogue: thread = row, a quarter of the columns
     const int h = (warp - NEPI0) >> 2, quad = warp & 3;
-    const int r = quad * 32 + lane;
-    const uint32_t addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(h * HALF);
+    const int r = quad * 32 + lane, chunks = a.ncols / 128;   // chunks of 32 columns
     bool ok = true;
     uint32_t it = 0;
     auto load = [&](const float* src, int64_t tl, float otherwise) -> float {
@@ -623,55 +674,67 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
       const RowTerms t = row_terms(nu_next, g_next);
       nu_next = load(a.norms, tile + 2 * nunits, 1.f);
       g_next = load(gsrc, tile + 2 * nunits, 0.f);
-      if (!(ok = mbar_wait(&dfull[h], it & 1u, abort_flag, a.status))) break;
+      const uint32_t d = it & 1u;
+      if (!(ok = mbar_wait(&dfull[d], (it >> 1) & 1u, abort_flag, a.status))) break;
       tc_fence_after();
+      const uint32_t addr = tmem_base + ((uint32_t)(quad * 32) << 16) + d * 256u;
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
-        const int q0 = h * HALF + 32 * c;
+      for (int c = 0; c < chunks; ++c) {
+        const int q0 = (h * chunks + c) * 32;
         uint32_t acc[32];
         __syncwarp();
-        tmem_ld32(addr + 32 * c, acc);
+        tmem_ld32(addr + q0, acc);
         tmem_ld_wait();
-        if (c == 3) {   // the last columns are in registers
+        if (c == chunks - 1) {   // the last columns are in registers
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive_leader(&dfree[h]);
+          if (lane == 0) mbar_arrive_leader(&dfree[d]);
         }
         if (q0 >= a.nqp) continue;
+        auto err_of = [&](int q) -> float { return reinterpret_cast<const float*>(et + (q >> 1))[q & 1]; };
         if (MODE == 0) {
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
-            const float low = fmaxf(fmaf(__uint_as_float(acc[i]), t.nu, -t.rho * et[q0 + i].x) * unscale[q0 + i], -FLT_MAX);
+            const float low = fmaxf(fmaf(__uint_as_float(acc[i]), t.nu, -t.rho * err_of(q0 + i)) * unscale[q0 + i], -FLT_MAX);
             if (row_ok && q0 + i < a.nqp && TQ_DEVICE_CHECK(row >= 0 && row < a.lds, a.status)) a.dense[(int64_t)(q0 + i) * a.lds + row] = low;
           }
-        } else {
+          continue;
+        }
+        // Sign bit clear: the row's upper bound reaches the threshold.  The signs of eight columns are ANDed, one three-input
+        // operation per pair, and looked at together.
+        float v[32];
+        uint32_t none[4] = {~0u, ~0u, ~0u, ~0u};
 #pragma unroll
-          for (int i8 = 0; i8 < 32; i8 += 8) {
-            float v[8], most = -INFINITY;
+        for (int i = 0; i < 32; i += 2) {
+          v[i] = __uint_as_float(acc[i]);
+          v[i + 1] = __uint_as_float(acc[i + 1]);
+          test_pair(v[i], v[i + 1], t.nu, t.rho, et[(q0 + i) >> 1]);
+          none[i >> 3] &= __float_as_uint(v[i]) & __float_as_uint(v[i + 1]);
+        }
+        if (!row_ok || (int)(none[0] & none[1] & none[2] & none[3]) < 0) continue;
 #pragma unroll
-            for (int i = 0; i < 8; i += 2) {
-              const float4 e = *reinterpret_cast<const float4*>(et + q0 + i8 + i);
-              v[i] = fmaf(__uint_as_float(acc[i8 + i]), t.nu, fmaf(t.rho, e.x, e.y));
-              v[i + 1] = fmaf(__uint_as_float(acc[i8 + i + 1]), t.nu, fmaf(t.rho, e.z, e.w));
-              most = fmaxf(most, fmaxf(v[i], v[i + 1]));
-            }
-            if (most >= 0.f && row_ok) {
+        for (int g = 0; g < 4; ++g) {
+          if ((int)none[g] < 0) continue;
+          uint32_t hits = 0u;
 #pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                if (v[i] >= 0.f) {
-                  const int q = q0 + i8 + i;
-                  const float low = fmaxf(fmaf(__uint_as_float(acc[i8 + i]), t.nu, -t.rho * et[q].x) * unscale[q], -FLT_MAX);
-                  const int ls = atomicAdd(&lcnt[q], 1);
-                  if (ls < LBUF) {
-                    lbuf[q * LBUF + ls] = make_uint2(__float_as_uint(low), (uint32_t)row);
-                  } else {   // the CTA's buffer is full: straight to the list
-                    const int slot = atomicAdd(a.count + q, 1);
-                    if (slot < a.cap) {
-                      a.cand_s[(int64_t)q * a.cap + slot] = low;
-                      a.cand_i[(int64_t)q * a.cap + slot] = (int)row;
-                    }
-                  }
-                }
+          for (int i = 0; i < 8; ++i) hits |= (~__float_as_uint(v[8 * g + i]) >> 31) << i;
+          while (hits != 0u) {   // a lane takes its own hits one after the other
+            const int i = __ffs((int)hits) - 1, q = q0 + 8 * g + i;
+            hits &= hits - 1u;
+            const float x0 = (i & 1) ? v[8 * g + 1] : v[8 * g], x1 = (i & 1) ? v[8 * g + 3] : v[8 * g + 2];
+            const float x2 = (i & 1) ? v[8 * g + 5] : v[8 * g + 4], x3 = (i & 1) ? v[8 * g + 7] : v[8 * g + 6];
+            const float y0 = (i & 2) ? x1 : x0, y1 = (i & 2) ? x3 : x2, val = (i & 4) ? y1 : y0;
+            const float* pair = reinterpret_cast<const float*>(et + (q >> 1)) + (q & 1);
+            // the lower bound: val + tau - 2 rho E
+            const float low = fmaf(-2.f * t.rho, pair[0], val) - pair[2];
+            const int ls = atomicAdd(&lcnt[q], 1);
+            if (ls < LBUF) {
+              lbuf[q * LBUF + ls] = make_uint2(__float_as_uint(low), (uint32_t)row);
+            } else {   // the CTA's buffer is full: straight to the list
+              const int slot = atomicAdd(a.count + q, 1);
+              if (slot < a.cap) {
+                a.cand_s[(int64_t)q * a.cap + slot] = fmaxf(low * unscale[q], -FLT_MAX);
+                a.cand_i[(int64_t)q * a.cap + slot] = (int)row;
               }
             }
           }
@@ -698,7 +761,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
         const int slot = base + i;
         if (slot < a.cap) {
           const uint2 e = lbuf[q * LBUF + i];
-          a.cand_s[(int64_t)q * a.cap + slot] = __uint_as_float(e.x);
+          a.cand_s[(int64_t)q * a.cap + slot] = fmaxf(__uint_as_float(e.x) * unscale[q], -FLT_MAX);   // (not finite: no lower bound)
           a.cand_i[(int64_t)q * a.cap + slot] = (int)e.y;
         }
       }
@@ -777,6 +840,7 @@ Table make_table(const tq_plan* plan) {
   return t;
 }
 
+int columns(int nqp) { return nqp > kQueries / 2 ? kQueries : kQueries / 2; }
 size_t operand_bytes(const Geo& g) { return (size_t)kQueries * g.kblocks() * 128; }
 
 }  // namespace
@@ -801,13 +865,11 @@ int prepare(const tq_plan* plan, const float* Qcat, int nqp, void* workspace, cu
   a.cmax = t.cmax;
   a.dcmax = t.dcmax;
   a.coef = plan->coef;
-  a.planes = plan->mse_bits == 3 ? 4 : plan->mse_bits == 4 ? 8 : plan->mse_bits;
-  a.amax2 = (float)(2.0 * plan->ms.amax);
-  a.delta = (float)plan->nb.delta;
+  a.engine = engine_rounding(plan);
   a.B = static_cast<__half*>(workspace);
   a.terms = const_cast<QueryTerms*>(query_terms(plan, workspace));
   count_launches(1);
-  TQ_CHECK_CUDA(launch_dependent(screen_prep_kernel, dim3((unsigned)(nqp > HALF ? 2 * HALF : HALF)), dim3(256), 0, st, a), who);
+  TQ_CHECK_CUDA(launch_dependent(screen_prep_kernel, dim3((unsigned)columns(nqp)), dim3(256), 0, st, a), who);
   return TQ_OK;
 }
 
@@ -822,7 +884,7 @@ int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8
   a.ngroups = g.nib ? g.nblk : ga + (g.kbs + S_GROUP_KB - 1) / S_GROUP_KB;
   a.n = n;
   a.nqp = nqp;
-  a.nhalf = nqp > HALF ? 2 : 1;
+  a.ncols = columns(nqp);
   a.terms = query_terms(plan, workspace);
   a.gamma = gamma;
   a.norms = norms;
@@ -848,7 +910,7 @@ int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8
     }
   }
   CUtensorMap mb, pa, ps;
-  TQ_REQUIRE(make_half_map(&mb, static_cast<const __half*>(workspace), kQueries, 64 * g.kblocks(), 64 * g.kblocks(), 64), TQ_ERR_CUDA,
+  TQ_REQUIRE(make_half_map(&mb, static_cast<const __half*>(workspace), kQueries, 64 * g.kblocks(), 64 * g.kblocks(), a.ncols / 2), TQ_ERR_CUDA,
              "%s: cuTensorMapEncodeTiled failed (query operand)", who);
   const int ab = g.nib ? 64 : a_group_bytes(g.bm), sb = g.nib ? 64 : S_GROUP_BYTES;
   if (g.bm > 0)

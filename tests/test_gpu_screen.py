@@ -1,4 +1,4 @@
-"""Top-k of many queries: bounds from one fp16 pass decide which rows are scored, so the results are those of sorting the dense
+"""Top-k by screening: bounds from one fp16 pass decide which rows are scored, so the results are those of sorting the dense
 estimates, bit for bit."""
 import pytest
 import torch
@@ -22,12 +22,12 @@ def check(su, Q, n, codes, k):
 
 
 # one to four bits with and without signs; d at the edges of K steps (16), k-blocks (64), row groups (128, 256) and of the nibble
-# layout's blocks; n and nq at the edges of the row tiles (256) and of the halves and passes (128, 256)
+# layout's blocks; n and nq at the edges of the row tiles (256) and of the passes' two widths (128, 256 queries)
 @pytest.mark.parametrize("d,bits,mode,layout", [
     (128, 1, tq.TQ_MSE, None), (257, 1, tq.TQ_PROD, None), (200, 2, tq.TQ_MSE, None), (384, 2, tq.TQ_PROD, None), (200, 3, tq.TQ_PROD, None),
     (136, 3, tq.TQ_MSE, None), (130, 4, tq.TQ_MSE, None), (768, 4, tq.TQ_PROD, None), (200, 4, tq.TQ_PROD, NIB), (1000, 4, tq.TQ_PROD, NIB),
-    (1536, 4, tq.TQ_PROD, NIB), (3072, 2, tq.TQ_PROD, None)])
-@pytest.mark.parametrize("n,nq,k", [(65_536, 193, 100), (65_793, 513, 1)])
+    (1536, 4, tq.TQ_PROD, NIB), (3072, 2, tq.TQ_PROD, None), (1537, 1, tq.TQ_MSE, None)])
+@pytest.mark.parametrize("n,nq,k", [(65_537, 65, 10), (70_000, 128, 1), (65_536, 193, 100), (65_793, 513, 1)])
 def test_screened_search_is_the_dense_one(d, bits, mode, layout, n, nq, k):
     su = P.Setup(d, bits, mode, layout=layout)
     g = torch.Generator(device=DEV).manual_seed(d + nq)
@@ -35,10 +35,11 @@ def test_screened_search_is_the_dense_one(d, bits, mode, layout, n, nq, k):
     check(su, Q, n, su.quantize(X), k)
 
 
-def test_rows_and_queries_that_the_bounds_do_not_cover():
+@pytest.mark.parametrize("nq", [80, 200])
+def test_rows_and_queries_that_the_bounds_do_not_cover(nq):
     """Norms and gammas outside what the fp16 operands hold, a query of zeros, one of very large and one of very small entries, and
     rows that are all alike (more candidates than the lists hold: every row is scored)."""
-    n, d, nq, k = 65_600, 200, 200, 10
+    n, d, k = 65_600, 200, 10
     su = P.Setup(d, 3, tq.TQ_PROD)
     g = torch.Generator(device=DEV).manual_seed(1)
     X, Q = torch.randn((n, d), generator=g, device=DEV), torch.randn((nq, d), generator=g, device=DEV)
@@ -55,4 +56,4 @@ def test_rows_and_queries_that_the_bounds_do_not_cover():
     Q[9] *= 1e-25
     check(su, Q, n, (idx, qjl, gamma, norms), k)
     same = su.quantize(X[:1].expand(n, d).contiguous())
-    check(su, Q[:195], n, same, k)
+    check(su, Q[:nq - 5], n, same, k)
