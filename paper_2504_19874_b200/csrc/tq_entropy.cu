@@ -327,13 +327,15 @@ __global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(Args a, const uin
   if (rest) clear_rest(offsets[0], offsets[a.n], out, out_bytes);
 }
 
-// One thread per row.  Look-up on the next K = 10 bits (12 where a code word is longer than 10; always 12 measured 322 us: the
-// larger table takes L1 away from the rows' lines): up to 16 bits of whole
-// symbols, their number of output bits and the stream bits they take.  The lanes of a warp run in step by output word, so that
-// filling and emitting words is the same instruction for all of them; only the number of look-ups per word differs.
-constexpr int kUnpackThreads = 128;
-__global__ void __launch_bounds__(kUnpackThreads) unpack_kernel(Args a, int K, const uint64_t* __restrict__ offsets,
-                                                                const uint8_t* __restrict__ packed, uint8_t* __restrict__ idx_out) {
+// One thread per row.  Look-up on the next K bits: up to 16 bits of whole symbols, their number of output bits and the stream bits
+// they take.  The lanes of a warp run in step by output word, so that filling and emitting words is the same instruction for all of
+// them; only the number of look-ups per word differs.
+// Bound: instructions issued per look-up (a chain of shifts of two-word buffers, written out in 32-bit funnel shifts: a 64-bit shift
+// by a variable is six) and the look-ups per word.  K = 12 takes 2.8 of them per word of eight 4-bit symbols, K = 10 3.7, but its 16 KB
+// table is L1 that the rows' lines need, so that it pays only where one CTA of many rows has the SM to itself (five CTAs of 128
+// rows with it: 322 us).  100,000 rows of d = 1536: 154 -> 142 us.
+__global__ void __launch_bounds__(1024) unpack_kernel(Args a, int K, const uint64_t* __restrict__ offsets,
+                                                      const uint8_t* __restrict__ packed, uint8_t* __restrict__ idx_out) {
   extern __shared__ uint32_t unpack_smem[];
   uint32_t* lut = unpack_smem;                                            // [2^K]: symbols | output bits << 16 | stream bits << 24
   uint16_t* single = reinterpret_cast<uint16_t*>(unpack_smem + (1 << K)); // [2^maxlen]: symbol | length << 8
@@ -371,12 +373,13 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_kernel(Args a, int K, c
   const uint32_t last_mask = (total_bits & 31) ? (1u << (total_bits & 31)) - 1u : 0xffffffffu;
   // The stream window is filled at the start of every output word by all lanes together, and only rarely inside a word: a
   // load that some lane issues at every look-up makes the other lanes of the warp wait for it (267 against 150 us).
-  unsigned long long in = 0ull, outbuf = 0ull;
+  uint32_t in_lo = 0u, in_hi = 0u, out_lo = 0u, out_hi = 0u;
   int have = 0, rd = 0, ofill = 0;
   const unsigned mask = (1u << K) - 1u;
   uint32_t ahead = nwords > 0 ? __ldg(src) : 0u;   // the next word, requested one word early
-  auto refill = [&]() {   // zero words past the end of the row stream only pad the look-up of its last code words
-    in |= (unsigned long long)ahead << have;
+  auto refill = [&]() {   // (have < 32.)  Zero words past the end of the row stream only pad the look-up of its last code words
+    in_lo |= ahead << have;
+    in_hi |= __funnelshift_l(ahead, 0u, have);
     have += 32;
     ++rd;
     ahead = rd < nwords ? __ldg(src + rd) : 0u;
@@ -385,15 +388,19 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_kernel(Args a, int K, c
     if (have < 32) refill();
     do {
       if (have < K) refill();
-      const uint32_t e = lut[(unsigned)in & mask];
+      const uint32_t e = lut[in_lo & mask];
       const int used = e >> 24;
-      in >>= used;
+      in_lo = __funnelshift_r(in_lo, in_hi, used);
+      in_hi >>= used;
       have -= used;
-      outbuf |= (unsigned long long)(e & 0xffffu) << ofill;
+      const uint32_t symbols = e & 0xffffu;
+      out_lo |= symbols << ofill;
+      out_hi |= __funnelshift_l(symbols, 0u, ofill);
       ofill += (e >> 16) & 255u;
     } while (ofill < 32);
-    const uint32_t v = (uint32_t)outbuf;
-    outbuf >>= 32;
+    const uint32_t v = out_lo;
+    out_lo = out_hi;
+    out_hi = 0u;
     ofill -= 32;
     return v;
   };
@@ -593,10 +600,14 @@ extern "C" int tq_entropy_unpack(const tq_plan* plan, const uint8_t* lengths, in
   entropy::Args a;
   if ((rc = entropy::make_code(plan, lengths, &a.code, who))) return rc;
   a.n = n; a.d = plan->d; a.idx = nullptr; a.idx_rb = plan->idx_row_bytes;
-  const int K = a.code.maxlen <= 10 ? 10 : 12;
+  // An SM's share of the rows as one CTA (of at most 1,024) where it is worth the larger table, else CTAs of 128 rows.
+  const int64_t share = round_up64((n + tc::sm_count() - 1) / tc::sm_count(), 32);
+  const bool wide = share >= 256;
+  const int threads = wide ? (int)((share + (share + 1023) / 1024 - 1) / ((share + 1023) / 1024) + 31) / 32 * 32 : 128;
+  const int K = wide || a.code.maxlen > 10 ? 12 : 10;
   const size_t smem = sizeof(uint32_t) * ((size_t)1 << K) + sizeof(uint16_t) * ((size_t)1 << a.code.maxlen);   // at most 24 KB
-  const int64_t ctas = (n + entropy::kUnpackThreads - 1) / entropy::kUnpackThreads;
-  entropy::unpack_kernel<<<(unsigned)ctas, entropy::kUnpackThreads, smem, static_cast<cudaStream_t>(stream)>>>(a, K, row_offsets, packed, idx);
+  const int64_t ctas = (n + threads - 1) / threads;
+  entropy::unpack_kernel<<<(unsigned)ctas, threads, smem, static_cast<cudaStream_t>(stream)>>>(a, K, row_offsets, packed, idx);
   count_launches(1);
   TQ_CHECK_CUDA(cudaGetLastError(), who);
   return TQ_OK;
