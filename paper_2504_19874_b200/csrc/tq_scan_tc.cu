@@ -1120,7 +1120,7 @@ int prepare_group(const tq_plan* plan, const float* Qcat, int nqg, void* workspa
   const int queries = (nqg + kQueriesPerPass - 1) / kQueriesPerPass * kQueriesPerPass;   // absent ones get zero rows
   const int words = (g.kba + g.kbs) * 32;
   // shares of an operand: one round of 256 words each, fewer rounds than that only where the queries fill the chip
-  const int shares = std::max(1, std::min((words + 255) / 256, 4 * tc::sm_count() / queries));
+  const int shares = std::max(1, std::min((words + 255) / 256, 16 * tc::sm_count() / queries));
   count_launches(1);
   const dim3 grid((unsigned)queries, (unsigned)shares);
   TQ_CHECK_CUDA(g.nib ? launch_dependent(toperand_kernel<true>, grid, dim3(256), 0, st, a)
