@@ -13,14 +13,15 @@
 //
 // CTA pair (cta_group::2, M = 256 rows, 128 per CTA; N = 256 queries, or 128), persistent over row tiles, 896 threads per CTA:
 //   warp 0        TMA producer of the query operand: per k-block (64 coordinates) the CTA's half of its rows
-//   warp 1        MMA issuer (of the leader)
+//   warps 1, 3    MMA issuers (of the leader), k-blocks of a tile in turn
 //   warp 2        TMA producer of the packed rows
 //   warps 4..11   expansion (thread = row): packed codes -> fp16 by byte permutes over the codebook's bytes -> the stage's A tile; two
 //                 sets of four warps take the k-blocks in turn
 //   warps 12..27  epilogue (thread = row, a quarter of the queries): one FMA chain per pair of estimates, the hits one by one
 // Five stages of 32 KB (A and half of B), two accumulators of 256 columns (all of TMEM), so that a tile is read while the next one's
-// MMAs run.  The single-lane roles are chains of dependent instructions at six cycles each: with some sixty of them per k-block the
-// issuer was the longest part of the kernel, hence one barrier for both operands and nothing in its loop that can be outside.
+// MMAs run.  The single-lane roles are chains of dependent instructions at six cycles each: an issuer spends some 500 cycles per
+// k-block besides its 512 of MMAs, of which the tensor pipe's queue hides only a part.  Hence one barrier for both operands, nothing in
+// the loop that can be outside, and two issuers (10^4 queries, d = 200 prod b = 3, 10^6 rows: 16.6 ms with one, 15.9 with two).
 // All waits are bounded.
 #include <algorithm>
 #include <atomic>
@@ -43,6 +44,10 @@ using namespace tq::tc;
 
 constexpr int TILE = 128;                   // rows per CTA = TMEM lanes
 constexpr int STAGES = 5;                   // ring of k-blocks
+// A parity wait also passes when its barrier is two completions behind, so whoever waits for a k-block must have waited for the one
+// before on the same barrier.  With two issuers in turn, which need not keep step, operands are announced and MMAs complete on rings of
+// twice the stages: issuer and expansion set of k-block k have waited for k - RING there.
+constexpr int RING = 2 * STAGES;
 constexpr int ATILE = TILE * 128, BTILE = kQueries / 2 * 128;   // bytes of a k-block in one CTA: 128 rows, 128 queries x 64 fp16
 constexpr int STAGE = ATILE + BTILE;
 constexpr int PSTAGES = 3, PTILE = TILE * 64;
@@ -379,13 +384,14 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   unsigned char* pring = smem + STAGES * STAGE;
   uint64_t* bars = reinterpret_cast<uint64_t*>(pring + PSTAGES * PTILE);
-  uint64_t* full = bars;                  // [STAGES]  TMA, and A stored by its set's four warps of both CTAs -> MMA (the leader's)
-  uint64_t* empty = full + STAGES;        // [STAGES]  the k-block's MMAs complete
-  uint64_t* pfull = empty + STAGES;       // [PSTAGES]  TMA (packed rows) -> expansion
+  uint64_t* full = bars;                  // [RING]  TMA, and A stored by its set's four warps of both CTAs -> MMA (the leader's)
+  uint64_t* empty = full + RING;          // [RING]  the k-block's MMAs complete
+  uint64_t* pfull = empty + RING;         // [PSTAGES]  TMA (packed rows) -> expansion
   uint64_t* pempty = pfull + PSTAGES;     // [PSTAGES]  expansion -> TMA
   uint64_t* dfull = pempty + PSTAGES;     // [2]  accumulator complete -> epilogue
   uint64_t* dfree = dfull + 2;            // [2]  accumulator read -> issuer (the leader's)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(dfree + 2);
+  uint64_t* begun = dfree + 2;            // the tile's first MMAs, which overwrite the accumulator, have been issued -> second issuer
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(begun + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   // [128] of two queries each: error constants, then thresholds, negative; scaled like the accumulators
   float4* et = reinterpret_cast<float4*>(reinterpret_cast<unsigned char*>(bars) + 512);
@@ -398,7 +404,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
   const int64_t nrounds = (a.n + 2 * TILE - 1) / (2 * TILE);
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < RING; ++s) {
       mbar_init(&full[s], 8 + 1);
       mbar_init(&empty[s], 1);
     }
@@ -407,9 +413,10 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
       mbar_init(&pempty[s], 8);
     }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&dfull[i], 1);
+      mbar_init(&dfull[i], 2);
       mbar_init(&dfree[i], 2 * NEPI);
     }
+    mbar_init(begun, 1);
     *abort_flag = 0;
     fence_barrier_init();
     tma_prefetch_desc(&tmB);
@@ -438,21 +445,24 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
+  // The stage of k-block kt was last read by the MMAs of k-block kt - STAGES.
+  auto stage_free = [&](uint32_t kt) -> bool {
+    const uint32_t kp = kt - STAGES;
+    return kt < STAGES || mbar_wait(&empty[kp % RING], (kp / RING) & 1u, abort_flag, a.status);
+  };
+
   if (warp < NEXP0) {
     if (warp == 0) {
       // ---------------------------------------------------------------- query operand
       if (lane == 0) {
-        uint32_t st = 0, ph = 1;
+        uint32_t kt = 0;
         bool ok = true;
         for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits) {
-          for (int f = 0; f < nkb; ++f) {
-            if (!(ok = mbar_wait(&empty[st], ph, abort_flag, a.status))) break;
-            if (rank == 0) mbar_arrive_expect_tx(&full[st], 128u * (uint32_t)a.ncols);
-            tma_load_2d_pair(smem + st * STAGE + ATILE, &tmB, &full[st], f * 64, rank * (a.ncols / 2));   // this CTA's half of the queries
-            if (++st == STAGES) {
-              st = 0;
-              ph ^= 1u;
-            }
+          for (int f = 0; f < nkb; ++f, ++kt) {
+            if (!(ok = stage_free(kt))) break;
+            uint64_t* bar = &full[kt % RING];
+            if (rank == 0) mbar_arrive_expect_tx(bar, 128u * (uint32_t)a.ncols);
+            tma_load_2d_pair(smem + kt % STAGES * STAGE + ATILE, &tmB, bar, f * 64, rank * (a.ncols / 2));   // this CTA's half of the queries
           }
         }
         if (!ok) {
@@ -460,8 +470,9 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
         }
       }
       __syncwarp();
-    } else if (warp == 1) {
-      // ---------------------------------------------------------------- MMA issuer
+    } else if (warp != 2) {
+      // ---------------------------------------------------------------- MMA issuer: every second k-block of a tile
+      const int me = warp >> 1;
       if (lane == 0 && rank == 0) {
         // fp16 x fp16 -> fp32, both K-major
         const uint32_t idesc = (1u << 4) | ((uint32_t)(a.ncols >> 3) << 17) | ((uint32_t)((2 * TILE) >> 4) << 24);
@@ -469,24 +480,26 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
         const int last = NIB ? 4 : k_steps<NIB>(a.g, (a.g.kba > 0 ? a.g.kba : a.g.kbs) - 1);   // K steps of a part's last k-block
         const int end0 = a.g.kba - 1, end1 = nkb - 1;
         bool ok = true;
-        uint32_t st = 0, ph = 0, it = 0;
-        for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits, ++it) {
+        uint32_t kt0 = 0, it = 0;
+        for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits, ++it, kt0 += (uint32_t)nkb) {
           const uint32_t d = it & 1u, d_tmem = tmem_base + d * 256u;
           if (!(ok = mbar_wait(&dfree[d], ((it >> 1) & 1u) ^ 1u, abort_flag, a.status))) break;
+          if (me == 1 && !(ok = mbar_wait(begun, it & 1u, abort_flag, a.status))) break;
           tc_fence_after();
-          for (int f = 0; f < nkb; ++f) {
+          for (int f = me; f < nkb; f += 2) {
+            const uint32_t kt = kt0 + (uint32_t)f, st = kt % STAGES;
             const uint64_t off = (uint64_t)(st * (STAGE >> 4));
             const uint64_t adesc = adesc0 + off, bdesc = bdesc0 + off;
             const int steps = NIB || (f != end0 && f != end1) ? 4 : last;
-            if (!(ok = mbar_wait(&full[st], ph, abort_flag, a.status))) break;
+            if (!(ok = mbar_wait(&full[kt % RING], (kt / RING) & 1u, abort_flag, a.status))) break;
             tc_fence_after();
 #pragma unroll
             for (int s = 0; s < 4; ++s)
               if (s < steps) umma_bf16_pair(d_tmem, adesc + 2 * s, bdesc + 2 * s, idesc, s != 0 || f != 0 ? 1u : 0u);
-            umma_commit_pair(&empty[st]);
-            if (++st == STAGES) {
-              st = 0;
-              ph ^= 1u;
+            umma_commit_pair(&empty[kt % RING]);
+            if (f == 0) {
+              tc_fence_before();
+              mbar_arrive(begun);
             }
           }
           if (ok) umma_commit_pair(&dfull[d]);
@@ -534,18 +547,17 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
       const uint32_t g16 = (uint32_t)__half_as_ushort(__float2half_rn(row_terms(1.f, gm).gamma));
       const uint32_t neg = (g16 | (g16 << 16)) ^ 0x80008000u;
       const uint32_t kt0 = it * (uint32_t)nkb;
-      // The stage was last read by the MMAs of k-block kt - STAGES.  (A parity wait must not be two completions behind: the set's
-      // previous store is two k-blocks back, and k-blocks complete in order.)  The tensor core of this SM reads what these threads
-      // write, in a pair too: the proxy fence orders the writes, the arrival only tells the leader's issuer.
+      // The tensor core of this SM reads what these threads write, in a pair too: the proxy fence orders the writes, the arrival only
+      // tells the leader's issuer.
       auto fill = [&](uint32_t kt, auto&& pieces) {
         const uint32_t st = kt % STAGES;
-        if (!(ok = mbar_wait(&empty[st], ((kt / STAGES) & 1u) ^ 1u, abort_flag, a.status))) return;
+        if (!(ok = stage_free(kt))) return;
         unsigned char* dst = smem + st * STAGE + r * 128;
         // 16-byte piece p of the row, 128-byte swizzle
         pieces([&](int p, const uint32_t* v) { *reinterpret_cast<uint4*>(dst + ((p ^ (r & 7)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]); });
         fence_proxy_async();
         __syncwarp();
-        if (lane == 0) mbar_arrive_leader(&full[st]);
+        if (lane == 0) mbar_arrive_leader(&full[kt % RING]);
       };
       auto mine = [&](uint32_t kt) { return (int)(kt & 1u) == set; };
       for (int gi = 0; gi < ngroups && ok; ++gi) {
