@@ -322,12 +322,15 @@ __device__ __forceinline__ RowGroup row_group(const Geo& g, int gi) {
   }
   return rg;
 }
-// K steps of 16 coordinates that k-block f needs.
-template <bool NIB>
+// K steps of 16 elements that k-block f needs.  A step holds 16 neighbouring codes of two bits or more; of one-bit streams, half of the
+// pairs (b, b + 16) of a word: with 9 to 15 coordinates of a word both of its steps.
+template <int BM, bool NIB>
 __device__ __forceinline__ int k_steps(const Geo& g, int f) {
   if (NIB) return 4;
-  const int kb = f < g.kba ? f : f - g.kba;
-  return min(4, (g.d - 64 * kb + 15) >> 4);
+  const int left = g.d - 64 * (f < g.kba ? f : f - g.kba);
+  if (left >= 64) return 4;
+  if (f < g.kba && BM >= 2) return (left + 15) >> 4;
+  return 2 * (left >> 5) + ((left & 31) == 0 ? 0 : (left & 31) <= 8 ? 1 : 2);
 }
 
 // Eight selectors (nibbles 0..7) -> eight fp16 centroids in natural order.
@@ -477,8 +480,9 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
         // fp16 x fp16 -> fp32, both K-major
         const uint32_t idesc = (1u << 4) | ((uint32_t)(a.ncols >> 3) << 17) | ((uint32_t)((2 * TILE) >> 4) << 24);
         const uint64_t adesc0 = smem_desc_sw128(smem_u32(smem)), bdesc0 = smem_desc_sw128(smem_u32(smem + ATILE));
-        const int last = NIB ? 4 : k_steps<NIB>(a.g, (a.g.kba > 0 ? a.g.kba : a.g.kbs) - 1);   // K steps of a part's last k-block
+        // K steps of the parts' last k-blocks
         const int end0 = a.g.kba - 1, end1 = nkb - 1;
+        const int last0 = k_steps<BM, NIB>(a.g, max(end0, 0)), last1 = k_steps<BM, NIB>(a.g, end1);
         bool ok = true;
         uint32_t kt0 = 0, it = 0;
         for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits, ++it, kt0 += (uint32_t)nkb) {
@@ -490,7 +494,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
             const uint32_t kt = kt0 + (uint32_t)f, st = kt % STAGES;
             const uint64_t off = (uint64_t)(st * (STAGE >> 4));
             const uint64_t adesc = adesc0 + off, bdesc = bdesc0 + off;
-            const int steps = NIB || (f != end0 && f != end1) ? 4 : last;
+            const int steps = NIB ? 4 : f == end0 ? last0 : f == end1 ? last1 : 4;
             if (!(ok = mbar_wait(&full[kt % RING], (kt / RING) & 1u, abort_flag, a.status))) break;
             tc_fence_after();
 #pragma unroll
@@ -591,6 +595,8 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
         __syncwarp();
         if (lane == 0) mbar_arrive(&pempty[pst]);
         const uint32_t kt = kt0 + (uint32_t)rg.f0;
+        // 16-byte pieces of a row that the K steps of the group's k-block j read (d = 200: 2 of 8 in each part's last one)
+        auto pieces_of = [&](int j) { return 2 * k_steps<BM, NIB>(a.g, rg.f0 + j); };
         if (NIB) {
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
@@ -620,8 +626,10 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
           for (int j = 0; j < 4; ++j) {
             if (ok && j < rg.cnt && mine(kt + j))
               fill(kt + j, [&](auto&& put) {
+                const int pieces = pieces_of(j);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {   // bits b and b + 16 of a word are a pair
+                  if (i >= pieces) break;
                   uint32_t v[4];
 #pragma unroll
                   for (int p = 0; p < 4; ++p) v[p] = pair ^ ((w[2 * j + (i >> 2)] << (15 - 4 * (i & 3) - p)) & 0x80008000u);
@@ -634,9 +642,11 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
           for (int j = 0; j < a_group_kb(BM); ++j) {
             if (ok && j < rg.cnt && mine(kt + j))
               fill(kt + j, [&](auto&& put) {
+                const int pieces = pieces_of(j);
                 if (BM == 2) {
 #pragma unroll
                   for (int i = 0; i < 4; ++i) {
+                    if (2 * i >= pieces) break;
                     uint32_t v[8];
                     centroids16_two(a.tab, w[4 * j + i], v);
                     put(2 * i, v);
@@ -649,6 +659,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
                     const uint32_t sel[4] = {x[0], __funnelshift_r(x[0], x[1], 24), __funnelshift_r(x[1], x[2], 16), x[2] >> 8};
 #pragma unroll
                     for (int p = 0; p < 4; ++p) {
+                      if (4 * i + p >= pieces) break;
                       uint32_t v[4];
                       centroids8(a.tab, spread3(sel[p] & 0xffffffu), v);
                       put(4 * i + p, v);
@@ -657,6 +668,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
                 } else {
 #pragma unroll
                   for (int i = 0; i < 8; ++i) {
+                    if (i >= pieces) break;
                     uint32_t v[4];
                     centroids8_wide(a.tab, w[8 * j + i], v);
                     put(i, v);

@@ -21,12 +21,13 @@ def check(su, Q, n, codes, k):
     assert torch.equal(ts, order.values[:, :k]) and torch.equal(ti.long(), order.indices[:, :k])
 
 
-# one to four bits with and without signs; d at the edges of K steps (16), k-blocks (64), row groups (128, 256) and of the nibble
+# one to four bits with and without signs; d at the edges of K steps (16; one-bit streams 8, 16, 32), k-blocks (64), row groups (128, 256) and of the nibble
 # layout's blocks; n and nq at the edges of the row tiles (256) and of the passes' two widths (128, 256 queries)
 @pytest.mark.parametrize("d,bits,mode,layout", [
     (128, 1, tq.TQ_MSE, None), (257, 1, tq.TQ_PROD, None), (200, 2, tq.TQ_MSE, None), (384, 2, tq.TQ_PROD, None), (200, 3, tq.TQ_PROD, None),
     (136, 3, tq.TQ_MSE, None), (130, 4, tq.TQ_MSE, None), (768, 4, tq.TQ_PROD, None), (200, 4, tq.TQ_PROD, NIB), (1000, 4, tq.TQ_PROD, NIB),
-    (1536, 4, tq.TQ_PROD, NIB), (3072, 2, tq.TQ_PROD, None), (1537, 1, tq.TQ_MSE, None)])
+    (1536, 4, tq.TQ_PROD, NIB), (3072, 2, tq.TQ_PROD, None), (1537, 1, tq.TQ_MSE, None),
+    (139, 3, tq.TQ_PROD, None), (171, 4, tq.TQ_PROD, None), (139, 1, tq.TQ_MSE, None), (207, 2, tq.TQ_PROD, None)])
 @pytest.mark.parametrize("n,nq,k", [(65_537, 65, 10), (70_000, 128, 1), (65_536, 193, 100), (65_793, 513, 1)])
 def test_screened_search_is_the_dense_one(d, bits, mode, layout, n, nq, k):
     su = P.Setup(d, bits, mode, layout=layout)
