@@ -595,8 +595,6 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
         __syncwarp();
         if (lane == 0) mbar_arrive(&pempty[pst]);
         const uint32_t kt = kt0 + (uint32_t)rg.f0;
-        // 16-byte pieces of a row that the K steps of the group's k-block j read (d = 200: 2 of 8 in each part's last one)
-        auto pieces_of = [&](int j) { return 2 * k_steps<BM, NIB>(a.g, rg.f0 + j); };
         if (NIB) {
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
@@ -626,10 +624,8 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
           for (int j = 0; j < 4; ++j) {
             if (ok && j < rg.cnt && mine(kt + j))
               fill(kt + j, [&](auto&& put) {
-                const int pieces = pieces_of(j);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {   // bits b and b + 16 of a word are a pair
-                  if (i >= pieces) break;
                   uint32_t v[4];
 #pragma unroll
                   for (int p = 0; p < 4; ++p) v[p] = pair ^ ((w[2 * j + (i >> 2)] << (15 - 4 * (i & 3) - p)) & 0x80008000u);
@@ -642,11 +638,9 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
           for (int j = 0; j < a_group_kb(BM); ++j) {
             if (ok && j < rg.cnt && mine(kt + j))
               fill(kt + j, [&](auto&& put) {
-                const int pieces = pieces_of(j);
                 if (BM == 2) {
 #pragma unroll
                   for (int i = 0; i < 4; ++i) {
-                    if (2 * i >= pieces) break;
                     uint32_t v[8];
                     centroids16_two(a.tab, w[4 * j + i], v);
                     put(2 * i, v);
@@ -659,7 +653,6 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
                     const uint32_t sel[4] = {x[0], __funnelshift_r(x[0], x[1], 24), __funnelshift_r(x[1], x[2], 16), x[2] >> 8};
 #pragma unroll
                     for (int p = 0; p < 4; ++p) {
-                      if (4 * i + p >= pieces) break;
                       uint32_t v[4];
                       centroids8(a.tab, spread3(sel[p] & 0xffffffu), v);
                       put(4 * i + p, v);
@@ -668,7 +661,6 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
                 } else {
 #pragma unroll
                   for (int i = 0; i < 8; ++i) {
-                    if (i >= pieces) break;
                     uint32_t v[4];
                     centroids8_wide(a.tab, w[8 * j + i], v);
                     put(i, v);
