@@ -737,6 +737,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
           while (hits != 0u) {   // a lane takes its own hits one after the other
             const int i = __ffs((int)hits) - 1, q = q0 + 8 * g + i;
             hits &= hits - 1u;
+            if (q >= a.nqp) break;   // absent queries have no list: rho E is NaN for them where a row's bound is infinite
             const float x0 = (i & 1) ? v[8 * g + 1] : v[8 * g], x1 = (i & 1) ? v[8 * g + 3] : v[8 * g + 2];
             const float x2 = (i & 1) ? v[8 * g + 5] : v[8 * g + 4], x3 = (i & 1) ? v[8 * g + 7] : v[8 * g + 6];
             const float y0 = (i & 2) ? x1 : x0, y1 = (i & 2) ? x3 : x2, val = (i & 4) ? y1 : y0;
@@ -748,7 +749,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
               lbuf[q * LBUF + ls] = make_uint2(__float_as_uint(low), (uint32_t)row);
             } else {   // the CTA's buffer is full: straight to the list
               const int slot = atomicAdd(a.count + q, 1);
-              if (slot < a.cap) {
+              if (slot < a.cap && TQ_DEVICE_CHECK(slot >= 0 && row < a.n, a.status)) {
                 a.cand_s[(int64_t)q * a.cap + slot] = fmaxf(low * unscale[q], -FLT_MAX);
                 a.cand_i[(int64_t)q * a.cap + slot] = (int)row;
               }
@@ -775,7 +776,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
       base = __shfl_sync(0xffffffffu, base, 0);
       for (int i = lane; i < m; i += 32) {
         const int slot = base + i;
-        if (slot < a.cap) {
+        if (slot < a.cap && TQ_DEVICE_CHECK(slot >= 0, a.status)) {
           const uint2 e = lbuf[q * LBUF + i];
           a.cand_s[(int64_t)q * a.cap + slot] = fmaxf(__uint_as_float(e.x) * unscale[q], -FLT_MAX);   // (not finite: no lower bound)
           a.cand_i[(int64_t)q * a.cap + slot] = (int)e.y;

@@ -58,3 +58,24 @@ def test_rows_and_queries_that_the_bounds_do_not_cover(nq):
     check(su, Q, n, (idx, qjl, gamma, norms), k)
     same = su.quantize(X[:1].expand(n, d).contiguous())
     check(su, Q[:nq - 5], n, same, k)
+
+
+@pytest.mark.parametrize("value", [-1.0, float("inf")])
+@pytest.mark.parametrize("nq", [65, 80, 300])
+def test_a_block_of_rows_that_the_bounds_do_not_cover(nq, value):
+    """More such rows in one CTA's share than it collects per query: absent queries (up to the next multiple of 32) have no list, and nothing
+    outside the outputs and the workspace changes, whatever the workspace held before."""
+    n, d, k, pad = 65_600, 200, 10, 1 << 20
+    su = P.Setup(d, 3, tq.TQ_PROD)
+    g = torch.Generator(device=DEV).manual_seed(nq)
+    X, Q = torch.randn((n, d), generator=g, device=DEV), torch.randn((nq, d), generator=g, device=DEV)
+    codes = su.quantize(X)
+    codes[3][1000:1200] = value
+    ts, ti = torch.empty((nq, k), device=DEV), torch.empty((nq, k), dtype=torch.int32, device=DEV)
+    need = (tq.tq_workspace_bytes(su.plan, tq.TQ_OP_TOPK, n, nq, k) + 255) // 256 * 256
+    whole = torch.full((need + 2 * pad,), 0xBF, dtype=torch.uint8, device=DEV)
+    tq.tq_topk(su.plan, Q, n, *codes, k, ts, ti, whole[pad:pad + need])
+    tq.tq_plan_status(su.plan)
+    assert bool((whole[:pad] == 0xBF).all()) and bool((whole[pad + need:] == 0xBF).all())
+    order = torch.sort(su.score(Q, n, *codes), dim=1, descending=True, stable=True)
+    assert torch.equal(ts, order.values[:, :k]) and torch.equal(ti.long(), order.indices[:, :k])
