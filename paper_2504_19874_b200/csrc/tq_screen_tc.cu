@@ -13,15 +13,17 @@
 //
 // CTA pair (cta_group::2, M = 256 rows, 128 per CTA; N = 256 queries, or 128), persistent over row tiles, 896 threads per CTA:
 //   warp 0        TMA producer of the query operand: per k-block (64 coordinates) the CTA's half of its rows
-//   warps 1, 3    MMA issuers (of the leader), k-blocks of a tile in turn
+//   warp 1        MMA issuer (of the leader)
 //   warp 2        TMA producer of the packed rows
 //   warps 4..11   expansion (thread = row): packed codes -> fp16 by byte permutes over the codebook's bytes -> the stage's A tile; two
 //                 sets of four warps take the k-blocks in turn
 //   warps 12..27  epilogue (thread = row, a quarter of the queries): one FMA chain per pair of estimates, the hits one by one
 // Five stages of 32 KB (A and half of B), two accumulators of 256 columns (all of TMEM), so that a tile is read while the next one's
-// MMAs run.  The single-lane roles are chains of dependent instructions at six cycles each: an issuer spends some 500 cycles per
-// k-block besides its 512 of MMAs, of which the tensor pipe's queue hides only a part.  Hence one barrier for both operands, nothing in
-// the loop that can be outside, and two issuers (10^4 queries, d = 200 prod b = 3, 10^6 rows: 16.6 ms with one, 15.9 with two).
+// MMAs run.  The single-lane roles are chains of dependent instructions at six cycles each, of which the tensor pipe's queue hides only
+// a part: with 128 columns the issuer's chain is longer than a k-block's 256 cycles of MMAs.  Hence one barrier for both operands and
+// counters instead of divisions in its loop.  One thread issues all MMAs of an accumulator: those of two threads are in order only
+// where the threads order them, and handing every k-block's turn over a barrier costs more than the second issuer gains (65 queries,
+// 10^6 rows of d = 768 prod b = 4: 659 us, 635 with one issuer; 256 queries 849 and 807; 10^4 queries of d = 200 prod b = 3 alike, 16.5 ms).
 // All waits are bounded.
 #include <algorithm>
 #include <atomic>
@@ -45,8 +47,8 @@ using namespace tq::tc;
 constexpr int TILE = 128;                   // rows per CTA = TMEM lanes
 constexpr int STAGES = 5;                   // ring of k-blocks
 // A parity wait also passes when its barrier is two completions behind, so whoever waits for a k-block must have waited for the one
-// before on the same barrier.  With two issuers in turn, which need not keep step, operands are announced and MMAs complete on rings of
-// twice the stages: issuer and expansion set of k-block k have waited for k - RING there.
+// before on the same barrier.  The two expansion sets take every second k-block, so operands are announced and MMAs complete on rings
+// of twice the stages: the set of k-block k has waited for k - RING there.
 constexpr int RING = 2 * STAGES;
 constexpr int ATILE = TILE * 128, BTILE = kQueries / 2 * 128;   // bytes of a k-block in one CTA: 128 rows, 128 queries x 64 fp16
 constexpr int STAGE = ATILE + BTILE;
@@ -393,8 +395,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
   uint64_t* pempty = pfull + PSTAGES;     // [PSTAGES]  expansion -> TMA
   uint64_t* dfull = pempty + PSTAGES;     // [2]  accumulator complete -> epilogue
   uint64_t* dfree = dfull + 2;            // [2]  accumulator read -> issuer (the leader's)
-  uint64_t* begun = dfree + 2;            // the tile's first MMAs, which overwrite the accumulator, have been issued -> second issuer
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(begun + 1);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(dfree + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   // [128] of two queries each: error constants, then thresholds, negative; scaled like the accumulators
   float4* et = reinterpret_cast<float4*>(reinterpret_cast<unsigned char*>(bars) + 512);
@@ -416,10 +417,9 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
       mbar_init(&pempty[s], 8);
     }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&dfull[i], 2);
+      mbar_init(&dfull[i], 1);
       mbar_init(&dfree[i], 2 * NEPI);
     }
-    mbar_init(begun, 1);
     *abort_flag = 0;
     fence_barrier_init();
     tma_prefetch_desc(&tmB);
@@ -473,9 +473,8 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
         }
       }
       __syncwarp();
-    } else if (warp != 2) {
-      // ---------------------------------------------------------------- MMA issuer: every second k-block of a tile
-      const int me = warp >> 1;
+    } else if (warp == 1) {
+      // ---------------------------------------------------------------- MMA issuer
       if (lane == 0 && rank == 0) {
         // fp16 x fp16 -> fp32, both K-major
         const uint32_t idesc = (1u << 4) | ((uint32_t)(a.ncols >> 3) << 17) | ((uint32_t)((2 * TILE) >> 4) << 24);
@@ -484,26 +483,24 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
         const int end0 = a.g.kba - 1, end1 = nkb - 1;
         const int last0 = k_steps<BM, NIB>(a.g, max(end0, 0)), last1 = k_steps<BM, NIB>(a.g, end1);
         bool ok = true;
-        uint32_t kt0 = 0, it = 0;
-        for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits, ++it, kt0 += (uint32_t)nkb) {
+        uint32_t it = 0, st = 0, at = 0, ph = 0;   // stage and barrier of the next k-block
+        for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits, ++it) {
           const uint32_t d = it & 1u, d_tmem = tmem_base + d * 256u;
           if (!(ok = mbar_wait(&dfree[d], ((it >> 1) & 1u) ^ 1u, abort_flag, a.status))) break;
-          if (me == 1 && !(ok = mbar_wait(begun, it & 1u, abort_flag, a.status))) break;
-          tc_fence_after();
-          for (int f = me; f < nkb; f += 2) {
-            const uint32_t kt = kt0 + (uint32_t)f, st = kt % STAGES;
+          for (int f = 0; f < nkb; ++f) {
             const uint64_t off = (uint64_t)(st * (STAGE >> 4));
             const uint64_t adesc = adesc0 + off, bdesc = bdesc0 + off;
             const int steps = NIB ? 4 : f == end0 ? last0 : f == end1 ? last1 : 4;
-            if (!(ok = mbar_wait(&full[kt % RING], (kt / RING) & 1u, abort_flag, a.status))) break;
+            if (!(ok = mbar_wait(&full[at], ph, abort_flag, a.status))) break;
             tc_fence_after();
 #pragma unroll
             for (int s = 0; s < 4; ++s)
               if (s < steps) umma_bf16_pair(d_tmem, adesc + 2 * s, bdesc + 2 * s, idesc, s != 0 || f != 0 ? 1u : 0u);
-            umma_commit_pair(&empty[kt % RING]);
-            if (f == 0) {
-              tc_fence_before();
-              mbar_arrive(begun);
+            umma_commit_pair(&empty[at]);
+            if (++st == STAGES) st = 0;
+            if (++at == RING) {
+              at = 0;
+              ph ^= 1u;
             }
           }
           if (ok) umma_commit_pair(&dfull[d]);

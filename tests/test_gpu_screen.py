@@ -79,3 +79,15 @@ def test_a_block_of_rows_that_the_bounds_do_not_cover(nq, value):
     assert bool((whole[:pad] == 0xBF).all()) and bool((whole[pad + need:] == 0xBF).all())
     order = torch.sort(su.score(Q, n, *codes), dim=1, descending=True, stable=True)
     assert torch.equal(ts, order.values[:, :k]) and torch.equal(ti.long(), order.indices[:, :k])
+
+
+@pytest.mark.parametrize("d,bits,mode", [(128, 2, tq.TQ_MSE), (128, 1, tq.TQ_PROD), (128, 3, tq.TQ_PROD), (130, 4, tq.TQ_MSE), (256, 3, tq.TQ_MSE),
+                                         (320, 2, tq.TQ_MSE), (130, 3, tq.TQ_PROD)])
+def test_few_k_blocks_per_tile(d, bits, mode):
+    """Two to six k-blocks per tile, even and odd, and some fifty tiles per CTA pair: several tiles within the ring of stages, and expansion
+    sets and accumulators that take their turns at any place of it."""
+    n, nq, k = 1_000_000, 200, 10
+    su = P.Setup(d, bits, mode)
+    g = torch.Generator(device=DEV).manual_seed(d)
+    X, Q = torch.randn((n, d), generator=g, device=DEV), torch.randn((nq, d), generator=g, device=DEV)
+    check(su, Q, n, su.quantize(X), k)
