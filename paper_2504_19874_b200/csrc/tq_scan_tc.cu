@@ -840,6 +840,7 @@ struct RescoreArgs {
   const float* norms;
   float coef;
   const screen::QueryTerms* terms;
+  const float* tau;        // threshold of the listing
   const float* kth;        // lower bound of the k-th best estimate
   const int* count;        // candidates: (lower bound, row)
   const float* cand_s;
@@ -876,7 +877,7 @@ __global__ void __launch_bounds__(kRescoreThreads, 2) rescore_kernel(const __gri
   const int q = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool signs = a.g.kbs > 0 || a.g.nib;
   const int m = min(a.count[q], a.cap);
-  const float kth = a.kth[q], err = a.terms[q].err, unscale = a.terms[q].unscale;
+  const float kth = a.kth[q], err = a.terms[q].err, unscale = a.terms[q].unscale, slack = 2.f * screen::kThresholdSlack * fabsf(a.tau[q]);
   // four candidates of a thread at a time: the loads of their scalars are a chain of two round trips
   const int stride = kRescoreThreads * (int)gridDim.y;
   for (int i0 = blockIdx.y * kRescoreThreads + threadIdx.x; i0 < m; i0 += 4 * stride) {
@@ -895,7 +896,7 @@ __global__ void __launch_bounds__(kRescoreThreads, 2) rescore_kernel(const __gri
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const float high = low[u] + 2.f * screen::row_terms(nu[u], gm[u]).rho * err * unscale;
+      const float high = low[u] + slack + 2.f * screen::row_terms(nu[u], gm[u]).rho * err * unscale;
       if (i0 + u * stride < m && !(high < kth)) {
         const int s = atomicAdd(&s_n, 1);
         if (s < screen::kSurvivors) ids[s] = id[u];
@@ -1206,8 +1207,9 @@ int run_pass(const tq_plan* plan, int pass, int nqp, int64_t n, const uint8_t* i
 }
 
 int rescore(const tq_plan* plan, int nqp, const uint8_t* idx, const uint8_t* qjl, const float* gamma, const float* norms,
-            const void* workspace, const screen::QueryTerms* terms, const float* kth, const int* count, const float* cand_s,
-            const int* cand_i, int cap, float* out_s, int* out_i, int* out_count, int* overflow, cudaStream_t st, const char* who) {
+            const void* workspace, const screen::QueryTerms* terms, const float* tau, const float* kth, const int* count,
+            const float* cand_s, const int* cand_i, int cap, float* out_s, int* out_i, int* out_count, int* overflow, cudaStream_t st,
+            const char* who) {
   RescoreArgs a;
   a.g = make_geo(plan);
   a.hi_a = plan->nb.hi_a; a.hi_b = plan->nb.hi_b; a.lo_a = plan->nb.lo_a; a.lo_b = plan->nb.lo_b;
@@ -1220,6 +1222,7 @@ int rescore(const tq_plan* plan, int nqp, const uint8_t* idx, const uint8_t* qjl
   a.norms = norms;
   a.coef = plan->coef;
   a.terms = terms;
+  a.tau = tau;
   a.kth = kth;
   a.count = count;
   a.cand_s = cand_s;

@@ -739,8 +739,8 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
             const float x2 = (i & 1) ? v[8 * g + 5] : v[8 * g + 4], x3 = (i & 1) ? v[8 * g + 7] : v[8 * g + 6];
             const float y0 = (i & 2) ? x1 : x0, y1 = (i & 2) ? x3 : x2, val = (i & 4) ? y1 : y0;
             const float* pair = reinterpret_cast<const float*>(et + (q >> 1)) + (q & 1);
-            // the lower bound: val + tau - 2 rho E
-            const float low = fmaf(-2.f * t.rho, pair[0], val) - pair[2];
+            // the lower bound: val + tau - 2 rho E.  val is rounded on the grid of tau, which a row of small norm may lie far below.
+            const float low = fmaf(fabsf(pair[2]), -kThresholdSlack, fmaf(-2.f * t.rho, pair[0], val) - pair[2]);
             const int ls = atomicAdd(&lcnt[q], 1);
             if (ls < LBUF) {
               lbuf[q * LBUF + ls] = make_uint2(__float_as_uint(low), (uint32_t)row);

@@ -8,6 +8,9 @@ namespace screen {
 
 constexpr int kQueries = 256;          // queries per pass over the codes
 constexpr int kSurvivors = 2048;       // rows of a query that are scored again at most
+// Lower bounds of listed rows are formed by four operations whose results are no larger than |tau| and the row's own terms: half a
+// place each, 2^-22 |tau| in all (the row's own terms are covered by its error constant).  Twice that is taken off.
+constexpr float kThresholdSlack = 4.76837158e-7f;   // 2^-21
 
 // Bytes of workspace for one pass: the fp16 query operand and the per-query constants.
 size_t workspace_bytes(const tq_plan* plan);
@@ -17,7 +20,8 @@ int prepare(const tq_plan* plan, const float* Qcat, int nqp, void* workspace, cu
 
 // Bounds of the estimates of vectors [0, n) (vector i is row i step of the arrays).
 //   dense != nullptr: dense[q lds + i] = a lower bound of the estimate that the exact engines return for (query q, vector i)
-//   else: the vectors whose upper bound reaches tau[q] are appended to query q's list as (lower bound, row)
+//   else: the vectors whose upper bound reaches tau[q] are appended to query q's list as (lower bound, row); the upper bound is at most
+//         the lower one + 2 rho E + 2 kThresholdSlack |tau[q]|
 int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma, const float* norms,
         float* dense, int64_t lds, const float* tau, int* count, float* cand_s, int* cand_i, int cap, const void* workspace,
         cudaStream_t st, const char* who, int64_t step);

@@ -91,3 +91,17 @@ def test_few_k_blocks_per_tile(d, bits, mode):
     g = torch.Generator(device=DEV).manual_seed(d)
     X, Q = torch.randn((n, d), generator=g, device=DEV), torch.randn((nq, d), generator=g, device=DEV)
     check(su, Q, n, su.quantize(X), k)
+
+
+def test_norms_far_apart_and_negative_estimates():
+    """Every estimate is negative and a few rows have norms 10^8 below the others': bounds of theirs that are rounded on the grid of the
+    threshold would stand above their estimates.  They lie where the first sample does not look and the second does."""
+    n, d, nq, k = 70_000, 200, 128, 10
+    su = P.Setup(d, 3, tq.TQ_PROD)
+    g = torch.Generator(device=DEV).manual_seed(5)
+    X, Q = torch.randn((n, d), generator=g, device=DEV) + 2.0, 0.1 * torch.randn((nq, d), generator=g, device=DEV) - 1.0
+    codes = su.quantize(X)
+    codes[3].uniform_(0.5e8, 1e8, generator=g)
+    codes[3][4:4 + 16 * 200:16] = 1.0
+    assert bool((su.score(Q, n, *codes) < 0).all())
+    check(su, Q, n, codes, k)
