@@ -265,7 +265,8 @@ int tq_score_static_max_queries(const tq_plan* plan);
 /*
  * The k vectors with the largest estimate per query (nearest-neighbour search by estimated
  * inner product, Section 4.4), sorted by descending score, equal scores by ascending id.
- * The nq x n score matrix is never formed.
+ * The nq x n score matrix is never formed.  A row whose estimate is NaN (codes of a row with NaN entries) is not in the
+ * result; where fewer than k rows are left the tail is (-inf, -1).
  *   k 1..min(n, TQ_MAX_K);  top_scores device out [nq, k] floats;  top_ids device out [nq, k] int32
  */
 int tq_topk(const tq_plan* plan, const void* Q, int q_dtype, int nq, int64_t ldq, int64_t n,
@@ -276,8 +277,8 @@ int tq_topk(const tq_plan* plan, const void* Q, int q_dtype, int nq, int64_t ldq
  * The k best of m candidate (score, id) pairs per query, sorted like tq_topk's output (descending
  * score, equal scores by ascending id).  This is the merge step of a sharded search: every shard
  * returns its local top-k (the search of Section 4.4 is independent per database vector), the lists
- * are concatenated per query and reduced to the global top-k here.  Pairs with a negative id are
- * empty slots and are ignored; ids must be distinct within a query.
+ * are concatenated per query and reduced to the global top-k here.  Pairs with a negative id or a
+ * NaN score are empty slots and are ignored; ids must be distinct within a query.
  *   cand_scores, cand_ids  device, nq rows of m entries, row stride ld
  *   k 1..TQ_MAX_K;  top_scores / top_ids device out [nq, k] (may not alias the candidates);
  *   if fewer than k candidates exist the tail is filled with (-inf, -1)

@@ -632,7 +632,9 @@ struct SelArgs {
   int* clear_flag;
 };
 
+// 0: an empty slot, which a score that is not a number is too (it has no rank, and passes no filter).
 __device__ __forceinline__ unsigned long long make_key(float s, int id) {
+  if (isnan(s)) return 0ull;
   if (s == 0.f) s = 0.f;   // -0 and +0 tie
   uint32_t u = __float_as_uint(s);
   u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);

@@ -683,7 +683,8 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
     float nu_next = load(a.norms, unit * 2 + rank, 1.f), g_next = load(gsrc, unit * 2 + rank, 0.f);
     for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits, ++it) {
       const int64_t tile = rnd * 2 + rank, row = tile * TILE + r;
-      const bool row_ok = row < a.n;
+      // (a NaN scalar makes every estimate NaN, which no list holds)
+      const bool row_ok = row < a.n && (MODE == 0 || !(isnan(nu_next) || isnan(g_next)));
       const RowTerms t = row_terms(nu_next, g_next);
       nu_next = load(a.norms, tile + 2 * nunits, 1.f);
       g_next = load(gsrc, tile + 2 * nunits, 0.f);

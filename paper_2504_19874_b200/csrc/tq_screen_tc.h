@@ -28,7 +28,7 @@ int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8
 
 // What the estimate of row (nu, gamma) may differ from its screened value by, per unit of the query's error constant; the row's
 // values as the screening uses them.  A row that the bounds do not hold for (negative or non-finite norm or gamma, a norm near the
-// ends of the range of fp32) has nu 0 and an infinite bound: it passes every threshold.
+// ends of the range of fp32) has nu 0 and an infinite bound: it passes every threshold, unless a scalar of it is NaN.
 struct RowTerms {
   float nu, rho, gamma;
 };

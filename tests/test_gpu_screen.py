@@ -105,3 +105,30 @@ def test_norms_far_apart_and_negative_estimates():
     codes[3][4:4 + 16 * 200:16] = 1.0
     assert bool((su.score(Q, n, *codes) < 0).all())
     check(su, Q, n, codes, k)
+
+
+def spoilt(n, rows, spread, g):
+    """A block of `rows` rows, or as many spread over the index."""
+    return torch.randperm(n, generator=g, device=DEV)[:rows] if spread else torch.arange(1000, 1000 + rows, device=DEV)
+
+
+@pytest.mark.parametrize("n,nq", [(3000, 3), (3000, 40), (65_600, 8), (65_600, 40), (65_600, 80), (65_600, 300)])
+@pytest.mark.parametrize("rows,spread,gamma", [(100, True, False), (200, False, True), (1900, True, True), (5000, True, False), (40_000, False, False)])
+def test_rows_without_a_number(n, nq, rows, spread, gamma):
+    """Rows whose norm or residual norm is NaN are in no result, however many there are and whichever path the search takes: the exact
+    one below 65,536 rows, thresholds, or screening from 65 queries on.  Where nearly all rows are such, the tail is empty."""
+    d, k = 200, 10
+    rows = min(rows, n - 5 if rows == 40_000 else n // 2)
+    su = P.Setup(d, 3, tq.TQ_PROD)
+    g = torch.Generator(device=DEV).manual_seed(rows + nq)
+    X, Q = torch.randn((n, d), generator=g, device=DEV), torch.randn((nq, d), generator=g, device=DEV)
+    codes = su.quantize(X)
+    at = spoilt(n, rows, spread, g) if rows < n - 5 else torch.arange(rows, device=DEV)
+    codes[2 if gamma else 3][at] = float("nan")
+    ts, ti = su.topk(Q, n, *codes, k)
+    tq.tq_plan_status(su.plan)
+    scores = su.score(Q, n, *codes)
+    assert bool(scores[:, at].isnan().all()) and int(scores.isnan().sum()) == nq * rows
+    order = torch.sort(scores.nan_to_num(nan=-float("inf")), dim=1, descending=True, stable=True)
+    values, ids = order.values[:, :k], order.indices[:, :k]
+    assert torch.equal(ts, values) and torch.equal(ti.long(), torch.where(values == -float("inf"), -1, ids))
