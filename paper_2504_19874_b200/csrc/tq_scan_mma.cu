@@ -457,8 +457,7 @@ scan_mma_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
             z[m][h][0] = v.x; z[m][h][1] = v.y; z[m][h][2] = v.z; z[m][h][3] = v.w;
           }
         }
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&empty[stage]);   // the stage now lives in registers
+      tc::release_stage(&empty[stage], lane);   // the stage now lives in registers
       if (++stage == a.stages) {
         stage = 0;
         phase ^= 1u;

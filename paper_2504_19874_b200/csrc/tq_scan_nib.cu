@@ -362,8 +362,7 @@ scan_nib_kernel(const __grid_constant__ CUtensorMap tmIdx, const __grid_constant
             w[h][4 * u] = v.x; w[h][4 * u + 1] = v.y; w[h][4 * u + 2] = v.z; w[h][4 * u + 3] = v.w;
           }
       }
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&empty[stage]);   // the stage now lives in registers
+      tc::release_stage(&empty[stage], lane);   // the stage now lives in registers
       if (++stage == a.stages) {
         stage = 0;
         phase ^= 1u;

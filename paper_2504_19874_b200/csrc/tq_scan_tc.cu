@@ -685,8 +685,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__
             const uint4 v4 = *reinterpret_cast<const uint4*>(ps + prow * 64 + ((j ^ ((prow >> 1) & 3)) << 4));
             x[4 * j] = v4.x; x[4 * j + 1] = v4.y; x[4 * j + 2] = v4.z; x[4 * j + 3] = v4.w;
           }
-          __syncwarp();
-          if (lane == 0) tc::mbar_arrive(&pempty[pstage]);
+          tc::release_stage(&pempty[pstage], lane);
           if (++pstage == P_STAGES) {
             pstage = 0;
             pphase ^= 1u;
@@ -746,8 +745,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__
             w[2 * j][0] = v.x; w[2 * j][1] = v.y; w[2 * j + 1][0] = v.z; w[2 * j + 1][1] = v.w;
           }
         }
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&pempty[pstage]);
+        tc::release_stage(&pempty[pstage], lane);
         if (++pstage == P_STAGES) {
           pstage = 0;
           pphase ^= 1u;

@@ -400,8 +400,7 @@ scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant_
             const uint4 v4 = *reinterpret_cast<const uint4*>(ps + r * 64 + ((j ^ ((r >> 1) & 3)) << 4));
             x[4 * j] = v4.x; x[4 * j + 1] = v4.y; x[4 * j + 2] = v4.z; x[4 * j + 3] = v4.w;
           }
-          __syncwarp();
-          if (lane == 0) tc::mbar_arrive(&pempty[pst]);
+          tc::release_stage(&pempty[pst], lane);
           const uint32_t kt = kt0 + (uint32_t)rg.f0;
           uint32_t v[32];
 #pragma unroll
@@ -452,8 +451,7 @@ scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant_
               w[2 * j][0] = v.x; w[2 * j][1] = v.y; w[2 * j + 1][0] = v.z; w[2 * j + 1][1] = v.w;
             }
           }
-          __syncwarp();
-          if (lane == 0) tc::mbar_arrive(&pempty[pst]);
+          tc::release_stage(&pempty[pst], lane);
 #pragma unroll
           for (int j = 0; j < 4; ++j)
             if (j < rg.cnt) ok = ok && emit(w[j], rg.f0 + j);

@@ -589,8 +589,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
 #pragma unroll
           for (int j = 8; j < 16; ++j) w[j] = 0u;
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&pempty[pst]);
+        release_stage(&pempty[pst], lane);
         const uint32_t kt = kt0 + (uint32_t)rg.f0;
         if (NIB) {
 #pragma unroll

@@ -99,6 +99,14 @@ __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// A warp gives a stage that TMA filled back to the producer, its bytes read into registers.  Reads of the generic proxy are ordered
+// before the next TMA write only by the proxy fence: without it that write overtook them where atomics kept the warps' loads waiting (a
+// list of all 65,600 rows for one query of 256: rows of other queries in the same tiles got estimates of mixed codes).
+__device__ __forceinline__ void release_stage(uint64_t* bar, int lane) {
+  fence_proxy_async();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(bar);
+}
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }

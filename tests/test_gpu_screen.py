@@ -132,3 +132,17 @@ def test_rows_without_a_number(n, nq, rows, spread, gamma):
     order = torch.sort(scores.nan_to_num(nan=-float("inf")), dim=1, descending=True, stable=True)
     values, ids = order.values[:, :k], order.indices[:, :k]
     assert torch.equal(ts, values) and torch.equal(ti.long(), torch.where(values == -float("inf"), -1, ids))
+
+
+@pytest.mark.parametrize("d,bits,mode,layout", [(200, 3, tq.TQ_PROD, None), (200, 2, tq.TQ_MSE, None), (768, 4, tq.TQ_PROD, NIB)])
+def test_a_query_that_every_row_passes(d, bits, mode, layout):
+    """The atomics of so many hits hold up the warps that read the packed rows: the other queries' estimates of the rows beside them are
+    formed from those rows all the same."""
+    n, nq, k = 65_600, 200, 10
+    su = P.Setup(d, bits, mode, layout=layout)
+    g = torch.Generator(device=DEV).manual_seed(d)
+    X, Q = torch.randn((n, d), generator=g, device=DEV), torch.randn((nq, d), generator=g, device=DEV)
+    Q[3:6] *= 1e19
+    codes = su.quantize(X)
+    for _ in range(4):
+        check(su, Q, n, codes, k)
