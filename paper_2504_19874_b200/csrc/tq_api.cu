@@ -167,7 +167,11 @@ size_t ms_topk_fixed(const tq_plan* plan, int nq) {
 // d = 1536 prod b = 4 nibble 797 / 1,163, 2,082 / 1,215, 3,013 / 1,583; d = 3072 prod b = 2 1,368 / 2,755, 3,422 / 2,798,
 // 5,293 / 3,611; n = 65,536: d = 200 84 / 107, 161 / 95, 259 / 148; d = 1536 mse b = 2 115 / 190, 248 / 161, 405 / 297).
 constexpr int kScreenFrom = 65;
-bool screens(const tq_plan* plan, int nq, int64_t n) { return nq >= kScreenFrom && n >= kFilterMinN && pick_engine(plan, nq).tc; }
+constexpr int kScreenPass = 64;   // queries of a pass of the exact engine in such calls: they share a flag
+bool screens(const tq_plan* plan, int nq, int64_t n) {
+  const ScanEngine e = pick_engine(plan, nq);
+  return nq >= kScreenFrom && n >= kFilterMinN && e.tc && e.qpp == kScreenPass;
+}
 // A query's list: 2,048 candidates are expected at most (screen_samples), and two CTAs of the selection fit an SM.
 constexpr int kScreenCap = 8192;
 // Workspace of a screened pass, between the exact engine's operand and the dense score buffer.
@@ -189,7 +193,7 @@ ScreenSpace screen_space(const tq_plan* plan) {
   s.count = take(Q * 4);
   s.count1 = take(Q * 4);
   s.left = take(Q * 4);
-  s.flag = take(8);
+  s.flag = take(3 * Q / kScreenPass * 4);
   s.left_s = take(Q * screen::kSurvivors * 4);
   s.left_i = take(Q * screen::kSurvivors * 4);
   s.cand_s = take(Q * kScreenCap * 4);
@@ -1043,7 +1047,7 @@ static int64_t pilot_rows(int64_t n, int k, int64_t most) {
   return std::min<int64_t>(m, std::min<int64_t>(most / 256 * 256, n));
 }
 
-// Dense block flow over the queries of one pass: the whole job for small n, the guarded rescue of a filtered search otherwise.
+// Dense block flow over the queries of one pass: the whole job for small n, the guarded last resort of a filtered search otherwise.
 static int topk_dense(const ScanEngine& eng, int q0, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma,
                       const float* norms, int k, float* ts, int32_t* ti, float* dense, int64_t dense_floats, const int* guard, void* msw,
                       cudaStream_t st, const char* who) {
@@ -1088,6 +1092,10 @@ static ScreenSamples screen_samples(int64_t n, int k, int64_t most) {
 
 // Top-k of many queries by screening: lower bounds of samples' estimates give a threshold that k rows reach, the rows whose upper
 // bounds reach it are listed, and those whose upper bounds reach the list's k-th lower bound are scored exactly.
+// A pass of the exact engine among whose queries one has more rows to score than that pays for (rows all alike at the top, rows that
+// the bounds do not cover) is run, with the k-th lower bounds as its thresholds.  Only where its lists overflow too the rows are
+// scored densely, whose selection out of all scores takes longer than the scan (12,000 equal rows at the top for 256 queries, d = 200,
+// k = 10, 10^6 rows: 12.6 ms without the filtered passes between, 4.7 with them; they cost 5 us per 256 queries where they are off).
 static int topk_screened(const ScanEngine& eng, const float* Qcat, int nq, int64_t n, const uint8_t* idx, const uint8_t* qjl,
                          const float* gamma, const float* norms, int k, float* top_scores, int32_t* top_ids, char* ws, size_t ws_bytes,
                          cudaStream_t st, const char* who) {
@@ -1105,6 +1113,13 @@ static int topk_screened(const ScanEngine& eng, const float* Qcat, int nq, int64
   const int64_t dense_floats = (int64_t)((ws + ws_bytes - reinterpret_cast<char*>(dense)) / sizeof(float));
   const ScreenSamples sm = screen_samples(n, k, dense_floats / screen::kQueries);
   static_assert(screen::kQueries == kGroupQueries, "one exact operand per screened pass");
+  constexpr int kFlags = screen::kQueries / kScreenPass;
+  int *flag2 = flag + kFlags, *unused = flag2 + kFlags;
+  // lists of the filtered exact passes: in the dense buffer where it has room for longer ones than the screening lists
+  const int64_t room = dense_floats / (2 * screen::kQueries);
+  const int xcap = (int)std::min<int64_t>(std::max<int64_t>(room, kScreenCap), kCandCap);
+  float* x_s = room > kScreenCap ? dense : cand_s;
+  int* x_i = room > kScreenCap ? reinterpret_cast<int*>(dense + (int64_t)screen::kQueries * xcap) : cand_i;
   const screen::QueryTerms* terms = screen::query_terms(plan, operand);
   for (int q0 = 0; q0 < nq; q0 += screen::kQueries) {
     const int nqp = std::min(screen::kQueries, nq - q0);
@@ -1115,25 +1130,30 @@ static int topk_screened(const ScanEngine& eng, const float* Qcat, int nq, int64
     auto filter = [&](int64_t rows, int64_t step, int* counts) {
       return screen::run(plan, nqp, rows, idx, qjl, gamma, norms, nullptr, 0, tau, counts, cand_s, cand_i, kScreenCap, operand, st, who, step);
     };
-    int* unused = flag + 1;
     if ((rc = screen::run(plan, nqp, sm.dense, idx, qjl, gamma, norms, dense, sm.dense, nullptr, nullptr, nullptr, nullptr, 0, operand, st, who,
                           sm.dense_step)))
       return rc;
     TQ_CHECK_CUDA(mscan::select_topk(dense, nullptr, nullptr, (int)sm.dense, (int)sm.dense, 0, nqp, k, 0, nullptr, nullptr, tau, nullptr, nullptr,
-                                     sm.first > 0 ? count1 : count, sm.first > 0 ? unused : flag, st), who);
+                                     sm.first > 0 ? count1 : count, sm.first > 0 ? unused : flag, st, eng.qpp), who);
     if (sm.first > 0) {   // (a list that is too short here still gives a threshold that k rows reach)
       if ((rc = filter(sm.first, sm.first_step, count1))) return rc;
-      TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count1, kScreenCap, 0, 0, nqp, k, 0, nullptr, nullptr, tau, nullptr, nullptr, count, flag, st), who);
+      TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count1, kScreenCap, 0, 0, nqp, k, 0, nullptr, nullptr, tau, nullptr, nullptr, count, flag, st,
+                                       eng.qpp), who);
     }
     if ((rc = filter(n, 1, count))) return rc;
-    TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count, kScreenCap, 0, 0, nqp, k, 0, nullptr, nullptr, kth, flag, nullptr, left, unused, st), who);
+    TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count, kScreenCap, 0, 0, nqp, k, 0, nullptr, nullptr, kth, nullptr, nullptr, left, unused, st,
+                                     eng.qpp), who);
     if ((rc = tscan::rescore(plan, nqp, idx, qjl, gamma, norms, msw, terms, tau, kth, count, cand_s, cand_i, kScreenCap,
-                             left_s, left_i, left, flag, st, who)))
+                             k, left_s, left_i, left, flag, eng.qpp, st, who)))
       return rc;
-    TQ_CHECK_CUDA(mscan::select_topk(left_s, left_i, left, screen::kSurvivors, 0, 0, nqp, k, 0, ts, ti, nullptr, nullptr, nullptr, nullptr, nullptr, st), who);
-    for (int s = 0; s < nqp; s += eng.qpp)
+    TQ_CHECK_CUDA(mscan::select_topk(left_s, left_i, left, screen::kSurvivors, 0, 0, nqp, k, 0, ts, ti, nullptr, nullptr, nullptr, count1, flag2, st,
+                                     eng.qpp), who);
+    mscan::Filter f{kth, count1, x_s, x_i, xcap};
+    if ((rc = engine_run(eng, q0, nqp, n, idx, qjl, gamma, norms, nullptr, 0, &f, flag, msw, st, who))) return rc;
+    TQ_CHECK_CUDA(mscan::select_topk(x_s, x_i, count1, xcap, 0, 0, nqp, k, 0, ts, ti, nullptr, flag2, flag, nullptr, nullptr, st, eng.qpp), who);
+    for (int s = 0; s < nqp; s += eng.qpp)   // (the buffer holds the scores of one pass)
       if ((rc = topk_dense(eng, q0 + s, std::min(eng.qpp, nqp - s), n, idx, qjl, gamma, norms, k, ts + (size_t)s * k, ti + (size_t)s * k, dense,
-                           dense_floats, flag, msw, st, who)))
+                           dense_floats, flag2 + s / eng.qpp, msw, st, who)))
         return rc;
   }
   return TQ_OK;

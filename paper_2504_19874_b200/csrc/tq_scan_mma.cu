@@ -625,10 +625,11 @@ struct SelArgs {
   float* top_s;           // nullable (with top_i, merge = 0): only kth is wanted, and any lower bound reached by k entries will do
   int* top_i;
   float* kth;             // nullable
-  int* overflow;          // nullable: set to 1 when count > cap for this query
+  int* overflow;          // nullable: the query's flag is set to 1 when its count > cap
   const int* run_if;      // nullable
-  int* clear_count;       // nullable: [nq] counters to zero, and with them the flag
+  int* clear_count;       // nullable: [nq] counters to zero, and with them the flags
   int* clear_flag;
+  int per_flag;           // queries that share one flag of overflow, run_if and clear_flag
 };
 
 // 0: an empty slot, which a score that is not a number is too (it has no rank, and passes no filter).
@@ -700,16 +701,16 @@ __global__ void __launch_bounds__(1024) select_kernel(SelArgs a) {
   skey[tid] = 0ull;
   hist[tid] = hist[tid + 1024] = 0;
   wait_for_predecessor();   // all inputs are outputs of kernels ahead in the stream
-  if (a.run_if != nullptr && *a.run_if == 0) return;
+  if (a.run_if != nullptr && a.run_if[q / a.per_flag] == 0) return;
   if (a.clear_count != nullptr && tid == 0) {   // the candidate counters of the pass that follows
     a.clear_count[q] = 0;
-    if (q == 0) *a.clear_flag = 0;
+    if (q % a.per_flag == 0) a.clear_flag[q / a.per_flag] = 0;
   }
   int m_new = a.m;
   if (a.count != nullptr) {
     const int c = a.count[q];
     m_new = min(c, a.cap);
-    if (a.overflow != nullptr && c > a.cap && tid == 0) atomicExch(a.overflow, 1);
+    if (a.overflow != nullptr && c > a.cap && tid == 0) atomicExch(a.overflow + q / a.per_flag, 1);
   }
   const int total = m_new + (a.merge ? a.k : 0);
   const bool cached = total <= kSelCached;
@@ -1171,7 +1172,7 @@ int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8
 
 cudaError_t select_topk(const float* cand_s, const int* cand_i, const int* count, int cap, int m, int id0, int nq, int k,
                         int merge, float* top_s, int* top_i, float* kth, int* overflow, const int* run_if, int* clear_count,
-                        int* clear_flag, cudaStream_t st) {
+                        int* clear_flag, cudaStream_t st, int per_flag) {
   SelArgs a;
   a.cand_s = cand_s;
   a.cand_i = cand_i;
@@ -1188,6 +1189,7 @@ cudaError_t select_topk(const float* cand_s, const int* cand_i, const int* count
   a.run_if = run_if;
   a.clear_count = clear_count;
   a.clear_flag = clear_flag;
+  a.per_flag = per_flag;
   // the shared-memory copy of the list: as much as this call can need (none where the list is known to be too long for it)
   const int64_t most = std::max<int64_t>(count != nullptr ? cap : m, 0) + (merge ? k : 0);
   const size_t smem = count == nullptr && most > kSelCached ? 0 : (size_t)std::min<int64_t>(most, kSelCached) * sizeof(unsigned long long);

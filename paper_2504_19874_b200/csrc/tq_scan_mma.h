@@ -39,11 +39,11 @@ int run(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8
 // cand_i is nullptr, out of the dense row cand_s[q*cap .. +m) with ids id0 + position.  Optionally merges
 // the previous best list (top_s/top_i, when merge != 0) and writes the k-th score to kth[q].
 // With top_s == nullptr only kth[q] is written: a lower bound of the k-th score that at least k entries reach.
-// *overflow is set to 1 if some count exceeded cap; run_if as above.  clear_count[0 .. nq) and *clear_flag are set to 0
-// (the counters of the filter pass that follows a pilot's selection).
+// overflow[q / per_flag] is set to 1 if the count of query q exceeded cap; run_if[q / per_flag] as above.  clear_count[0 .. nq) and the
+// flags clear_flag[q / per_flag] are set to 0 (the counters of the filter pass that follows a pilot's selection).
 cudaError_t select_topk(const float* cand_s, const int* cand_i, const int* count, int cap, int m, int id0, int nq, int k,
                         int merge, float* top_s, int* top_i, float* kth, int* overflow, const int* run_if, int* clear_count,
-                        int* clear_flag, cudaStream_t st);
+                        int* clear_flag, cudaStream_t st, int per_flag = 1 << 30);
 
 // The k best of m candidate pairs per query (row stride ld); pairs with id < 0 are skipped.
 cudaError_t select_pairs(const float* cand_s, const int* cand_i, int ld, int m, int nq, int k, float* top_s, int* top_i,

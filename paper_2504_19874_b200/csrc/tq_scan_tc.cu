@@ -843,11 +843,12 @@ struct RescoreArgs {
   const int* count;        // candidates: (lower bound, row)
   const float* cand_s;
   const int* cand_i;
-  int cap;
+  int cap, k;
   float* out_s;            // [queries][kSurvivors]
   int* out_i;
   int* out_count;
   int* overflow;
+  int per_flag;
 };
 
 __device__ __forceinline__ int dp4a_us(uint32_t a, uint32_t b, int c) {
@@ -874,7 +875,11 @@ __global__ void __launch_bounds__(kRescoreThreads, 2) rescore_kernel(const __gri
   wait_for_predecessor();   // the lists are its output
   const int q = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool signs = a.g.kbs > 0 || a.g.nib;
-  const int m = min(a.count[q], a.cap);
+  const int m = a.count[q];
+  if (m > a.cap || m < a.k) {   // too long for the list; too short: no threshold that k rows reach keeps fewer
+    if (threadIdx.x == 0) atomicExch(a.overflow + q / a.per_flag, 1);
+    return;
+  }
   const float kth = a.kth[q], err = a.terms[q].err, unscale = a.terms[q].unscale, slack = 2.f * screen::kThresholdSlack * fabsf(a.tau[q]);
   // four candidates of a thread at a time: the loads of their scalars are a chain of two round trips
   const int stride = kRescoreThreads * (int)gridDim.y;
@@ -902,14 +907,14 @@ __global__ void __launch_bounds__(kRescoreThreads, 2) rescore_kernel(const __gri
     }
   }
   __syncthreads();
-  int n = min(s_n, screen::kSurvivors);
+  const int n = s_n;
   if (threadIdx.x == 0) {
     s_base = atomicAdd(a.out_count + q, n);
-    if (s_n > screen::kSurvivors || s_base + n > screen::kSurvivors) atomicExch(a.overflow, 1);
+    if (s_base + n > screen::kSurvivors) atomicExch(a.overflow + q / a.per_flag, 1);
   }
   __syncthreads();
   const int base = s_base;
-  n = min(n, screen::kSurvivors - base);
+  if (base + n > screen::kSurvivors) return;   // the pass is scored by the scan kernels
   const QConst c = a.qc[q];
   const int row0 = q / kQueriesPerPass * NCOL + q % kQueriesPerPass;
   const size_t pa = (size_t)a.g.kba * KB_BYTES, psn = (size_t)a.g.kbs * KB_BYTES;
@@ -1018,12 +1023,13 @@ cudaError_t launch_wide_c(const CUtensorMap& ma, const CUtensorMap& ms, const CU
   }
   count_launches(1);
   const int64_t ntiles = (args.n + TILE - 1) / TILE;
+  const unsigned passes = (unsigned)((args.nqp + W_QPP - 1) / W_QPP);
   if (CTAS == 1)
-    return launch_dependent(kern, dim3((unsigned)std::min<int64_t>(ntiles, tc::sm_count())), dim3(W_NTHREADS), kWideSmemBytes, st, ma, ms, pa,
-                            ps, args);
+    return launch_dependent(kern, dim3((unsigned)std::min<int64_t>(ntiles, tc::sm_count()), passes), dim3(W_NTHREADS), kWideSmemBytes, st, ma,
+                            ms, pa, ps, args);
   const int units = (int)std::min<int64_t>((ntiles + CTAS - 1) / CTAS, tc::sm_count() / CTAS);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(units * CTAS));
+  cfg.gridDim = dim3((unsigned)(units * CTAS), passes);
   cfg.blockDim = dim3(W_NTHREADS);
   cfg.dynamicSmemBytes = kWideSmemBytes;
   cfg.stream = st;
@@ -1137,7 +1143,7 @@ int run_pass(const tq_plan* plan, int pass, int nqp, int64_t n, const uint8_t* i
   // more than 32 queries: the wide kernel takes the B rows of this pass and the next as one box of 192 rows and one
   // 128-vector tile at a time
   const bool wide = nqp > kQueriesPerPass;
-  TQ_REQUIRE(nqp <= (wide ? W_QPP : kQueriesPerPass) && (!wide || (pass % 2 == 0 && pass + 2 <= kPassesPerGroup)), TQ_ERR_INVALID_ARG,
+  TQ_REQUIRE(!wide || (pass % 2 == 0 && pass * kQueriesPerPass + nqp <= kPassesPerGroup * kQueriesPerPass), TQ_ERR_INVALID_ARG,
              "%s: pass %d of %d queries", who, pass, nqp);
   // The wide kernel runs on CTA pairs wherever there is more than one tile (M = 256, each CTA loads half of a B box's
   // rows into one of twelve half-size stages: measured 316 against 339 us per 32 queries at d = 1536, n = 10^6).
@@ -1206,8 +1212,8 @@ int run_pass(const tq_plan* plan, int pass, int nqp, int64_t n, const uint8_t* i
 
 int rescore(const tq_plan* plan, int nqp, const uint8_t* idx, const uint8_t* qjl, const float* gamma, const float* norms,
             const void* workspace, const screen::QueryTerms* terms, const float* tau, const float* kth, const int* count,
-            const float* cand_s, const int* cand_i, int cap, float* out_s, int* out_i, int* out_count, int* overflow, cudaStream_t st,
-            const char* who) {
+            const float* cand_s, const int* cand_i, int cap, int k, float* out_s, int* out_i, int* out_count, int* overflow, int per_flag,
+            cudaStream_t st, const char* who) {
   RescoreArgs a;
   a.g = make_geo(plan);
   a.hi_a = plan->nb.hi_a; a.hi_b = plan->nb.hi_b; a.lo_a = plan->nb.lo_a; a.lo_b = plan->nb.lo_b;
@@ -1226,10 +1232,12 @@ int rescore(const tq_plan* plan, int nqp, const uint8_t* idx, const uint8_t* qjl
   a.cand_s = cand_s;
   a.cand_i = cand_i;
   a.cap = cap;
+  a.k = k;
   a.out_s = out_s;
   a.out_i = out_i;
   a.out_count = out_count;
   a.overflow = overflow;
+  a.per_flag = per_flag;
   count_launches(1);
   TQ_CHECK_CUDA(launch_dependent(rescore_kernel, dim3((unsigned)nqp, (unsigned)std::max(1, std::min(8, 2 * tc::sm_count() / nqp))), dim3(kRescoreThreads), 0, st, a), who);
   return TQ_OK;

@@ -25,7 +25,8 @@ int prepare_group(const tq_plan* plan, const float* Qcat, int nqg, void* workspa
 
 // One pass of up to 32 queries (pass index `pass` inside the prepared group), or of 33 to 64 queries (the queries of
 // passes `pass` and `pass + 1`, `pass` even), over vectors [0, n): dense estimates into scores[nqp, lds] or the pairs
-// admitted by the filter.  run_if and step as in mscan::run.
+// admitted by the filter.  run_if and step as in mscan::run.  More queries, up to the end of the group: several passes of 64 in one
+// launch, run_if[i] the switch of the i-th.
 int run_pass(const tq_plan* plan, int pass, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma,
              const float* norms, float* scores, int64_t lds, const mscan::Filter* filter, const int* run_if,
              const void* workspace, cudaStream_t st, const char* who, int64_t step = 1);
@@ -33,11 +34,11 @@ int run_pass(const tq_plan* plan, int pass, int nqp, int64_t n, const uint8_t* i
 // The candidates (lower bound, row; listed with thresholds tau) of nqp queries of a prepared group whose upper bound reaches kth[q],
 // scored exactly -- the bits of run_pass -- into out_s / out_i [nqp, screen::kSurvivors] (NaN estimates as empty slots), their numbers added to
 // out_count (zero before).
-// *overflow is set to 1 where more are left than fit.
+// overflow[q / per_flag] is set to 1 where more are left than fit, or where the list is longer than cap or has fewer than k entries.
 int rescore(const tq_plan* plan, int nqp, const uint8_t* idx, const uint8_t* qjl, const float* gamma, const float* norms,
             const void* workspace, const screen::QueryTerms* terms, const float* tau, const float* kth, const int* count,
-            const float* cand_s, const int* cand_i, int cap, float* out_s, int* out_i, int* out_count, int* overflow, cudaStream_t st,
-            const char* who);
+            const float* cand_s, const int* cand_i, int cap, int k, float* out_s, int* out_i, int* out_count, int* overflow, int per_flag,
+            cudaStream_t st, const char* who);
 
 }  // namespace tscan
 }  // namespace tq

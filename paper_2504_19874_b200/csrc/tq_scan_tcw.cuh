@@ -98,6 +98,21 @@ __global__ void __launch_bounds__(W_NTHREADS, 1)
 scan_tcw_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__ CUtensorMap tmBs,
                 const __grid_constant__ CUtensorMap tmPa, const __grid_constant__ CUtensorMap tmPs, ScanArgs a) {
   allow_successor();
+  {   // several passes of one group: the grid's second dimension
+    const int y = (int)blockIdx.y, q = W_QPP * y;
+    a.pass += W_QPP / kQueriesPerPass * y;
+    a.nqp = min(W_QPP, a.nqp - q);
+    a.qc += q;
+    if (MODE == 0) {
+      a.scores += q * a.lds;
+    } else {
+      a.tau += q;
+      a.count += q;
+      a.cand_s += (int64_t)q * a.cap;
+      a.cand_i += (int64_t)q * a.cap;
+    }
+    if (a.run_if != nullptr) a.run_if += y;
+  }
   if (a.run_if != nullptr) {
     wait_for_predecessor();   // it may write the switch
     if (*a.run_if == 0) return;

@@ -7,7 +7,10 @@ namespace tq {
 namespace screen {
 
 constexpr int kQueries = 256;          // queries per pass over the codes
-constexpr int kSurvivors = 2048;       // rows of a query that are scored again at most
+// Rows of a query that are scored again at most.  One costs 1.0 ns at d = 200 prod b = 3 and 1.4 at d = 1536 prod b = 4 (256 queries with
+// as many each, 10^6 rows), so that 8,192 cost about what the exact passes do that stand in for them (6,000 equal rows at the top, a
+// limit of 4,096: 3.4 and 5.1 ms; scored one by one 2.0 and 3.6).
+constexpr int kSurvivors = 8192;
 // Lower bounds of listed rows are formed by four operations whose results are no larger than |tau| and the row's own terms: half a
 // place each, 2^-22 |tau| in all (the row's own terms are covered by its error constant).  Twice that is taken off.
 constexpr float kThresholdSlack = 4.76837158e-7f;   // 2^-21

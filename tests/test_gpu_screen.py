@@ -146,3 +146,18 @@ def test_a_query_that_every_row_passes(d, bits, mode, layout):
     codes = su.quantize(X)
     for _ in range(4):
         check(su, Q, n, codes, k)
+
+
+@pytest.mark.parametrize("copies", [3000, 7000, 20_000, 40_000])
+@pytest.mark.parametrize("d,bits,mode,layout", [(200, 3, tq.TQ_PROD, None), (768, 4, tq.TQ_PROD, NIB)])
+def test_equal_rows_at_the_top(d, bits, mode, layout, copies):
+    """More equal rows at the top of some queries' results than are scored one by one, than the screening lists hold, and than the lists of the
+    exact passes hold: ties go to the lowest ids.  The other queries' passes are not touched by it."""
+    n, nq, k = 70_000, 300, 100
+    su = P.Setup(d, bits, mode, layout=layout)
+    g = torch.Generator(device=DEV).manual_seed(copies)
+    X, Q = torch.randn((n, d), generator=g, device=DEV), torch.randn((nq, d), generator=g, device=DEV)
+    X[torch.randperm(n, generator=g, device=DEV)[:copies]] = X[0].clone()
+    Q[70:90] += 2.0 * X[0]
+    Q[280:] += 2.0 * X[0]
+    check(su, Q, n, su.quantize(X), k)
