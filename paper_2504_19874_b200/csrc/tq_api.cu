@@ -1143,7 +1143,7 @@ static int topk_screened(const ScanEngine& eng, const float* Qcat, int nq, int64
     if ((rc = filter(n, 1, count))) return rc;
     TQ_CHECK_CUDA(mscan::select_topk(cand_s, cand_i, count, kScreenCap, 0, 0, nqp, k, 0, nullptr, nullptr, kth, nullptr, nullptr, left, unused, st,
                                      eng.qpp), who);
-    if ((rc = tscan::rescore(plan, nqp, idx, qjl, gamma, norms, msw, terms, tau, kth, count, cand_s, cand_i, kScreenCap,
+    if ((rc = tscan::rescore(plan, nqp, n, idx, qjl, gamma, norms, msw, terms, tau, kth, count, cand_s, cand_i, kScreenCap,
                              k, left_s, left_i, left, flag, eng.qpp, st, who)))
       return rc;
     TQ_CHECK_CUDA(mscan::select_topk(left_s, left_i, left, screen::kSurvivors, 0, 0, nqp, k, 0, ts, ti, nullptr, nullptr, nullptr, count1, flag2, st,

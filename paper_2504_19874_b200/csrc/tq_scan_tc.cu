@@ -827,6 +827,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmBa, const __grid_constant__
 // For the rows that a screening pass leaves: the same digit sums as the scan kernels, hence the same estimates, by byte dot
 // products on CUDA cores over the digit rows of B that the scan kernels read.
 struct RescoreArgs {
+  int64_t n;
   Geo g;
   uint32_t hi_a, hi_b, lo_a, lo_b;
   const QConst* qc;
@@ -868,19 +869,26 @@ __device__ __forceinline__ int dp4a_ss(uint32_t a, uint32_t b, int c) {
 constexpr int kRescoreThreads = 512;
 __global__ void __launch_bounds__(kRescoreThreads, 2) rescore_kernel(const __grid_constant__ RescoreArgs a) {
   __shared__ int ids[screen::kSurvivors];
-  __shared__ int s_n, s_base;
+  __shared__ int s_n, s_base, s_numbers;
   allow_successor();
-  if (threadIdx.x == 0) s_n = 0;
+  if (threadIdx.x == 0) s_n = s_numbers = 0;
   __syncthreads();
   wait_for_predecessor();   // the lists are its output
   const int q = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool signs = a.g.kbs > 0 || a.g.nib;
-  const int m = a.count[q];
-  if (m > a.cap || m < a.k) {   // too long for the list; too short: no threshold that k rows reach keeps fewer
+  const float err = a.terms[q].err, unscale = a.terms[q].unscale;
+  const bool zero = err == screen::kZeroQuery;
+  if (err == screen::kNanQuery || (zero && blockIdx.y > 0)) return;
+  const int m = zero ? 0 : a.count[q];
+  if (zero) {   // the first rows
+    const int rows = (int)min(a.n, (int64_t)a.k + screen::kZeroSpare);
+    for (int i = threadIdx.x; i < rows; i += kRescoreThreads) ids[i] = i;
+    if (threadIdx.x == 0) s_n = rows;
+  } else if (m > a.cap || m < a.k) {   // too long for the list; too short: no threshold that k rows reach keeps fewer
     if (threadIdx.x == 0) atomicExch(a.overflow + q / a.per_flag, 1);
     return;
   }
-  const float kth = a.kth[q], err = a.terms[q].err, unscale = a.terms[q].unscale, slack = 2.f * screen::kThresholdSlack * fabsf(a.tau[q]);
+  const float kth = a.kth[q], slack = 2.f * screen::kThresholdSlack * fabsf(a.tau[q]);
   // four candidates of a thread at a time: the loads of their scalars are a chain of two round trips
   const int stride = kRescoreThreads * (int)gridDim.y;
   for (int i0 = blockIdx.y * kRescoreThreads + threadIdx.x; i0 < m; i0 += 4 * stride) {
@@ -981,7 +989,12 @@ __global__ void __launch_bounds__(kRescoreThreads, 2) rescore_kernel(const __gri
       const float e = __fmul_rn(nu, fmaf(cg, sv, av));
       a.out_s[(int64_t)q * screen::kSurvivors + base + s] = e;
       a.out_i[(int64_t)q * screen::kSurvivors + base + s] = isnan(e) ? -1 : (int)row;   // a negative id is an empty slot
+      if (zero && !isnan(e)) atomicAdd(&s_numbers, 1);
     }
+  }
+  if (zero) {
+    __syncthreads();
+    if (threadIdx.x == 0 && s_numbers < a.k) atomicExch(a.overflow + q / a.per_flag, 1);
   }
 }
 
@@ -1210,11 +1223,12 @@ int run_pass(const tq_plan* plan, int pass, int nqp, int64_t n, const uint8_t* i
   return TQ_OK;
 }
 
-int rescore(const tq_plan* plan, int nqp, const uint8_t* idx, const uint8_t* qjl, const float* gamma, const float* norms,
+int rescore(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma, const float* norms,
             const void* workspace, const screen::QueryTerms* terms, const float* tau, const float* kth, const int* count,
             const float* cand_s, const int* cand_i, int cap, int k, float* out_s, int* out_i, int* out_count, int* overflow, int per_flag,
             cudaStream_t st, const char* who) {
   RescoreArgs a;
+  a.n = n;
   a.g = make_geo(plan);
   a.hi_a = plan->nb.hi_a; a.hi_b = plan->nb.hi_b; a.lo_a = plan->nb.lo_a; a.lo_b = plan->nb.lo_b;
   a.qc = static_cast<const QConst*>(workspace);

@@ -31,11 +31,11 @@ int run_pass(const tq_plan* plan, int pass, int nqp, int64_t n, const uint8_t* i
              const float* norms, float* scores, int64_t lds, const mscan::Filter* filter, const int* run_if,
              const void* workspace, cudaStream_t st, const char* who, int64_t step = 1);
 
-// The candidates (lower bound, row; listed with thresholds tau) of nqp queries of a prepared group whose upper bound reaches kth[q],
+// The candidates (lower bound, row of n; listed with thresholds tau) of nqp queries of a prepared group whose upper bound reaches kth[q],
 // scored exactly -- the bits of run_pass -- into out_s / out_i [nqp, screen::kSurvivors] (NaN estimates as empty slots), their numbers added to
 // out_count (zero before).
 // overflow[q / per_flag] is set to 1 where more are left than fit, or where the list is longer than cap or has fewer than k entries.
-int rescore(const tq_plan* plan, int nqp, const uint8_t* idx, const uint8_t* qjl, const float* gamma, const float* norms,
+int rescore(const tq_plan* plan, int nqp, int64_t n, const uint8_t* idx, const uint8_t* qjl, const float* gamma, const float* norms,
             const void* workspace, const screen::QueryTerms* terms, const float* tau, const float* kth, const int* count,
             const float* cand_s, const int* cand_i, int cap, int k, float* out_s, int* out_i, int* out_count, int* overflow, int per_flag,
             cudaStream_t st, const char* who);

@@ -204,16 +204,18 @@ __global__ void __launch_bounds__(256) screen_prep_kernel(PrepArgs a) {
   const float* qa = a.Qcat + (int64_t)q * a.ldq;
   const float* qs = qa + a.dpad;
   float mx1 = 0.f, mx2 = 0.f;
-  bool odd = false;
+  bool odd = false, nan = false;
   if (q < a.nq) {
     for (int j = tid; j < d; j += 256) {
       const float u = qa[j], v = a.prod ? qs[j] : 0.f;
       odd |= !(fabsf(u) <= FLT_MAX) || !(fabsf(v) <= FLT_MAX);
+      nan |= isnan(a.prod ? v : u);   // the estimate's constant term is the sum of these
       mx1 = fmaxf(mx1, fabsf(u));
       mx2 = fmaxf(mx2, fabsf(v));
     }
   }
   odd = __syncthreads_or(odd) != 0;
+  nan = __syncthreads_or(nan) != 0;
   mx1 = block_max(mx1, red);
   mx2 = block_max(mx2, red);
   // the largest operand entry goes to [2^9, 2^10)
@@ -222,9 +224,10 @@ __global__ void __launch_bounds__(256) screen_prep_kernel(PrepArgs a) {
   int x = 0;
   if (mx > 0.f && mx <= FLT_MAX) x = 9 - ilogbf(mx);
   odd = odd || !(mx <= FLT_MAX) || x > 60 || x < -60;
-  if (q >= a.nq || odd) {   // an absent query, or one whose estimates the bounds do not cover: every row passes
+  const bool zero = !odd && (a.g.bm == 0 || mx1 == 0.f) && mx2 == 0.f;
+  if (q >= a.nq || odd || zero) {   // an absent query, or one whose estimates the bounds do not cover: every row passes
     for (int i = tid; i < words; i += 256) out[i] = 0u;
-    if (tid == 0) a.terms[q] = {q < a.nq ? 1e30f : 0.f, 1.f};
+    if (tid == 0) a.terms[q] = {q >= a.nq ? 0.f : nan ? kNanQuery : zero ? kZeroQuery : 1e30f, 1.f};
     return;
   }
   const float sa = ldexpf(1.f, x), ss = sgn * sa;
@@ -433,7 +436,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
     float un = 0.f;
     if (q < a.nqp) {
       const QueryTerms t = a.terms[q];
-      v = make_float2(t.err, MODE == 1 ? -a.tau[q] / t.unscale : 0.f);   // the scale is a power of two
+      if (t.err >= 0.f) v = make_float2(t.err, MODE == 1 ? -a.tau[q] / t.unscale : 0.f);   // the scale is a power of two
       un = t.unscale;
     }
     float* pair = reinterpret_cast<float*>(et + (q >> 1)) + (q & 1);

@@ -47,10 +47,13 @@ __device__ __forceinline__ RowTerms row_terms(float nu, float gamma) {
 #endif
 
 // Per-query constants (device array in the workspace): error constant (scaled like the screened values) and the power of two
-// that scales them back.
+// that scales them back.  Two queries have no bounds and list no row: one of zeros, whose estimates all are zero, so that its result
+// is the first k rows (of the first k + kZeroSpare, some of whose estimates may be NaN), and one with a NaN, whose estimates all are.
 struct QueryTerms {
   float err, unscale;
 };
+constexpr float kZeroQuery = -1.f, kNanQuery = -2.f;   // their error constants
+constexpr int kZeroSpare = 128;
 const QueryTerms* query_terms(const tq_plan* plan, const void* workspace);
 
 }  // namespace screen

@@ -161,3 +161,23 @@ def test_equal_rows_at_the_top(d, bits, mode, layout, copies):
     Q[70:90] += 2.0 * X[0]
     Q[280:] += 2.0 * X[0]
     check(su, Q, n, su.quantize(X), k)
+
+
+@pytest.mark.parametrize("d,bits,mode,layout", [(200, 3, tq.TQ_PROD, None), (139, 1, tq.TQ_PROD, None), (200, 2, tq.TQ_MSE, None), (200, 4, tq.TQ_PROD, NIB)])
+@pytest.mark.parametrize("rows", [0, 50, 1500])
+def test_queries_of_zeros_and_without_a_number(d, bits, mode, layout, rows):
+    """A batch padded with zeros gets the first k rows that have an estimate (behind `rows` rows without one), a query with a NaN an empty
+    result, and the other queries what they get without them."""
+    n, nq, k = 70_000, 200, 100
+    su = P.Setup(d, bits, mode, layout=layout)
+    g = torch.Generator(device=DEV).manual_seed(rows)
+    X, Q = torch.randn((n, d), generator=g, device=DEV), torch.randn((nq, d), generator=g, device=DEV)
+    codes = su.quantize(X)
+    codes[3][:rows] = float("nan")
+    Q[150:], Q[7, 3] = 0.0, float("nan")
+    ts, ti = su.topk(Q, n, *codes, k)
+    tq.tq_plan_status(su.plan)
+    order = torch.sort(su.score(Q, n, *codes).nan_to_num(nan=-float("inf")), dim=1, descending=True, stable=True)
+    values, ids = order.values[:, :k], order.indices[:, :k]
+    assert torch.equal(ts, values) and torch.equal(ti.long(), torch.where(values == -float("inf"), -1, ids))
+    assert bool((ti[7] == -1).all()) and torch.equal(ti[199].long(), torch.arange(rows, rows + k, device=DEV))
