@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(256) topk_merge_kernel(const float* __restrict
   }
   for (int t = threadIdx.x; t < k; t += blockDim.x) {
     top_s[(int64_t)q * k + t] = ss[t];
-    top_i[(int64_t)q * k + t] = si[t];
+    top_i[(int64_t)q * k + t] = si[t] == 0x7fffffff ? -1 : si[t];   // (an empty slot: fewer than k estimates are numbers)
   }
 }
 

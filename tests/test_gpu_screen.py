@@ -181,3 +181,16 @@ def test_queries_of_zeros_and_without_a_number(d, bits, mode, layout, rows):
     values, ids = order.values[:, :k], order.indices[:, :k]
     assert torch.equal(ts, values) and torch.equal(ti.long(), torch.where(values == -float("inf"), -1, ids))
     assert bool((ti[7] == -1).all()) and torch.equal(ti[199].long(), torch.arange(rows, rows + k, device=DEV))
+
+
+@pytest.mark.parametrize("n", [100, 9000])
+def test_rows_without_a_number_in_short_vectors(n):
+    """The same rule where the scans run on CUDA cores: what is left of k is empty."""
+    d, k, nq = 64, 10, 3
+    su = P.Setup(d, 3, tq.TQ_PROD)
+    g = torch.Generator(device=DEV).manual_seed(n)
+    codes = su.quantize(torch.randn((n, d), generator=g, device=DEV))
+    codes[3][4:] = float("nan")
+    ts, ti = su.topk(torch.randn((nq, d), generator=g, device=DEV), n, *codes, k)
+    assert bool((ti[:, 4:] == -1).all()) and bool((ts[:, 4:] == -float("inf")).all())
+    assert torch.equal(ti[:, :4].sort(dim=1).values.long(), torch.arange(4, device=DEV).expand(nq, 4))
