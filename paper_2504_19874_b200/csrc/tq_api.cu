@@ -161,16 +161,44 @@ size_t ms_topk_fixed(const tq_plan* plan, int nq) {
   return ms_score_fixed(plan, nq) + 1024 /* tau, count, overflow */ + (size_t)pick_engine(plan, nq).qpp * kCandCap * 8;
 }
 
-// Top-k of kScreenFrom queries or more over at least kFilterMinN vectors: bounds of the estimates from one fp16 pass per 256 queries,
-// exact estimates only for the rows that the bounds leave (tq_screen_tc.cu).  The line lies where the exact engine needs a second
-// pass of 64 queries (us, exact / screened, n = 10^6: d = 200 prod b = 3, 64 queries 353 / 308, 130 795 / 303, 256 1,365 / 426;
-// d = 1536 prod b = 4 nibble 797 / 1,163, 2,082 / 1,215, 3,013 / 1,583; d = 3072 prod b = 2 1,368 / 2,755, 3,422 / 2,798,
-// 5,293 / 3,611; n = 65,536: d = 200 84 / 107, 161 / 95, 259 / 148; d = 1536 mse b = 2 115 / 190, 248 / 161, 405 / 297).
-constexpr int kScreenFrom = 65;
+// Samples of a screened search: `dense` rows whose lower bounds are written out give a threshold that k rows reach, `first` rows (0:
+// none) are filtered with it and give the threshold of the pass over all rows.  That one then keeps k n / first candidates: a hit
+// costs its warp as much as testing 30 estimates, and with one sample of 13,312 of 10^6 rows (one hit in 132) the pass took
+// 939 us instead of 130.
+// The rows written out are among the first sample's, so that at least k of that one reach the threshold.
+struct ScreenSamples {
+  int64_t dense, dense_step, first, first_step;
+};
+ScreenSamples screen_samples(int64_t n, int k, int64_t most) {
+  const double expect = 2048.0 / (k + 8);   // rows per sampled row that make a list of 2,048
+  const double dense0 = std::max(4096.0, std::min(160.0 * (k + 8), std::max(16384.0, 16.0 * (k + 8))));
+  double first = std::max(std::sqrt((double)n * dense0), n / expect), dense = std::max(dense0, first / expect);
+  ScreenSamples s;
+  if ((double)n <= 16.0 * dense0 && n / dense0 <= expect) {
+    first = 0.0;
+    dense = dense0;
+  }
+  s.first = std::min<int64_t>(round_up64((int64_t)first, 256), n);
+  s.dense = std::min<int64_t>(round_up64((int64_t)dense, 256), std::min<int64_t>(most / 256 * 256, s.first > 0 ? s.first : n));
+  s.first_step = s.first > 0 ? n / s.first : 1;
+  s.dense_step = s.first > 0 ? s.first_step * (s.first / s.dense) : n / s.dense;
+  return s;
+}
+
+// Top-k of many queries over at least kFilterMinN vectors: bounds of the estimates from one fp16 pass per 256 queries, exact estimates only
+// for the rows that the bounds leave (tq_screen_tc.cu).  It pays where the exact engine needs several passes of 64 queries, and the
+// less so the more rows the samples add and the more k-blocks a row has: with up to 128 queries their issue, not the MMAs, bounds the
+// pass, and selecting among the rows written out grows with k.  The line is a fit to 630 searches measured both ways (us, exact /
+// screened): d = 200 prod b = 3, 10^6 rows, k = 10, 65 queries 477 / 287, 256 queries 1,289 / 358; d = 768 prod b = 4, 65,536 rows, k = 100,
+// 128 queries 223 / 243, 192 queries 304 / 275; d = 3072 prod b = 2, 500,000 rows, k = 10, 128 queries 1,379 / 1,466, 129 queries
+// 1,676 / 1,516; d = 1536 mse b = 2, k = 1,024, 256 queries, 10^6 rows 2,821 / 2,356, 65,536 rows 594 / 902.
 constexpr int kScreenPass = 64;   // queries of a pass of the exact engine in such calls: they share a flag
-bool screens(const tq_plan* plan, int nq, int64_t n) {
+bool screens(const tq_plan* plan, int nq, int64_t n, int k) {
   const ScanEngine e = pick_engine(plan, nq);
-  return nq >= kScreenFrom && n >= kFilterMinN && e.tc && e.qpp == kScreenPass;
+  if (nq <= kScreenPass || n < kFilterMinN || !e.tc || e.qpp != kScreenPass) return false;
+  const ScreenSamples s = screen_samples(n, k, std::max<int64_t>(std::min<int64_t>(n, e.dense_rows_pref) / 4, 16384));
+  const double passes = (nq + kScreenPass - 1) / kScreenPass, rows = (double)n + (double)s.first + (double)s.dense + 1e4 + 200.0 * k;
+  return passes * (double)n >= rows * (1.0 + screen::k_blocks(plan) / 96.0);
 }
 // A query's list: 2,048 candidates are expected at most (screen_samples), and two CTAs of the selection fit an SM.
 constexpr int kScreenCap = 8192;
@@ -767,7 +795,7 @@ extern "C" size_t tq_workspace_bytes(const tq_plan* plan, int op, int64_t n, int
       return plan->ms.ok ? ms_score_fixed(plan, nq) : qcat_bytes(plan, nq);
     case TQ_OP_TOPK:
       if (plan->ms.ok)
-        return std::max(screens(plan, nq, n) ? qcat_bytes(plan, nq) + screen_pref(plan, nq, n) : 0,
+        return std::max(screens(plan, nq, n, k) ? qcat_bytes(plan, nq) + screen_pref(plan, nq, n) : 0,
                         ms_topk_fixed(plan, nq) + align_up((size_t)pick_engine(plan, nq).qpp *
                                                                std::max<int64_t>(std::min<int64_t>(n, pick_engine(plan, nq).dense_rows_pref), kDenseRowsMin) *
                                                                sizeof(float),
@@ -1066,30 +1094,6 @@ static int topk_dense(const ScanEngine& eng, int q0, int nqp, int64_t n, const u
   return TQ_OK;
 }
 
-// Samples of a screened search: `dense` rows whose lower bounds are written out give a threshold that k rows reach, `first` rows (0:
-// none) are filtered with it and give the threshold of the pass over all rows.  That one then keeps k n / first candidates: a hit
-// costs its warp as much as testing 30 estimates, and with one sample of 13,312 of 10^6 rows (one hit in 132) the pass took
-// 939 us instead of 130.
-// The rows written out are among the first sample's, so that at least k of that one reach the threshold.
-struct ScreenSamples {
-  int64_t dense, dense_step, first, first_step;
-};
-static ScreenSamples screen_samples(int64_t n, int k, int64_t most) {
-  const double expect = 2048.0 / (k + 8);   // rows per sampled row that make a list of 2,048
-  const double dense0 = std::max(4096.0, std::min(160.0 * (k + 8), std::max(16384.0, 16.0 * (k + 8))));
-  double first = std::max(std::sqrt((double)n * dense0), n / expect), dense = std::max(dense0, first / expect);
-  ScreenSamples s;
-  if ((double)n <= 16.0 * dense0 && n / dense0 <= expect) {
-    first = 0.0;
-    dense = dense0;
-  }
-  s.first = std::min<int64_t>(round_up64((int64_t)first, 256), n);
-  s.dense = std::min<int64_t>(round_up64((int64_t)dense, 256), std::min<int64_t>(most / 256 * 256, s.first > 0 ? s.first : n));
-  s.first_step = s.first > 0 ? n / s.first : 1;
-  s.dense_step = s.first > 0 ? s.first_step * (s.first / s.dense) : n / s.dense;
-  return s;
-}
-
 // Top-k of many queries by screening: lower bounds of samples' estimates give a threshold that k rows reach, the rows whose upper
 // bounds reach it are listed, and those whose upper bounds reach the list's k-th lower bound are scored exactly.
 // A pass of the exact engine among whose queries one has more rows to score than that pays for (rows all alike at the top, rows that
@@ -1169,7 +1173,7 @@ static int topk_ms(const tq_plan* plan, const float* Qcat, int nq, int64_t n, co
                    size_t ws_bytes, cudaStream_t st, const char* who) {
   int rc;
   // (a workspace of the documented minimum has no room for the lists)
-  if (screens(plan, nq, n) && ws_bytes >= screen_least(plan))
+  if (screens(plan, nq, n, k) && ws_bytes >= screen_least(plan))
     return topk_screened(pick_engine(plan, nq), Qcat, nq, n, idx, qjl, gamma, norms, k, top_scores, top_ids, ws, ws_bytes, st, who);
   const ScanEngine eng = pick_engine(plan, nq);
   void* msw = ws;

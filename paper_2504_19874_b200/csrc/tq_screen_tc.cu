@@ -862,6 +862,8 @@ size_t operand_bytes(const Geo& g) { return (size_t)kQueries * g.kblocks() * 128
 
 }  // namespace
 
+int k_blocks(const tq_plan* plan) { return make_geo(plan).kblocks(); }
+
 size_t workspace_bytes(const tq_plan* plan) { return (operand_bytes(make_geo(plan)) + kQueries * sizeof(QueryTerms) + 255) / 256 * 256; }
 
 const QueryTerms* query_terms(const tq_plan* plan, const void* workspace) {

@@ -15,6 +15,9 @@ constexpr int kSurvivors = 8192;
 // place each, 2^-22 |tau| in all (the row's own terms are covered by its error constant).  Twice that is taken off.
 constexpr float kThresholdSlack = 4.76837158e-7f;   // 2^-21
 
+// K-blocks of 64 coordinates that a row takes.
+int k_blocks(const tq_plan* plan);
+
 // Bytes of workspace for one pass: the fp16 query operand and the per-query constants.
 size_t workspace_bytes(const tq_plan* plan);
 
