@@ -351,8 +351,9 @@ __global__ void __launch_bounds__(256) scale_rows_kernel(const __nv_bfloat16* __
   }
 }
 
-// MODE 0: idx.  MODE 1: idx + residual limbs + partial ||e||^2.  MODE 2: sign bits.
-template <int BN, int MODE, int BITS, int CTAS>
+// MODE 0: idx.  MODE 1: idx + residual limbs + partial ||e||^2.  MODE 2: sign bits.  ONE: A has one limb.  (An instance of its own: with
+// number, size and offsets of the stages at run time, calls of fp32 rows were slower, 300 rows of d = 384 mse b = 2 10.0 -> 10.4 us.)
+template <int BN, int MODE, int BITS, int CTAS, bool ONE>
 __global__ void __launch_bounds__(Cfg<BN, CTAS>::kThreads, 1)
 quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmA2,
                      const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2,
@@ -363,9 +364,8 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
   const int64_t unit = blockIdx.x / CTAS, nunits = gridDim.x / CTAS;   // a unit = one CTA or one pair
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const bool one = MODE != 2 && a.one_limb != 0;                       // A has one limb
-  const int stages = one ? C::kStages1 : C::kStages, stage_bytes = one ? C::kStageBytes1 : C::kStageBytes;
-  const int b_off = one ? BM * BK * 2 : 2 * BM * BK * 2;               // B's limbs in a stage
+  constexpr int stages = ONE ? C::kStages1 : C::kStages, stage_bytes = ONE ? C::kStageBytes1 : C::kStageBytes;
+  constexpr int b_off = ONE ? BM * BK * 2 : 2 * BM * BK * 2;           // B's limbs in a stage
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kStages * C::kStageBytes);
   uint64_t* full = bars;                    // [stages]   TMA -> MMA
   uint64_t* empty = bars + stages;          // [stages]   MMA -> TMA
@@ -426,13 +426,13 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
             // both CTAs' bytes are counted on the leader's barrier, which the leader arms for both
             if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * stage_bytes);
             tma_load_2d_pair(sa, &tmA1, &full[stage], kb * BK, m0);
-            if (!one) tma_load_2d_pair(sa + BM * BK * 2, &tmA2, &full[stage], kb * BK, m0);
+            if (!ONE) tma_load_2d_pair(sa + BM * BK * 2, &tmA2, &full[stage], kb * BK, m0);
             tma_load_2d_pair(sa + b_off, &tmB1, &full[stage], kb * BK, n0);
             tma_load_2d_pair(sa + b_off + C::kBRows * BK * 2, &tmB2, &full[stage], kb * BK, n0);
           } else {
             mbar_arrive_expect_tx(&full[stage], stage_bytes);
             tma_load_2d(sa, &tmA1, &full[stage], kb * BK, m0);
-            if (!one) tma_load_2d(sa + BM * BK * 2, &tmA2, &full[stage], kb * BK, m0);
+            if (!ONE) tma_load_2d(sa + BM * BK * 2, &tmA2, &full[stage], kb * BK, m0);
             tma_load_2d(sa + b_off, &tmB1, &full[stage], kb * BK, n0);
             tma_load_2d(sa + b_off + BN * BK * 2, &tmB2, &full[stage], kb * BK, n0);
           }
@@ -473,11 +473,11 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
             const uint64_t off = (uint64_t)((k * UMMA_K * 2) >> 4);   // 32 bytes per K step
             if (CTAS == 2) {
               umma_bf16_pair(d_tmem, a1 + off, b2 + off, idesc, (kb | k) != 0 ? 1u : 0u);   // hi * lo
-              if (!one) umma_bf16_pair(d_tmem, a2 + off, b1 + off, idesc, 1u);              // lo * hi
+              if (!ONE) umma_bf16_pair(d_tmem, a2 + off, b1 + off, idesc, 1u);              // lo * hi
               umma_bf16_pair(d_tmem, a1 + off, b1 + off, idesc, 1u);                        // hi * hi
             } else {
               umma_bf16(d_tmem, a1 + off, b2 + off, idesc, (kb | k) != 0 ? 1u : 0u);
-              if (!one) umma_bf16(d_tmem, a2 + off, b1 + off, idesc, 1u);
+              if (!ONE) umma_bf16(d_tmem, a2 + off, b1 + off, idesc, 1u);
               umma_bf16(d_tmem, a1 + off, b1 + off, idesc, 1u);
             }
           }
@@ -537,10 +537,10 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
       const bool row_ok = row < a.M;
       bool zero_row = false;
       float back = 1.f;
-      if (MODE != 2 && a.nu != nullptr && row_ok) {
+      if ((MODE == 1 || ONE) && a.nu != nullptr && row_ok) {
         const float nu = __ldg(a.nu + row);
         zero_row = nu == 0.f;
-        if (one) back = row_scale(nu).back;
+        if (ONE) back = row_scale(nu).back;
       }
       float gsum = 0.f;
       uint32_t* out_row = reinterpret_cast<uint32_t*>(a.out + (size_t)(row_ok ? row : 0) * a.out_rb);
@@ -588,7 +588,7 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
               const int i = 2 * i2 + q;
-              const float y = __uint_as_float(v[i]) * back;
+              const float y = ONE ? __uint_as_float(v[i]) * back : __uint_as_float(v[i]);
               const bool col_ok = (col0 + i < a.N);
               int code = 0;
 #pragma unroll
@@ -802,10 +802,10 @@ int sm_count() {
 
 namespace {
 
-template <int BN, int MODE, int BITS, int CTAS>
+template <int BN, int MODE, int BITS, int CTAS, bool ONE>
 cudaError_t launch_gemm_t(const CUtensorMap& a1, const CUtensorMap& a2, const CUtensorMap& b1, const CUtensorMap& b2,
                           const GemmArgs& args, cudaStream_t st) {
-  auto kern = quantize_gemm_kernel<BN, MODE, BITS, CTAS>;
+  auto kern = quantize_gemm_kernel<BN, MODE, BITS, CTAS, ONE>;
   using C = Cfg<BN, CTAS>;
   // function attributes are per device: remember the devices this launcher has prepared
   static std::atomic<unsigned long long> attr_devices{0};   // written by any thread that launches
@@ -840,35 +840,37 @@ cudaError_t launch_gemm_t(const CUtensorMap& a1, const CUtensorMap& a2, const CU
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <int BN, int MODE, int CTAS>
+template <int BN, int MODE, int CTAS, bool ONE>
 cudaError_t launch_gemm_bits(int bits, const CUtensorMap& a1, const CUtensorMap& a2, const CUtensorMap& b1,
                              const CUtensorMap& b2, const GemmArgs& args, cudaStream_t st) {
   if constexpr (MODE == 2) {
-    return launch_gemm_t<BN, 2, 1, CTAS>(a1, a2, b1, b2, args, st);
+    return launch_gemm_t<BN, 2, 1, CTAS, false>(a1, a2, b1, b2, args, st);
   } else {
     switch (bits) {
-      case 0: return launch_gemm_t<BN, MODE, 0, CTAS>(a1, a2, b1, b2, args, st);
-      case 1: return launch_gemm_t<BN, MODE, 1, CTAS>(a1, a2, b1, b2, args, st);
-      case 2: return launch_gemm_t<BN, MODE, 2, CTAS>(a1, a2, b1, b2, args, st);
-      case 3: return launch_gemm_t<BN, MODE, 3, CTAS>(a1, a2, b1, b2, args, st);
-      default: return launch_gemm_t<BN, MODE, 4, CTAS>(a1, a2, b1, b2, args, st);
+      case 0: return launch_gemm_t<BN, MODE, 0, CTAS, ONE>(a1, a2, b1, b2, args, st);
+      case 1: return launch_gemm_t<BN, MODE, 1, CTAS, ONE>(a1, a2, b1, b2, args, st);
+      case 2: return launch_gemm_t<BN, MODE, 2, CTAS, ONE>(a1, a2, b1, b2, args, st);
+      case 3: return launch_gemm_t<BN, MODE, 3, CTAS, ONE>(a1, a2, b1, b2, args, st);
+      default: return launch_gemm_t<BN, MODE, 4, CTAS, ONE>(a1, a2, b1, b2, args, st);
     }
   }
 }
 
-template <int MODE>
+template <int MODE, bool ONE = false>
 cudaError_t launch_gemm(const Tile& t, int bits, const CUtensorMap& a1, const CUtensorMap& a2, const MatrixLimbs& b,
                         const GemmArgs& args, cudaStream_t st) {
+  if constexpr (MODE != 2 && !ONE)
+    if (args.one_limb) return launch_gemm<MODE, true>(t, bits, a1, a2, b, args, st);
   const int box = t.bn / t.ctas / 32 - 1;   // maps by the rows of B that a CTA loads
   const CUtensorMap &b1 = b.map_hi[box], &b2 = b.map_lo[box];
   if (t.ctas == 1) {
-    if (t.bn == 128) return launch_gemm_bits<128, MODE, 1>(bits, a1, a2, b1, b2, args, st);
-    return launch_gemm_bits<64, MODE, 1>(bits, a1, a2, b1, b2, args, st);
+    if (t.bn == 128) return launch_gemm_bits<128, MODE, 1, ONE>(bits, a1, a2, b1, b2, args, st);
+    return launch_gemm_bits<64, MODE, 1, ONE>(bits, a1, a2, b1, b2, args, st);
   }
   switch (t.bn) {
-    case 128: return launch_gemm_bits<128, MODE, 2>(bits, a1, a2, b1, b2, args, st);
-    case 192: return launch_gemm_bits<192, MODE, 2>(bits, a1, a2, b1, b2, args, st);
-    default: return launch_gemm_bits<256, MODE, 2>(bits, a1, a2, b1, b2, args, st);
+    case 128: return launch_gemm_bits<128, MODE, 2, ONE>(bits, a1, a2, b1, b2, args, st);
+    case 192: return launch_gemm_bits<192, MODE, 2, ONE>(bits, a1, a2, b1, b2, args, st);
+    default: return launch_gemm_bits<256, MODE, 2, ONE>(bits, a1, a2, b1, b2, args, st);
   }
 }
 
