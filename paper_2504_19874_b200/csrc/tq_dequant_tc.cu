@@ -284,7 +284,7 @@ dequant_kernel(const __grid_constant__ CUtensorMap tmP1, const __grid_constant__
         for (int c = c_begin; c < c_end && ok; ++c)
           for (int term = first_term; term <= last_term && ok; ++term)
             for (int kb = c * kChunk; kb < min((c + 1) * kChunk, a.num_kb); ++kb) {
-              if (!(ok = mbar_wait(&empty[stage], phase ^ 1u, abort_flag, a.status))) break;
+              if (!(ok = mbar_wait_suspended(&empty[stage], phase ^ 1u, abort_flag, a.status))) break;
               unsigned char* sb = smem + stage * C::kStageBytes + 2 * C::kABytes;
               const CUtensorMap* m1 = term == 0 ? &tmP1 : &tmS1;
               const CUtensorMap* m2 = term == 0 ? &tmP2 : &tmS2;
@@ -327,13 +327,13 @@ dequant_kernel(const __grid_constant__ CUtensorMap tmP1, const __grid_constant__
         for (int c = c_begin; c < c_end && ok; ++c)
           for (int term = first_term; term <= last_term && ok; ++term, ++it) {
             const uint32_t acc = it & 1u, acc_phase = (it >> 1) & 1u;
-            if (!(ok = mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, a.status))) break;
+            if (!(ok = mbar_wait_suspended(&tempty[acc], acc_phase ^ 1u, abort_flag, a.status))) break;
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + acc * BN;
             uint32_t accumulate = 0u;
             for (int kb = c * kChunk; kb < min((c + 1) * kChunk, a.num_kb); ++kb) {
-              if (!(ok = mbar_wait(&full_b[stage], phase, abort_flag, a.status))) break;
-              if (!(ok = mbar_wait(&full_a[stage], phase, abort_flag, a.status))) break;
+              if (!(ok = mbar_wait_suspended(&full_b[stage], phase, abort_flag, a.status))) break;
+              if (!(ok = mbar_wait_suspended(&full_a[stage], phase, abort_flag, a.status))) break;
               tc_fence_after();
               const uint32_t sa = smem_u32(smem + stage * C::kStageBytes);
               const uint64_t a1 = smem_desc_sw128(sa), a2 = smem_desc_sw128(sa + C::kABytes);
@@ -404,7 +404,7 @@ dequant_kernel(const __grid_constant__ CUtensorMap tmP1, const __grid_constant__
             else if (j + 1 < jobs) load_part(a, src_row, (c_begin + (j + 1) / nterms) * kChunk, part, first_term + (j + 1) % nterms, nxt);
             if (term == 0) unpack_indices(a, w, nib);
             else unpack_signs(a, w, nib);
-            if (!(ok = mbar_wait(&empty[stage], phase ^ 1u, abort_flag, a.status))) break;
+            if (!(ok = mbar_wait_suspended(&empty[stage], phase ^ 1u, abort_flag, a.status))) break;
             unsigned char* dst = smem + stage * C::kStageBytes + rt * 128;
             if (term == 0) expand_indices(a, nib, dst, C::kABytes, 2u * part, swz);
             else expand_signs(nib, dst, 2u * part, swz);
@@ -428,7 +428,7 @@ dequant_kernel(const __grid_constant__ CUtensorMap tmP1, const __grid_constant__
         const uint32_t acc = it & 1u, acc_phase = (it >> 1) & 1u;
         const int drained_term = first_term + (j - 1) % nterms;
         ++it;
-        if (!(ok = mbar_wait(&tfull[acc], acc_phase, abort_flag, a.status))) break;
+        if (!(ok = mbar_wait_suspended(&tfull[acc], acc_phase, abort_flag, a.status))) break;
         tc_fence_after();
         const float s = drained_term == 0 ? a.oscale : g;
         const uint32_t base = tmem_base + ((uint32_t)(lg * 32) << 16) + acc * BN + part * NC;

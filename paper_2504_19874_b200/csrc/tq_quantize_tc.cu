@@ -420,7 +420,7 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
       for (int64_t t = unit; t < num_tiles && ok; t += nunits) {
         const int m0 = ((int)(t / a.tiles_n) * CTAS + rank) * BM, n0 = (int)(t % a.tiles_n) * BN + rank * C::kBRows;
         for (int kb = 0; kb < num_kb; ++kb) {
-          if (!(ok = mbar_wait(&empty[stage], phase ^ 1u, abort_flag, a.status))) break;
+          if (!(ok = mbar_wait_suspended(&empty[stage], phase ^ 1u, abort_flag, a.status))) break;
           unsigned char* sa = smem + stage * stage_bytes;
           if (CTAS == 2) {
             // both CTAs' bytes are counted on the leader's barrier, which the leader arms for both
@@ -458,11 +458,11 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
       int64_t it = 0;
       for (int64_t t = unit; t < num_tiles && ok; t += nunits, ++it) {
         const uint32_t acc = (uint32_t)(it & 1), acc_phase = (uint32_t)((it >> 1) & 1);
-        if (!(ok = mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, a.status))) break;
+        if (!(ok = mbar_wait_suspended(&tempty[acc], acc_phase ^ 1u, abort_flag, a.status))) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * C::kAccCols;
         for (int kb = 0; kb < num_kb; ++kb) {
-          if (!(ok = mbar_wait(&full[stage], phase, abort_flag, a.status))) break;
+          if (!(ok = mbar_wait_suspended(&full[stage], phase, abort_flag, a.status))) break;
           tc_fence_after();
           const uint32_t sa = smem_u32(smem + stage * stage_bytes);
           const uint64_t a1 = smem_desc_sw128(sa), a2 = smem_desc_sw128(sa + BM * BK * 2);
@@ -532,7 +532,7 @@ quantize_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_cons
       const int tm = (int)(t / a.tiles_n), tn = (int)(t % a.tiles_n);
       const int64_t row = (int64_t)(tm * CTAS + rank) * BM + lg * 32 + lane;
       const int n0 = tn * BN;
-      if (!(ok = mbar_wait(&tfull[acc], acc_phase, abort_flag, a.status))) break;
+      if (!(ok = mbar_wait_suspended(&tfull[acc], acc_phase, abort_flag, a.status))) break;
       tc_fence_after();
       const bool row_ok = row < a.M;
       bool zero_row = false;

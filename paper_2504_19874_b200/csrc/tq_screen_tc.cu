@@ -454,7 +454,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
   // The stage of k-block kt was last read by the MMAs of k-block kt - STAGES.
   auto stage_free = [&](uint32_t kt) -> bool {
     const uint32_t kp = kt - STAGES;
-    return kt < STAGES || mbar_wait(&empty[kp % RING], (kp / RING) & 1u, abort_flag, a.status);
+    return kt < STAGES || mbar_wait_suspended(&empty[kp % RING], (kp / RING) & 1u, abort_flag, a.status);
   };
 
   if (warp < NEXP0) {
@@ -489,12 +489,12 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
         uint32_t it = 0, st = 0, at = 0, ph = 0;   // stage and barrier of the next k-block
         for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits, ++it) {
           const uint32_t d = it & 1u, d_tmem = tmem_base + d * 256u;
-          if (!(ok = mbar_wait(&dfree[d], ((it >> 1) & 1u) ^ 1u, abort_flag, a.status))) break;
+          if (!(ok = mbar_wait_suspended(&dfree[d], ((it >> 1) & 1u) ^ 1u, abort_flag, a.status))) break;
           for (int f = 0; f < nkb; ++f) {
             const uint64_t off = (uint64_t)(st * (STAGE >> 4));
             const uint64_t adesc = adesc0 + off, bdesc = bdesc0 + off;
             const int steps = NIB ? 4 : f == end0 ? last0 : f == end1 ? last1 : 4;
-            if (!(ok = mbar_wait(&full[at], ph, abort_flag, a.status))) break;
+            if (!(ok = mbar_wait_suspended(&full[at], ph, abort_flag, a.status))) break;
             tc_fence_after();
 #pragma unroll
             for (int s = 0; s < 4; ++s)
@@ -518,7 +518,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
         for (int64_t rnd = unit; rnd < nrounds && ok; rnd += nunits) {   // rows past the last one read zeros
           for (int gi = 0; gi < ngroups; ++gi) {
             const RowGroup rg = row_group<BM, NIB>(a.g, gi);
-            if (!(ok = mbar_wait(&pempty[pst], ph, abort_flag, a.status))) break;
+            if (!(ok = mbar_wait_suspended(&pempty[pst], ph, abort_flag, a.status))) break;
             mbar_arrive_expect_tx(&pfull[pst], (uint32_t)(TILE * rg.bytes));
             tma_load_2d(pring + pst * PTILE, rg.from_qjl ? &tmPs : &tmPa, &pfull[pst], rg.x, (int)((rnd * 2 + rank) * TILE));
             if (++pst == PSTAGES) {
@@ -567,7 +567,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
       for (int gi = 0; gi < ngroups && ok; ++gi) {
         const RowGroup rg = row_group<BM, NIB>(a.g, gi);
         const uint32_t gc = it * (uint32_t)ngroups + (uint32_t)gi, pst = gc % PSTAGES;
-        if (!(ok = mbar_wait(&pfull[pst], (gc / PSTAGES) & 1u, abort_flag, a.status))) break;
+        if (!(ok = mbar_wait_suspended(&pfull[pst], (gc / PSTAGES) & 1u, abort_flag, a.status))) break;
         const unsigned char* ps = pring + pst * PTILE;
         uint32_t w[16];
         if (rg.bytes == 64) {          // 64-byte swizzle: piece c at c ^ ((row >> 1) & 3)
@@ -691,7 +691,7 @@ screen_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ C
       nu_next = load(a.norms, tile + 2 * nunits, 1.f);
       g_next = load(gsrc, tile + 2 * nunits, 0.f);
       const uint32_t d = it & 1u;
-      if (!(ok = mbar_wait(&dfull[d], (it >> 1) & 1u, abort_flag, a.status))) break;
+      if (!(ok = mbar_wait_suspended(&dfull[d], (it >> 1) & 1u, abort_flag, a.status))) break;
       tc_fence_after();
       const uint32_t addr = tmem_base + ((uint32_t)(quad * 32) << 16) + d * 256u;
 #pragma unroll 1

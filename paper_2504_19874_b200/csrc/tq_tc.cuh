@@ -27,9 +27,22 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// The hint lets the hardware suspend the warp for up to 16 us before it says no.  Without one the waiting warps of a CTA poll so often
-// that they take issue slots and shared-memory cycles from the others (10^6 rows of d = 1536 quantised: 22.3 -> 21.2 ms).
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// The same with a hint that lets the hardware suspend the warp for up to 16 us before it says no.  The GEMM-shaped kernels wait so
+// (quantiser, reconstruction, screening: 100 rows of d = 384 mse b = 2 10.4 -> 10.0 us, 2,000 rows of d = 1536 prod b = 4 read back
+// 65.6 -> 63.6, 10^4 queries of d = 200 17.4 -> 17.1 ms); the exact scans, whose warps wait often and briefly, lose by it (64 queries, 500,000 rows: d = 1536 mse b = 2 307 -> 319 us, d = 3072 prod
+// b = 4 831 -> 859).
+__device__ __forceinline__ bool mbar_try_wait_suspended(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
@@ -58,13 +71,14 @@ constexpr long long kWaitLimitCycles = 4000000000LL;  // ~2-3 s of SM clock
 
 // Bounded wait.  `abort_flag` lives in shared memory; once any thread of the CTA gives up,
 // every other wait of that CTA returns false at its next check.
+template <bool SUSPEND = false>
 static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
                                                    long long limit_cycles = kWaitLimitCycles) {
   const long long t0 = clock64();
   uint32_t polls = 0;
   while (true) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((++polls & 63u) == 0u) {
+    if (SUSPEND ? mbar_try_wait_suspended(bar, parity) : mbar_try_wait(bar, parity)) return true;
+    if ((++polls & (SUSPEND ? 63u : 255u)) == 0u) {
       if (*abort_flag) return false;
       if (clock64() - t0 > limit_cycles) {
         *abort_flag = 1;
@@ -78,6 +92,10 @@ static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parit
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
   if (mbar_try_wait(bar, parity)) return true;
   return mbar_wait_slow(bar, parity, abort_flag, status);
+}
+__device__ __forceinline__ bool mbar_wait_suspended(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
+  if (mbar_try_wait_suspended(bar, parity)) return true;
+  return mbar_wait_slow<true>(bar, parity, abort_flag, status);
 }
 
 // ---------------------------------------------------------------- TMA
