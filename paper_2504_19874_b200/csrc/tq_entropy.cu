@@ -600,9 +600,11 @@ extern "C" int tq_entropy_unpack(const tq_plan* plan, const uint8_t* lengths, in
   entropy::Args a;
   if ((rc = entropy::make_code(plan, lengths, &a.code, who))) return rc;
   a.n = n; a.d = plan->d; a.idx = nullptr; a.idx_rb = plan->idx_row_bytes;
-  // An SM's share of the rows as one CTA (of at most 1,024) where it is worth the larger table, else CTAs of 128 rows.
+  // An SM's share of the rows as one CTA (of at most 1,024) where it is worth the larger table, else CTAs of 128 rows.  Packing and
+  // unpacking, CTAs of 128 rows / of the share: 37,000 rows (256 per SM) d = 128 b = 3 67.9 / 75.7 us, d = 1536 b = 2 140 / 148; 60,000 rows
+  // (416 per SM) 87.3 / 87.9 and 189 / 187; 100,000 rows d = 1536 b = 4 349 / 339.
   const int64_t share = round_up64((n + tc::sm_count() - 1) / tc::sm_count(), 32);
-  const bool wide = share >= 256;
+  const bool wide = share >= 384;
   const int threads = wide ? (int)((share + (share + 1023) / 1024 - 1) / ((share + 1023) / 1024) + 31) / 32 * 32 : 128;
   const int K = wide || a.code.maxlen > 10 ? 12 : 10;
   const size_t smem = sizeof(uint32_t) * ((size_t)1 << K) + sizeof(uint16_t) * ((size_t)1 << a.code.maxlen);   // at most 24 KB
