@@ -1254,6 +1254,30 @@ extern "C" int tq_topk(const tq_plan* plan, const void* Q, int q_dtype, int nq, 
   return TQ_OK;
 }
 
+#ifdef TQ_DEBUG
+// Hook for the tests of the debug build: the screening pass's lower bound of every pair's estimate into low [nq, n], and per query the
+// error constant and the scale (screen::QueryTerms) into terms [nq, 2].  Queries fp32, rows of d; nq <= 256.
+extern "C" int tq_debug_screen_bounds(const tq_plan* plan, const float* Q, int nq, int64_t n, const uint8_t* idx, const uint8_t* qjl,
+                                      const float* gamma, const float* norms, float* low, float* terms, void* workspace,
+                                      size_t workspace_bytes, void* stream) {
+  const char* who = "tq_debug_screen_bounds";
+  int rc = check_plan(plan, who);
+  if (rc) return rc;
+  TQ_REQUIRE(nq > 0 && nq <= screen::kQueries && n > 0 && plan->ms.ok && tscan::available(plan), TQ_ERR_INVALID_ARG, "%s: sizes", who);
+  const size_t qb = qcat_bytes(plan, nq);
+  TQ_REQUIRE(workspace != nullptr && aligned(workspace, 256) && workspace_bytes >= qb + screen::workspace_bytes(plan), TQ_ERR_WORKSPACE,
+             "%s: workspace", who);
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  float* Qcat = static_cast<float*>(workspace);
+  void* operand = static_cast<char*>(workspace) + qb;
+  TQ_CHECK_CUDA(prepare_queries(plan, Q, TQ_F32, nq, plan->d, Qcat, st), who);
+  if ((rc = screen::prepare(plan, Qcat, nq, operand, st, who))) return rc;
+  if ((rc = screen::run(plan, nq, n, idx, qjl, gamma, norms, low, n, nullptr, nullptr, nullptr, nullptr, 0, operand, st, who, 1))) return rc;
+  TQ_CHECK_CUDA(cudaMemcpyAsync(terms, screen::query_terms(plan, operand), (size_t)nq * sizeof(screen::QueryTerms), cudaMemcpyDeviceToDevice, st), who);
+  return TQ_OK;
+}
+#endif
+
 template <int BITS>
 static cudaError_t launch_wsum_partial(const tq_plan* plan, const attend::WsumArgs& a, dim3 grid, cudaStream_t st) {
   if (plan->mode == TQ_PROD) attend::wsum_partial_kernel<BITS, true><<<grid, 128, 0, st>>>(a);
